@@ -22,8 +22,6 @@
 // Every mbarrier wait is bounded (about a second): after the limit the kernel raises the error flag, all
 // roles leave their loops, TMEM is freed and the kernel returns.  No multicast loads anywhere (the only
 // multicast is tcgen05.commit arriving on both CTAs of a pair).
-#include <cuda.h>
-
 #include <cstdio>
 #include <cstdlib>
 #include <cmath>
@@ -32,90 +30,14 @@
 #include <mutex>
 #include <unordered_map>
 
-#include "internal.h"
+#include "gemm_common.cuh"
 
 namespace hbsjd {
 
 namespace {
 
 constexpr int BM = 128;
-constexpr int BK = 64;  // 64 bf16 = 128 bytes = one swizzle row
 constexpr int NUM_THREADS = 192;
-
-enum { EPI_STORE = 0, EPI_ADD = 1, EPI_SWIGLU = 2, EPI_QKV = 3, EPI_ADDNORM = 4 };
-
-struct GemmArgs {
-    float* C;        // STORE / ADD
-    bf16* out;       // SWIGLU: [M, N/2];  QKV: q [M, D]
-    int M, N, K;
-    int32_t* error_flag;
-    // RMSNorm folded around the GEMMs (bf16 model): the operand A is the bf16 copy of the UNNORMALISED residual
-    // stream and the norm's gain is folded into W, so that norm(x) W^T = r (x W'^T) with the row factor
-    // r = rsqrt(mean(x^2) + eps) applied here, in the epilogue, from partial sums of squares
-    const float* ssq_in;   // [M][ssq_n] partial sums of squares of A's rows (null: no row factor)
-    int ssq_n;             // partials per row = K / 32
-    float inv_dim, eps;
-    // ADDNORM: C (fp32 residual) += acc, plus what the next GEMM needs
-    bf16* hb;              // [M][N] bf16 copy of the updated residual
-    float* ssq_out;        // [M][N / 32] sums of squares of the updated residual per 32-column chunk
-    int w_constant;   // W never changes while the stream runs (model weights): its tiles may be fetched early
-    unsigned int acc_wait_ns;  // 0, or a shorter limit for the epilogue's accumulator wait (time-out test)
-    // QKV epilogue
-    State st;
-    int S, layer;
-    const float* rope_cs;  // [T][dh/2][2]
-    KvView kv;
-};
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-// Bounded wait (about one second unless a shorter limit is given).  Returns false when it gave up or another
-// role raised `abort`.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort,
-                                          unsigned long long limit_ns = 1000000000ull) {
-    if (mbar_try(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer_ns();
-    const int polls = limit_ns < 1000000ull ? 1 : 128;  // a short limit is checked after every poll
-    for (;;) {
-        for (int it = 0; it < polls; ++it)
-            if (mbar_try(bar, parity)) return true;
-        if (*abort) return false;
-        if (globaltimer_ns() - t0 > limit_ns) return false;
-    }
-}
-
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
 
 // CTA-pair variants (cta_group::2): the load may signal the mbarrier of the pair's leader.
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
@@ -209,11 +131,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32]) {
         : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-    __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<uint32_t*>(&v);
-}
-
 // PAIR: two CTAs of a cluster compute one 256 x BN tile with cta_group::2 MMAs; each CTA stages its own 128 rows
 // of A and its own BN/2 rows of W, which cuts the operand bytes per FLOP by a third against a 128 x BN tile.
 // WIDE: the epilogue stages a bf16 tile beside every fp32 tile (EPI_ADDNORM), 48 KB instead of 32 KB; the operand
@@ -238,13 +155,6 @@ struct Cfg {
     static constexpr int SMEM = STAGES * STAGE_BYTES + STAGING_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
     static_assert(16 * STAGES + 32 + 8 + 8 <= 256, "barrier area");
     static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
-};
-
-// Per-row context of the QKV epilogue: where the token row's q / k / v go.
-struct RowDst {
-    bool valid;
-    int s;        // sequence index (RoPE position)
-    size_t kvoff; // element offset of the row's K/V vector in the page pool
 };
 
 template <int BN, int EPI, bool PAIR>
@@ -466,14 +376,7 @@ __global__ void __launch_bounds__(NUM_THREADS) k_gemm_tcgen05(const __grid_const
             // row factor of the folded RMSNorm: the partial sums of squares of this row of A, added in a fixed order
             float rscale = 1.0f;
             if (EPI != EPI_ADD && EPI != EPI_ADDNORM && g.ssq_in != nullptr && row < M) {
-                const float2* pp = reinterpret_cast<const float2*>(g.ssq_in + (size_t)row * g.ssq_n);
-                float ss = 0.f;
-                for (int v = 0; v < g.ssq_n / 2; ++v) {
-                    const float2 t = pp[v];
-                    ss += t.x;
-                    ss += t.y;
-                }
-                rscale = 1.0f / sqrtf(ss * g.inv_dim + g.eps);
+                rscale = norm_row_factor(g, row);
             }
             // ADDNORM: the residual values this thread's row adds to, fetched three 32-column chunks ahead through a
             // ring of four register buffers (a chunk is 128 contiguous bytes of the row; the first three are
@@ -504,21 +407,7 @@ __global__ void __launch_bounds__(NUM_THREADS) k_gemm_tcgen05(const __grid_const
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-            RowDst rd;
-            rd.valid = row < M;
-            rd.s = 0;
-            rd.kvoff = 0;
-            if (EPI == EPI_QKV && rd.valid) {
-                const State& st = g.st;
-                const int i = row % st.W;
-                const int slot = (row / st.W) % g.S;
-                const int br = row / (st.W * g.S);
-                rd.valid = i < st.slot_n[slot];
-                if (rd.valid) {
-                    rd.s = st.slot_c[slot] + i;
-                    rd.kvoff = g.kv.offset(g.layer, br * st.Bmax + st.slot_img[slot], rd.s);
-                }
-            }
+            const RowDst rd = EPI == EPI_QKV ? qkv_row(g, row, row < M) : RowDst{row < M, 0, 0};
             // cos/sin of this row's sequence index, fetched once per tile (all loads in flight together):
             // rotation pairs 0..15 and 16..31 of a head (head sizes 64: both halves; 32: the first)
             float4 rope_lo[8], rope_hi[8];
@@ -656,14 +545,7 @@ __global__ void __launch_bounds__(NUM_THREADS) k_gemm_tcgen05(const __grid_const
                     // columns (2f, 2f+1) = (gate_f, up_f)
                     uint4* dst = reinterpret_cast<uint4*>(g.out + (size_t)row * (N / 2) + col / 2);
                     uint32_t o[8];
-#pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        const float g0 = __uint_as_float(r[4 * v]) * rscale, u0 = __uint_as_float(r[4 * v + 1]) * rscale;
-                        const float g1 = __uint_as_float(r[4 * v + 2]) * rscale, u1 = __uint_as_float(r[4 * v + 3]) * rscale;
-                        // silu(g) * u with ex2.approx and rcp.approx (about 1e-6 relative, far below bf16)
-                        o[v] = pack_bf16x2(__fdividef(g0, 1.0f + __expf(-g0)) * u0,
-                                           __fdividef(g1, 1.0f + __expf(-g1)) * u1);
-                    }
+                    swiglu_chunk(r, rscale, o);
                     dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
                     dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
                 } else {  // EPI_QKV
@@ -671,22 +553,10 @@ __global__ void __launch_bounds__(NUM_THREADS) k_gemm_tcgen05(const __grid_const
                     const int D = st.D;
                     const int sec = col / D, cs = col % D;  // 0 q, 1 k, 2 v; a tile never straddles sections
                     uint32_t o[16];
-                    if (sec < 2) {
-                        // the chunk's 16 rotation pairs: first or second half of the row's cos/sin table
-                        const bool hi = ((cs % st.dh) / 2) >= 16;
-#pragma unroll
-                        for (int v = 0; v < 8; ++v) {
-                            const float4 t = hi ? rope_hi[v] : rope_lo[v];  // cos, sin of pairs 2v and 2v+1
-                            const float a0 = __uint_as_float(r[4 * v]) * rscale, b0 = __uint_as_float(r[4 * v + 1]) * rscale;
-                            const float a1 = __uint_as_float(r[4 * v + 2]) * rscale, b1 = __uint_as_float(r[4 * v + 3]) * rscale;
-                            o[2 * v] = pack_bf16x2(a0 * t.x - b0 * t.y, a0 * t.y + b0 * t.x);
-                            o[2 * v + 1] = pack_bf16x2(a1 * t.z - b1 * t.w, a1 * t.w + b1 * t.z);
-                        }
-                    } else {
-#pragma unroll
-                        for (int v = 0; v < 16; ++v)
-                            o[v] = pack_bf16x2(__uint_as_float(r[2 * v]) * rscale, __uint_as_float(r[2 * v + 1]) * rscale);
-                    }
+                    if (sec < 2)  // the chunk's 16 rotation pairs: first or second half of the row's cos/sin table
+                        rope_chunk(r, rscale, ((cs % st.dh) / 2) >= 16 ? rope_hi : rope_lo, o);
+                    else
+                        plain_chunk(r, rscale, o);
                     bf16* base = sec == 0 ? g.out + (size_t)row * D + cs
                                           : (bf16*)(sec == 1 ? g.kv.k : g.kv.v) + rd.kvoff + cs;
                     uint4* dst = reinterpret_cast<uint4*>(base);
@@ -762,7 +632,7 @@ struct MapKeyHash {
         size_t h = std::hash<const void*>()(k.base);
         h = h * 1000003u ^ (size_t)k.rows;
         h = h * 1000003u ^ (size_t)k.inner;
-        h = h * 1000003u ^ (size_t)(k.box_rows * 4 + k.kind);
+        h = h * 1000003u ^ (size_t)(k.box_rows * 8 + k.kind);
         return h;
     }
 };
@@ -791,6 +661,20 @@ bool encode_map_ab(CUtensorMap* map, const void* base, int rows, int K, int box_
     const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 3D view of a bf16 row-major [rows, K] tensor: (64 columns, rows, k-blocks), box = 64 x box_rows x KB.
+template <int KB>
+bool encode_map_kb(CUtensorMap* map, const void* base, int rows, int K, int box_rows) {
+    EncodeFn enc = get_encode();
+    if (!enc) return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)BK, (cuuint64_t)rows, (cuuint64_t)(K / BK)};
+    const cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)BK * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, (cuuint32_t)KB};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -893,9 +777,20 @@ int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int ma
                  M, N, K);
         return -1;
     }
+    const int map_rows = m_cap >= M ? m_cap : M;
+    // few rows: the kernel without the tensor memory round trip (a shortened accumulator wait is the tcgen05 kernel's)
+    if (!force_bn && !g.acc_wait_ns) force_bn = skinny_tile_code(M, N, num_sms());
+    if (skinny_tile_exists(force_bn)) {
+        if (N % (force_bn % 1000) != 0) {
+            snprintf(err, errlen, "gemm: N=%d is not a multiple of the tile width %d", N, force_bn % 1000);
+            return -1;
+        }
+        return gemm_skinny_launch(epi, force_bn, A, W, g, map_rows, s, err, errlen);
+    }
     if (force_bn != 0 && force_bn != 32 && force_bn != 64 && force_bn != 128 && force_bn != 256 && force_bn != 512 &&
         force_bn != 640) {
-        snprintf(err, errlen, "gemm: tile %d is not one of 32, 64, 128, 256 (one CTA) or 512, 640 (CTA pair)", force_bn);
+        snprintf(err, errlen, "gemm: tile %d is not one of 32, 64, 128, 256 (one CTA), 512, 640 (CTA pair) or 16032, "
+                              "16064, 32032, 32064 (few rows)", force_bn);
         return -1;
     }
     const bool force_pair = force_bn >= 512;
@@ -914,7 +809,6 @@ int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int ma
     CUtensorMap ma, mw, mc, mh;
     memset(&mc, 0, sizeof(mc));
     memset(&mh, 0, sizeof(mh));
-    const int map_rows = m_cap >= M ? m_cap : M;
     if ((epi == EPI_STORE || epi == EPI_ADD || epi == EPI_ADDNORM) && !make_map_c(&mc, g.C, map_rows, N)) {
         snprintf(err, errlen, "gemm: cuTensorMapEncodeTiled failed for the output (M=%d N=%d)", M, N);
         return -3;
@@ -952,6 +846,11 @@ int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int ma
 // ones with the widest tile that still fits one wave.
 bool make_tensor_map_bf16(::CUtensorMap_st* map, const void* base, int rows, int cols, int box_rows) {
     return make_map(map, base, rows, cols, box_rows);
+}
+
+bool make_tensor_map_kblocks(CUtensorMap* map, const void* base, int rows, int K, int box_rows, int box_kb) {
+    if (box_kb == 2) return cached_map(map, MapKey{base, rows, K, box_rows, 3}, encode_map_kb<2>);
+    return box_kb == 4 && cached_map(map, MapKey{base, rows, K, box_rows, 4}, encode_map_kb<4>);
 }
 
 int gemm_tcgen05_tile_n(int M, int N, int K) {

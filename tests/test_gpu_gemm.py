@@ -98,3 +98,21 @@ def test_bounded_wait_runs_out_and_the_context_recovers(ctx_bf16):
     C3 = torch.zeros(M, N, device="cuda")
     ctx_bf16.hbsjd_debug_gemm(A, W, C3, reps=3)
     assert torch.equal(C3, C2)
+
+
+@pytest.mark.parametrize("tile", [16032, 16064, 32032, 32064])
+@pytest.mark.parametrize("M,N,K", [(1, 64, 64), (15, 128, 192), (17, 64, 320), (33, 192, 1088), (128, 1024, 2816),
+                                   (301, 576, 1024)])
+def test_few_row_kernel_gives_the_tcgen05_kernels_bits(ctx_bf16, tile, M, N, K):
+    """The kernel for few rows sums each element's products in the tcgen05 kernel's order: equal bits, whatever the
+    remainder of rows and of k-blocks per copy (1, 3, 5, 17, 44 and 16 k-blocks against copies of two or four)."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A = torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    W = (torch.randn(N, K, generator=g, device="cuda") * 0.05).bfloat16()
+    for acc in (False, True):
+        C0 = torch.randn(M, N, generator=g, device="cuda")
+        want, got = C0.clone(), C0.clone()
+        ctx_bf16.hbsjd_debug_gemm(A, W, want, accumulate=acc, tile=64)
+        ctx_bf16.hbsjd_debug_gemm(A, W, got, accumulate=acc, tile=tile)
+        assert torch.equal(got, want)
