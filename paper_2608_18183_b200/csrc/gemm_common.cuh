@@ -158,6 +158,14 @@ __device__ __forceinline__ void plain_chunk(const uint32_t r[32], float rscale, 
         o[v] = pack_bf16x2(__uint_as_float(r[2 * v]) * rscale, __uint_as_float(r[2 * v + 1]) * rscale);
 }
 
+// 32 bytes to a 32-byte aligned address: one whole sector per thread and instruction (two 16-byte stores leave every
+// sector half written until the second one arrives, and a warp's rows are too far apart to be merged otherwise).
+__device__ __forceinline__ void store_32b(void* dst, const uint32_t* o) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+                 "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
+                 : "memory");
+}
+
 // Row-major bf16 [rows, K] as (64 columns, rows, K / 64) with a box of 64 x box_rows x box_kb (2 or 4): one copy brings
 // box_kb consecutive k-blocks, each a 128-byte-swizzled tile of box_rows rows; zero fill past the last k-block.
 bool make_tensor_map_kblocks(CUtensorMap* map, const void* base, int rows, int K, int box_rows, int box_kb);

@@ -158,7 +158,7 @@ struct Cfg {
 };
 
 template <int BN, int EPI, bool PAIR>
-__global__ void __launch_bounds__(NUM_THREADS) k_gemm_tcgen05(const __grid_constant__ CUtensorMap map_a,
+__global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_constant__ CUtensorMap map_a,
                                                               const __grid_constant__ CUtensorMap map_w,
                                                               const __grid_constant__ CUtensorMap map_c,
                                                               const __grid_constant__ CUtensorMap map_hb,
@@ -398,16 +398,9 @@ __global__ void __launch_bounds__(NUM_THREADS) k_gemm_tcgen05(const __grid_const
                         }
                 }
             }
-            if (!mbar_wait(accf0 + 8 * buf, aph, abort_flag, g.acc_wait_ns ? g.acc_wait_ns : 1000000000ull)) {
-                if (lane == 0) {
-                    raise_abort<PAIR>(abort_flag, rank);
-                    atomicExch(g.error_flag, 3);
-                }
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-
             const RowDst rd = EPI == EPI_QKV ? qkv_row(g, row, row < M) : RowDst{row < M, 0, 0};
+            // Where the row goes and its cos / sin sit behind three dependent global loads: also requested before the
+            // accumulator is waited for (behind it they cost every tile about a microsecond).
             // cos/sin of this row's sequence index, fetched once per tile (all loads in flight together):
             // rotation pairs 0..15 and 16..31 of a head (head sizes 64: both halves; 32: the first)
             float4 rope_lo[8], rope_hi[8];
@@ -421,6 +414,15 @@ __global__ void __launch_bounds__(NUM_THREADS) k_gemm_tcgen05(const __grid_const
                     for (int v = 0; v < 8; ++v) rope_hi[v] = tab[8 + v];
                 }
             }
+            if (!mbar_wait(accf0 + 8 * buf, aph, abort_flag, g.acc_wait_ns ? g.acc_wait_ns : 1000000000ull)) {
+                if (lane == 0) {
+                    raise_abort<PAIR>(abort_flag, rank);
+                    atomicExch(g.error_flag, 3);
+                }
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+
 #pragma unroll 1
             for (int cg = 0; cg < BN; cg += 32 * UNR) {
               float ssq4[UNR];  // ADDNORM: sums of squares of this group's chunks
@@ -543,11 +545,9 @@ __global__ void __launch_bounds__(NUM_THREADS) k_gemm_tcgen05(const __grid_const
                 if (!rd.valid) continue;
                 if (EPI == EPI_SWIGLU) {
                     // columns (2f, 2f+1) = (gate_f, up_f)
-                    uint4* dst = reinterpret_cast<uint4*>(g.out + (size_t)row * (N / 2) + col / 2);
                     uint32_t o[8];
                     swiglu_chunk(r, rscale, o);
-                    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+                    store_32b(g.out + (size_t)row * (N / 2) + col / 2, o);
                 } else {  // EPI_QKV
                     const State& st = g.st;
                     const int D = st.D;
@@ -559,9 +559,8 @@ __global__ void __launch_bounds__(NUM_THREADS) k_gemm_tcgen05(const __grid_const
                         plain_chunk(r, rscale, o);
                     bf16* base = sec == 0 ? g.out + (size_t)row * D + cs
                                           : (bf16*)(sec == 1 ? g.kv.k : g.kv.v) + rd.kvoff + cs;
-                    uint4* dst = reinterpret_cast<uint4*>(base);
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) dst[v] = make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
+                    store_32b(base, o);
+                    store_32b(base + 16, o + 8);
                 }
               }
               if (EPI == EPI_ADDNORM && row < M) {  // the group's partial sums: 16 contiguous bytes per row
