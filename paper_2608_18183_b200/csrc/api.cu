@@ -155,11 +155,11 @@ int gemm(hbsjd_ctx* c, const void* A, const void* W, float* C, int M, int N, int
          int w_constant = 1, unsigned int acc_wait_ns = 0, int tile = 0);
 
 template <>
-int gemm<float>(hbsjd_ctx* c, const void* A, const void* W, float* C, int M, int N, int K, int accumulate, int, int,
-                unsigned int, int) {
+int gemm<float>(hbsjd_ctx* c, const void* A, const void* W, float* C, int M, int N, int K, int accumulate, int,
+                int w_constant, unsigned int, int) {
     const int ps = prof_begin(c, HBSJD_PROF_GEMM, 2.0 * M * N * K, M,
                               4.0 * ((double)M * K + (double)N * K) + 4.0 * M * N * (accumulate ? 2 : 1));
-    launch_gemm_simt<float>((const float*)A, (const float*)W, C, M, N, K, accumulate, c->stream);
+    launch_gemm_simt<float>((const float*)A, (const float*)W, C, M, N, K, accumulate, w_constant, c->stream);
     prof_end(c, ps);
     c->launches++;
     return 0;
@@ -1260,7 +1260,7 @@ int hbsjd_debug_gemm(hbsjd_ctx* c, const void* A, const void* W, float* C, int M
         } else {
             // W is the caller's buffer, possibly written by earlier work of the stream: no early fetch of its tiles
             rc = c->bf16_model ? gemm<bf16>(c, A, W, C, M, N, K, accumulate, 0, 0, acc_wait_ns, tile)
-                               : gemm<float>(c, A, W, C, M, N, K, accumulate);
+                               : gemm<float>(c, A, W, C, M, N, K, accumulate, 0, 0);
         }
         if (rc) return rc;
     }

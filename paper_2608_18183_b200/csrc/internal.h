@@ -68,8 +68,10 @@ template <typename TA>
 void launch_attention_ref(const State& st, int S, int layer, const TA* q, KvView kv, TA* out, cudaStream_t s);
 template <typename TA>
 void launch_swiglu(const float* gu, TA* act, int M, int F, cudaStream_t s);
+// w_constant: W is a model weight (never written while the stream runs): fetched before the preceding kernel has finished
 template <typename TA>
-void launch_gemm_simt(const TA* A, const TA* W, float* C, int M, int N, int K, int accumulate, cudaStream_t s);
+void launch_gemm_simt(const TA* A, const TA* W, float* C, int M, int N, int K, int accumulate, int w_constant,
+                      cudaStream_t s);
 
 // Scratch of the stand-alone verification step, carved from one allocation.
 struct VerifyScratch {

@@ -313,6 +313,7 @@ __global__ void k_attention_ref(State st, int S, int layer, const TA* __restrict
     for (int t = lane; t <= s; t += 32) {
         const TA* k = (const TA*)kv.k + kv.offset(layer, crow, t) + head * dh;
         float dot = 0.f;
+#pragma unroll 16
         for (int e = 0; e < dh; ++e) dot += qs[e] * to_f<TA>(k[e]);
         dot *= scale;
         sc[t] = dot;
@@ -328,10 +329,13 @@ __global__ void k_attention_ref(State st, int S, int layer, const TA* __restrict
     den = warp_sum(den);
     __syncwarp();
     for (int e = lane; e < dh; e += 32) {
+        // the values of one page at a time, sixteen loads in flight; the sum runs over t in order
         float acc = 0.f;
-        for (int t = 0; t <= s; ++t) {
-            const TA* v = (const TA*)kv.v + kv.offset(layer, crow, t) + head * dh;
-            acc += sc[t] * to_f<TA>(v[e]);
+        for (int t0 = 0; t0 <= s; t0 += kv.page) {
+            const TA* v = (const TA*)kv.v + kv.offset(layer, crow, t0) + head * dh + e;
+            const int cnt = min(kv.page, s + 1 - t0);
+#pragma unroll 16
+            for (int t = 0; t < cnt; ++t) acc += sc[t0 + t] * to_f<TA>(v[(size_t)t * st.D]);
         }
         o[e] = from_f<TA>(acc / den);
     }
@@ -367,7 +371,7 @@ void launch_swiglu(const float* gu, TA* act, int M, int F, cudaStream_t s) {
 template void launch_swiglu<float>(const float*, float*, int, int, cudaStream_t);
 template void launch_swiglu<bf16>(const float*, bf16*, int, int, cudaStream_t);
 
-// ------------------------------------------------------------------ CUDA-core GEMM (fp32 model; bf16 checker)
+// ------------------------------------------------------------------ CUDA-core GEMM (fp32 model)
 // C[M,N] (+)= A[M,K] . W[N,K]^T, fp32 accumulation in increasing k, 64x64 tile, 4x4 outputs per thread.
 template <typename TA>
 __global__ void __launch_bounds__(256) k_gemm_simt(const TA* __restrict__ A, const TA* __restrict__ W,
@@ -420,12 +424,109 @@ __global__ void __launch_bounds__(256) k_gemm_simt(const TA* __restrict__ A, con
     }
 }
 
+// The same product for problems too small to fill the chip with 64 x 64 tiles (the fp32 decoder's rows of a round):
+// bound by latency, not by arithmetic, so a CTA of 64 threads takes a 16 x 16 tile, has every operand panel of its
+// ring requested before it needs the first (W's before the preceding kernel has finished when W is a model weight)
+// and runs one chain of fused multiply-adds per output in increasing k -- the sum of the 64 x 64 kernel, bit for bit.
+// A rollout of four images of the two-layer fp32 model (32 rows, N 64..384, K 64 and 192) spent 11.8 us per launch in
+// the 64 x 64 kernel and took 10.4 ms; with this one 5.9 ms.
+constexpr int SS_T = 16, SS_K = 64, SS_PITCH = SS_K + 4, SS_STAGES = 4;
+
+__global__ void __launch_bounds__(64) k_gemm_simt_small(const float* __restrict__ A, const float* __restrict__ W,
+                                                        float* __restrict__ C, int M, int N, int K, int accumulate,
+                                                        int w_constant) {
+    pdl_trigger();
+    __shared__ __align__(16) float As[SS_STAGES][SS_T * SS_PITCH], Ws[SS_STAGES][SS_T * SS_PITCH];
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int m0 = blockIdx.y * SS_T, n0 = blockIdx.x * SS_T;
+    const int panels = (K + SS_K - 1) / SS_K;
+    // 16 bytes per thread and step; rows past the edge and columns past K read as zero (size 0: nothing is fetched)
+    auto fetch = [&](const float* __restrict__ src, int rows, int r0, float* dst, int p) {
+        for (int idx = tid; idx < SS_T * SS_K / 4; idx += 64) {
+            const int r = idx / (SS_K / 4), k = p * SS_K + idx % (SS_K / 4) * 4;
+            const int row = r0 + r;
+            const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + r * SS_PITCH + idx % (SS_K / 4) * 4);
+            const bool in = row < rows && k < K;
+            const float* from = in ? src + (size_t)row * K + k : src;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(from), "r"(in ? 16 : 0)
+                         : "memory");
+        }
+    };
+    if (w_constant)
+        for (int p = 0; p < SS_STAGES && p < panels; ++p) fetch(W, N, n0, Ws[p], p);
+    pdl_wait();
+    for (int p = 0; p < SS_STAGES; ++p) {  // one group per panel, empty ones included, so that the counts below fit
+        if (p < panels) {
+            if (!w_constant) fetch(W, N, n0, Ws[p], p);
+            fetch(A, M, m0, As[p], p);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, old[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+    if (accumulate) {
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const int gm = m0 + ty + 8 * x, gn = n0 + tx + 8 * y;
+                if (gm < M && gn < N) old[x][y] = C[(size_t)gm * N + gn];
+            }
+    }
+    for (int p = 0; p < panels; ++p) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(SS_STAGES - 1) : "memory");
+        __syncthreads();
+        const float* a = As[p % SS_STAGES] + ty * SS_PITCH;
+        const float* w = Ws[p % SS_STAGES] + tx * SS_PITCH;
+#pragma unroll
+        for (int k = 0; k < SS_K; k += 4) {
+            float4 av[2], wv[2];
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                av[x] = *reinterpret_cast<const float4*>(a + 8 * x * SS_PITCH + k);
+                wv[x] = *reinterpret_cast<const float4*>(w + 8 * x * SS_PITCH + k);
+            }
+#pragma unroll
+            for (int x = 0; x < 2; ++x)
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    acc[x][y] = fmaf(av[x].x, wv[y].x, acc[x][y]);
+                    acc[x][y] = fmaf(av[x].y, wv[y].y, acc[x][y]);
+                    acc[x][y] = fmaf(av[x].z, wv[y].z, acc[x][y]);
+                    acc[x][y] = fmaf(av[x].w, wv[y].w, acc[x][y]);
+                }
+        }
+        __syncthreads();
+        if (p + SS_STAGES < panels) {
+            fetch(W, N, n0, Ws[p % SS_STAGES], p + SS_STAGES);
+            fetch(A, M, m0, As[p % SS_STAGES], p + SS_STAGES);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            const int gm = m0 + ty + 8 * x, gn = n0 + tx + 8 * y;
+            if (gm < M && gn < N) C[(size_t)gm * N + gn] = accumulate ? old[x][y] + acc[x][y] : acc[x][y];
+        }
+}
+
 template <typename TA>
-void launch_gemm_simt(const TA* A, const TA* W, float* C, int M, int N, int K, int accumulate, cudaStream_t s) {
+void launch_gemm_simt(const TA* A, const TA* W, float* C, int M, int N, int K, int accumulate, int w_constant,
+                      cudaStream_t s) {
+    if constexpr (sizeof(TA) == 4) {
+        // up to four 16 x 16 tiles per SM (they are resident together); beyond that the 64 x 64 kernel has at least 37
+        // tiles and reads every operand four times less often
+        const long tiles = (long)((M + SS_T - 1) / SS_T) * ((N + SS_T - 1) / SS_T);
+        if (K % 4 == 0 && (((uintptr_t)A | (uintptr_t)W) & 15) == 0 && tiles <= 4L * device_sm_count()) {
+            launch_k(k_gemm_simt_small, dim3((N + SS_T - 1) / SS_T, (M + SS_T - 1) / SS_T), dim3(64), 0, s, A, W, C, M,
+                     N, K, accumulate, w_constant);
+            return;
+        }
+    }
     dim3 grid((N + 63) / 64, (M + 63) / 64);
     launch_k(k_gemm_simt<TA>, dim3(grid), dim3(256), 0, s, A, W, C, M, N, K, accumulate);
 }
-template void launch_gemm_simt<float>(const float*, const float*, float*, int, int, int, int, cudaStream_t);
-template void launch_gemm_simt<bf16>(const bf16*, const bf16*, float*, int, int, int, int, cudaStream_t);
+template void launch_gemm_simt<float>(const float*, const float*, float*, int, int, int, int, int, cudaStream_t);
 
 }  // namespace hbsjd

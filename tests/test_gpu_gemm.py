@@ -116,3 +116,24 @@ def test_few_row_kernel_gives_the_tcgen05_kernels_bits(ctx_bf16, tile, M, N, K):
         ctx_bf16.hbsjd_debug_gemm(A, W, want, accumulate=acc, tile=64)
         ctx_bf16.hbsjd_debug_gemm(A, W, got, accumulate=acc, tile=tile)
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 16, 4), (17, 33, 68), (32, 192, 64), (31, 64, 260), (32, 64, 1028), (5, 40, 7),
+                                   (304, 496, 64), (320, 496, 64)])
+def test_fp32_gemm_small_tiles(ctx_fp32, M, N, K):
+    """The 16 x 16 tiles of small fp32 problems: edges of tiles and K panels, more panels than the ring holds, K not a
+    multiple of four (the 64 x 64 kernel), and both sides of the largest problem that takes them (19 x 31 tiles = 589,
+    20 x 31 = 620 of 4 x 148 = 592).  Bound: K fused multiply-adds, each within half an ulp of the running sum."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A = torch.randn(M, K, generator=g, device="cuda")
+    W = torch.randn(N, K, generator=g, device="cuda") * 0.1
+    C0 = torch.randn(M, N, generator=g, device="cuda")
+    ref = A.double() @ W.double().T
+    tol = 2.0 ** -24 * (K + 2) * (A.double().abs() @ W.double().abs().T + C0.abs())
+    C = torch.zeros(M, N, device="cuda")
+    ctx_fp32.hbsjd_gemm(A, W, C)
+    assert bool(((C.double() - ref).abs() <= tol).all())
+    C = C0.clone()
+    ctx_fp32.hbsjd_gemm(A, W, C, accumulate=True)
+    assert bool(((C.double() - C0.double() - ref).abs() <= tol).all())
