@@ -1,5 +1,6 @@
 // C ABI of the rollout library (see include/hbsjd.h): context, host-side round loop, debug helpers.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -51,6 +52,11 @@ struct hbsjd_ctx {
     float* ssq;             // [rows][dim / 32] partial sums of squares of the residual rows (bf16 model)
     // host side
     int32_t* h_counters;  // pinned [8]
+    RoundPost* post;      // mapped host memory [2], by round parity: the counters of the last rounds
+    RoundPost* post_dev;  // the same, as the GPU addresses it
+    int32_t* tally;       // [2] device, see AcceptArgs
+    uint32_t post_seq;    // stamp of the last round enqueued
+    int min_left;         // fewest tokens left of a live image, after the last collected round
     cudaEvent_t ev0, ev1, ev2;
     hbsjd_params P;
     bool have_rollout;
@@ -345,6 +351,22 @@ int choose_compact(const hbsjd_ctx* c, int live) {
     return live > c->P.gamma ? 0 : 1;  // Eq. 6
 }
 
+// Error counter of the device (as read into h_counters) -> return code; clears it.
+int check_error(hbsjd_ctx* c) {
+    if (c->h_counters[CNT_ERROR] == 0) return 0;
+    const int code = c->h_counters[CNT_ERROR];
+    cudaStreamSynchronize(c->stream);  // nothing of a later round may still run
+    cudaMemsetAsync(c->st.counters + CNT_ERROR, 0, sizeof(int32_t), c->stream);
+    if (code >= 16) {  // a kernel met rollout state that cannot be valid; it skipped the access
+        snprintf(c->err, sizeof(c->err), "invalid rollout state on the device (code %d: %s)", code,
+                 code == 16 ? "cursor out of range" : code == 17 ? "draft token out of range"
+                                                                 : "proposal row out of range");
+        return HBSJD_EINVAL;
+    }
+    snprintf(c->err, sizeof(c->err), "a bounded device-side wait gave up (code %d)", code);
+    return HBSJD_ETIMEOUT;
+}
+
 int sync_counters(hbsjd_ctx* c) {
     CK(cudaMemcpyAsync(c->h_counters, c->st.counters, 8 * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -356,23 +378,11 @@ int sync_counters(hbsjd_ctx* c) {
         const double keys = c->h_counters[CNT_SUM_KEYS], n = c->h_counters[CNT_SUM_N];
         prof_resolve(c, nb * (keys * 2.0 * D * es + n * 2.0 * D * es), n * (nb + 1.0) * V * 4.0);
     }
-    if (c->h_counters[CNT_ERROR] != 0) {
-        const int code = c->h_counters[CNT_ERROR];
-        cudaMemsetAsync(c->st.counters + CNT_ERROR, 0, sizeof(int32_t), c->stream);
-        if (code >= 16) {  // a kernel met rollout state that cannot be valid; it skipped the access
-            snprintf(c->err, sizeof(c->err), "invalid rollout state on the device (code %d: %s)", code,
-                     code == 16 ? "cursor out of range" : code == 17 ? "draft token out of range"
-                                                                     : "proposal row out of range");
-            return HBSJD_EINVAL;
-        }
-        snprintf(c->err, sizeof(c->err), "a bounded device-side wait gave up (code %d)", code);
-        return HBSJD_ETIMEOUT;
-    }
-    return 0;
+    return check_error(c);
 }
 
-int run_round(hbsjd_ctx* c) {
-    if (c->live == 0) return 0;
+// Enqueues one round for c->live images, which must be the live count that the round will find.
+int enqueue_round(hbsjd_ctx* c) {
     const int compact = choose_compact(c, c->live);
     const int S = compact ? c->live : c->st.B;
     launch_setup(c->st, 0, compact, c->stream);
@@ -395,6 +405,9 @@ int run_round(hbsjd_ctx* c) {
     a.seed_hi = (uint32_t)(c->P.seed >> 32);
     a.round = (uint32_t)c->round;
     a.m_sync = c->P.exec_mode == HBSJD_EXEC_SYNC ? c->m_sync : nullptr;
+    a.post_stamp = ++c->post_seq;
+    a.post = c->post_dev + (a.post_stamp & 1u);
+    a.tally = c->tally;
     {
         const int ps = prof_begin(c, HBSJD_PROF_ACCEPT, 0.0);
         launch_prob_accept(c->st, a, c->stream);
@@ -407,8 +420,35 @@ int run_round(hbsjd_ctx* c) {
     }
     c->launches += 2;
     CK(cudaGetLastError());
-    rc = sync_counters(c);
-    if (rc) return rc;
+    c->last_S = S;
+    c->last_compact = compact;
+    c->round += 1;
+    c->parity ^= 1;
+    return 0;
+}
+
+// Waits for the round with this stamp and takes over its counters.  sync: by a stream synchronisation (the round is
+// the last one enqueued), else by polling what the round posts.
+int collect_round(hbsjd_ctx* c, uint32_t stamp, bool sync) {
+    const volatile RoundPost* p = c->post + (stamp & 1u);
+    int rc;
+    if (sync) {
+        if ((rc = sync_counters(c))) return rc;
+    } else {
+        // the stream is asked now and then: after a CUDA error nothing will be posted
+        for (unsigned spins = 1; p->stamp != stamp; ++spins)
+            if (spins % (1u << 20) == 0) {
+                const cudaError_t e = cudaStreamQuery(c->stream);
+                if (e != cudaErrorNotReady && p->stamp != stamp) {
+                    CK(e);
+                    snprintf(c->err, sizeof(c->err), "a round ended without its counters");
+                    return HBSJD_ECUDA;
+                }
+            }
+        std::atomic_thread_fence(std::memory_order_acquire);
+        for (int x = 0; x < 8; ++x) c->h_counters[x] = p->counters[x];
+        if ((rc = check_error(c))) return rc;
+    }
     if (c->h_counters[CNT_LIVE_SETUP] != c->live) {
         snprintf(c->err, sizeof(c->err), "live count mismatch: host %d device %d", c->live,
                  c->h_counters[CNT_LIVE_SETUP]);
@@ -416,16 +456,35 @@ int run_round(hbsjd_ctx* c) {
     }
     c->stats.rounds += 1;
     c->stats.image_forwards += c->live;
-    if (compact) c->stats.compact_rounds += 1;
+    if (choose_compact(c, c->live)) c->stats.compact_rounds += 1;
     else c->stats.full_rounds += 1;
     c->stats.committed = c->h_counters[CNT_COMMITTED];
     c->stats.rejects = c->h_counters[CNT_REJECTS];
     c->live = c->h_counters[CNT_LIVE];
-    c->last_S = S;
-    c->last_compact = compact;
-    c->round += 1;
-    c->parity ^= 1;
+    c->min_left = p->min_left;
     return 0;
+}
+
+// Rounds until every image is complete (max_rounds < 0) or that many are done.  The live count decides the next
+// round's shape, so a round is normally enqueued once the one before has been collected; but an image commits at most
+// `window` tokens per round, so while every live image has more than that left the round in flight cannot change the
+// count, and the next one is enqueued behind it (the GPU then never waits for the host between rounds).
+int run_rounds(hbsjd_ctx* c, int max_rounds) {
+    int enqueued = 0, in_flight = 0, rc;
+    while (true) {
+        const bool more = max_rounds < 0 || enqueued < max_rounds;
+        // (event times of a round are folded at its synchronisation: no running ahead while they are taken)
+        if (more && c->live > 0 && (in_flight == 0 || (in_flight == 1 && c->min_left > c->st.W && !c->profiling))) {
+            if ((rc = enqueue_round(c))) return rc;
+            ++enqueued;
+            ++in_flight;
+        } else if (in_flight > 0) {
+            if ((rc = collect_round(c, c->post_seq - (uint32_t)in_flight + 1u, c->profiling))) return rc;
+            --in_flight;
+        } else {
+            return 0;
+        }
+    }
 }
 
 void free_all(hbsjd_ctx* c) {
@@ -434,10 +493,11 @@ void free_all(hbsjd_ctx* c) {
                     c->st.counters, c->st.m_last, c->st.j_last, c->pbuf[0], c->pbuf[1], c->flag, c->cand_rep,
                     c->cand_ref, c->h, c->qkv, c->gu, c->logits, c->a, c->q, c->o, c->act, c->ssq,
                     c->stage_tok, c->stage_len, c->stage_lab, c->stage_out, c->verify_scratch,
-                    c->score_pos, c->score_img, c->score_loss, c->m_sync};
+                    c->score_pos, c->score_img, c->score_loss, c->m_sync, c->tally};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c->h_counters) cudaFreeHost(c->h_counters);
+    if (c->post) cudaFreeHost(c->post);
     for (auto& s : c->pool) {
         if (s.a) cudaEventDestroy(s.a);
         if (s.b) cudaEventDestroy(s.b);
@@ -624,6 +684,14 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
         CK(cudaEventCreate(&s.b));
     }
     CK(cudaMallocHost((void**)&c->h_counters, 8 * sizeof(int32_t)));
+    CK(cudaHostAlloc((void**)&c->post, 2 * sizeof(RoundPost), cudaHostAllocMapped));
+    memset(c->post, 0, 2 * sizeof(RoundPost));
+    CK(cudaHostGetDevicePointer((void**)&c->post_dev, c->post, 0));
+    if ((rc = dev_alloc(c, &c->tally, (size_t)2))) return rc;
+    {
+        const int32_t none = 0x7fffffff;
+        CK(cudaMemcpyAsync(c->tally + 1, &none, sizeof(none), cudaMemcpyHostToDevice, c->stream));
+    }
     CK(cudaEventCreate(&c->ev0));
     CK(cudaEventCreate(&c->ev1));
     CK(cudaEventCreate(&c->ev2));
@@ -723,7 +791,7 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
     CK(cudaMemcpyAsync(ht.data(), prefix_tokens, (size_t)batch * T * sizeof(int32_t), cudaMemcpyDeviceToHost,
                        c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    int kmax = 0, live = 0;
+    int live = 0, min_left = T;
     for (int b = 0; b < batch; ++b) {
         if (hk[b] < 0 || hk[b] > T || hl[b] < 0 || hl[b] > c->d.n_classes) {
             snprintf(c->err, sizeof(c->err), "image %d: prefix_len %d or label %d out of range", b, hk[b], hl[b]);
@@ -734,8 +802,10 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
                 snprintf(c->err, sizeof(c->err), "image %d: prefix token %d out of range", b, t);
                 return HBSJD_EINVAL;
             }
-        kmax = hk[b] > kmax ? hk[b] : kmax;
-        live += hk[b] < T;
+        if (hk[b] < T) {
+            ++live;
+            min_left = std::min(min_left, T - hk[b]);
+        }
     }
     c->P = *p;
     State& st = c->st;
@@ -758,6 +828,7 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
     c->round = 0;
     c->parity = 0;
     c->live = live;
+    c->min_left = min_left;
     c->have_rollout = false;
 
     CK(cudaEventRecord(c->ev0, c->stream));
@@ -791,11 +862,9 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
     CK(cudaGetLastError());
     c->have_rollout = true;
 
-    int rounds = 0;
-    while (c->live > 0 && (p->max_rounds < 0 || rounds < p->max_rounds)) {
-        const int rc = run_round(c);
+    {
+        const int rc = run_rounds(c, p->max_rounds);
         if (rc) return rc;
-        ++rounds;
     }
     launch_export_tokens(st, out_tokens, c->stream);
     c->launches++;
@@ -1084,8 +1153,10 @@ int hbsjd_round(hbsjd_ctx* c, int* live_out) {
         snprintf(c->err, sizeof(c->err), "hbsjd_round needs a preceding hbsjd_rollout");
         return HBSJD_ESTATE;
     }
-    const int rc = run_round(c);
-    if (rc) return rc;
+    if (c->live > 0) {
+        int rc = enqueue_round(c);
+        if (rc || (rc = collect_round(c, c->post_seq, true))) return rc;
+    }
     if (live_out) *live_out = c->live;
     return HBSJD_OK;
 }

@@ -38,6 +38,14 @@ struct State {
 enum { CNT_LIVE = 0, CNT_COMMITTED = 1, CNT_REJECTS = 2, CNT_LIVE_SETUP = 3, CNT_SLOTS = 4, CNT_ERROR = 5,
        CNT_SUM_KEYS = 6 /* sum over active slots of c+n */, CNT_SUM_N = 7 /* sum of n */ };
 
+// What the host needs to know of a finished round, written by the GPU into mapped host memory; stamp last.
+struct RoundPost {
+    int32_t counters[8];
+    int32_t min_left;  // fewest tokens still to commit over the images that are live after the round
+    uint32_t stamp;
+    int32_t pad[6];
+};
+
 struct AcceptArgs {
     const float* logits;  // [nb][S][W][V]
     float* pcur;          // [Bmax][Wmax][V] this round's probabilities (next round's proposals)
@@ -50,6 +58,10 @@ struct AcceptArgs {
     int top_k, greedy;
     uint32_t seed_lo, seed_hi, round;
     const int32_t* m_sync;  // batch-synchronous progress: the smallest commit of the batch (null: independent)
+    // k_commit's last CTA posts the round's counters to the host (null: not wanted)
+    RoundPost* post;         // mapped host memory
+    int32_t* tally;          // [2] device: CTAs done, fewest tokens left of a live image; left at {0, INT_MAX}
+    uint32_t post_stamp;
 };
 
 // ---- row operations (model_kernels.cu)

@@ -656,6 +656,24 @@ void launch_prob_accept(const State& st, const AcceptArgs& a, cudaStream_t s) {
 // of (image, position, round); the probabilities are read back from this round's p rows.  Thread 0 then
 // commits, advances the cursor -- the KV commit is this cursor move: entries at and after the new cursor are
 // recomputed by the next forward (Sec. 4.2 "Independent progress") -- and rebuilds the window.
+// One thread of every CTA of k_commit, when the CTA's slot is done (left: tokens the slot's image still has to commit,
+// INT_MAX if it has none or no image).  The last one hands the round's counters to the host, which polls the stamp in
+// its own memory, in place of a copy and a stream synchronisation.
+__device__ __forceinline__ void post_round(const State& st, const AcceptArgs& a, int left) {
+    if (a.post == nullptr) return;
+    if (left != 0x7fffffff) atomicMin(&a.tally[1], left);
+    __threadfence();
+    if (atomicAdd(&a.tally[0], 1) != (int)gridDim.x - 1) return;
+    __threadfence();
+    volatile RoundPost* p = a.post;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) p->counters[x] = atomicAdd(&st.counters[x], 0);
+    p->min_left = atomicExch(&a.tally[1], 0x7fffffff);
+    a.tally[0] = 0;
+    __threadfence_system();
+    p->stamp = a.post_stamp;
+}
+
 __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) {
     pdl_trigger();
     pdl_wait();
@@ -665,7 +683,10 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int slot = blockIdx.x;
     const int n = st.slot_n[slot];
-    if (n == 0) return;
+    if (n == 0) {
+        if (tid == 0) post_round(st, a, 0x7fffffff);
+        return;
+    }
     const int V = st.V;
     const int img = st.slot_img[slot], c = st.slot_c[slot];
     int32_t* seq = st.seq + (size_t)img * (st.T + 1);
@@ -791,6 +812,7 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
     }
     atomicAdd(&st.counters[CNT_COMMITTED], m);
     if (j >= 0) atomicAdd(&st.counters[CNT_REJECTS], 1);
+    post_round(st, a, c2 < st.T ? st.T - c2 : 0x7fffffff);
 }
 
 // One CTA: every thread walks the accept flags of its slots; block-wide minimum of the commits.
@@ -892,6 +914,9 @@ cudaError_t verify_enqueue(const VerifyDesc& d, const VerifyScratch& sc, const f
     a.seed_hi = (uint32_t)(d.seed >> 32);
     a.round = d.round;
     a.m_sync = nullptr;
+    a.post = nullptr;
+    a.tally = nullptr;
+    a.post_stamp = 0;
     // the commit counters accumulate with atomics: they must start at zero on every call
     cudaError_t e = cudaMemsetAsync(sc.counters, 0, 8 * sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
