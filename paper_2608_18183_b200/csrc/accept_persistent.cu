@@ -144,7 +144,9 @@ __device__ __forceinline__ unsigned int radix_select_regs(const float (&x)[NCH][
     return sh.sel_bin;
 }
 
-template <bool CFG>
+// PROBS: the probability pipeline alone (hbsjd_probs): item = row of a.logits (and a.logits_u), probabilities to a.pcur;
+// st has V, W = 1 and a place for the error code.
+template <bool CFG, bool PROBS>
 __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArgs a) {
     pdl_trigger();
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
     int* s_n = (int*)(smem_raw + (size_t)(CFG ? 2 : 1) * V * sizeof(float) + sizeof(PShared));
     int* s_img = s_n + a.S;
     int* s_c = s_img + a.S;
-    for (int sidx = tid; sidx < a.S; sidx += PT) {
+    for (int sidx = tid; !PROBS && sidx < a.S; sidx += PT) {
         s_n[sidx] = st.slot_n[sidx];
         s_img[sidx] = st.slot_img[sidx];
         s_c[sidx] = st.slot_c[sidx];
@@ -174,14 +176,14 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
     __syncthreads();
 
     const int total = a.S * W;
-    auto valid = [&](int it) { return (it % W) < s_n[it / W]; };
+    auto valid = [&](int it) { return PROBS || (it % W) < s_n[it / W]; };
     auto issue = [&](int it) {  // thread 0: both rows of item `it` into the staging area
         const int slot = it / W, i = it % W;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
                      "r"(CFG ? 2u * row_bytes : row_bytes)
                      : "memory");
         bulk_load(smem_addr(stage_c), a.logits + ((size_t)slot * W + i) * V, row_bytes, bar);
-        if (CFG) bulk_load(smem_addr(stage_u), a.logits + ((size_t)(a.S + slot) * W + i) * V, row_bytes, bar);
+        if (CFG) bulk_load(smem_addr(stage_u), a.logits_u + ((size_t)slot * W + i) * V, row_bytes, bar);
     };
     // The state an item needs besides its logits -- the draft token under test, whether its proposal is a point
     // mass, the proposal row and the proposal's entry q(z) -- sits behind three levels of dependent global loads.
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
     const bool select = a.top_k > 0 && a.top_k < V;
     Raw raw = {0, 0, 0};
     float qz = 1.0f;
-    if (it < total) {
+    if (!PROBS && it < total) {
         raw = fetch_raw(it);
         qz = fetch_qz(it, raw);
     }
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
         philox4x32_10((uint32_t)s_img[slot], (uint32_t)(s_c[slot] + i + 1), a.round, 0u, a.seed_lo, a.seed_hi, dst);
     };
     uint32_t par = 0;  // item parity
-    if (it < total && tid == PT - 32) make_words(it, sh.words[0]);
+    if (!PROBS && it < total && tid == PT - 32) make_words(it, sh.words[0]);
     sh.hist[tid] = 0u;  // SEL_BINS == PT
     // threshold guess carried from the previous item of this CTA: lower end and bin scale of the selection histogram
     float g_lo = 0.f, g_scale = 0.f;
@@ -243,12 +245,10 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
         int nxt = it + gridDim.x;
         while (nxt < total && !valid(nxt)) nxt += gridDim.x;
         Raw raw_next = {0, 0, 0};
-        if (nxt < total) raw_next = fetch_raw(nxt);  // consumed after barrier (1)
+        if (!PROBS && nxt < total) raw_next = fetch_raw(nxt);  // consumed after barrier (1)
         const int slot = it / W, i = it % W;
-        const int n = s_n[slot], img = s_img[slot], c = s_c[slot];
-        const int t = c + i + 1;  // token position this distribution decides
-        const bool last = (i == n - 1);
-        const size_t oidx = (size_t)img * st.Wmax + i;
+        const bool last = PROBS || i == s_n[slot] - 1;
+        const size_t oidx = PROBS ? (size_t)it : (size_t)s_img[slot] * st.Wmax + i;
         float* pout = a.pcur + oidx * V;
 
         int z = -1;
@@ -340,9 +340,9 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
             break;  // a copy never arrived; nothing else is in flight (the next item's copies are issued below)
         }
         if (tid == 0 && nxt < total) issue(nxt);  // the next item's rows stream in behind the rest of this one
-        if (tid == PT - 32 && nxt < total) make_words(nxt, sh.words[par ^ 1u]);
+        if (!PROBS && tid == PT - 32 && nxt < total) make_words(nxt, sh.words[par ^ 1u]);
         float qz_next = 1.0f;
-        if (nxt < total) qz_next = fetch_qz(nxt, raw_next);
+        if (!PROBS && nxt < total) qz_next = fetch_qz(nxt, raw_next);
         mn = key_float(__reduce_min_sync(0xffffffffu, sh.redk[0][lane]));
         mx = key_float(__reduce_max_sync(0xffffffffu, sh.redk[1][lane]));
 
@@ -499,11 +499,13 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
             const int v = ch * CHUNK + tid * 4;
 #pragma unroll
             for (int e = 0; e < 4; ++e) x[ch][e] *= inv;
-            wc[ch] = fixed_weight(x[ch][0]) + fixed_weight(x[ch][1]) + fixed_weight(x[ch][2]) + fixed_weight(x[ch][3]);
+            if (!PROBS) wc[ch] = fixed_weight(x[ch][0]) + fixed_weight(x[ch][1]) + fixed_weight(x[ch][2]) + fixed_weight(x[ch][3]);
             if (v < V) *reinterpret_cast<float4*>(pout + v) = make_float4(x[ch][0], x[ch][1], x[ch][2], x[ch][3]);
         }
 
-        if (a.greedy) {
+        if (PROBS) {
+            // the probabilities are all that is wanted
+        } else if (a.greedy) {
             // argmax, lowest index on ties: the largest probability bits, then the lowest index that holds them
             unsigned int bb = 0u;
 #pragma unroll
@@ -619,19 +621,37 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
 
 bool accept_persistent_supported(const State& st) { return st.V <= NCH * CHUNK && st.V % 4 == 0; }
 
-void launch_accept_persistent(const State& st, const AcceptArgs& a, int n_sms, cudaStream_t s) {
-    const int nb = st.nb;
-    const int bytes = nb * st.V * (int)sizeof(float) + (int)sizeof(PShared) + 3 * a.S * (int)sizeof(int);
+template <bool CFG, bool PROBS>
+static void launch(const State& st, const AcceptArgs& a, int n_sms, cudaStream_t s) {
+    static int configured[64] = {0};
+    const int bytes = (CFG ? 2 : 1) * st.V * (int)sizeof(float) + (int)sizeof(PShared) +
+                      (PROBS ? 0 : 3 * a.S * (int)sizeof(int));
     const int items = a.S * st.W;
-    const int grid = items < n_sms ? items : n_sms;
-    static int configured[2][64] = {{0}, {0}};
-    if (nb == 2) {
-        ensure_dynamic_smem(k_accept_persistent<true>, bytes, configured[1]);
-        launch_k(k_accept_persistent<true>, dim3(grid), dim3(PT), bytes, s, st, a);
-    } else {
-        ensure_dynamic_smem(k_accept_persistent<false>, bytes, configured[0]);
-        launch_k(k_accept_persistent<false>, dim3(grid), dim3(PT), bytes, s, st, a);
-    }
+    ensure_dynamic_smem(k_accept_persistent<CFG, PROBS>, bytes, configured);
+    launch_k(k_accept_persistent<CFG, PROBS>, dim3(items < n_sms ? items : n_sms), dim3(PT), bytes, s, st, a);
+}
+
+void launch_accept_persistent(const State& st, const AcceptArgs& a, int n_sms, cudaStream_t s) {
+    if (st.nb == 2) launch<true, false>(st, a, n_sms, s);
+    else launch<false, false>(st, a, n_sms, s);
+}
+
+void launch_probs_persistent(const float* lc, const float* lu, int rows, int V, float cfg_scale, float temperature,
+                             int top_k, float* p, int32_t* counters, int n_sms, cudaStream_t s) {
+    State st{};
+    st.V = V;
+    st.W = 1;
+    st.counters = counters;
+    AcceptArgs a{};
+    a.logits = lc;
+    a.logits_u = lu;
+    a.pcur = p;
+    a.S = rows;
+    a.cfg_scale = cfg_scale;
+    a.temperature = temperature;
+    a.top_k = top_k;
+    if (lu) launch<true, true>(st, a, n_sms, s);
+    else launch<false, true>(st, a, n_sms, s);
 }
 
 }  // namespace hbsjd

@@ -52,7 +52,7 @@ struct hbsjd_ctx {
     float* ssq;             // [rows][dim / 32] partial sums of squares of the residual rows (bf16 model)
     // host side
     int32_t* h_counters;  // pinned [8]
-    RoundPost* post;      // mapped host memory [2], by round parity: the counters of the last rounds
+    RoundPost* post;      // mapped host memory [3]: by round parity the counters of the last rounds; error code of hbsjd_probs
     RoundPost* post_dev;  // the same, as the GPU addresses it
     int32_t* tally;       // [2] device, see AcceptArgs
     uint32_t post_seq;    // stamp of the last round enqueued
@@ -391,6 +391,7 @@ int enqueue_round(hbsjd_ctx* c) {
     if (rc) return rc;
     AcceptArgs a;
     a.logits = c->logits;
+    a.logits_u = c->logits + (size_t)S * c->st.W * c->st.V;
     a.pcur = c->pbuf[c->parity];
     a.pprev = c->pbuf[c->parity ^ 1];
     a.flag = c->flag;
@@ -684,8 +685,8 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
         CK(cudaEventCreate(&s.b));
     }
     CK(cudaMallocHost((void**)&c->h_counters, 8 * sizeof(int32_t)));
-    CK(cudaHostAlloc((void**)&c->post, 2 * sizeof(RoundPost), cudaHostAllocMapped));
-    memset(c->post, 0, 2 * sizeof(RoundPost));
+    CK(cudaHostAlloc((void**)&c->post, 3 * sizeof(RoundPost), cudaHostAllocMapped));
+    memset(c->post, 0, 3 * sizeof(RoundPost));
     CK(cudaHostGetDevicePointer((void**)&c->post_dev, c->post, 0));
     if ((rc = dev_alloc(c, &c->tally, (size_t)2))) return rc;
     {
@@ -901,9 +902,17 @@ int hbsjd_probs(hbsjd_ctx* c, const float* logits_c, const float* logits_u, int 
     if (!c || !logits_c || !probs || rows < 1 || !(temperature > 0.f) || top_k < 0 ||
         (((uintptr_t)logits_c | (uintptr_t)logits_u | (uintptr_t)probs) & 15))
         return HBSJD_EINVAL;
-    launch_probs(logits_c, logits_u, rows, c->d.vocab, cfg_scale, temperature, top_k, probs, c->stream);
+    volatile RoundPost* post = c->post + 2;  // (only its error code is used)
+    post->counters[CNT_ERROR] = 0;
+    launch_probs(logits_c, logits_u, rows, c->d.vocab, cfg_scale, temperature, top_k, probs, c->post_dev[2].counters,
+                 c->stream);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->stream));
+    if (post->counters[CNT_ERROR] != 0) {
+        snprintf(c->err, sizeof(c->err), "hbsjd_probs: a bounded device-side wait gave up (code %d)",
+                 post->counters[CNT_ERROR]);
+        return HBSJD_ETIMEOUT;
+    }
     return HBSJD_OK;
 }
 

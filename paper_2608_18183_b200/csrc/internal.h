@@ -47,7 +47,8 @@ struct RoundPost {
 };
 
 struct AcceptArgs {
-    const float* logits;  // [nb][S][W][V]
+    const float* logits;    // [S][W][V], conditional
+    const float* logits_u;  // [S][W][V], unconditional (guidance)
     float* pcur;          // [Bmax][Wmax][V] this round's probabilities (next round's proposals)
     const float* pprev;   // [Bmax][Wmax][V]
     uint8_t* flag;        // [Bmax][Wmax] 1 = draft accepted
@@ -128,8 +129,11 @@ bool accept_persistent_supported(const State& st);
 void launch_accept_persistent(const State& st, const AcceptArgs& a, int n_sms, cudaStream_t s);
 // streaming multiprocessors of the current device
 int device_sm_count();
+// counters: place of CNT_ERROR (a bounded wait that gave up), in memory that the host can read
 void launch_probs(const float* lc, const float* lu, int rows, int V, float cfg_scale, float temperature, int top_k,
-                  float* p, cudaStream_t s);
+                  float* p, int32_t* counters, cudaStream_t s);
+void launch_probs_persistent(const float* lc, const float* lu, int rows, int V, float cfg_scale, float temperature,
+                             int top_k, float* p, int32_t* counters, int n_sms, cudaStream_t s);
 
 // empty kernel launched like every other (timing aid, model_kernels.cu)
 void launch_noop(cudaStream_t s);

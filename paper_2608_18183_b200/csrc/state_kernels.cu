@@ -545,11 +545,11 @@ __global__ void __launch_bounds__(ACC_THREADS, 2) k_prob_accept(State st, Accept
     const int img = st.slot_img[slot], c = st.slot_c[slot];
     const int t = c + i + 1;  // token position this distribution decides
     const float* lc = a.logits + ((size_t)slot * st.W + i) * V;
-    const float* lu = a.logits + ((size_t)(a.S + slot) * st.W + i) * V;
+    const float* lu = st.nb == 2 ? a.logits_u + ((size_t)slot * st.W + i) * V : nullptr;
     if (tid == 0) philox4x32_10((uint32_t)img, (uint32_t)t, a.round, 0u, a.seed_lo, a.seed_hi, sh.words);
 
     float* pout = a.pcur + ((size_t)img * st.Wmax + i) * V;
-    prob_pipeline(g, lc, st.nb == 2 ? lu : nullptr, V, a.cfg_scale, a.temperature, a.top_k, pout, sh);
+    prob_pipeline(g, lc, lu, V, a.cfg_scale, a.temperature, a.top_k, pout, sh);
 
     const size_t oidx = (size_t)img * st.Wmax + i;
     const bool last = (i == n - 1);
@@ -618,7 +618,15 @@ __global__ void __launch_bounds__(ACC_THREADS, 2) k_prob_accept(State st, Accept
 int accept_smem_bytes(int V) { return V * (int)sizeof(float) + (int)sizeof(AccShared); }
 
 void launch_probs(const float* lc, const float* lu, int rows, int V, float cfg_scale, float temperature, int top_k,
-                  float* p, cudaStream_t s) {
+                  float* p, int32_t* counters, cudaStream_t s) {
+    // The persistent kernel has one CTA of 1024 threads per SM, this file's k_probs two of 512: up to 4096 entries a row
+    // leaves the wide CTA a group of four per thread and its latency counts (4096 rows of 4096: 67 us against 75);
+    // above, its prefetched rows win (2048 rows of 8192 with guidance 62 -> 56 us, 1024 rows of 16384 56 -> 42 us
+    // plain and 85 -> 72 us with every option, 3 rows of 16384 26 -> 20 us).
+    if (V > 4096 && V <= 16384) {
+        launch_probs_persistent(lc, lu, rows, V, cfg_scale, temperature, top_k, p, counters, device_sm_count(), s);
+        return;
+    }
     static int configured[64] = {0};
     const int bytes = accept_smem_bytes(V);
     ensure_dynamic_smem(k_probs, bytes, configured);
@@ -900,6 +908,7 @@ cudaError_t verify_enqueue(const VerifyDesc& d, const VerifyScratch& sc, const f
     st.j_last = sc.j_last;
     AcceptArgs a;
     a.logits = logits;
+    a.logits_u = logits + (size_t)d.batch * d.window * d.V;
     a.pcur = p_out;
     a.pprev = q_prev;
     a.flag = sc.flag;

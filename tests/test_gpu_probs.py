@@ -62,3 +62,25 @@ def test_ties_and_crowded_bins(ctx16k):
     lc = np.stack(rows)
     for k in (1, 5, 1000, 4000, 16000):
         _check(ctx16k, lc, None, 1.0, 1.0, k)
+
+
+@pytest.mark.parametrize("V", [4096, 4160, 8256, 16384])
+def test_more_rows_than_ctas(V):
+    """Several rows per CTA of the persistent kernel (V above 4096; 4096 runs the other one), rows of very different
+    scale behind one another, so that the threshold guess carried from row to row is often useless; V that leaves
+    threads without entries (4160, 8256)."""
+    rng = np.random.default_rng(V)
+    sh = synth.ModelShape(1, 64, 1, 64, V, 4, 4, 3, "bf16")
+    ctx = binding.Context(sh, synth.make_weights(sh, 3, target_entropy=None), 2, 4)
+    rows = 311
+    scale = 10.0 ** rng.uniform(-3, 1, size=(rows, 1))
+    lc = (rng.normal(size=(rows, V)) * scale + rng.normal(size=(rows, 1)) * 5).astype(np.float32)
+    lc[::37] = np.round(lc[::37])
+    lu = (rng.normal(size=(rows, V)) * scale).astype(np.float32)
+    _check(ctx, lc, None, 1.0, 0.9, 500)
+    _check(ctx, lc, None, 1.0, 1.0, 0)
+    # the oracle rounds the guided logit once, the kernels after each of three steps, which can swap the k-th largest with
+    # a neighbour in the narrow rows: with guidance, multiples of 2^-10 below 2^7, on which every fp32 step is exact
+    lc, lu = (np.round(np.clip(x, -40, 40) * 1024).astype(np.float32) / 1024 for x in (lc, lu))
+    _check(ctx, lc, lu, 2.0, 0.5, 100)
+    ctx.hbsjd_destroy()
