@@ -4,10 +4,11 @@
 // Work item = one physical row (branch, slot) x HPC heads.  The items of a forward are dealt to the CTAs from a
 // list sorted by context length (longest first, alternate stripes reversed), so every CTA streams about the
 // same number of key blocks.  Inside a CTA
-//   warp 0 (one lane)   producer: for every item, its K and V blocks of 32 keys, each one cp.async.bulk.tensor copy
-//                       (128-byte swizzle) into a ring of STAGES stages, completion on mbarriers.  The producer
-//                       runs ahead across item boundaries: the next item's first blocks are in flight while the
-//                       current item's last ones are used.
+//   warp 0 (one lane)   producer: for every item, its keys in stages of one or two blocks of 32, K and V of a block and
+//                       all heads of the item one cp.async.bulk.tensor copy each (128-byte swizzle), completion on
+//                       mbarriers; an item's last stage brings only the blocks that it needs.  The producer runs ahead
+//                       across item boundaries: the next item's first keys are in flight while the current item's
+//                       last ones are used.
 //   warps 1..QB*HPC     consumers: warp (head, q-block) owns 16 consecutive window inputs of one head (its query
 //                       fragments come straight from global memory, once per item); online
 //                       softmax in fp32, products on mma.sync m16n8k16 (the work is about W FLOP per byte of K, V:
@@ -34,10 +35,24 @@ namespace {
 
 constexpr int DH = 64;   // head size
 constexpr int KB = 32;   // keys per block
-constexpr int HPC = 2;   // heads per work item
-constexpr int STAGES = 3;
-constexpr int TILE_BYTES = KB * DH * 2;             // one K or V tile of one head: 4 KB
-constexpr int STAGE_BYTES = HPC * 2 * TILE_BYTES;   // 16 KB
+constexpr int TILE_BYTES = KB * DH * 2;  // one K or V tile of one head: 4 KB
+
+// Split by the window's 16-query blocks QB.  A consumer warp takes 16 queries of one head; windows above 32 inputs have
+// three or four consumer warps with one head, smaller ones two heads.  What bounds an item is the latency of its chain
+// of key blocks, so windows above 16 take two blocks at a time (see attend), at the price of registers for two CTAs per
+// SM instead of three: 6 images of 36 layers, contexts up to 576: 16.6 -> 12.9 us per launch, rollout 876 -> 832 ms;
+// scoring of 128 images (windows of 64) 80.1 -> 78.9 ms.  Up to 16 inputs three CTAs with one block at a time stay
+// ahead (two at a time: 24 images one token at a time 303 -> 307 to 317 ms, 64 images of 16 inputs 84.2 -> 85.7 ms).
+template <int QB>
+struct AttnCfg {
+    static constexpr int HPC = QB >= 3 ? 1 : 2;
+    static constexpr int NCW = QB * HPC;                      // consumer warps
+    static constexpr int NBLK = QB == 1 ? 1 : 2;              // key blocks per stage
+    static constexpr int BLOCK_BYTES = HPC * 2 * TILE_BYTES;  // K and V of 32 keys, all heads of the item
+    static constexpr int STAGE_BYTES = NBLK * BLOCK_BYTES;
+    static constexpr int STAGES = QB == 1 ? 3 : 98304 / STAGE_BYTES;
+    static constexpr int CTAS = QB == 1 ? 3 : 2;              // per SM
+};
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -74,10 +89,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         if (t1 - t0 > 1000000000ull) return false;
     }
 }
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
         : "memory");
 }
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
@@ -108,7 +123,7 @@ __device__ __forceinline__ uint32_t tile_off(int row, int chunk) { return row * 
 
 struct AttnArgs {
     State st;
-    int S, layer, G;  // slots, layer, head groups (heads / HPC)
+    int S, layer, G, hpc;  // slots, layer, head groups (heads / hpc), heads per group
     KvView kv;
     const bf16* q;
     bf16* out;
@@ -130,21 +145,151 @@ __device__ __forceinline__ bool item_at(const AttnArgs& a, const int* s_tab, int
     it.c = s_tab[2 * a.S + slot];
     it.prow = br * a.S + slot;
     it.crow = br * st.Bmax + s_tab[3 * a.S + slot];
-    it.head0 = g * HPC;
+    it.head0 = g * a.hpc;
     return true;
 }
 
+// One or two consecutive blocks of 32 keys of one head for the 16 queries of a warp: S = Q K^T, causal mask, online
+// softmax in fp32, O += P V.  The blocks' score products, maxima, exponentials and row sums do not depend on one
+// another (the running maximum is the only link, and a maximum is exact in any order), so two blocks at a time hide
+// each other's latencies; the accumulation into the normaliser and into O stays block after block, so the result is
+// the same bits as one block at a time.  An all-masked block is an exact no-op.
+// kt / vt: shared addresses of the first block's K and V tile; the second block's lie block_bytes further.
+template <int NB>
+__device__ __forceinline__ void attend(uint32_t kt, uint32_t vt, uint32_t block_bytes, int key0, int s0, int s1,
+                                       int q_first, int lane, const uint32_t (&qa)[4][4], float (&o)[8][4], float& m0,
+                                       float& m1, float& l0, float& l1) {
+    const float sl2 = 0.125f * 1.4426950408889634f;  // 1/sqrt(64) * log2(e)
+    float sc[NB][4][4], bx0[NB], bx1[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        // 32 keys: 4 n-tiles of 8 keys
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt) {
+            sc[b][nt][0] = sc[b][nt][1] = sc[b][nt][2] = sc[b][nt][3] = 0.f;
+            const int krow = nt * 8 + (lane & 7);
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t b0, b1, b2, b3;  // k-chunks 2*half (b0,b1) and 2*half+1 (b2,b3)
+                ldmatrix_x4(kt + b * block_bytes + tile_off(krow, half * 4 + (lane >> 3)), b0, b1, b2, b3);
+                mma_bf16(sc[b][nt], qa[half * 2], b0, b1);
+                mma_bf16(sc[b][nt], qa[half * 2 + 1], b2, b3);
+            }
+        }
+    }
+    // causal mask and block maxima (rows r0 = lane/4 and r0+8; columns (lane%4)*2 + {0,1} per n-tile).  A block wholly
+    // at or before the warp's first query needs no mask; scaling a visible score is the same multiplication either
+    // way, so the two paths agree bit for bit.
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        const int kb0 = key0 + b * KB;
+        float mx0 = -INFINITY, mx1 = -INFINITY;
+        if (kb0 + KB - 1 <= q_first) {
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+                sc[b][nt][0] *= sl2;
+                sc[b][nt][1] *= sl2;
+                sc[b][nt][2] *= sl2;
+                sc[b][nt][3] *= sl2;
+                mx0 = fmaxf(mx0, fmaxf(sc[b][nt][0], sc[b][nt][1]));
+                mx1 = fmaxf(mx1, fmaxf(sc[b][nt][2], sc[b][nt][3]));
+            }
+        } else {
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+                const int key = kb0 + nt * 8 + (lane & 3) * 2;
+                sc[b][nt][0] = key <= s0 ? sc[b][nt][0] * sl2 : -INFINITY;
+                sc[b][nt][1] = key + 1 <= s0 ? sc[b][nt][1] * sl2 : -INFINITY;
+                sc[b][nt][2] = key <= s1 ? sc[b][nt][2] * sl2 : -INFINITY;
+                sc[b][nt][3] = key + 1 <= s1 ? sc[b][nt][3] * sl2 : -INFINITY;
+                mx0 = fmaxf(mx0, fmaxf(sc[b][nt][0], sc[b][nt][1]));
+                mx1 = fmaxf(mx1, fmaxf(sc[b][nt][2], sc[b][nt][3]));
+            }
+        }
+        bx0[b] = mx0;
+        bx1[b] = mx1;
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        bx0[b] = fmaxf(bx0[b], __shfl_xor_sync(0xffffffffu, bx0[b], 1));
+        bx1[b] = fmaxf(bx1[b], __shfl_xor_sync(0xffffffffu, bx1[b], 1));
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        bx0[b] = fmaxf(bx0[b], __shfl_xor_sync(0xffffffffu, bx0[b], 2));
+        bx1[b] = fmaxf(bx1[b], __shfl_xor_sync(0xffffffffu, bx1[b], 2));
+    }
+    float corr0[NB], corr1[NB], rs0[NB], rs1[NB];
+    uint32_t pa[NB][2][4];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        // key 0 is visible to every query, so the running maximum is finite from the first block on
+        const float mx0 = fmaxf(m0, bx0[b]), mx1 = fmaxf(m1, bx1[b]);
+        corr0[b] = exp2f(m0 - mx0);
+        corr1[b] = exp2f(m1 - mx1);
+        m0 = mx0;
+        m1 = mx1;
+        rs0[b] = rs1[b] = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt) {
+            const float p0 = exp2f(sc[b][nt][0] - mx0), p1 = exp2f(sc[b][nt][1] - mx0);
+            const float p2 = exp2f(sc[b][nt][2] - mx1), p3 = exp2f(sc[b][nt][3] - mx1);
+            rs0[b] += p0 + p1;
+            rs1[b] += p2 + p3;
+            // the softmax weights enter the P.V product as bf16 (the normaliser keeps the fp32 values)
+            pa[b][nt >> 1][(nt & 1) * 2] = pack_bf16(p0, p1);
+            pa[b][nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            o[t][0] *= corr0[b];
+            o[t][1] *= corr0[b];
+            o[t][2] *= corr1[b];
+            o[t][3] *= corr1[b];
+        }
+        // O += P V: two k-chunks of 16 keys, 8 n-tiles of 8 dims
+#pragma unroll
+        for (int kc = 0; kc < 2; ++kc) {
+            const int vrow = kc * 16 + ((lane >> 3) & 1) * 8 + (lane & 7);
+#pragma unroll
+            for (int dp = 0; dp < 4; ++dp) {  // pairs of n-tiles: dims dp*16 .. dp*16+15
+                uint32_t b0, b1, b2, b3;
+                ldmatrix_x4_trans(vt + b * block_bytes + tile_off(vrow, dp * 2 + (lane >> 4)), b0, b1, b2, b3);
+                mma_bf16(o[dp * 2], pa[b][kc], b0, b1);
+                mma_bf16(o[dp * 2 + 1], pa[b][kc], b2, b3);
+            }
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        rs0[b] += __shfl_xor_sync(0xffffffffu, rs0[b], 1);
+        rs1[b] += __shfl_xor_sync(0xffffffffu, rs1[b], 1);
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        rs0[b] += __shfl_xor_sync(0xffffffffu, rs0[b], 2);
+        rs1[b] += __shfl_xor_sync(0xffffffffu, rs1[b], 2);
+        l0 = l0 * corr0[b] + rs0[b];
+        l1 = l1 * corr1[b] + rs1[b];
+    }
+}
+
 template <int QB>
-__global__ void __launch_bounds__((QB * HPC + 1) * 32, QB >= 3 ? 2 : 3) k_attention_tma(const __grid_constant__ CUtensorMap map_k,
-                                                                       const __grid_constant__ CUtensorMap map_v,
-                                                                       const AttnArgs a) {
+__global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS)
+    k_attention_tma(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                    const AttnArgs a) {
     pdl_trigger();
-    constexpr int NCW = QB * HPC;                 // consumer warps
+    using cfg = AttnCfg<QB>;
+    constexpr int NCW = cfg::NCW, HPC = cfg::HPC, STAGES = cfg::STAGES;
+    constexpr int SK = cfg::NBLK * KB;  // keys per stage
     extern __shared__ unsigned char smem_raw[];
     const State& st = a.st;
     const uint32_t raw = smem_u32(smem_raw);
-    const uint32_t ring = (raw + 1023u) & ~1023u;               // [STAGES][HPC][K tile | V tile]
-    const uint32_t bars = ring + STAGES * STAGE_BYTES;          // full[STAGES], empty[STAGES]
+    const uint32_t ring = (raw + 1023u) & ~1023u;               // [STAGES][block][K tiles | V tiles]
+    const uint32_t bars = ring + STAGES * cfg::STAGE_BYTES;          // full[STAGES], empty[STAGES]
     const uint32_t full0 = bars, empty0 = bars + 8 * STAGES;
     unsigned char* tail = smem_raw + (bars - raw) + 16 * STAGES;
     volatile uint32_t* abort_flag = (volatile uint32_t*)tail;
@@ -184,24 +329,28 @@ __global__ void __launch_bounds__((QB * HPC + 1) * 32, QB >= 3 ? 2 : 3) k_attent
                 const int pos = position(stripe);
                 Item it;
                 if (pos >= n_items || !item_at(a, s_tab, pos, it)) continue;
-                const int nblocks = (it.c + it.n + KB - 1) / KB;
+                const int keys = it.c + it.n, nstages = (keys + SK - 1) / SK;
                 const int32_t* pages = a.kv.table + (size_t)it.crow * a.kv.pages_per_row;
                 const int layer_row0 = a.layer * a.kv.n_pages * a.kv.page;
-                for (int blk = 0; blk < nblocks; ++blk, ++gc) {
+                int page = pages[0];  // one page holds whole stages (the page size is a multiple of 64)
+                for (int sg = 0; sg < nstages; ++sg, ++gc) {
+                    const int key0 = sg * SK;
+                    // the next stage's page is looked up while this one's turn is waited for
+                    const int page_next = sg + 1 < nstages ? pages[(key0 + SK) / a.kv.page] : 0;
                     const uint32_t gs = gc % STAGES, ph = (gc / STAGES) & 1u;
                     if (!mbar_wait(empty0 + 8 * gs, ph ^ 1u, abort_flag)) {
                         ok = false;
                         break;
                     }
-                    const int key0 = blk * KB;
-                    // one page holds whole blocks (the page size is a multiple of 32)
-                    const int y = layer_row0 + pages[key0 / a.kv.page] * a.kv.page + key0 % a.kv.page;
-                    mbar_expect_tx(full0 + 8 * gs, STAGE_BYTES);
-                    for (int h = 0; h < HPC; ++h) {
-                        const uint32_t dst = ring + gs * STAGE_BYTES + h * 2 * TILE_BYTES;
-                        tma_load_2d(dst, &map_k, (it.head0 + h) * DH, y, full0 + 8 * gs);
-                        tma_load_2d(dst + TILE_BYTES, &map_v, (it.head0 + h) * DH, y, full0 + 8 * gs);
+                    const int y = layer_row0 + page * a.kv.page + key0 % a.kv.page;
+                    const int blocks = min(cfg::NBLK, (keys - key0 + KB - 1) / KB);
+                    mbar_expect_tx(full0 + 8 * gs, blocks * cfg::BLOCK_BYTES);
+                    for (int b = 0; b < blocks; ++b) {
+                        const uint32_t dst = ring + gs * cfg::STAGE_BYTES + b * cfg::BLOCK_BYTES;
+                        tma_load_3d(dst, &map_k, 0, y + b * KB, it.head0, full0 + 8 * gs);
+                        tma_load_3d(dst + HPC * TILE_BYTES, &map_v, 0, y + b * KB, it.head0, full0 + 8 * gs);
                     }
+                    page = page_next;
                 }
             }
             if (!ok) {
@@ -224,14 +373,13 @@ __global__ void __launch_bounds__((QB * HPC + 1) * 32, QB >= 3 ? 2 : 3) k_attent
         const int cw = warp - 1;
         const int wh = cw / QB, wq = cw % QB;  // head within the item, q-block
         uint32_t gc = 0;
-        const float sl2 = 0.125f * 1.4426950408889634f;  // 1/sqrt(64) * log2(e)
         bool ok = true;
         for (int stripe = 0; ok && stripe * grid < n_items; ++stripe) {
             const int pos = position(stripe);
             Item it;
             if (pos >= n_items || !item_at(a, s_tab, pos, it)) continue;
             const int c = it.c, n = it.n;
-            const int nblocks = (c + n + KB - 1) / KB;
+            const int keys = c + n, nstages = (keys + SK - 1) / SK;
             // ---- this warp's queries: 16 rows x 64 dims as A fragments.  Rows at or past n hold whatever the buffer
             // holds (finite values of older forwards): their results are never written back.
             const int i0 = wq * 16 + (lane >> 2), i1 = i0 + 8;
@@ -264,105 +412,21 @@ __global__ void __launch_bounds__((QB * HPC + 1) * 32, QB >= 3 ? 2 : 3) k_attent
             for (int t = 0; t < 8; ++t) o[t][0] = o[t][1] = o[t][2] = o[t][3] = 0.f;
             float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
 
-            for (int blk = 0; blk < nblocks; ++blk, ++gc) {
+            for (int sg = 0; sg < nstages; ++sg, ++gc) {
                 const uint32_t gs = gc % STAGES, ph = (gc / STAGES) & 1u;
                 if (!mbar_wait(full0 + 8 * gs, ph, abort_flag)) {
                     ok = false;
                     break;
                 }
-                const int key0 = blk * KB;
-                // rows of this warp whose last visible key precedes the block contribute nothing: skip the math
-                // (an all-masked block is an exact no-op of the online softmax, so skipping changes no bits)
+                const int key0 = sg * SK;
+                // keys behind the last one visible to this warp contribute nothing: skip the math (an all-masked
+                // block is an exact no-op of the online softmax, so skipping changes no bits)
                 const int smax_warp = c + min(wq * 16 + 15, n - 1);
-                if (warp_active && key0 <= smax_warp) {
-                    const uint32_t kt = ring + gs * STAGE_BYTES + wh * 2 * TILE_BYTES;
-                    const uint32_t vt = kt + TILE_BYTES;
-                    // S = Q K^T for 32 keys: 4 n-tiles of 8 keys
-                    float sc[4][4];
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt) {
-                        sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
-                        const int krow = nt * 8 + (lane & 7);
-#pragma unroll
-                        for (int half = 0; half < 2; ++half) {
-                            uint32_t b0, b1, b2, b3;  // k-chunks 2*half (b0,b1) and 2*half+1 (b2,b3)
-                            ldmatrix_x4(kt + tile_off(krow, half * 4 + (lane >> 3)), b0, b1, b2, b3);
-                            mma_bf16(sc[nt], qa[half * 2], b0, b1);
-                            mma_bf16(sc[nt], qa[half * 2 + 1], b2, b3);
-                        }
-                    }
-                    // causal mask + online softmax (rows r0 = lane/4 and r0+8; columns (lane%4)*2 + {0,1} per
-                    // n-tile).  A block wholly at or before the warp's first query needs no mask; scaling a
-                    // visible score is the same multiplication either way, so the two paths agree bit for bit.
-                    float mx0 = m0, mx1 = m1;
-                    if (key0 + KB - 1 <= c + wq * 16) {
-#pragma unroll
-                        for (int nt = 0; nt < 4; ++nt) {
-                            sc[nt][0] *= sl2;
-                            sc[nt][1] *= sl2;
-                            sc[nt][2] *= sl2;
-                            sc[nt][3] *= sl2;
-                            mx0 = fmaxf(mx0, fmaxf(sc[nt][0], sc[nt][1]));
-                            mx1 = fmaxf(mx1, fmaxf(sc[nt][2], sc[nt][3]));
-                        }
-                    } else {
-#pragma unroll
-                        for (int nt = 0; nt < 4; ++nt) {
-                            const int key = key0 + nt * 8 + (lane & 3) * 2;
-                            sc[nt][0] = key <= s0 ? sc[nt][0] * sl2 : -INFINITY;
-                            sc[nt][1] = key + 1 <= s0 ? sc[nt][1] * sl2 : -INFINITY;
-                            sc[nt][2] = key <= s1 ? sc[nt][2] * sl2 : -INFINITY;
-                            sc[nt][3] = key + 1 <= s1 ? sc[nt][3] * sl2 : -INFINITY;
-                            mx0 = fmaxf(mx0, fmaxf(sc[nt][0], sc[nt][1]));
-                            mx1 = fmaxf(mx1, fmaxf(sc[nt][2], sc[nt][3]));
-                        }
-                    }
-                    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
-                    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-                    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
-                    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-                    // key 0 is visible to every query, so mx is finite from the first block on
-                    const float corr0 = exp2f(m0 - mx0), corr1 = exp2f(m1 - mx1);
-                    m0 = mx0;
-                    m1 = mx1;
-                    float rs0 = 0.f, rs1 = 0.f;
-                    uint32_t pa[2][4];
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt) {
-                        const float p0 = exp2f(sc[nt][0] - mx0), p1 = exp2f(sc[nt][1] - mx0);
-                        const float p2 = exp2f(sc[nt][2] - mx1), p3 = exp2f(sc[nt][3] - mx1);
-                        rs0 += p0 + p1;
-                        rs1 += p2 + p3;
-                        // the softmax weights enter the P.V product as bf16 (the normaliser keeps the fp32 values)
-                        pa[nt >> 1][(nt & 1) * 2] = pack_bf16(p0, p1);
-                        pa[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
-                    }
-                    rs0 += __shfl_xor_sync(0xffffffffu, rs0, 1);
-                    rs0 += __shfl_xor_sync(0xffffffffu, rs0, 2);
-                    rs1 += __shfl_xor_sync(0xffffffffu, rs1, 1);
-                    rs1 += __shfl_xor_sync(0xffffffffu, rs1, 2);
-                    l0 = l0 * corr0 + rs0;
-                    l1 = l1 * corr1 + rs1;
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) {
-                        o[t][0] *= corr0;
-                        o[t][1] *= corr0;
-                        o[t][2] *= corr1;
-                        o[t][3] *= corr1;
-                    }
-                    // O += P V: two k-chunks of 16 keys, 8 n-tiles of 8 dims
-#pragma unroll
-                    for (int kc = 0; kc < 2; ++kc) {
-                        const int vrow = kc * 16 + ((lane >> 3) & 1) * 8 + (lane & 7);
-#pragma unroll
-                        for (int dp = 0; dp < 4; ++dp) {  // pairs of n-tiles: dims dp*16 .. dp*16+15
-                            uint32_t b0, b1, b2, b3;
-                            ldmatrix_x4_trans(vt + tile_off(vrow, dp * 2 + (lane >> 4)), b0, b1, b2, b3);
-                            mma_bf16(o[dp * 2], pa[kc], b0, b1);
-                            mma_bf16(o[dp * 2 + 1], pa[kc], b2, b3);
-                        }
-                    }
-                }
+                const uint32_t kt = ring + gs * cfg::STAGE_BYTES + wh * TILE_BYTES, vt = kt + HPC * TILE_BYTES;
+                if (cfg::NBLK == 2 && warp_active && key0 + KB <= smax_warp)
+                    attend<cfg::NBLK>(kt, vt, cfg::BLOCK_BYTES, key0, s0, s1, c + wq * 16, lane, qa, o, m0, m1, l0, l1);
+                else if (warp_active && key0 <= smax_warp)
+                    attend<1>(kt, vt, cfg::BLOCK_BYTES, key0, s0, s1, c + wq * 16, lane, qa, o, m0, m1, l0, l1);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty0 + 8 * gs);  // this warp is done with the stage
             }
@@ -389,12 +453,13 @@ __global__ void __launch_bounds__((QB * HPC + 1) * 32, QB >= 3 ? 2 : 3) k_attent
 
 template <int QB>
 cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, const AttnArgs& a, cudaStream_t s) {
-    constexpr int threads = (QB * HPC + 1) * 32;
-    const int smem = 1024 + STAGES * STAGE_BYTES + 16 * STAGES + 16 + 16 * a.S;
+    using cfg = AttnCfg<QB>;
+    constexpr int threads = (cfg::NCW + 1) * 32;
+    const int smem = 1024 + cfg::STAGES * cfg::STAGE_BYTES + 16 * cfg::STAGES + 16 + 16 * a.S;
     static int configured[64] = {0};
     cudaError_t e = ensure_dynamic_smem(k_attention_tma<QB>, smem, configured);
     if (e != cudaSuccess) return e;
-    // resident CTAs per SM (registers and shared memory), at most 3: the grid is exactly what is resident at once
+    // resident CTAs per SM (registers and shared memory): the grid is exactly what is resident at once
     static int resident[64] = {0};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -403,7 +468,7 @@ cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, const AttnAr
         int n = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_attention_tma<QB>, threads, (size_t)smem);
         if (e != cudaSuccess) return e;
-        resident[dev] = n < 1 ? 1 : (n > 3 ? 3 : n);
+        resident[dev] = n < 1 ? 1 : (n > cfg::CTAS ? cfg::CTAS : n);
     }
     const int per_sm = resident[dev];
     const long items = (long)a.S * a.st.nb * a.G;
@@ -415,7 +480,7 @@ cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, const AttnAr
 }  // namespace
 
 bool attention_tma_supported(const State& st, const KvView& kv) {
-    return st.dh == DH && st.W <= 64 && kv.page % KB == 0 && st.Hh % HPC == 0 && st.slot_order != nullptr;
+    return st.dh == DH && st.W <= 64 && kv.page % (2 * KB) == 0 && st.Hh % 2 == 0 && st.slot_order != nullptr;
 }
 
 int launch_attention_tma(const State& st, int S, int layer, const bf16* q, int q_rows_cap, KvView kv, bf16* out,
@@ -424,8 +489,10 @@ int launch_attention_tma(const State& st, int S, int layer, const bf16* q, int q
     const int qb = (st.W + 15) / 16;
     const long kv_rows = (long)st.L * kv.n_pages * kv.page;
     (void)q_rows_cap;
-    if (kv_rows > 0x7fffffffL || !make_tensor_map_bf16(&mk, kv.k, (int)kv_rows, st.D, KB) ||
-        !make_tensor_map_bf16(&mv, kv.v, (int)kv_rows, st.D, KB)) {
+    const int hpc = qb == 1 ? AttnCfg<1>::HPC : qb == 2 ? AttnCfg<2>::HPC : AttnCfg<3>::HPC;
+    // the pool as (64 columns of a head, rows, heads): the same form as a GEMM operand's k-blocks
+    if (kv_rows > 0x7fffffffL || !make_tensor_map_kblocks(&mk, kv.k, (int)kv_rows, st.D, KB, hpc) ||
+        !make_tensor_map_kblocks(&mv, kv.v, (int)kv_rows, st.D, KB, hpc)) {
         snprintf(err, errlen, "attention: cuTensorMapEncodeTiled failed");
         return -3;
     }
@@ -433,7 +500,8 @@ int launch_attention_tma(const State& st, int S, int layer, const bf16* q, int q
     a.st = st;
     a.S = S;
     a.layer = layer;
-    a.G = st.Hh / HPC;
+    a.hpc = hpc;
+    a.G = st.Hh / hpc;
     a.kv = kv;
     a.out = out;
     a.q = q;

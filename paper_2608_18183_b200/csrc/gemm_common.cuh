@@ -166,10 +166,6 @@ __device__ __forceinline__ void store_32b(void* dst, const uint32_t* o) {
                  : "memory");
 }
 
-// Row-major bf16 [rows, K] as (64 columns, rows, K / 64) with a box of 64 x box_rows x box_kb (2 or 4): one copy brings
-// box_kb consecutive k-blocks, each a 128-byte-swizzled tile of box_rows rows; zero fill past the last k-block.
-bool make_tensor_map_kblocks(CUtensorMap* map, const void* base, int rows, int K, int box_rows, int box_kb);
-
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"

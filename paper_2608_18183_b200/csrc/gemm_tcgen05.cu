@@ -843,11 +843,8 @@ int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int ma
 // 16 KB activation tile of every k-block has to cross from L2 whatever N is, and about 160 KB can be in flight
 // per SM); the epilogue adds about 0.15 us per 32 columns.  Large problems end up with 256 (CTA pairs), small
 // ones with the widest tile that still fits one wave.
-bool make_tensor_map_bf16(::CUtensorMap_st* map, const void* base, int rows, int cols, int box_rows) {
-    return make_map(map, base, rows, cols, box_rows);
-}
-
-bool make_tensor_map_kblocks(CUtensorMap* map, const void* base, int rows, int K, int box_rows, int box_kb) {
+bool make_tensor_map_kblocks(::CUtensorMap_st* map, const void* base, int rows, int K, int box_rows, int box_kb) {
+    if (box_kb == 1) return cached_map(map, MapKey{base, rows, K, box_rows, 5}, encode_map_kb<1>);
     if (box_kb == 2) return cached_map(map, MapKey{base, rows, K, box_rows, 3}, encode_map_kb<2>);
     return box_kb == 4 && cached_map(map, MapKey{base, rows, K, box_rows, 4}, encode_map_kb<4>);
 }

@@ -159,8 +159,10 @@ int gemm_tcgen05_run(const bf16* A, const bf16* W, float* C, int M, int N, int K
                      int m_cap, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int w_constant = 1,
                      unsigned int acc_wait_ns = 0);
 int gemm_tcgen05_tile_n(int M, int N, int K);
-// Cached TMA descriptor of a row-major bf16 matrix [rows, cols]: box = 64 columns x box_rows rows, 128-byte swizzle.
-bool make_tensor_map_bf16(::CUtensorMap_st* map, const void* base, int rows, int cols, int box_rows);
+// Cached TMA descriptor of a row-major bf16 [rows, K] matrix seen as (64 columns, rows, K / 64) with a box of
+// 64 x box_rows x box_kb (box_kb 1, 2 or 4): one copy brings box_kb consecutive 64-column blocks, each a
+// 128-byte-swizzled tile of box_rows rows; zero fill past the last one.
+bool make_tensor_map_kblocks(::CUtensorMap_st* map, const void* base, int rows, int K, int box_rows, int box_kb);
 // RMSNorm folded around a GEMM: A holds the bf16 copy of the unnormalised residual rows x, W has the norm's gain
 // folded in, and the epilogue multiplies row m by rsqrt(sum(ssq[m][0 .. K/32)) / K + eps).  ssq null: no factor.
 struct NormIn {
