@@ -1,5 +1,7 @@
 // Row-wise kernels of the verifier forward (Sec. 4.2 "Batched verification"): slot set-up / compaction,
 // embedding gather, RMSNorm, 2D RoPE + paged KV write, reference attention, SwiGLU, CUDA-core GEMM.
+#include <cstring>
+
 #include "internal.h"
 
 namespace hbsjd {
@@ -312,9 +314,19 @@ __global__ void k_attention_ref(State st, int S, int layer, const TA* __restrict
     float mx = -INFINITY;
     for (int t = lane; t <= s; t += 32) {
         const TA* k = (const TA*)kv.k + kv.offset(layer, crow, t) + head * dh;
+        // the value row will be wanted behind the softmax: towards L1 meanwhile
+        for (int b = 0; b < dh * (int)sizeof(TA); b += 128)
+            asm volatile("prefetch.global.L1 [%0];" ::"l"((const char*)kv.v + ((const char*)k - (const char*)kv.k) + b));
         float dot = 0.f;
-#pragma unroll 16
-        for (int e = 0; e < dh; ++e) dot += qs[e] * to_f<TA>(k[e]);
+        constexpr int PER = 16 / (int)sizeof(TA);  // elements per 16-byte load (head sizes are multiples of 16)
+#pragma unroll 4
+        for (int e = 0; e < dh; e += PER) {
+            const uint4 raw = *reinterpret_cast<const uint4*>(k + e);
+            TA v[PER];
+            memcpy(v, &raw, 16);
+#pragma unroll
+            for (int x = 0; x < PER; ++x) dot += qs[e + x] * to_f<TA>(v[x]);
+        }
         dot *= scale;
         sc[t] = dot;
         mx = fmaxf(mx, dot);

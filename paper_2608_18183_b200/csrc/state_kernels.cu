@@ -675,9 +675,10 @@ __device__ __forceinline__ void post_round(const State& st, const AcceptArgs& a,
     __threadfence();
     volatile RoundPost* p = a.post;
 #pragma unroll
-    for (int x = 0; x < 8; ++x) p->counters[x] = atomicAdd(&st.counters[x], 0);
-    p->min_left = atomicExch(&a.tally[1], 0x7fffffff);
+    for (int x = 0; x < 8; ++x) p->counters[x] = *(volatile int32_t*)&st.counters[x];
+    p->min_left = *(volatile int32_t*)&a.tally[1];
     a.tally[0] = 0;
+    a.tally[1] = 0x7fffffff;
     __threadfence_system();
     p->stamp = a.post_stamp;
 }
@@ -690,13 +691,12 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
     AccShared& sh = *(AccShared*)(smem_raw + (size_t)st.V * sizeof(float));
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int slot = blockIdx.x;
-    const int n = st.slot_n[slot];
+    const int n = st.slot_n[slot], img = st.slot_img[slot], c = st.slot_c[slot];
     if (n == 0) {
         if (tid == 0) post_round(st, a, 0x7fffffff);
         return;
     }
     const int V = st.V;
-    const int img = st.slot_img[slot], c = st.slot_c[slot];
     int32_t* seq = st.seq + (size_t)img * (st.T + 1);
     uint8_t* dl = st.delta + (size_t)img * (st.T + 1);
     if (wid == 0) {
@@ -724,12 +724,12 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
     // many of its accepted drafts (no replacement token is drawn: the token at the new cursor was accepted)
     const bool held_back = a.m_sync != nullptr && *a.m_sync < m;
     if (held_back) {
-        if (tid != 0) return;
+        if (wid != 0) return;
         m = *a.m_sync;
         j = -1;
         tok = seq[c + m];
     } else if (a.greedy) {
-        if (tid != 0) return;
+        if (wid != 0) return;
         tok = a.cand_rep[(size_t)img * st.Wmax + (m - 1)];
     } else {
         const int is = m - 1, t = c + m;
@@ -749,10 +749,11 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
             // pass 0: the residual (or p itself for the bonus token); pass 1, only after an empty residual:
             // p_j itself with the same word
             unsigned long long wsum = 0;
-            for (int v0 = wid * seg + lane * 4; v0 < vend; v0 += 128 * 4) {
-                float4 p4[4], q4[4];
+            // (eight float4 per lane and row in flight: the whole segment of a 16384-entry vocabulary)
+            for (int v0 = wid * seg + lane * 4; v0 < vend; v0 += 128 * 8) {
+                float4 p4[8], q4[8];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
+                for (int k = 0; k < 8; ++k) {
                     const int v = v0 + k * 128;
                     if (v < vend) {
                         p4[k] = *reinterpret_cast<const float4*>(prow + v);
@@ -760,7 +761,7 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
                     }
                 }
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
+                for (int k = 0; k < 8; ++k) {
                     const int v = v0 + k * 128;
                     if (v < vend) {
                         float4 x = p4[k];
@@ -789,23 +790,32 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
             tok = block_pick(g, V, sh.words[1], sh);
             if (tok >= 0 || !reject) break;
         }
-        if (tid != 0) return;
+        if (wid != 0) return;
     }
-    seq[c + m] = tok;
-    dl[c + m] = 0;
+    // warp 0: commit and draft refresh.  A serial walk over the window (a load and a store per draft that the compiler
+    // may not reorder) was most of the work behind the sampled token.
     const int c2 = c + m;
-    st.cursor[img] = c2;
-    st.qbase[img] = c;
-    st.m_last[img] = m;
-    st.j_last[img] = j;
+    if (lane == 0) {
+        seq[c2] = tok;
+        dl[c2] = 0;
+        st.cursor[img] = c2;
+        st.qbase[img] = c;
+        st.m_last[img] = m;
+        st.j_last[img] = j;
+    }
+    __syncwarp();
     if (c2 < st.T) {
-        const int n2 = min(st.W, st.T - c2);
-        for (int t = c2 + 1; t <= c2 + n2 - 1; ++t) {
-            if (t <= c + n) {
-                seq[t] = a.cand_ref[(size_t)img * st.Wmax + (t - c - 1)];
-                dl[t] = 0;
-            } else {
-                const int src = t - st.H;
+        const int end = c2 + min(st.W, st.T - c2) - 1;  // last draft position
+        for (int t = c2 + 1 + lane; t <= min(end, c + n); t += 32) {
+            seq[t] = a.cand_ref[(size_t)img * st.Wmax + (t - c - 1)];
+            dl[t] = 0;
+        }
+        __syncwarp();
+        // history drafts copy the token H back, which may itself be one of them: H positions at a time
+        const int step = min(32, st.H);
+        for (int t0 = c + n + 1; t0 <= end; t0 += step) {
+            const int t = t0 + lane, src = t - st.H;
+            if (lane < step && t <= end) {
                 if (src >= 1) {
                     seq[t] = seq[src];
                 } else {
@@ -815,9 +825,11 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
                 }
                 dl[t] = 1;
             }
+            __syncwarp();
         }
-        atomicAdd(&st.counters[CNT_LIVE], 1);
     }
+    if (lane != 0) return;
+    if (c2 < st.T) atomicAdd(&st.counters[CNT_LIVE], 1);
     atomicAdd(&st.counters[CNT_COMMITTED], m);
     if (j >= 0) atomicAdd(&st.counters[CNT_REJECTS], 1);
     post_round(st, a, c2 < st.T ? st.T - c2 : 0x7fffffff);
