@@ -157,3 +157,26 @@ def test_score_of_a_model_against_itself_is_zero_and_the_call_is_repeatable():
     assert e.value.code == -1
     for c in (a, b, tea):
         c.hbsjd_destroy()
+
+
+def test_score_does_not_depend_on_the_chunk():
+    """Chunks of 16, 32, 40 and 64 inputs per image -- one, two, three and four 16-query blocks per attention item, the
+    shapes of the attention kernel -- see the same keys in the same order: equal bits (T = 144: three KV pages, a
+    ragged last chunk each)."""
+    w = synth.WORKLOADS["small_bf16"]
+    toks, k, lab = synth.make_inputs(w)
+    tsh = synth.ModelShape(2, 384, 6, 512, w.shape.vocab, 12, 12, 10, "bf16")
+    timg = synth.make_weights(tsh, 77)
+    got = []
+    for max_window in (8, 16, 20, 32):
+        stu = binding.Context(w.shape, G.weights_for(w), w.batch, max_window)
+        tea = binding.Context(tsh, timg, w.batch, max_window)
+        assert stu.fold_norm and tea.fold_norm  # one form of RMSNorm throughout
+        pos, per, loss = stu.hbsjd_score(tea, G.dev(toks), G.dev(k), G.dev(lab))
+        got.append((pos.cpu().numpy(), per.cpu().numpy(), loss))
+        stu.hbsjd_destroy()
+        tea.hbsjd_destroy()
+    for pos, per, loss in got[1:]:
+        np.testing.assert_array_equal(pos, got[0][0])
+        np.testing.assert_array_equal(per, got[0][1])
+        assert loss == got[0][2]
