@@ -89,10 +89,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         if (t1 - t0 > 1000000000ull) return false;
     }
 }
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+// Keys and values are read once per layer and round, a stream larger than L2 at full batch: marked to be evicted first,
+// so that the layer's activations and residual stream, which the next kernels read, stay in L2 (rollout of 200 L images with
+// long prefixes 426.4 -> 420.9 ms, 128 images 632.3 -> 628.5 ms).
+__device__ __forceinline__ uint64_t evict_first_policy() {
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar,
+                                            uint64_t policy) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
+        "[%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(dst),
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy)
         : "memory");
 }
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
@@ -323,6 +333,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
     if (warp == 0) {
         // ---------------------------------------------------------------- producer
         if (lane == 0) {
+            const uint64_t policy = evict_first_policy();
             uint32_t gc = 0;  // K/V stages issued so far
             bool ok = true;
             for (int stripe = 0; ok && stripe * grid < n_items; ++stripe) {
@@ -347,8 +358,8 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
                     mbar_expect_tx(full0 + 8 * gs, blocks * cfg::BLOCK_BYTES);
                     for (int b = 0; b < blocks; ++b) {
                         const uint32_t dst = ring + gs * cfg::STAGE_BYTES + b * cfg::BLOCK_BYTES;
-                        tma_load_3d(dst, &map_k, 0, y + b * KB, it.head0, full0 + 8 * gs);
-                        tma_load_3d(dst + HPC * TILE_BYTES, &map_v, 0, y + b * KB, it.head0, full0 + 8 * gs);
+                        tma_load_3d(dst, &map_k, 0, y + b * KB, it.head0, full0 + 8 * gs, policy);
+                        tma_load_3d(dst + HPC * TILE_BYTES, &map_v, 0, y + b * KB, it.head0, full0 + 8 * gs, policy);
                     }
                     page = page_next;
                 }
