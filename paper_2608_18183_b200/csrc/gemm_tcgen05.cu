@@ -133,24 +133,24 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32]) {
 }
 // PAIR: two CTAs of a cluster compute one 256 x BN tile with cta_group::2 MMAs; each CTA stages its own 128 rows
 // of A and its own BN/2 rows of W, which cuts the operand bytes per FLOP by a third against a 128 x BN tile.
-// WIDE: the epilogue stages a bf16 tile beside every fp32 tile (EPI_ADDNORM), 48 KB instead of 32 KB; the operand
-// ring gives up a stage or two for it.
+// WIDE: the epilogue stages a bf16 tile beside every fp32 tile (EPI_ADDNORM).
 template <int BN, bool PAIR = false, bool WIDE = false>
 struct Cfg {
     // as many stages as fit beside the epilogue staging: small tiles are latency-bound (one TMA round trip per ring
     // revolution), so a narrow tile gets a deep ring
-    static constexpr int STAGES = WIDE ? (PAIR ? 5 : (BN >= 256 ? 3 : (BN == 128 ? 5 : (BN == 64 ? 6 : 8))))
-                                       : (PAIR ? 6 : (BN >= 256 ? 4 : (BN == 128 ? 6 : 8)));
-    // k-blocks that share one full / empty barrier pair (one wait and one commit per KG x 4 MMAs)
-    static constexpr int KG = WIDE ? ((PAIR || BN >= 128) ? 1 : (BN == 64 ? 2 : 4)) : ((!PAIR && BN <= 64) ? 4 : 2);
+    static constexpr int STAGES = PAIR ? 6 : (BN >= 256 ? 4 : (BN == 128 ? 6 : 8));
+    // k-blocks that share one full / empty barrier pair (one wait and one commit per KG x 4 MMAs).  Every group costs the
+    // MMA stream about 190 clocks, as much as half a k-block of a narrow tile, so narrow tiles take four at a time.
+    static constexpr int KG = !PAIR && BN <= 64 ? 4 : 2;
     static constexpr int GROUPS = STAGES / KG;
     static_assert(GROUPS * KG == STAGES && GROUPS >= 2, "ring stages must split into whole barrier groups");
     static constexpr int A_BYTES = BM * BK * 2;
     static constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * BK * 2;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
     static constexpr int TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;  // two accumulators
-    // 4 epilogue warps x 2 buffers x (32 rows x 128 bytes fp32 [+ 32 rows x 64 bytes bf16])
-    static constexpr int WARP_STAGING = WIDE ? 2 * 6144 : 2 * 4096;
+    // 4 epilogue warps x 2 buffers x (32 rows x 128 bytes fp32 [+ 32 rows x 64 bytes bf16]); one buffer where the second
+    // would cost the ring a group: deeper groups win more than the epilogue loses (see the rule above)
+    static constexpr int WARP_STAGING = WIDE ? (BN == 32 ? 2 : 1) * 6144 : 2 * 4096;
     static constexpr int STAGING_BYTES = 4 * WARP_STAGING;
     static constexpr int SMEM = STAGES * STAGE_BYTES + STAGING_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
     static_assert(16 * STAGES + 32 + 8 + 8 <= 256, "barrier area");
@@ -438,7 +438,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                 if (EPI == EPI_ADDNORM) {
                     // this warp's staging: two buffers of (fp32 tile 4 KB, swizzled | bf16 tile 2 KB, dense)
                     const uint32_t sb32 =
-                        staging + (uint32_t)(warp - 2) * (uint32_t)cfg::WARP_STAGING + (uint32_t)(nchunk++ & 1u) * 6144u;
+                        staging + (uint32_t)(warp - 2) * (uint32_t)cfg::WARP_STAGING +
+                        (cfg::WARP_STAGING > 6144 ? (uint32_t)(nchunk++ & 1u) * 6144u : 0u);
                     const uint32_t sb16 = sb32 + 4096u;
                     float4 hcur[8];
 #pragma unroll
@@ -461,9 +462,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                         r[4 * v + 3] = __float_as_uint(x3);
                     }
                     ssq4[u] = ss;
-                    // one bulk tensor store per tile (the pair is one bulk group: the buffer used two chunks ago is
-                    // free once at most one group is still reading); rows past the buffers' capacity are clipped
-                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                    // one bulk tensor store per tile (the pair is one bulk group: of two buffers, the one used two chunks
+                    // ago is free once at most one group is still reading); rows past the buffers' capacity are clipped
+                    if (lane == 0) {
+                        if (cfg::WARP_STAGING > 6144) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                        else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                    }
                     __syncwarp();
 #pragma unroll
                     for (int v = 0; v < 8; ++v) {
