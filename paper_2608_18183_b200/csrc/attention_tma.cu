@@ -159,6 +159,16 @@ __device__ __forceinline__ bool item_at(const AttnArgs& a, const int* s_tab, int
     return true;
 }
 
+// 2^x for the softmax weights and corrections, by the one instruction.  exp2f also returns results below 2^-126; here they
+// meet a normaliser of at least 1 and outputs of the values' size, whose last bits they cannot reach, and the range
+// handling was a sixth of this kernel's instructions (rollout of six XL images 823.4 -> 813.9 ms, 24 L images one token
+// at a time 307.3 -> 303.3 ms).
+__device__ __forceinline__ float ex2(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // One or two consecutive blocks of 32 keys of one head for the 16 queries of a warp: S = Q K^T, causal mask, online
 // softmax in fp32, O += P V.  The blocks' score products, maxima, exponentials and row sums do not depend on one
 // another (the running maximum is the only link, and a maximum is exact in any order), so two blocks at a time hide
@@ -235,15 +245,15 @@ __device__ __forceinline__ void attend(uint32_t kt, uint32_t vt, uint32_t block_
     for (int b = 0; b < NB; ++b) {
         // key 0 is visible to every query, so the running maximum is finite from the first block on
         const float mx0 = fmaxf(m0, bx0[b]), mx1 = fmaxf(m1, bx1[b]);
-        corr0[b] = exp2f(m0 - mx0);
-        corr1[b] = exp2f(m1 - mx1);
+        corr0[b] = ex2(m0 - mx0);
+        corr1[b] = ex2(m1 - mx1);
         m0 = mx0;
         m1 = mx1;
         rs0[b] = rs1[b] = 0.f;
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
-            const float p0 = exp2f(sc[b][nt][0] - mx0), p1 = exp2f(sc[b][nt][1] - mx0);
-            const float p2 = exp2f(sc[b][nt][2] - mx1), p3 = exp2f(sc[b][nt][3] - mx1);
+            const float p0 = ex2(sc[b][nt][0] - mx0), p1 = ex2(sc[b][nt][1] - mx0);
+            const float p2 = ex2(sc[b][nt][2] - mx1), p3 = ex2(sc[b][nt][3] - mx1);
             rs0[b] += p0 + p1;
             rs1[b] += p2 + p3;
             // the softmax weights enter the P.V product as bf16 (the normaliser keeps the fp32 values)
