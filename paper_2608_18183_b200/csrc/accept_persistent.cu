@@ -471,8 +471,10 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                 }
                 thr = key_float(theta);
                 // the next item's guess: a lower end a little below this threshold, a top a little above this maximum
-                g_lo = thr - 0.3f * (mx - thr);
-                g_scale = (float)SEL_BINS / (1.4f * (mx - thr));
+                // (0.1 of the span: a step at 128 images, window 32, top-k 1000 took 310 us with 0.3, 303 with 0.1 and
+                // 0.05, 307 with 0.02, where rows start to miss the guess; the rollouts do not care)
+                g_lo = thr - 0.1f * (mx - thr);
+                g_scale = (float)SEL_BINS / (1.2f * (mx - thr));
                 have_guess = mx > thr;
             }
         }
