@@ -1,4 +1,6 @@
 """Distillation score on the GPU (Eq. 3) against the oracle, through the C ABI."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -180,3 +182,38 @@ def test_score_does_not_depend_on_the_chunk():
         np.testing.assert_array_equal(pos, got[0][0])
         np.testing.assert_array_equal(per, got[0][1])
         assert loss == got[0][2]
+
+
+@pytest.mark.parametrize("model,batch", [("tiny", 1), ("B", 3)])
+def test_score_of_contexts_on_one_stream_and_on_two_is_the_same(model, batch):
+    """Contexts that share a stream run side by side inside the call.  The same kernels do the same arithmetic in the
+    same order whatever the streams are, so every bit is equal; work of the shared stream before and after the call (the
+    tokens it reads, an overwrite of them) is ordered with it; an invalid argument leaves the contexts usable."""
+    import torch
+    w = synth.WORKLOADS[model]
+    w = synth.with_shape(w, shape=dataclasses.replace(w.shape, n_layers=2))
+    rng = np.random.default_rng(8)
+    toks = rng.integers(0, w.shape.vocab, size=(batch, w.shape.T)).astype(np.int32)
+    k = rng.integers(0, w.shape.T // 2, size=batch).astype(np.int32)
+    lab = rng.integers(0, w.shape.n_classes, size=batch).astype(np.int32)
+    simg, timg = (synth.make_weights(w.shape, s, target_entropy=None) for s in (5, 6))
+    out = []
+    for streams in ((torch.cuda.Stream(),) * 2, (torch.cuda.Stream(), torch.cuda.Stream()), (None, None)):
+        stu, tea = (binding.Context(w.shape, img, batch, w.window, stream=s) for img, s in zip((simg, timg), streams))
+        dk, dl, dt = G.dev(k), G.dev(lab), G.dev(toks)
+        bad = dk + w.shape.T
+        torch.cuda.synchronize()
+        with pytest.raises(binding.HbsjdError):
+            stu.hbsjd_score(tea, dt, bad, dl)
+        for _ in range(2):
+            if streams[0] is streams[1]:
+                with torch.cuda.stream(streams[0]):
+                    dt.fill_(0)
+                    dt.copy_(G.dev(toks))
+            pos, per, loss = stu.hbsjd_score(tea, dt, dk, dl)
+            out.append((pos.cpu().numpy(), per.cpu().numpy(), loss))
+        stu.hbsjd_destroy()
+        tea.hbsjd_destroy()
+    for pos, per, loss in out[1:]:
+        assert np.array_equal(pos, out[0][0]) and np.array_equal(per, out[0][1]) and loss == out[0][2]
+    assert out[0][2] > 0
