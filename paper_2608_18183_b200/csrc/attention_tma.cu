@@ -326,12 +326,17 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
     }
-    pdl_wait();
+    // The kernel before this one is the QKV projection, which lets this grid start only once its own wait is over: all
+    // that precedes the projection is complete here, the slot tables and the keys and values of earlier rounds among it
+    // (read through L2).  Queries and the window's own keys come after the wait.  The chain of look-ups and the first
+    // stages' copies, two microseconds, so lie beside the projection's tail: rollouts of 24 L images token by token
+    // 294.0 -> 284.5 ms, one L image 42.8 -> 41.0, 64 B images 82.9 -> 80.7, six XL images 813 -> 796, 128 L images 624 ->
+    // 617 ms.
     for (int s = threadIdx.x; s < a.S; s += blockDim.x) {
-        s_tab[s] = st.slot_order[s];
-        s_tab[a.S + s] = st.slot_n[s];
-        s_tab[2 * a.S + s] = st.slot_c[s];
-        s_tab[3 * a.S + s] = st.slot_img[s];
+        s_tab[s] = __ldcg(st.slot_order + s);
+        s_tab[a.S + s] = __ldcg(st.slot_n + s);
+        s_tab[2 * a.S + s] = __ldcg(st.slot_c + s);
+        s_tab[3 * a.S + s] = __ldcg(st.slot_img + s);
     }
     __syncthreads();
 
@@ -345,7 +350,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
         if (lane == 0) {
             const uint64_t policy = evict_first_policy();
             uint32_t gc = 0;  // K/V stages issued so far
-            bool ok = true;
+            bool ok = true, waited = false;
             for (int stripe = 0; ok && stripe * grid < n_items; ++stripe) {
                 const int pos = position(stripe);
                 Item it;
@@ -362,6 +367,10 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
                     if (!mbar_wait(empty0 + 8 * gs, ph ^ 1u, abort_flag)) {
                         ok = false;
                         break;
+                    }
+                    if (!waited && key0 + SK > it.c) {  // the first stage with keys of this forward
+                        pdl_wait();
+                        waited = true;
                     }
                     const int y = layer_row0 + page * a.kv.page + key0 % a.kv.page;
                     const int blocks = min(cfg::NBLK, (keys - key0 + KB - 1) / KB);
@@ -391,6 +400,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
         }
     } else {
         // ---------------------------------------------------------------- consumers
+        pdl_wait();
         const int cw = warp - 1;
         const int wh = cw / QB, wq = cw % QB;  // head within the item, q-block
         uint32_t gc = 0;

@@ -107,6 +107,7 @@ cudaError_t verify_enqueue(const VerifyDesc& d, const VerifyScratch& sc, const f
 
 // ---- persistent tensor-core ragged attention, bf16, head size 64 (attention_tma.cu)
 bool attention_tma_supported(const State& st, const KvView& kv);
+// To be launched directly behind a QKV projection of the same forward (whose late trigger it relies on, see pdl_wait).
 // q_rows_cap: row capacity of the q buffer.  Returns 0 or a negative code with a message in err.
 int launch_attention_tma(const State& st, int S, int layer, const bf16* q, int q_rows_cap, KvView kv, bf16* out,
                          int32_t* error_flag, cudaStream_t s, char* err, size_t errlen);
