@@ -148,7 +148,6 @@ __device__ __forceinline__ unsigned int radix_select_regs(const float (&x)[NCH][
 // st has V, W = 1 and a place for the error code.
 template <bool CFG, bool PROBS>
 __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArgs a) {
-    pdl_trigger();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int V = st.V, W = st.W;
     float* stage_c = (float*)smem_raw;
@@ -162,6 +161,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     pdl_wait();
+    pdl_trigger();  // k_commit reads what precedes this kernel before its own wait
     __syncthreads();
 
     // slot tables of the round in shared memory: the item walk below reads them at every step

@@ -1,6 +1,5 @@
 // C ABI of the rollout library (see include/hbsjd.h): context, host-side round loop, debug helpers.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -432,23 +431,26 @@ int enqueue_round(hbsjd_ctx* c) {
 // Waits for the round with this stamp and takes over its counters.  sync: by a stream synchronisation (the round is
 // the last one enqueued), else by polling what the round posts.
 int collect_round(hbsjd_ctx* c, uint32_t stamp, bool sync) {
-    const volatile RoundPost* p = c->post + (stamp & 1u);
+    const volatile unsigned long long* word = c->post[stamp & 1u].word;
     int rc;
     if (sync) {
         if ((rc = sync_counters(c))) return rc;
     } else {
         // the stream is asked now and then: after a CUDA error nothing will be posted
-        for (unsigned spins = 1; p->stamp != stamp; ++spins)
-            if (spins % (1u << 20) == 0) {
-                const cudaError_t e = cudaStreamQuery(c->stream);
-                if (e != cudaErrorNotReady && p->stamp != stamp) {
-                    CK(e);
-                    snprintf(c->err, sizeof(c->err), "a round ended without its counters");
-                    return HBSJD_ECUDA;
+        unsigned spins = 0;
+        for (int x = 8; x >= 0; --x) {
+            unsigned long long w;
+            while ((uint32_t)((w = word[x]) >> 32) != stamp)
+                if (++spins % (1u << 20) == 0) {
+                    const cudaError_t e = cudaStreamQuery(c->stream);
+                    if (e != cudaErrorNotReady && (uint32_t)(word[x] >> 32) != stamp) {
+                        CK(e);
+                        snprintf(c->err, sizeof(c->err), "a round ended without its counters");
+                        return HBSJD_ECUDA;
+                    }
                 }
-            }
-        std::atomic_thread_fence(std::memory_order_acquire);
-        for (int x = 0; x < 8; ++x) c->h_counters[x] = p->counters[x];
+            if (x < 8) c->h_counters[x] = (int32_t)(uint32_t)w;
+        }
         if ((rc = check_error(c))) return rc;
     }
     if (c->h_counters[CNT_LIVE_SETUP] != c->live) {
@@ -463,7 +465,7 @@ int collect_round(hbsjd_ctx* c, uint32_t stamp, bool sync) {
     c->stats.committed = c->h_counters[CNT_COMMITTED];
     c->stats.rejects = c->h_counters[CNT_REJECTS];
     c->live = c->h_counters[CNT_LIVE];
-    c->min_left = p->min_left;
+    c->min_left = (int)(uint32_t)word[8];
     return 0;
 }
 
@@ -905,15 +907,15 @@ int hbsjd_probs(hbsjd_ctx* c, const float* logits_c, const float* logits_u, int 
     if (!c || !logits_c || !probs || rows < 1 || !(temperature > 0.f) || top_k < 0 ||
         (((uintptr_t)logits_c | (uintptr_t)logits_u | (uintptr_t)probs) & 15))
         return HBSJD_EINVAL;
-    volatile RoundPost* post = c->post + 2;  // (only its error code is used)
-    post->counters[CNT_ERROR] = 0;
-    launch_probs(logits_c, logits_u, rows, c->d.vocab, cfg_scale, temperature, top_k, probs, c->post_dev[2].counters,
+    volatile int32_t* counters = (volatile int32_t*)c->post[2].word;  // (only the error code is used)
+    counters[CNT_ERROR] = 0;
+    launch_probs(logits_c, logits_u, rows, c->d.vocab, cfg_scale, temperature, top_k, probs, (int32_t*)c->post_dev[2].word,
                  c->stream);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->stream));
-    if (post->counters[CNT_ERROR] != 0) {
+    if (counters[CNT_ERROR] != 0) {
         snprintf(c->err, sizeof(c->err), "hbsjd_probs: a bounded device-side wait gave up (code %d)",
-                 post->counters[CNT_ERROR]);
+                 counters[CNT_ERROR]);
         return HBSJD_ETIMEOUT;
     }
     return HBSJD_OK;

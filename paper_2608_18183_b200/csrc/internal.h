@@ -40,10 +40,10 @@ enum { CNT_LIVE = 0, CNT_COMMITTED = 1, CNT_REJECTS = 2, CNT_LIVE_SETUP = 3, CNT
 
 // What the host needs to know of a finished round, written by the GPU into mapped host memory; stamp last.
 struct RoundPost {
-    int32_t counters[8];
-    int32_t min_left;  // fewest tokens still to commit over the images that are live after the round
-    uint32_t stamp;
-    int32_t pad[6];
+    // low half: the eight counters, then the fewest tokens still to commit over the images that are live after the
+    // round; high half: the round's stamp.  Eight bytes are written at once: a word with the stamp is the round's.
+    unsigned long long word[9];
+    unsigned long long pad[7];
 };
 
 struct AcceptArgs {

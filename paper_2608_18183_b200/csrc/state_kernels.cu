@@ -532,8 +532,8 @@ __global__ void __launch_bounds__(ACC_THREADS, 2) k_probs(const float* __restric
 }
 
 __global__ void __launch_bounds__(ACC_THREADS, 2) k_prob_accept(State st, AcceptArgs a) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();  // k_commit reads what precedes this kernel before its own wait
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* g = (float*)smem_raw;  // [V]
     AccShared& sh = *(AccShared*)(smem_raw + (size_t)st.V * sizeof(float));
@@ -665,7 +665,7 @@ void launch_prob_accept(const State& st, const AcceptArgs& a, cudaStream_t s) {
 // commits, advances the cursor -- the KV commit is this cursor move: entries at and after the new cursor are
 // recomputed by the next forward (Sec. 4.2 "Independent progress") -- and rebuilds the window.
 // One thread of every CTA of k_commit, when the CTA's slot is done (left: tokens the slot's image still has to commit,
-// INT_MAX if it has none or no image).  The last one hands the round's counters to the host, which polls the stamp in
+// INT_MAX if it has none or no image).  The last one hands the round's counters to the host, which polls the words in
 // its own memory, in place of a copy and a stream synchronisation.
 __device__ __forceinline__ void post_round(const State& st, const AcceptArgs& a, int left) {
     if (a.post == nullptr) return;
@@ -673,42 +673,62 @@ __device__ __forceinline__ void post_round(const State& st, const AcceptArgs& a,
     __threadfence();
     if (atomicAdd(&a.tally[0], 1) != (int)gridDim.x - 1) return;
     __threadfence();
-    volatile RoundPost* p = a.post;
+    // every word carries the stamp, so no fence across the bus has to order one word behind the others
+    const unsigned long long stamp = (unsigned long long)a.post_stamp << 32;
+    volatile unsigned long long* w = a.post->word;
 #pragma unroll
-    for (int x = 0; x < 8; ++x) p->counters[x] = *(volatile int32_t*)&st.counters[x];
-    p->min_left = *(volatile int32_t*)&a.tally[1];
+    for (int x = 0; x < 8; ++x) w[x] = stamp | *(volatile uint32_t*)&st.counters[x];
+    w[8] = stamp | *(volatile uint32_t*)&a.tally[1];
     a.tally[0] = 0;
     a.tally[1] = 0x7fffffff;
-    __threadfence_system();
-    p->stamp = a.post_stamp;
 }
 
+// What bounds it is a chain of look-ups, each a round trip to L2, with one token to draw in between.  The slot's entries
+// and the old window are therefore read before the wait (the kernel before this one triggers after its own, see
+// pdl_wait), flags and candidates together behind it, and the new window is put together in shared memory (rollouts of
+// four tiny images 4.74 -> 4.60 ms, one L image 40.9 -> 40.7, 64 B images 80.1 -> 79.9).
 __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) {
     pdl_trigger();
-    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* g = (float*)smem_raw;  // [V]
     AccShared& sh = *(AccShared*)(smem_raw + (size_t)st.V * sizeof(float));
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int slot = blockIdx.x;
-    const int n = st.slot_n[slot], img = st.slot_img[slot], c = st.slot_c[slot];
+    const int n = __ldcg(st.slot_n + slot), img = __ldcg(st.slot_img + slot), c = __ldcg(st.slot_c + slot);
     if (n == 0) {
+        pdl_wait();
         if (tid == 0) post_round(st, a, 0x7fffffff);
         return;
     }
-    const int V = st.V;
+    const int V = st.V, W = st.W, H = st.H;
     int32_t* seq = st.seq + (size_t)img * (st.T + 1);
     uint8_t* dl = st.delta + (size_t)img * (st.T + 1);
+    // by window position x = t - c - 1 (all in the selection's work area, W <= 64):
+    int32_t* old = (int32_t*)sh.work;  // [n] the drafts that were verified
+    int32_t* odl = old + W;            // [n] whether they were point masses
+    int32_t* win = odl + W;            // [2 W] refreshed candidates, then the new window
+    int32_t* hist = win + 2 * W;       // [W] the committed token H positions before x = n, n + 1, ...
+    static_assert(5 * 64 <= SEL_BINS + SEL_CAP, "window of the commit");
+    const int qbase = __ldcg(st.qbase + img);
+    if (wid == 0) {
+        for (int x = lane; x < W; x += 32) {
+            const int src = c + 1 + n + x - H;
+            if (x < n) {
+                old[x] = __ldcg(seq + c + 1 + x);
+                odl[x] = __ldcg(dl + c + 1 + x);
+            }
+            if (src >= 1 && src <= c) hist[x] = __ldcg(seq + src);
+        }
+    }
+    pdl_wait();
     if (wid == 0) {
         int j = -1;
-        for (int base = 0; base < n - 1; base += 32) {
-            const int i = base + lane;
-            const bool rej = (i < n - 1) && (a.flag[(size_t)img * st.Wmax + i] == 0);
+        for (int base = 0; base < n; base += 32) {
+            const int x = base + lane;
+            if (x < n) win[x] = a.cand_ref[(size_t)img * st.Wmax + x];
+            const bool rej = (x < n - 1) && (a.flag[(size_t)img * st.Wmax + x] == 0);
             const unsigned int b = __ballot_sync(0xffffffffu, rej);
-            if (b) {
-                j = base + __ffs(b) - 1;
-                break;
-            }
+            if (b && j < 0) j = base + __ffs(b) - 1;
         }
         if (lane == 0) {
             sh.jfirst = j;
@@ -727,7 +747,7 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
         if (wid != 0) return;
         m = *a.m_sync;
         j = -1;
-        tok = seq[c + m];
+        tok = old[m - 1];
     } else if (a.greedy) {
         if (wid != 0) return;
         tok = a.cand_rep[(size_t)img * st.Wmax + (m - 1)];
@@ -735,9 +755,9 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
         const int is = m - 1, t = c + m;
         const float* prow = a.pcur + ((size_t)img * st.Wmax + is) * V;
         const bool reject = j >= 0;
-        const int z = reject ? seq[t] : -1;
-        bool is_delta = reject && dl[t] != 0;
-        int qi = t - st.qbase[img] - 1;
+        const int z = reject ? old[is] : -1;
+        bool is_delta = reject && odl[is] != 0;
+        int qi = t - qbase - 1;
         if (reject && !is_delta && (qi < 0 || qi >= st.Wmax)) {  // cannot be valid: record it, skip the access
             if (tid == 0) atomicExch(&st.counters[CNT_ERROR], ERR_BAD_PROPOSAL_ROW);
             is_delta = true;
@@ -792,42 +812,42 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
         }
         if (wid != 0) return;
     }
-    // warp 0: commit and draft refresh.  A serial walk over the window (a load and a store per draft that the compiler
-    // may not reorder) was most of the work behind the sampled token.
+    // warp 0: commit and draft refresh
     const int c2 = c + m;
     if (lane == 0) {
-        seq[c2] = tok;
-        dl[c2] = 0;
         st.cursor[img] = c2;
         st.qbase[img] = c;
         st.m_last[img] = m;
         st.j_last[img] = j;
     }
+    const int last = c2 < st.T ? m - 1 + min(W, st.T - c2) : m;  // positions of the new window end before x = last
+    for (int x = lane; x < n; x += 32)
+        if (x < m) win[x] = x == m - 1 ? tok : old[x];
     __syncwarp();
-    if (c2 < st.T) {
-        const int end = c2 + min(st.W, st.T - c2) - 1;  // last draft position
-        for (int t = c2 + 1 + lane; t <= min(end, c + n); t += 32) {
-            seq[t] = a.cand_ref[(size_t)img * st.Wmax + (t - c - 1)];
-            dl[t] = 0;
+    // history drafts copy the token H back, which may itself be one of them: H positions at a time
+    const int step = min(32, H);
+    for (int x0 = n; x0 < last; x0 += step) {
+        const int x = x0 + lane;
+        if (lane < step && x < last) {
+            int32_t v;
+            if (x >= H) {
+                v = win[x - H];
+            } else if (c + 1 + x - H >= 1) {
+                v = hist[x - n];
+            } else {
+                uint32_t w[4];
+                philox4x32_10((uint32_t)img, (uint32_t)(c + 1 + x), a.round, 0u, a.seed_lo, a.seed_hi, w);
+                v = (int32_t)(((uint64_t)w[3] * (uint64_t)st.V) >> 32);
+            }
+            win[x] = v;
         }
         __syncwarp();
-        // history drafts copy the token H back, which may itself be one of them: H positions at a time
-        const int step = min(32, st.H);
-        for (int t0 = c + n + 1; t0 <= end; t0 += step) {
-            const int t = t0 + lane, src = t - st.H;
-            if (lane < step && t <= end) {
-                if (src >= 1) {
-                    seq[t] = seq[src];
-                } else {
-                    uint32_t w[4];
-                    philox4x32_10((uint32_t)img, (uint32_t)t, a.round, 0u, a.seed_lo, a.seed_hi, w);
-                    seq[t] = (int32_t)(((uint64_t)w[3] * (uint64_t)st.V) >> 32);
-                }
-                dl[t] = 1;
-            }
-            __syncwarp();
-        }
     }
+    for (int x = m - 1 + lane; x < last; x += 32) {
+        seq[c + 1 + x] = win[x];
+        dl[c + 1 + x] = x >= n ? 1 : 0;
+    }
+    __syncwarp();
     if (lane != 0) return;
     if (c2 < st.T) atomicAdd(&st.counters[CNT_LIVE], 1);
     atomicAdd(&st.counters[CNT_COMMITTED], m);
@@ -837,8 +857,8 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
 
 // One CTA: every thread walks the accept flags of its slots; block-wide minimum of the commits.
 __global__ void k_sync_min(State st, AcceptArgs a, int32_t* __restrict__ m_sync) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();  // k_commit reads what precedes this kernel before its own wait
     __shared__ int red[32];
     int best = 0x7fffffff;
     for (int slot = threadIdx.x; slot < a.S; slot += blockDim.x) {

@@ -120,3 +120,33 @@ def test_verify_reports_invalid_state_arrays_instead_of_touching_memory(ctx, wha
     ctx.hbsjd_verify(G.verify_desc(good, 1, 0), dg["logits"], dg["q"], p_out, dg["cursor"], dg["seq"], dg["delta"],
                      dg["qbase"], m_out)
     assert int(m_out.cpu().numpy()[good["cursor"] < good["T"]].min()) >= 1
+
+
+@pytest.mark.parametrize("W,H", [(1, 1), (2, 1), (16, 40), (33, 1), (33, 32), (64, 7), (64, 64), (64, 100)])
+@pytest.mark.parametrize("greedy", [False, True])
+def test_commit_of_every_window_and_history_offset(W, H, greedy):
+    """The new window is put together from old drafts, candidates and history tokens: windows of one lane step and of
+    two, history that copies itself (H below the window), that reaches back before the first token (random drafts), and
+    that lies wholly in the committed part; a cursor at 0, near the end and at it.  All whole numbers: equal."""
+    import torch
+    w = synth.WORKLOADS["tiny_bf16"]
+    ctx = binding.Context(w.shape, G.weights_for(w), 12, W)
+    case = G.verify_case(W + H, B=12, W=W, T=128, V=256, H=H)
+    d = {k: G.dev(case[k]) for k in ("logits", "q", "cursor", "seq", "delta", "qbase")}
+    p_out = torch.zeros((12, W, 256), device="cuda")
+    m_out = torch.zeros(12, dtype=torch.int32, device="cuda")
+    ctx.hbsjd_verify(G.verify_desc(case, 5, 3, greedy), d["logits"], d["q"], p_out, d["cursor"], d["seq"], d["delta"],
+                     d["qbase"], m_out)
+    p, cur, seq, dl = (x.cpu().numpy() for x in (p_out, d["cursor"], d["seq"], d["delta"]))
+    for b in range(12):
+        c = int(case["cursor"][b])
+        if c >= 128:
+            assert np.array_equal(seq[b], case["seq"][b])
+            continue
+        s2, d2 = case["seq"][b].copy(), case["delta"][b].copy()
+        nc, m, _ = O.replay_round(256, 128, W, H, greedy, 5, b, 3, c, s2, d2, p[b, :min(W, 128 - c)], case["q"][b],
+                                  int(case["qbase"][b]))
+        assert nc == cur[b] and m == int(m_out[b])
+        np.testing.assert_array_equal(s2, seq[b])
+        np.testing.assert_array_equal(d2[nc + 1:nc + W], dl[b][nc + 1:nc + W])
+    ctx.hbsjd_destroy()
