@@ -409,6 +409,7 @@ int enqueue_round(hbsjd_ctx* c) {
     a.post_stamp = ++c->post_seq;
     a.post = c->post_dev + (a.post_stamp & 1u);
     a.tally = c->tally;
+    a.early = c->bf16_model;
     {
         const int ps = prof_begin(c, HBSJD_PROF_ACCEPT, 0.0);
         launch_prob_accept(c->st, a, c->stream);

@@ -81,7 +81,8 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
     constexpr int KG = cfg::KG;
     constexpr bool RES = cfg::RES;
     extern __shared__ unsigned char smem_raw[];
-    if (EPI != EPI_QKV) pdl_trigger();
+    constexpr bool LATE = EPI == EPI_QKV || EPI == EPI_STORE;  // see pdl_wait
+    if (!LATE) pdl_trigger();
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t ring = (raw + 1023u) & ~1023u;
     const uint32_t tile_at = ring + cfg::STAGES * cfg::STAGE_BYTES - raw;  // byte offset of the accumulator tile
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
 
     // -------------------------------------------------------------------- consumers
     pdl_wait();
-    if (EPI == EPI_QKV) pdl_trigger();  // attention reads what precedes this kernel before its own wait
+    if (LATE) pdl_trigger();  // the next kernel reads what precedes this one before its own wait
     const int row = m0 + lane, col = n0 + warp * 32;  // epilogue warp w: columns 32 w .. 32 w + 31 of the tile
     const bool finisher = warp * 32 < TN && lane < TM && row < g.M;
     float4 pre[8];  // old residual values: they travel while the main loop runs

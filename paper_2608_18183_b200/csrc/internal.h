@@ -63,6 +63,7 @@ struct AcceptArgs {
     RoundPost* post;         // mapped host memory
     int32_t* tally;          // [2] device: CTAs done, fewest tokens left of a live image; left at {0, INT_MAX}
     uint32_t post_stamp;
+    bool early;  // the kernel before is a forward's LM head, which triggers after its own wait (see pdl_wait)
 };
 
 // ---- row operations (model_kernels.cu)

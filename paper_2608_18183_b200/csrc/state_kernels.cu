@@ -958,6 +958,7 @@ cudaError_t verify_enqueue(const VerifyDesc& d, const VerifyScratch& sc, const f
     a.post = nullptr;
     a.tally = nullptr;
     a.post_stamp = 0;
+    a.early = false;
     // the commit counters accumulate with atomics: they must start at zero on every call
     cudaError_t e = cudaMemsetAsync(sc.counters, 0, 8 * sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
