@@ -15,9 +15,10 @@ typedef __nv_bfloat16 bf16;
 // preceding grid in the stream has completed and its writes are visible) after pdl_trigger() (lets the
 // next grid's CTAs be scheduled as SMs free up), so launch latency and kernel prologues overlap the
 // previous kernel's tail.  Nothing before pdl_wait() touches global memory that any kernel writes, but
-// for pairs whose first kernel triggers after its own wait, so that all that precedes it is complete
-// when the second starts and may be read there before the wait: the QKV projection and attention; a
-// forward's LM head and the accept kernel; the accept kernel (or k_sync_min) and k_commit.
+// for pairs whose first kernel triggers after its own wait, so that all that precedes it is complete when
+// the second starts and may be read there before the wait: embedding, RMSNorm or the folded residual
+// projection and the QKV projection; the QKV projection and attention; a forward's LM head and the
+// accept kernel; the accept kernel (or k_sync_min) and k_commit.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -121,10 +121,10 @@ __device__ __forceinline__ RowDst qkv_row(const GemmArgs& g, int row, bool valid
         const int i = row % st.W;
         const int slot = (row / st.W) % g.S;
         const int br = row / (st.W * g.S);
-        rd.valid = i < st.slot_n[slot];
+        rd.valid = i < __ldcg(st.slot_n + slot);  // (through L2: may be read before the grid wait)
         if (rd.valid) {
-            rd.s = st.slot_c[slot] + i;
-            rd.kvoff = g.kv.offset(g.layer, br * st.Bmax + st.slot_img[slot], rd.s);
+            rd.s = __ldcg(st.slot_c + slot) + i;
+            rd.kvoff = g.kv.offset(g.layer, br * st.Bmax + __ldcg(st.slot_img + slot), rd.s);
         }
     }
     return rd;

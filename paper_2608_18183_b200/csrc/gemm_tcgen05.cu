@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                                                               const GemmArgs g) {
     using cfg = Cfg<BN, PAIR, EPI == EPI_ADDNORM>;
     extern __shared__ unsigned char smem_raw[];
-    constexpr bool LATE = EPI == EPI_QKV || EPI == EPI_STORE;  // see pdl_wait
+    constexpr bool LATE = EPI == EPI_QKV || EPI == EPI_STORE || EPI == EPI_ADDNORM;  // see pdl_wait
     if (!LATE) pdl_trigger();
     const uint32_t rank = PAIR ? cluster_rank() : 0u;       // 0 = leader of the pair
     const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;  // tile walker id

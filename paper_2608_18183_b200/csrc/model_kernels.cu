@@ -108,8 +108,8 @@ template <typename TA>
 __global__ void __launch_bounds__(128) k_embed(State st, int S, const TA* __restrict__ tok_emb,
                                                const TA* __restrict__ cls_emb, float* __restrict__ h,
                                                bf16* __restrict__ hb, float* __restrict__ ssq) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int row = blockIdx.x;
     const int i = row % st.W;
     const int slot = (row / st.W) % S;
@@ -156,12 +156,12 @@ template void launch_embed<bf16>(const State&, int, const bf16*, const bf16*, fl
 template <typename TA, int VEC_ITERS>
 __global__ void __launch_bounds__(256) k_rmsnorm_warp(const float* __restrict__ h, const TA* __restrict__ gain,
                                                       TA* __restrict__ out, int M, int D, float eps) {
-    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     // gain read four at a time: 32 two-byte loads per thread in their place cost the rollout of 128 L images 12 of 645 ms
     struct __align__(4 * sizeof(TA)) Gain4 { TA g[4]; };
     pdl_wait();
+    pdl_trigger();
     if (row >= M) return;
     const float4* x4 = reinterpret_cast<const float4*>(h + (size_t)row * D);
     float4 v[VEC_ITERS];
@@ -201,8 +201,8 @@ __global__ void __launch_bounds__(256) k_rmsnorm_warp(const float* __restrict__ 
 template <typename TA>
 __global__ void k_rmsnorm(const float* __restrict__ h, const TA* __restrict__ gain, TA* __restrict__ out, int D,
                           float eps) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     __shared__ float red[32];
     const int row = blockIdx.x;
     const float* x = h + (size_t)row * D;
