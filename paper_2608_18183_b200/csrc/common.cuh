@@ -11,14 +11,16 @@ namespace hbsjd {
 
 typedef __nv_bfloat16 bf16;
 
-// Programmatic dependent launch: every kernel of the library starts with pdl_wait() (blocks until the
-// preceding grid in the stream has completed and its writes are visible) after pdl_trigger() (lets the
-// next grid's CTAs be scheduled as SMs free up), so launch latency and kernel prologues overlap the
-// previous kernel's tail.  Nothing before pdl_wait() touches global memory that any kernel writes, but
-// for pairs whose first kernel triggers after its own wait, so that all that precedes it is complete when
-// the second starts and may be read there before the wait: embedding, RMSNorm or the folded residual
-// projection and the QKV projection; the QKV projection and attention; a forward's LM head and the
-// accept kernel; the accept kernel (or k_sync_min) and k_commit.
+// Programmatic dependent launch: every kernel of the library has a pdl_wait() (blocks until the preceding
+// grid in the stream has completed and its writes are visible) and a pdl_trigger() (lets the next grid's
+// CTAs be scheduled as SMs free up), so launch latency and kernel prologues overlap the previous kernel's
+// tail.  The decoder's kernels trigger after their own wait: triggered before it, a third kernel's CTAs took
+// the shared memory that the second's would have had (one L image 39.4 -> 37.0 ms with the gate/up projection
+// triggering late, 24 L images token by token 274.0 -> 271.1).  All that precedes such a kernel is complete
+// when the next one starts and may be read there before the wait; else nothing before pdl_wait() touches
+// global memory that any kernel writes.  The pairs that make use of it: embedding, RMSNorm or the folded
+// residual projection and the QKV projection; the QKV projection and attention; a forward's LM head and
+// the accept kernel; the accept kernel (or k_sync_min) and k_commit.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -81,8 +81,6 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
     constexpr int KG = cfg::KG;
     constexpr bool RES = cfg::RES;
     extern __shared__ unsigned char smem_raw[];
-    constexpr bool LATE = EPI == EPI_QKV || EPI == EPI_STORE || EPI == EPI_ADDNORM;  // see pdl_wait
-    if (!LATE) pdl_trigger();
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t ring = (raw + 1023u) & ~1023u;
     const uint32_t tile_at = ring + cfg::STAGES * cfg::STAGE_BYTES - raw;  // byte offset of the accumulator tile
@@ -178,7 +176,7 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
 
     // -------------------------------------------------------------------- consumers
     pdl_wait();
-    if (LATE) pdl_trigger();  // the next kernel reads what precedes this one before its own wait
+    pdl_trigger();  // (late: see pdl_wait)
     const int row = m0 + lane, col = n0 + warp * 32;  // epilogue warp w: columns 32 w .. 32 w + 31 of the tile
     const bool finisher = warp * 32 < TN && lane < TM && row < g.M;
     float4 pre[8];  // old residual values: they travel while the main loop runs

@@ -169,8 +169,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                                                               const GemmArgs g) {
     using cfg = Cfg<BN, PAIR, EPI == EPI_ADDNORM>;
     extern __shared__ unsigned char smem_raw[];
-    constexpr bool LATE = EPI == EPI_QKV || EPI == EPI_STORE || EPI == EPI_ADDNORM;  // see pdl_wait
-    if (!LATE) pdl_trigger();
     const uint32_t rank = PAIR ? cluster_rank() : 0u;       // 0 = leader of the pair
     const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;  // tile walker id
     const int units = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
@@ -262,7 +260,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
         for (int kb = cfg::GROUPS * cfg::KG; kb < num_kb; ++kb) tma_prefetch_2d(&map_w, kb * BK, n0);
     }
     pdl_wait();
-    if (LATE) pdl_trigger();  // the next kernel reads what precedes this one before its own wait
+    pdl_trigger();  // (late: see pdl_wait)
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
