@@ -14,9 +14,10 @@ typedef __nv_bfloat16 bf16;
 // Programmatic dependent launch: every kernel of the library has a pdl_wait() (blocks until the preceding
 // grid in the stream has completed and its writes are visible) and a pdl_trigger() (lets the next grid's
 // CTAs be scheduled as SMs free up), so launch latency and kernel prologues overlap the previous kernel's
-// tail.  The decoder's kernels trigger after their own wait: triggered before it, a third kernel's CTAs took
-// the shared memory that the second's would have had (one L image 39.4 -> 37.0 ms with the gate/up projection
-// triggering late, 24 L images token by token 274.0 -> 271.1).  All that precedes such a kernel is complete
+// tail.  All but k_commit, the small fp32 GEMM and attention's small grids trigger after their own wait:
+// triggered before it, a third kernel's CTAs took the shared memory that the second's would have had (one L
+// image 39.4 -> 37.0 ms with the gate/up projection triggering late, 24 L images token by token 274.0 ->
+// 271.1, the small kernels of four tiny images 4.50 -> 4.46).  All that precedes such a kernel is complete
 // when the next one starts and may be read there before the wait; else nothing before pdl_wait() touches
 // global memory that any kernel writes.  The pairs that make use of it: embedding, RMSNorm or the folded
 // residual projection and the QKV projection; the QKV projection and attention; a forward's LM head and

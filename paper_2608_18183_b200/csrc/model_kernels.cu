@@ -10,8 +10,8 @@ namespace hbsjd {
 // One block.  Builds the slot tables of the next forward.  Full: slot b = image b, n = 0 for inactive
 // images.  Compact: active images gathered in increasing image order (block-wide exclusive scan).
 __global__ void k_setup(State st, int phase, int compact) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     __shared__ int warp_tot[32];
     __shared__ int carry, sum_keys, sum_n;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -96,8 +96,8 @@ void launch_setup(const State& st, int phase, int compact, cudaStream_t s) {
 }
 
 __global__ void k_noop() {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
 }
 void launch_noop(cudaStream_t s) { launch_k(k_noop, dim3(1), dim3(32), 0, s); }
 
@@ -238,8 +238,8 @@ template void launch_rmsnorm<bf16>(const float*, const bf16*, bf16*, int, int, f
 template <typename TA>
 __global__ void k_rope_kv(State st, int S, int layer, const float* __restrict__ qkv,
                           const float* __restrict__ rope_cs, TA* __restrict__ q, KvView kv) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int row = blockIdx.x;
     const int i = row % st.W;
     const int slot = (row / st.W) % S;
@@ -289,8 +289,8 @@ template void launch_rope_kv<bf16>(const State&, int, int, const float*, const f
 template <typename TA>
 __global__ void k_attention_ref(State st, int S, int layer, const TA* __restrict__ q, KvView kv,
                                 TA* __restrict__ out) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     extern __shared__ float smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int row = blockIdx.x;
@@ -370,8 +370,8 @@ template void launch_attention_ref<bf16>(const State&, int, int, const bf16*, Kv
 // ------------------------------------------------------------------ SwiGLU: act = silu(gate) * up
 template <typename TA>
 __global__ void k_swiglu(const float* __restrict__ gu, TA* __restrict__ act, int F) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int row = blockIdx.y;
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= F) return;
@@ -392,8 +392,8 @@ template void launch_swiglu<bf16>(const float*, bf16*, int, int, cudaStream_t);
 template <typename TA>
 __global__ void __launch_bounds__(256) k_gemm_simt(const TA* __restrict__ A, const TA* __restrict__ W,
                                                    float* __restrict__ C, int M, int N, int K, int accumulate) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     __shared__ float As[16][64 + 4];
     __shared__ float Bs[16][64 + 4];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;

@@ -116,8 +116,8 @@ __device__ float bikl_row(const float* __restrict__ s, const float* __restrict__
 
 __global__ void __launch_bounds__(BK_THREADS) k_bikl_rows(const float* __restrict__ ls, const float* __restrict__ lt,
                                                           int V, float* __restrict__ out) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const size_t row = blockIdx.x;
     const float d = bikl_row(ls + row * V, lt + row * V, V);
     if (threadIdx.x == 0) out[row] = d;
@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(BK_THREADS) k_bikl_slots(State st, const float
                                                            const float* __restrict__ lt,
                                                            const int32_t* __restrict__ prefix_len,
                                                            float* __restrict__ pos) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int i = blockIdx.x, slot = blockIdx.y;
     if (i >= st.slot_n[slot]) return;
     const int img = st.slot_img[slot];
@@ -145,8 +145,8 @@ __global__ void __launch_bounds__(BK_THREADS) k_bikl_slots(State st, const float
 // 0..T-1 = class token, x_1..x_{T-1}), processed like a prefix of length T.
 __global__ void k_score_init(State st, const int32_t* __restrict__ tokens, const int32_t* __restrict__ labels,
                              const int32_t* __restrict__ prefix_len, float* __restrict__ pos) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.x;
     int32_t* seq = st.seq + (size_t)b * (st.T + 1);
     uint8_t* dl = st.delta + (size_t)b * (st.T + 1);
@@ -173,8 +173,8 @@ __global__ void k_score_init(State st, const int32_t* __restrict__ tokens, const
 // One CTA; fixed summation order (lane-strided partial sums, shuffle tree, then images in index order).
 __global__ void k_score_reduce(int B, int T, const int32_t* __restrict__ prefix_len, const float* __restrict__ pos,
                                float* __restrict__ per_image, float* __restrict__ loss) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int b = wid; b < B; b += nw) {
         const int k = prefix_len[b];

@@ -12,8 +12,8 @@ namespace hbsjd {
 // ------------------------------------------------------------------ state init (Sec. 4.2 "Independent rollout states")
 __global__ void k_init_state(State st, const int32_t* __restrict__ prefix_tokens,
                              const int32_t* __restrict__ prefix_len, const int32_t* __restrict__ labels) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.x;
     const int k = prefix_len[b];
     int32_t* seq = st.seq + (size_t)b * (st.T + 1);
@@ -42,8 +42,8 @@ void launch_init_state(const State& st, const int32_t* prefix_tokens, const int3
 }
 
 __global__ void k_prefill_advance(State st, int S) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int slot = blockIdx.x * blockDim.x + threadIdx.x;
     if (slot >= S) return;
     const int n = st.slot_n[slot];
@@ -57,8 +57,8 @@ void launch_prefill_advance(const State& st, int S, cudaStream_t s) {
 // Initial window: every draft is the token H positions back, or a keyed uniform token where that
 // position does not exist; all are point-mass proposals.  Reserved round value 0xFFFFFFFF.
 __global__ void k_init_window(State st, uint32_t seed_lo, uint32_t seed_hi) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= st.B) return;
     const int c = st.cursor[b];
@@ -84,8 +84,8 @@ void launch_init_window(const State& st, uint32_t seed_lo, uint32_t seed_hi, cud
 }
 
 __global__ void k_export_tokens(State st, int32_t* __restrict__ out) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.x;
     for (int t = threadIdx.x; t < st.T; t += blockDim.x)
         out[(size_t)b * st.T + t] = st.seq[(size_t)b * (st.T + 1) + t + 1];
@@ -96,8 +96,8 @@ void launch_export_tokens(const State& st, int32_t* out, cudaStream_t s) {
 }
 
 __global__ void k_calib_state(State st, int live) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.x;
     int32_t* seq = st.seq + (size_t)b * (st.T + 1);
     uint8_t* dl = st.delta + (size_t)b * (st.T + 1);
@@ -522,8 +522,8 @@ __device__ void prob_pipeline(float* g, const float* __restrict__ lc, const floa
 __global__ void __launch_bounds__(ACC_THREADS, 2) k_probs(const float* __restrict__ lc, const float* __restrict__ lu,
                                                        int V, float cfg_scale, float temperature, int top_k,
                                                        float* __restrict__ p) {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* g = (float*)smem_raw;
     AccShared& sh = *(AccShared*)(smem_raw + (size_t)V * sizeof(float));
