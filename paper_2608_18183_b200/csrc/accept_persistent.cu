@@ -367,6 +367,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                 const unsigned int k = (unsigned int)a.top_k;
                 unsigned int theta = 0u;
                 float lo = g_lo, scale = g_scale;
+                bool found = false;
                 for (int source = have_guess ? 0 : 1; source < 3; ++source) {
                     if (source > 0) {
                         if (source == 1) {
@@ -381,6 +382,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                             lo = mn;
                         }
                         scale = (float)SEL_BINS / (mx - lo);
+                        if (!(scale > 0.f)) break;  // -inf among the entries, or a span beyond fp32: no bins
 #pragma unroll
                         for (int ch = 0; ch < NCH; ++ch)
 #pragma unroll
@@ -471,7 +473,13 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                         __syncthreads();  // (6)
                         theta = sh.theta;
                     }
+                    found = true;
                     break;
+                }
+                if (!found) {  // no histogram, or fewer than k entries that compare (NaN among them): by the keys
+                    theta = radix_select_regs(x, tid, V, k, sh);
+                    __syncthreads();
+                    sh.hist[tid] = 0u;  // the radix passes used the first 256 bins
                 }
                 thr = key_float(theta);
                 // the next item's guess: a lower end a little below this threshold, a top a little above this maximum
@@ -479,7 +487,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                 // 0.05, 307 with 0.02, where rows start to miss the guess; the rollouts do not care)
                 g_lo = thr - 0.1f * (mx - thr);
                 g_scale = (float)SEL_BINS / (1.2f * (mx - thr));
-                have_guess = mx > thr;
+                have_guess = mx > thr && g_scale > 0.f && g_lo > -INFINITY;
             }
         }
 

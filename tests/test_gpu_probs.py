@@ -84,3 +84,45 @@ def test_more_rows_than_ctas(V):
     lc, lu = (np.round(np.clip(x, -40, 40) * 1024).astype(np.float32) / 1024 for x in (lc, lu))
     _check(ctx, lc, lu, 2.0, 0.5, 100)
     ctx.hbsjd_destroy()
+
+
+@pytest.mark.parametrize("V", [4096, 4160, 8192, 16384, 20480])
+def test_masked_huge_and_nan_logits(V):
+    """Rows as masks leave them, through both kernels (the persistent one runs 4160 to 16384): -inf or the type's lowest
+    value in nearly every place, in every other row only (the threshold guess goes from row to row), a span beyond
+    fp32 with the threshold inside its upper end, NaN where both branches are masked under guidance, and more NaN than
+    V - k, which count among the k largest.  Against the pipeline in 64 bits."""
+    import torch
+    sh = synth.ModelShape(1, 64, 1, 64, V, 4, 4, 3, "bf16")
+    ctx = binding.Context(sh, synth.make_weights(sh, 3, target_entropy=None), 2, 4)
+    g = torch.Generator(device="cuda").manual_seed(V)
+    rows, low = 300, torch.finfo(torch.float32).min
+    base = torch.randn(rows, V, generator=g, device="cuda") * 3
+    hide = torch.rand(rows, V, generator=g, device="cuda") < 0.9
+
+    def check(lc, k, lu=None, kept=None):
+        p = ctx.hbsjd_probs(lc, lu, 2.0 if lu is not None else 1.0, 1.0, k)
+        x = (lc if lu is None else lu + 2.0 * (lc - lu)).double()
+        x = x.masked_fill(torch.isnan(x), float("-inf"))
+        kth = torch.topk(x, kept or k, dim=-1).values[:, -1:]
+        ref = torch.softmax(x.masked_fill(x < kth, float("-inf")), -1)
+        assert bool(((p.double() - ref).abs() <= 1e-6 + 1e-5 * ref).all())
+
+    for value in (float("-inf"), low):
+        for every in (1, 2):
+            lc = base.clone()
+            lc[::every][hide[::every]] = value
+            check(lc, 1000)
+            check(lc, 40)
+    lc = base.clone()
+    lc[:, 100:107] = 3e38
+    lc[:, 107:3000] = -3e38
+    for k in (5, 7, 8, 1000):
+        check(lc, k)
+    masked = [torch.where(hide, float("-inf"), x) for x in (base, base.flip(0))]
+    check(masked[0], 200, lu=masked[1])
+    lc = base.clone()
+    lc[::3, 50:150] = float("nan")
+    check(lc[::3].contiguous(), V - 40, kept=V - 140)
+    check(lc, 1000)
+    ctx.hbsjd_destroy()
