@@ -456,9 +456,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                         const unsigned int hit = __ballot_sync(0xffffffffu, lane < nc && gt < krem && krem <= ge);
                         theta = __shfl_sync(0xffffffffu, ku, __ffs(hit) - 1);
                     } else if (nc > SEL_CAP) {
-                        theta = radix_select_regs(x, tid, V, k, sh);
-                        __syncthreads();
-                        sh.hist[tid] = 0u;  // the radix passes used the first 256 bins
+                        break;
                     } else {
                         for (int u = tid; u < nc; u += PT) {
                             const unsigned int ku = sh.cand[u];
@@ -476,7 +474,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                     found = true;
                     break;
                 }
-                if (!found) {  // no histogram, or fewer than k entries that compare (NaN among them): by the keys
+                if (!found) {  // no histogram, a crowded bin, or fewer than k entries that compare (NaN): by the keys
                     theta = radix_select_regs(x, tid, V, k, sh);
                     __syncthreads();
                     sh.hist[tid] = 0u;  // the radix passes used the first 256 bins
