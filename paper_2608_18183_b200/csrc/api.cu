@@ -494,7 +494,7 @@ int run_rounds(hbsjd_ctx* c, int max_rounds) {
 
 void free_all(hbsjd_ctx* c) {
     void* ptrs[] = {c->w_img, c->rope_cs, c->kc, c->vc, c->page_table, c->st.cursor, c->st.seq, c->st.delta,
-                    c->st.qbase, c->st.label, c->st.klen, c->st.pfill, c->st.slot_img, c->st.slot_c, c->st.slot_n, c->st.slot_order,
+                    c->st.qbase, c->st.label, c->st.klen, c->st.pfill, c->st.slot_img, c->st.slot_c, c->st.slot_n, c->st.slot_sorted,
                     c->st.counters, c->st.m_last, c->st.j_last, c->pbuf[0], c->pbuf[1], c->flag, c->cand_rep,
                     c->cand_ref, c->h, c->qkv, c->gu, c->logits, c->a, c->q, c->o, c->act, c->ssq,
                     c->stage_tok, c->stage_len, c->stage_lab, c->stage_out, c->verify_scratch,
@@ -651,7 +651,7 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
         (rc = dev_alloc(c, &st.label, Bm)) || (rc = dev_alloc(c, &st.klen, Bm)) ||
         (rc = dev_alloc(c, &st.pfill, Bm)) || (rc = dev_alloc(c, &st.slot_img, Bm)) ||
         (rc = dev_alloc(c, &st.slot_c, Bm)) || (rc = dev_alloc(c, &st.slot_n, Bm)) ||
-        (rc = dev_alloc(c, &st.slot_order, Bm)) ||
+        (rc = dev_alloc(c, &st.slot_sorted, Bm)) ||
         (rc = dev_alloc(c, &st.counters, (size_t)8)) || (rc = dev_alloc(c, &st.m_last, Bm)) ||
         (rc = dev_alloc(c, &st.j_last, Bm)) || (rc = dev_alloc(c, &c->pbuf[0], Bm * Wm * V)) ||
         (rc = dev_alloc(c, &c->pbuf[1], Bm * Wm * V)) || (rc = dev_alloc(c, &c->flag, Bm * Wm)) ||

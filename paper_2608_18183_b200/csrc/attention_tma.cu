@@ -53,6 +53,9 @@ struct AttnCfg {
     static constexpr int STAGES = QB == 1 ? 3 : 98304 / STAGE_BYTES;
     static constexpr int CTAS = QB == 1 ? 3 : 2;              // per SM
 };
+// A CTA's work list in shared memory: as many entries as leave the CTAs per SM alone; later items (beyond 148 x CTAS x 512)
+// are looked up in global memory.
+constexpr int LIST_MAX = 512;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -141,21 +144,27 @@ struct AttnArgs {
     bool few;  // the grid leaves half of the SMs free
 };
 
-// Position `pos` of the sorted item list -> work item.  Returns false for an inactive slot.
+// Position `pos` of the sorted item list, the CTA's item number `stripe` -> work item.  Returns false for an inactive slot.
 struct Item {
     int prow, crow, c, n, head0;
 };
-__device__ __forceinline__ bool item_at(const AttnArgs& a, const int* s_tab, int pos, Item& it) {
+__device__ __forceinline__ bool item_at(const AttnArgs& a, uint32_t list, int stripe, int pos, Item& it) {
     const State& st = a.st;
     const int per_slot = st.nb * a.G;
     const int r = pos / per_slot, rem = pos % per_slot;
     const int br = rem / a.G, g = rem % a.G;
-    const int slot = s_tab[r];  // slot with the r-th longest context
-    it.n = s_tab[a.S + slot];
+    // slot, n, c, image of the slot with the r-th longest context
+    int4 e;
+    if (stripe < LIST_MAX)
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(e.x), "=r"(e.y), "=r"(e.z), "=r"(e.w)
+                     : "r"(list + 16u * stripe));
+    else
+        e = __ldcg(st.slot_sorted + r);
+    it.n = e.y;
     if (it.n == 0) return false;
-    it.c = s_tab[2 * a.S + slot];
-    it.prow = br * a.S + slot;
-    it.crow = br * st.Bmax + s_tab[3 * a.S + slot];
+    it.c = e.z;
+    it.prow = br * a.S + e.x;
+    it.crow = br * st.Bmax + e.w;
     it.head0 = g * a.hpc;
     return true;
 }
@@ -317,7 +326,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
     const uint32_t full0 = bars, empty0 = bars + 8 * STAGES;
     unsigned char* tail = smem_raw + (bars - raw) + 16 * STAGES;
     volatile uint32_t* abort_flag = (volatile uint32_t*)tail;
-    int* s_tab = (int*)(tail + 16);  // [4][S]: order, n, c, image of every slot
+    const uint32_t list = bars + 16 * STAGES + 16;  // [min(stripes, LIST_MAX)] int4: slots of this CTA's items
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -336,18 +345,16 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
     // stages' copies, two microseconds, so lie beside the projection's tail: rollouts of 24 L images token by token
     // 294.0 -> 284.5 ms, one L image 42.8 -> 41.0, 64 B images 82.9 -> 80.7, six XL images 813 -> 796, 128 L images 624 ->
     // 617 ms.
-    for (int s = threadIdx.x; s < a.S; s += blockDim.x) {
-        s_tab[s] = __ldcg(st.slot_order + s);
-        s_tab[a.S + s] = __ldcg(st.slot_n + s);
-        s_tab[2 * a.S + s] = __ldcg(st.slot_c + s);
-        s_tab[3 * a.S + s] = __ldcg(st.slot_img + s);
-    }
-    __syncthreads();
-
     const int n_items = a.S * st.nb * a.G;
     const int grid = (int)gridDim.x, cta = (int)blockIdx.x;
     // stripe s of the sorted list: CTA j takes position s * grid + j, in reversed order on odd stripes
     auto position = [&](int stripe) { return stripe * grid + ((stripe & 1) ? grid - 1 - cta : cta); };
+    // (warp 0 has the barriers to set up)
+    for (int s = threadIdx.x - 32; warp > 0 && s < LIST_MAX && s * grid < n_items; s += NCW * 32) {
+        const int pos = position(s);
+        if (pos < n_items) ((int4*)(tail + 16))[s] = __ldcg(st.slot_sorted + pos / (st.nb * a.G));
+    }
+    __syncthreads();
 
     if (warp == 0) {
         // ---------------------------------------------------------------- producer
@@ -358,7 +365,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
             for (int stripe = 0; ok && stripe * grid < n_items; ++stripe) {
                 const int pos = position(stripe);
                 Item it;
-                if (pos >= n_items || !item_at(a, s_tab, pos, it)) continue;
+                if (pos >= n_items || !item_at(a, list, stripe, pos, it)) continue;
                 const int keys = it.c + it.n, nstages = (keys + SK - 1) / SK;
                 const int32_t* pages = a.kv.table + (size_t)it.crow * a.kv.pages_per_row;
                 const int layer_row0 = a.layer * a.kv.n_pages * a.kv.page;
@@ -413,7 +420,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
         for (int stripe = 0; ok && stripe * grid < n_items; ++stripe) {
             const int pos = position(stripe);
             Item it;
-            if (pos >= n_items || !item_at(a, s_tab, pos, it)) continue;
+            if (pos >= n_items || !item_at(a, list, stripe, pos, it)) continue;
             const int c = it.c, n = it.n;
             const int keys = c + n, nstages = (keys + SK - 1) / SK;
             // ---- this warp's queries: 16 rows x 64 dims as A fragments.  Rows at or past n hold whatever the buffer
@@ -435,7 +442,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
             {   // the next item's query rows towards L1 while this item's keys stream (one 128-byte line per row)
                 const int pos2 = (stripe + 1) * grid < n_items ? position(stripe + 1) : n_items;
                 Item nx;
-                if (lane < 16 && pos2 < n_items && item_at(a, s_tab, pos2, nx)) {
+                if (lane < 16 && pos2 < n_items && item_at(a, list, stripe + 1, pos2, nx)) {
                     const bf16* nq = a.q + ((size_t)nx.prow * st.W + min(wq * 16 + lane, st.W - 1)) * st.D +
                                      (nx.head0 + wh) * DH;
                     asm volatile("prefetch.global.L1 [%0];" ::"l"(nq));
@@ -491,9 +498,9 @@ template <int QB>
 cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, AttnArgs a, cudaStream_t s) {
     using cfg = AttnCfg<QB>;
     constexpr int threads = (cfg::NCW + 1) * 32;
-    const int smem = 1024 + cfg::STAGES * cfg::STAGE_BYTES + 16 * cfg::STAGES + 16 + 16 * a.S;
+    constexpr int fixed = 1024 + cfg::STAGES * cfg::STAGE_BYTES + 16 * cfg::STAGES + 16, most = fixed + 16 * LIST_MAX;
     static int configured[64] = {0};
-    cudaError_t e = ensure_dynamic_smem(k_attention_tma<QB>, smem, configured);
+    cudaError_t e = ensure_dynamic_smem(k_attention_tma<QB>, most, configured);
     if (e != cudaSuccess) return e;
     // resident CTAs per SM (registers and shared memory): the grid is exactly what is resident at once
     static int resident[64] = {0};
@@ -502,7 +509,7 @@ cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, AttnArgs a, 
     dev &= 63;
     if (resident[dev] == 0) {
         int n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_attention_tma<QB>, threads, (size_t)smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_attention_tma<QB>, threads, (size_t)most);
         if (e != cudaSuccess) return e;
         resident[dev] = n < 1 ? 1 : (n > cfg::CTAS ? cfg::CTAS : n);
     }
@@ -511,13 +518,15 @@ cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, AttnArgs a, 
     long grid = (long)device_sm_count() * per_sm;
     if (grid > items) grid = items;
     a.few = 2 * grid <= device_sm_count();
+    const long stripes = (items + grid - 1) / grid;
+    const int smem = fixed + 16 * (int)(stripes < LIST_MAX ? stripes : LIST_MAX);
     return launch_k(k_attention_tma<QB>, dim3((unsigned)grid), dim3(threads), (size_t)smem, s, mk, mv, a);
 }
 
 }  // namespace
 
 bool attention_tma_supported(const State& st, const KvView& kv) {
-    return st.dh == DH && st.W <= 64 && kv.page % (2 * KB) == 0 && st.Hh % 2 == 0 && st.slot_order != nullptr;
+    return st.dh == DH && st.W <= 64 && kv.page % (2 * KB) == 0 && st.Hh % 2 == 0 && st.slot_sorted != nullptr;
 }
 
 int launch_attention_tma(const State& st, int S, int layer, const bf16* q, int q_rows_cap, KvView kv, bf16* out,

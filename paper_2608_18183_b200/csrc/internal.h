@@ -29,7 +29,7 @@ struct State {
     int32_t* slot_img; // [Bmax]
     int32_t* slot_c;   // [Bmax] first sequence index of the slot's inputs
     int32_t* slot_n;   // [Bmax] number of inputs (0: inactive slot)
-    int32_t* slot_order;  // [Bmax] slots by context length c + n, longest first (null: not built)
+    int4* slot_sorted; // [Bmax] (slot, n, c, image) by context length c + n, longest first (null: not built)
     int32_t* counters; // [8], see CNT_*
     int32_t* m_last;   // [Bmax] tokens committed in the last round
     int32_t* j_last;   // [Bmax] first-reject index of the last round (-1 none)

@@ -250,3 +250,23 @@ def test_kernel_profile_bins_add_up():
     assert ctx.hbsjd_profile_read()["gemm"]["launches"] == g["launches"]
     ctx.hbsjd_destroy()
 
+
+
+@pytest.mark.parametrize("batch,dim,window", [(9000, 128, 20), (5000, 1024, 33), (300, 128, 16)])
+def test_batches_beyond_a_ctas_work_list(batch, dim, window):
+    """Thousands of images in one forward: the attention kernel's share of the work list does not depend on the batch (a
+    table of every slot did not fit beside the key ring above 8300 images), and at 5000 images of 16 heads with guidance
+    a CTA has more items (541) than the 512 entries it holds.  An image's tokens do not depend on the others."""
+    sh = synth.ModelShape(1, dim, dim // 64, 64, 64, 4, 4, 3, "bf16")
+    c = binding.Context(sh, synth.make_weights(sh, 3, target_entropy=None), batch, window)
+    rng = np.random.default_rng(batch)
+    toks = rng.integers(0, 64, size=(batch, 16)).astype(np.int32)
+    k = rng.integers(0, 16, size=batch).astype(np.int32)
+    lab = rng.integers(0, 3, size=batch).astype(np.int32)
+    few = 150
+    p = binding.make_params(window, 4, cfg_scale=2.0, exec_mode=binding.EXEC_FULL, seed=5)
+    out, st = c.hbsjd_rollout(G.dev(toks), G.dev(k), G.dev(lab), p)
+    assert st["committed"] == int((16 - k).sum())
+    out2, _ = c.hbsjd_rollout(G.dev(toks[:few]), G.dev(k[:few]), G.dev(lab[:few]), p)
+    np.testing.assert_array_equal(out[:few].cpu().numpy(), out2.cpu().numpy())
+    c.hbsjd_destroy()
