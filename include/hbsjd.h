@@ -143,7 +143,9 @@ int hbsjd_calibrate_gamma(hbsjd_ctx *c, int batch, int window, int guidance, int
 /* One verification round (Sec. 4.2 "Batched verification" .. "Independent progress") on the state left
  * by hbsjd_rollout or a previous hbsjd_round.  *live_out (HOST) = images still incomplete afterwards.
  * A sequence of hbsjd_rollout(max_rounds = 0) and hbsjd_round calls yields the same tokens as one
- * monolithic hbsjd_rollout.  Errors: HBSJD_ESTATE without a preceding hbsjd_rollout. */
+ * monolithic hbsjd_rollout.  Errors: HBSJD_ESTATE without a preceding hbsjd_rollout.
+ * A round that ends in an error (here or inside hbsjd_rollout) is not counted: nothing runs any more when the call
+ * returns, and the round index, statistics and proposals stand as before it. */
 int hbsjd_round(hbsjd_ctx *c, int *live_out);
 
 /* Copies the current token rows (committed tokens, then drafts) to DEVICE int32 [batch, T]. */
@@ -226,6 +228,11 @@ int hbsjd_debug_fold_norm(hbsjd_ctx *c, int on);
  * check that results do not depend on where a row's pages lie (Sec. 4.2: per-image KV-cache locations).  Only
  * before the first rollout of the context; HBSJD_ESTATE afterwards. */
 int hbsjd_debug_shuffle_pages(hbsjd_ctx *c, uint64_t seed);
+
+/* Plants the error that a bounded device wait leaves when it gives up in the next round with this index (host memory only
+ * until then; -1 takes it back), so that tests can check what a failed round leaves (Sec. 4.2 rounds; the paper has no
+ * counterpart). */
+int hbsjd_debug_fail_round(hbsjd_ctx *c, int round);
 
 /* Probability pipeline of the verification step on caller-supplied logits (Sec. 4.2: "verification uses the
  * fused guided logits"): p = softmax(top_k((l_u + s (l_c - l_u)) / temperature)), ties at the k-th value kept.

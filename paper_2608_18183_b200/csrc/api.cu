@@ -61,6 +61,7 @@ struct hbsjd_ctx {
     hbsjd_params P;
     bool have_rollout;
     int live, round, last_S, last_compact;
+    int fail_round;  // debugging: the round in which an error is planted (-1: none)
     int dbg_layer;  // layer of the last hbsjd_debug_forward (-1: none); selects the KV rows of hbsjd_debug_read
     hbsjd_stats stats;
     long long launches;
@@ -386,6 +387,10 @@ int enqueue_round(hbsjd_ctx* c) {
     const int compact = choose_compact(c, c->live);
     const int S = compact ? c->live : c->st.B;
     launch_setup(c->st, 0, compact, c->stream);
+    if (c->round == c->fail_round) {  // code 1: a bounded wait that gave up
+        c->fail_round = -1;
+        CK(cudaMemsetAsync(c->st.counters + CNT_ERROR, 1, 1, c->stream));
+    }
     c->launches++;
     int rc = forward_any(c, S, true);
     if (rc) return rc;
@@ -470,21 +475,35 @@ int collect_round(hbsjd_ctx* c, uint32_t stamp, bool sync) {
     return 0;
 }
 
+// A round (the oldest of `in_flight` ones) failed: nothing runs any more when the call returns, and the host's record is
+// the one before that round.  Rounds behind it found its error and changed nothing (see k_setup).
+int round_failed(hbsjd_ctx* c, int rc, int in_flight) {
+    cudaStreamSynchronize(c->stream);
+    c->round -= in_flight;
+    c->parity ^= in_flight & 1;
+    return rc;
+}
+
 // Rounds until every image is complete (max_rounds < 0) or that many are done.  The live count decides the next
 // round's shape, so a round is normally enqueued once the one before has been collected; but an image commits at most
 // `window` tokens per round, so while every live image has more than that left the round in flight cannot change the
 // count, and the next one is enqueued behind it (the GPU then never waits for the host between rounds).
 int run_rounds(hbsjd_ctx* c, int max_rounds) {
     int enqueued = 0, in_flight = 0, rc;
+    uint32_t oldest = c->post_seq + 1u;  // stamp of the oldest round in flight
     while (true) {
         const bool more = max_rounds < 0 || enqueued < max_rounds;
         // (event times of a round are folded at its synchronisation: no running ahead while they are taken)
         if (more && c->live > 0 && (in_flight == 0 || (in_flight == 1 && c->min_left > c->st.W && !c->profiling))) {
-            if ((rc = enqueue_round(c))) return rc;
+            if ((rc = enqueue_round(c))) {  // it left no trace; the round before it still counts
+                const int rb = in_flight > 0 ? collect_round(c, oldest, c->profiling) : 0;
+                return rb ? round_failed(c, rb, in_flight) : rc;
+            }
             ++enqueued;
             ++in_flight;
         } else if (in_flight > 0) {
-            if ((rc = collect_round(c, c->post_seq - (uint32_t)in_flight + 1u, c->profiling))) return rc;
+            if ((rc = collect_round(c, oldest, c->profiling))) return round_failed(c, rc, in_flight);
+            ++oldest;
             --in_flight;
         } else {
             return 0;
@@ -756,6 +775,7 @@ int hbsjd_create(hbsjd_ctx** out, const hbsjd_model_desc* m, const void* weights
     c->ref_attention = false;
     c->stream = (cudaStream_t)cuda_stream;
     c->dbg_layer = -1;
+    c->fail_round = -1;
     c->err[0] = 0;
     const int rc = create_impl(c, weights, weight_bytes);
     if (rc != 0) {
@@ -1207,7 +1227,8 @@ int hbsjd_round(hbsjd_ctx* c, int* live_out) {
     }
     if (c->live > 0) {
         int rc = enqueue_round(c);
-        if (rc || (rc = collect_round(c, c->post_seq, true))) return rc;
+        if (rc) return rc;
+        if ((rc = collect_round(c, c->post_seq, true))) return round_failed(c, rc, 1);
     }
     if (live_out) *live_out = c->live;
     return HBSJD_OK;
@@ -1399,6 +1420,12 @@ int hbsjd_debug_fold_norm(hbsjd_ctx* c, int on) {
         return HBSJD_ESTATE;
     }
     c->fold_norm = on != 0;
+    return HBSJD_OK;
+}
+
+int hbsjd_debug_fail_round(hbsjd_ctx* c, int round) {
+    if (!c) return HBSJD_EINVAL;
+    c->fail_round = round;
     return HBSJD_OK;
 }
 

@@ -282,3 +282,58 @@ def test_window_one_probabilistic_rollout_is_the_oracle_ar_sampler():
         same += int(np.array_equal(out.cpu().numpy(), ar))
     assert same >= 2  # fp32: a flip needs a sampling target within ~1e-6 of a bin edge
     ctx.hbsjd_destroy()
+
+
+@pytest.mark.parametrize("name,mode", [("tiny", "FULL"), ("small_bf16", "COMPACT"), ("small_bf16", "SYNC")])
+def test_a_failed_round_leaves_the_state_that_a_single_round_leaves(name, mode):
+    """Inside hbsjd_rollout the next round is already enqueued when a round's error is read.  It must not move the state:
+    round index, cursors, tokens, drafts and proposals after the failed call are those of the same rounds called one by
+    one, the context goes on from there to the same tokens, and a new rollout is unaffected."""
+    w = synth.WORKLOADS[name]
+    toks, k, lab = synth.make_inputs(w)
+    k = np.minimum(k, 5)  # every image is far from its end: rounds run ahead
+    args = [G.dev(x) for x in (toks, k, lab)]
+    par = dict(exec_mode=getattr(binding, "EXEC_" + mode))
+    ctxs = [binding.Context(w.shape, G.weights_for(w), w.batch, w.window) for _ in range(2)]
+    want, _ = ctxs[0].hbsjd_rollout(*args, G.gpu_params(w, 3, **par))
+    for c in ctxs:
+        c.hbsjd_rollout(*args, G.gpu_params(w, 3, max_rounds=0, **par))
+    for _ in range(3):
+        ctxs[0].hbsjd_round()
+    for c in ctxs:
+        c.hbsjd_debug_fail_round(3)
+    with pytest.raises(binding.HbsjdError) as e:
+        ctxs[0].hbsjd_round()
+    assert e.value.code == -5
+    with pytest.raises(binding.HbsjdError) as e:
+        ctxs[1].hbsjd_rollout(*args, G.gpu_params(w, 3, **par))
+    assert e.value.code == -5
+    states = [c.hbsjd_get_state() for c in ctxs]
+    assert states[0][0] == 3
+    for x, y in zip(*states):
+        np.testing.assert_array_equal(x, y)
+    for c in ctxs:
+        while c.hbsjd_round():
+            pass
+    np.testing.assert_array_equal(*(c.hbsjd_tokens().cpu().numpy() for c in ctxs))
+    for c in ctxs:
+        out, _ = c.hbsjd_rollout(*args, G.gpu_params(w, 3, **par))
+        assert bool((out == want).all())
+        c.hbsjd_destroy()
+
+
+@pytest.mark.parametrize("first", [2, 3, 7])
+def test_rounds_after_a_rollout_stopped_early(first):
+    """max_rounds of two and more ends with rounds run ahead; single rounds go on from there."""
+    w = synth.WORKLOADS["small_bf16"]
+    toks, k, lab = synth.make_inputs(w)
+    args = [G.dev(x) for x in (toks, k, lab)]
+    c = binding.Context(w.shape, G.weights_for(w), w.batch, w.window)
+    want, st = c.hbsjd_rollout(*args, G.gpu_params(w, 9))
+    assert st["rounds"] > first
+    _, st = c.hbsjd_rollout(*args, G.gpu_params(w, 9, max_rounds=first))
+    assert st["rounds"] == first
+    while c.hbsjd_round():
+        pass
+    assert bool((c.hbsjd_tokens() == want).all())
+    c.hbsjd_destroy()
