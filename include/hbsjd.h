@@ -17,7 +17,9 @@
  *     all scratch, allocated in hbsjd_create and freed in hbsjd_destroy.
  *   - All GPU work is enqueued on the stream given to hbsjd_create (a
  *     cudaStream_t passed as void*, NULL = the legacy default stream).  Calls
- *     that report a live count synchronise that stream before returning.
+ *     that report a live count synchronise that stream before returning.  A
+ *     rollout waits for its rounds as the process has set the device's schedule
+ *     flag (cudaSetDeviceFlags): by default it polls.
  *   - A context is not thread-safe; use one context per host thread / stream.
  *   - There is no CPU path: if no CUDA device is usable the calls fail with
  *     HBSJD_ECUDA.

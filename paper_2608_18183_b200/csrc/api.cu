@@ -7,6 +7,8 @@
 #include <type_traits>
 #include <vector>
 
+#include <sched.h>
+
 #include "../../include/hbsjd.h"
 #include "internal.h"
 
@@ -434,19 +436,32 @@ int enqueue_round(hbsjd_ctx* c) {
     return 0;
 }
 
-// Waits for the round with this stamp and takes over its counters.  sync: by a stream synchronisation (the round is
-// the last one enqueued), else by polling what the round posts.
-int collect_round(hbsjd_ctx* c, uint32_t stamp, bool sync) {
+// How the host waits for a round: BLOCK by a stream synchronisation (the round is the last one enqueued), else by polling
+// what the round posts, YIELD giving up the processor between polls.
+enum Wait { BLOCK, YIELD, SPIN };
+
+// The way of waiting that the process has asked CUDA for (cudaSetDeviceFlags); BLOCK while event times are taken, which
+// are folded at the round's synchronisation.
+Wait host_wait(const hbsjd_ctx* c) {
+    unsigned flags = 0;
+    if (c->profiling || cudaGetDeviceFlags(&flags) != cudaSuccess) return BLOCK;
+    flags &= cudaDeviceScheduleMask;
+    return flags == cudaDeviceScheduleBlockingSync ? BLOCK : flags == cudaDeviceScheduleYield ? YIELD : SPIN;
+}
+
+// Waits for the round with this stamp and takes over its counters.
+int collect_round(hbsjd_ctx* c, uint32_t stamp, Wait wait) {
     const volatile unsigned long long* word = c->post[stamp & 1u].word;
     int rc;
-    if (sync) {
+    if (wait == BLOCK) {
         if ((rc = sync_counters(c))) return rc;
     } else {
         // the stream is asked now and then: after a CUDA error nothing will be posted
         unsigned spins = 0;
         for (int x = 8; x >= 0; --x) {
             unsigned long long w;
-            while ((uint32_t)((w = word[x]) >> 32) != stamp)
+            while ((uint32_t)((w = word[x]) >> 32) != stamp) {
+                if (wait == YIELD) sched_yield();
                 if (++spins % (1u << 20) == 0) {
                     const cudaError_t e = cudaStreamQuery(c->stream);
                     if (e != cudaErrorNotReady && (uint32_t)(word[x] >> 32) != stamp) {
@@ -455,6 +470,7 @@ int collect_round(hbsjd_ctx* c, uint32_t stamp, bool sync) {
                         return HBSJD_ECUDA;
                     }
                 }
+            }
             if (x < 8) c->h_counters[x] = (int32_t)(uint32_t)w;
         }
         if ((rc = check_error(c))) return rc;
@@ -489,20 +505,20 @@ int round_failed(hbsjd_ctx* c, int rc, int in_flight) {
 // `window` tokens per round, so while every live image has more than that left the round in flight cannot change the
 // count, and the next one is enqueued behind it (the GPU then never waits for the host between rounds).
 int run_rounds(hbsjd_ctx* c, int max_rounds) {
+    const Wait wait = host_wait(c);
     int enqueued = 0, in_flight = 0, rc;
     uint32_t oldest = c->post_seq + 1u;  // stamp of the oldest round in flight
     while (true) {
         const bool more = max_rounds < 0 || enqueued < max_rounds;
-        // (event times of a round are folded at its synchronisation: no running ahead while they are taken)
-        if (more && c->live > 0 && (in_flight == 0 || (in_flight == 1 && c->min_left > c->st.W && !c->profiling))) {
+        if (more && c->live > 0 && (in_flight == 0 || (in_flight == 1 && c->min_left > c->st.W && wait != BLOCK))) {
             if ((rc = enqueue_round(c))) {  // it left no trace; the round before it still counts
-                const int rb = in_flight > 0 ? collect_round(c, oldest, c->profiling) : 0;
+                const int rb = in_flight > 0 ? collect_round(c, oldest, wait) : 0;
                 return rb ? round_failed(c, rb, in_flight) : rc;
             }
             ++enqueued;
             ++in_flight;
         } else if (in_flight > 0) {
-            if ((rc = collect_round(c, oldest, c->profiling))) return round_failed(c, rc, in_flight);
+            if ((rc = collect_round(c, oldest, wait))) return round_failed(c, rc, in_flight);
             ++oldest;
             --in_flight;
         } else {
@@ -1228,7 +1244,7 @@ int hbsjd_round(hbsjd_ctx* c, int* live_out) {
     if (c->live > 0) {
         int rc = enqueue_round(c);
         if (rc) return rc;
-        if ((rc = collect_round(c, c->post_seq, true))) return round_failed(c, rc, 1);
+        if ((rc = collect_round(c, c->post_seq, BLOCK))) return round_failed(c, rc, 1);
     }
     if (live_out) *live_out = c->live;
     return HBSJD_OK;

@@ -1,6 +1,9 @@
 """Edge and degenerate cases of the rollout on the GPU: nothing to generate, one token to generate, one image,
 one kept token, no-op guidance, temperature and history offsets the standard workloads do not use, the largest
 vocabulary of the verification kernels."""
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -270,3 +273,41 @@ def test_batches_beyond_a_ctas_work_list(batch, dim, window):
     out2, _ = c.hbsjd_rollout(G.dev(toks[:few]), G.dev(k[:few]), G.dev(lab[:few]), p)
     np.testing.assert_array_equal(out[:few].cpu().numpy(), out2.cpu().numpy())
     c.hbsjd_destroy()
+
+
+_WAIT = """
+import ctypes, sys, time
+flags = int(sys.argv[1])
+cu = ctypes.CDLL("libcuda.so.1")
+dev = ctypes.c_int()
+assert cu.cuInit(0) == 0 and cu.cuDeviceGet(ctypes.byref(dev), 0) == 0
+assert cu.cuDevicePrimaryCtxSetFlags_v2(dev, flags) == 0
+import torch
+from paper_2608_18183_b200 import binding, synth
+sh = synth.ModelShape(4, 1024, 16, 1024, 256, 16, 16, 3, "bf16")
+c = binding.Context(sh, synth.make_weights(sh, 3, target_entropy=None), 600, 32)
+g = torch.Generator(device="cuda").manual_seed(1)
+toks = torch.randint(0, 256, (600, 256), device="cuda", dtype=torch.int32, generator=g)
+k = torch.full((600,), 100, device="cuda", dtype=torch.int32)
+lab = torch.zeros_like(k)
+p = binding.make_params(32, 16, seed=4, max_rounds=20, exec_mode=binding.EXEC_FULL)
+out, _ = c.hbsjd_rollout(toks, k, lab, p)
+wall, cpu = time.perf_counter(), time.thread_time()
+for _ in range(3):
+    c.hbsjd_rollout(toks, k, lab, p, out)
+wall, cpu = time.perf_counter() - wall, time.thread_time() - cpu
+print(cpu / wall, int(out.long().sum()))
+"""
+
+
+def test_a_process_that_asked_for_blocking_waits_does_not_poll():
+    """The schedule flag of the device (4: blocking synchronisation, 2: yield) is the process's choice of how its threads
+    wait.  Rounds here take milliseconds and about a tenth of that to enqueue: a thread that blocks is mostly asleep, one
+    that polls never is.  The tokens do not depend on it."""
+    out = {}
+    for flags in (0, 2, 4):
+        r = subprocess.run([sys.executable, "-c", _WAIT, str(flags)], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        out[flags] = r.stdout.split()
+    assert float(out[4][0]) < 0.5, out
+    assert out[0][1] == out[2][1] == out[4][1]
