@@ -204,9 +204,10 @@ int hbsjd_gemm(hbsjd_ctx *c, const void *A, const void *W, float *C, int M, int 
  * forward itself uses, C += A W^T together with the bf16 copy and the per-row partial sums of squares of the new C
  * (written to buffers of the context), so that it can be timed and checked alone.
  * hbsjd_gemm `reps` times back to back before the one synchronisation (micro-benchmarks time the decoder's GEMM
- * shapes the way a forward issues them), and -- acc_wait_ns > 0, bf16 contexts -- with the bounded wait of the
- * epilogue warps on their accumulator shortened to that many nanoseconds (Sec. 4.2 verifier forward; the paper has
- * no counterpart of the failure path).  A limit shorter than the main loop makes a healthy pipeline take the
+ * shapes the way a forward issues them), and -- acc_wait_ns > 0, bf16 contexts -- with a bounded wait shortened to that
+ * many nanoseconds (Sec. 4.2 verifier forward; the paper has no counterpart of the failure path): of the epilogue
+ * warps on their accumulator, or, with a tile of the kernel for few rows, of its warps on their operands (tile 0
+ * then means the former).  A limit shorter than the main loop makes a healthy pipeline take the
  * time-out path: every role leaves its loop, copies and MMAs in flight are drained, TMEM is freed, the call
  * returns HBSJD_ETIMEOUT with C partly written, and the context stays usable.  Tests use it to exercise that path.
  * tile (bf16 contexts, accumulate 0 or 1): 0 = the library's own choice for the shape; 32, 64, 128, 256 = one CTA

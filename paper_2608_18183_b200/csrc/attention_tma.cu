@@ -397,17 +397,15 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
             if (!ok) {
                 *abort_flag = 1;
                 atomicExch(a.error_flag, 5);
-                // copies already issued must land before shared memory is released: wait for the stages armed last
-                const uint32_t first = gc > (uint32_t)STAGES ? gc - STAGES : 0u;
-                for (uint32_t g2 = first; g2 < gc; ++g2) {
-                    unsigned long long t0, t1;
-                    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-                    while (!mbar_try(full0 + 8 * (g2 % STAGES), (g2 / STAGES) & 1u)) {
-                        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
-                        if (t1 - t0 > 1000000000ull) break;
-                    }
-                }
             }
+            // copies must land before shared memory is released (they have, unless somebody gave up): the stages armed last
+            unsigned long long t0, t1;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+            for (uint32_t g2 = gc > (uint32_t)STAGES ? gc - STAGES : 0u; g2 < gc; ++g2)
+                while (!mbar_try(full0 + 8 * (g2 % STAGES), (g2 / STAGES) & 1u)) {
+                    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+                    if (t1 - t0 > 1000000000ull) break;
+                }
         }
     } else {
         // ---------------------------------------------------------------- consumers
@@ -457,7 +455,8 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
 
             for (int sg = 0; sg < nstages; ++sg, ++gc) {
                 const uint32_t gs = gc % STAGES, ph = (gc / STAGES) & 1u;
-                if (!mbar_wait(full0 + 8 * gs, ph, abort_flag)) {
+                // one answer for the warp: the products take all its lanes
+                if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * gs, ph, abort_flag))) {
                     ok = false;
                     break;
                 }

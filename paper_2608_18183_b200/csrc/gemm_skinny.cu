@@ -161,15 +161,12 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
                 tma_load_3d(dst0 + st * cfg::STAGE_BYTES, map, 0, y, gi * KG, full0 + 8 * st);
                 ++armed;
             }
-            if (*abort_flag) {
-                // leaving early: what this thread has requested must have landed before shared memory is released
-                // (the other producer's bytes too: the barrier completes with both, or the limit ends the wait)
-                for (int gi = armed > cfg::STAGES ? armed - cfg::STAGES : 0; gi < armed; ++gi) {
-                    const unsigned long long t0 = globaltimer_ns();
-                    while (!mbar_try(full0 + 8 * (gi % cfg::STAGES), (uint32_t)(gi / cfg::STAGES) & 1u))
-                        if (globaltimer_ns() - t0 > 1000000000ull) break;
-                }
-            }
+            // What this thread has requested must have landed before shared memory is released.  It has, unless
+            // somebody gave up: a stage completes with both producers' bytes, or the limit ends the wait.
+            const unsigned long long t0 = globaltimer_ns();
+            for (int gi = armed > cfg::STAGES ? armed - cfg::STAGES : 0; gi < armed; ++gi)
+                while (!mbar_try(full0 + 8 * (gi % cfg::STAGES), (uint32_t)(gi / cfg::STAGES) & 1u))
+                    if (globaltimer_ns() - t0 > 1000000000ull) break;
         }
         return;
     }
@@ -211,10 +208,12 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
             return ring + ((uint32_t)(kb / KG) % cfg::STAGES) * cfg::STAGE_BYTES + KG * cfg::A_BYTES +
                    (uint32_t)(kb % KG) * cfg::W_BYTES + b_row;
         };
-        auto ready = [&](int kb) {  // the k-block's stage has landed
+        const unsigned long long limit = g.acc_wait_ns ? g.acc_wait_ns : 1000000000ull;
+        auto ready = [&](int kb) {  // the k-block's stage has landed: one answer for the warp, whose lanes stay together
             if (kb % KG) return true;
             const uint32_t gi = (uint32_t)(kb / KG);
-            return mbar_wait(full0 + 8 * (gi % cfg::STAGES), (gi / cfg::STAGES) & 1u, abort_flag);
+            const bool in = mbar_wait(full0 + 8 * (gi % cfg::STAGES), (gi / cfg::STAGES) & 1u, abort_flag, limit);
+            return __all_sync(0xffffffffu, in) != 0;
         };
         bool ok = ready(0);
         if (ok) {
@@ -260,17 +259,7 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
             }
     }
     asm volatile("bar.sync 1, %0;" ::"n"((cfg::NW + cfg::HELP) * 32) : "memory");
-    if (*abort_flag) {
-        // a copy that is still on its way must land (or the limit run out) before shared memory is released
-        if (threadIdx.x == 0) {
-            const unsigned long long t0 = globaltimer_ns();
-            for (int gi = groups > cfg::STAGES ? groups - cfg::STAGES : 0; gi < groups; ++gi)
-                while (!mbar_try(full0 + 8 * (gi % cfg::STAGES), (uint32_t)(gi / cfg::STAGES) & 1u))
-                    if (globaltimer_ns() - t0 > 1000000000ull) break;
-        }
-        return;
-    }
-    if (!finisher) return;
+    if (*abort_flag || !finisher) return;
     const float rscale = RES ? 1.0f : row_scale[lane];
 
     uint32_t r[32];

@@ -425,7 +425,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                     for (int v = 0; v < 8; ++v) rope_hi[v] = tab[8 + v];
                 }
             }
-            if (!mbar_wait(accf0 + 8 * buf, aph, abort_flag, g.acc_wait_ns ? g.acc_wait_ns : 1000000000ull)) {
+            const bool acc_in = mbar_wait(accf0 + 8 * buf, aph, abort_flag, g.acc_wait_ns ? g.acc_wait_ns : 1000000000ull);
+            if (!__all_sync(0xffffffffu, acc_in)) {  // (one answer for the warp: tcgen05.ld takes all its lanes)
                 if (lane == 0) {
                     raise_abort<PAIR>(abort_flag, rank);
                     atomicExch(g.error_flag, 3);
@@ -792,7 +793,7 @@ int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int ma
         return -1;
     }
     const int map_rows = m_cap >= M ? m_cap : M;
-    // few rows: the kernel without the tensor memory round trip (a shortened accumulator wait is the tcgen05 kernel's)
+    // few rows: the kernel without the tensor memory round trip (a shortened wait without a tile is the tcgen05 kernel's)
     if (!force_bn && !g.acc_wait_ns) force_bn = skinny_tile_code(M, N, num_sms());
     if (skinny_tile_exists(force_bn)) {
         if (N % (force_bn % 1000) != 0) {

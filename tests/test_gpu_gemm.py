@@ -137,3 +137,24 @@ def test_fp32_gemm_small_tiles(ctx_fp32, M, N, K):
     C = C0.clone()
     ctx_fp32.hbsjd_gemm(A, W, C, accumulate=True)
     assert bool(((C.double() - C0.double() - ref).abs() <= tol).all())
+
+
+@pytest.mark.parametrize("tile", [16032, 16064, 32032, 32064])
+def test_bounded_wait_of_the_few_row_kernel_runs_out(ctx_bf16, tile):
+    """The same failure path in the kernel for few rows: 40 ns are shorter than any copy's way from memory, so the warps
+    that wait for their first operands give up, both producers leave and wait for what they have requested, and the
+    call returns HBSJD_ETIMEOUT.  The next call is correct."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(tile)
+    M, N, K = 40, 256, 8192
+    A = (torch.randn(M, K, generator=g, device="cuda") * 0.5).bfloat16()
+    W = (torch.randn(N, K, generator=g, device="cuda") * 0.05).bfloat16()
+    C = torch.zeros(M, N, device="cuda")
+    with pytest.raises(binding.HbsjdError) as e:
+        ctx_bf16.hbsjd_debug_gemm(A, W, C, acc_wait_ns=40, tile=tile)
+    assert e.value.code == -5
+    torch.cuda.synchronize()
+    want, got = torch.zeros(M, N, device="cuda"), torch.zeros(M, N, device="cuda")
+    ctx_bf16.hbsjd_debug_gemm(A, W, want, tile=64)
+    ctx_bf16.hbsjd_debug_gemm(A, W, got, tile=tile)
+    assert torch.equal(got, want)
