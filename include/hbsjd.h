@@ -232,6 +232,11 @@ int hbsjd_debug_fold_norm(hbsjd_ctx *c, int on);
  * before the first rollout of the context; HBSJD_ESTATE afterwards. */
 int hbsjd_debug_shuffle_pages(hbsjd_ctx *c, uint64_t seed);
 
+/* The tile (see hbsjd_debug_gemm: 0, 64 or one of the kernel for few rows) of every decoder GEMM of a bf16 context's
+ * forwards, so that tests can compare the two kernels in each fused epilogue (Sec. 4.2 verifier forward).  Every choice
+ * gives the same bits. */
+int hbsjd_debug_force_tile(hbsjd_ctx *c, int tile);
+
 /* Plants the error that a bounded device wait leaves when it gives up in the next round with this index (host memory only
  * until then; -1 takes it back), so that tests can check what a failed round leaves (Sec. 4.2 rounds; the paper has no
  * counterpart). */

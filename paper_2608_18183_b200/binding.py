@@ -19,7 +19,8 @@ DBG_ACT_A, DBG_ACT_Q, DBG_ACT_O, DBG_ACT_FFN, DBG_ACT_H, DBG_KV_K, DBG_KV_V = 3,
 
 EXPORTS = ["hbsjd_create", "hbsjd_rollout", "hbsjd_rollout_host", "hbsjd_profile", "hbsjd_profile_read", "hbsjd_profile_launch_floor", "hbsjd_probs", "hbsjd_verify", "hbsjd_verify_static", "hbsjd_calibrate_gamma", "hbsjd_round", "hbsjd_tokens", "hbsjd_destroy", "hbsjd_get_state",
            "hbsjd_set_state", "hbsjd_debug_read", "hbsjd_debug_forward", "hbsjd_debug_gemm",
-           "hbsjd_debug_shuffle_pages", "hbsjd_debug_fold_norm", "hbsjd_debug_fail_round", "hbsjd_gemm", "hbsjd_bikl", "hbsjd_score", "hbsjd_strerror",
+           "hbsjd_debug_shuffle_pages", "hbsjd_debug_fold_norm", "hbsjd_debug_fail_round",
+           "hbsjd_debug_force_tile", "hbsjd_gemm", "hbsjd_bikl", "hbsjd_score", "hbsjd_strerror",
            "hbsjd_last_error"]
 
 
@@ -108,6 +109,7 @@ def load():
         L.hbsjd_debug_shuffle_pages.argtypes = [vp, C.c_uint64]
         L.hbsjd_debug_fold_norm.argtypes = [vp, C.c_int]
         L.hbsjd_debug_fail_round.argtypes = [vp, C.c_int]
+        L.hbsjd_debug_force_tile.argtypes = [vp, C.c_int]
         L.hbsjd_bikl.argtypes = [vp, vp, vp, C.c_int, vp]
         L.hbsjd_score.argtypes = [vp, vp, C.c_int, vp, vp, vp, vp, vp, C.POINTER(C.c_float)]
         L.hbsjd_strerror.argtypes = [C.c_int]
@@ -315,6 +317,10 @@ class Context:
         """RMSNorm folded into the GEMM epilogues (True) or as its own kernel (False); before the first rollout."""
         self._check(self.lib.hbsjd_debug_fold_norm(self.h, 1 if on else 0), "hbsjd_debug_fold_norm")
         self.fold_norm = bool(on)
+
+    def hbsjd_debug_force_tile(self, tile: int):
+        """Tile of every decoder GEMM of this context's forwards (0: the library's choice)."""
+        self._check(self.lib.hbsjd_debug_force_tile(self.h, tile), "hbsjd_debug_force_tile")
 
     def hbsjd_debug_fail_round(self, rnd: int):
         """Plants a bounded wait's error in the next round with this index."""

@@ -63,6 +63,7 @@ struct hbsjd_ctx {
     hbsjd_params P;
     bool have_rollout;
     int live, round, last_S, last_compact;
+    int force_tile;  // debugging: tile of the decoder GEMMs of a bf16 forward (0: the library's choice)
     int fail_round;  // debugging: the round in which an error is planted (-1: none)
     int dbg_layer;  // layer of the last hbsjd_debug_forward (-1: none); selects the KV rows of hbsjd_debug_read
     hbsjd_stats stats;
@@ -281,9 +282,9 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
         int rc;
         if (fold)
             rc = gemm_tcgen05_addnorm((const bf16*)A, (const bf16*)W, c->h, a, c->ssq, M, D, K, Mcap, eflag, s, c->err,
-                                      sizeof(c->err));
+                                      sizeof(c->err), c->force_tile);
         else
-            rc = gemm_tcgen05_run((const bf16*)A, (const bf16*)W, c->h, M, D, K, 1, 0, Mcap, eflag, s, c->err,
+            rc = gemm_tcgen05_run((const bf16*)A, (const bf16*)W, c->h, M, D, K, 1, c->force_tile, Mcap, eflag, s, c->err,
                                   sizeof(c->err));
         prof_end(c, ps);
         c->launches++;
@@ -299,7 +300,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
         ps = prof_begin(c, HBSJD_PROF_GEMM, 2.0 * M * 3 * D * D, M,
                         es * ((double)M * D + 3.0 * D * D) + es * 3.0 * M * D);  // q, k, v written
         rc = gemm_tcgen05_qkv(a, (const bf16*)w.w_qkv, (bf16*)c->q, st, S, l, c->rope_cs, kv, Mcap, nin, eflag, s,
-                              c->err, sizeof(c->err));
+                              c->err, sizeof(c->err), c->force_tile);
         prof_end(c, ps);
         if (rc) return done(rc);
         ps = prof_begin(c, HBSJD_PROF_ATTENTION, 0.0);
@@ -318,7 +319,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
         ps = prof_begin(c, HBSJD_PROF_GEMM, 2.0 * M * 2 * F * D, M,
                         es * ((double)M * D + 2.0 * F * D) + es * (double)M * F);
         rc = gemm_tcgen05_swiglu(a, (const bf16*)w.w_13, (bf16*)c->act, M, 2 * F, D, Mcap, nin, eflag, s, c->err,
-                                 sizeof(c->err));
+                                 sizeof(c->err), c->force_tile);
         prof_end(c, ps);
         if (rc) return done(rc);
         c->launches++;
@@ -330,7 +331,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
         const int ps = prof_begin(c, HBSJD_PROF_GEMM, 2.0 * M * st.V * D, M,
                                   es * ((double)M * D + (double)st.V * D) + 4.0 * M * st.V);
         const int rc = gemm_tcgen05_head(a, (const bf16*)c->w_head, c->logits, M, st.V, D, Mcap, nin, eflag, s,
-                                         c->err, sizeof(c->err));
+                                         c->err, sizeof(c->err), c->force_tile);
         prof_end(c, ps);
         if (rc) return done(rc);
         c->launches++;
@@ -791,6 +792,7 @@ int hbsjd_create(hbsjd_ctx** out, const hbsjd_model_desc* m, const void* weights
     c->ref_attention = false;
     c->stream = (cudaStream_t)cuda_stream;
     c->dbg_layer = -1;
+    c->force_tile = 0;
     c->fail_round = -1;
     c->err[0] = 0;
     const int rc = create_impl(c, weights, weight_bytes);
@@ -1436,6 +1438,17 @@ int hbsjd_debug_fold_norm(hbsjd_ctx* c, int on) {
         return HBSJD_ESTATE;
     }
     c->fold_norm = on != 0;
+    return HBSJD_OK;
+}
+
+int hbsjd_debug_force_tile(hbsjd_ctx* c, int tile) {
+    if (!c) return HBSJD_EINVAL;
+    if (!c->bf16_model || (tile != 0 && tile != 64 && tile != 16032 && tile != 16064 && tile != 32032 && tile != 32064)) {
+        snprintf(c->err, sizeof(c->err), "hbsjd_debug_force_tile: needs a bf16 context and a tile of 0, 64, 16032, 16064, "
+                                         "32032 or 32064");
+        return HBSJD_EINVAL;
+    }
+    c->force_tile = tile;
     return HBSJD_OK;
 }
 

@@ -1,7 +1,9 @@
 // Shared pieces of the two bf16 GEMM kernels (gemm_tcgen05.cu, gemm_skinny.cu): the argument block, mbarrier / TMA
 // wrappers and the arithmetic of the fused epilogues.  A row's epilogue is one thread's work on 32 consecutive
 // columns in both kernels, through the functions below, so that an output element's bits do not depend on which
-// kernel computed it.
+// kernel computed it.  A sum of two products is spelled out as the fused operation that it is: left to the compiler,
+// which of the two is fused could differ from one instantiation to the next.  (One product, as in the sums of squares,
+// leaves no choice; spelled out there it cost the 256-wide residual tiles 50 registers and spills.)
 #pragma once
 #include <cuda.h>
 
@@ -124,7 +126,7 @@ __device__ __forceinline__ float norm_row_factor(const GemmArgs& g, int row) {
         ss += t.x;
         ss += t.y;
     }
-    return 1.0f / sqrtf(ss * g.inv_dim + g.eps);
+    return 1.0f / sqrtf(__fmaf_rn(ss, g.inv_dim, g.eps));
 }
 
 __device__ __forceinline__ RowDst qkv_row(const GemmArgs& g, int row, bool valid) {
@@ -163,9 +165,31 @@ __device__ __forceinline__ void rope_chunk(const uint32_t r[32], float rscale, c
     for (int v = 0; v < 8; ++v) {
         const float a0 = __uint_as_float(r[4 * v]) * rscale, b0 = __uint_as_float(r[4 * v + 1]) * rscale;
         const float a1 = __uint_as_float(r[4 * v + 2]) * rscale, b1 = __uint_as_float(r[4 * v + 3]) * rscale;
-        o[2 * v] = pack_bf16x2(a0 * t[v].x - b0 * t[v].y, a0 * t[v].y + b0 * t[v].x);
-        o[2 * v + 1] = pack_bf16x2(a1 * t[v].z - b1 * t[v].w, a1 * t[v].w + b1 * t[v].z);
+        o[2 * v] = pack_bf16x2(__fmaf_rn(a0, t[v].x, -(b0 * t[v].y)), __fmaf_rn(a0, t[v].y, b0 * t[v].x));
+        o[2 * v + 1] = pack_bf16x2(__fmaf_rn(a1, t[v].z, -(b1 * t[v].w)), __fmaf_rn(a1, t[v].w, b1 * t[v].z));
     }
+}
+
+// Residual update of one chunk: r becomes old + r (one fp32 addition per element), the return value is the new chunk's
+// sum of squares.
+__device__ __forceinline__ float residual_chunk(const float4 old[8], uint32_t r[32]) {
+    float ss = 0.f;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        const float x0 = old[v].x + __uint_as_float(r[4 * v]);
+        const float x1 = old[v].y + __uint_as_float(r[4 * v + 1]);
+        const float x2 = old[v].z + __uint_as_float(r[4 * v + 2]);
+        const float x3 = old[v].w + __uint_as_float(r[4 * v + 3]);
+        ss += x0 * x0;
+        ss += x1 * x1;
+        ss += x2 * x2;
+        ss += x3 * x3;
+        r[4 * v] = __float_as_uint(x0);
+        r[4 * v + 1] = __float_as_uint(x1);
+        r[4 * v + 2] = __float_as_uint(x2);
+        r[4 * v + 3] = __float_as_uint(x3);
+    }
+    return ss;
 }
 
 __device__ __forceinline__ void plain_chunk(const uint32_t r[32], float rscale, uint32_t o[16]) {

@@ -276,29 +276,18 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
     }
     if (RES) {
         // new residual = old + acc, its bf16 copy and the chunk's sum of squares
-        float ss = 0.f;
-        float4* cp = reinterpret_cast<float4*>(g.C + (size_t)row * N + col);
+        const float ss = residual_chunk(pre, r);
+        uint4* cp = reinterpret_cast<uint4*>(g.C + (size_t)row * N + col);
 #pragma unroll
-        for (int v = 0; v < 8; ++v) {
-            float4 x;
-            x.x = pre[v].x + __uint_as_float(r[4 * v]);
-            x.y = pre[v].y + __uint_as_float(r[4 * v + 1]);
-            x.z = pre[v].z + __uint_as_float(r[4 * v + 2]);
-            x.w = pre[v].w + __uint_as_float(r[4 * v + 3]);
-            ss += x.x * x.x;
-            ss += x.y * x.y;
-            ss += x.z * x.z;
-            ss += x.w * x.w;
-            pre[v] = x;
-            cp[v] = x;
-        }
+        for (int v = 0; v < 8; ++v) cp[v] = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
         if (EPI == EPI_ADDNORM) {
             uint4* hp = reinterpret_cast<uint4*>(g.hb + (size_t)row * N + col);
 #pragma unroll
             for (int v = 0; v < 4; ++v)
-                hp[v] = make_uint4(pack_bf16x2(pre[2 * v].x, pre[2 * v].y), pack_bf16x2(pre[2 * v].z, pre[2 * v].w),
-                                   pack_bf16x2(pre[2 * v + 1].x, pre[2 * v + 1].y),
-                                   pack_bf16x2(pre[2 * v + 1].z, pre[2 * v + 1].w));
+                hp[v] = make_uint4(pack_bf16x2(__uint_as_float(r[8 * v]), __uint_as_float(r[8 * v + 1])),
+                                   pack_bf16x2(__uint_as_float(r[8 * v + 2]), __uint_as_float(r[8 * v + 3])),
+                                   pack_bf16x2(__uint_as_float(r[8 * v + 4]), __uint_as_float(r[8 * v + 5])),
+                                   pack_bf16x2(__uint_as_float(r[8 * v + 6]), __uint_as_float(r[8 * v + 7])));
             g.ssq_out[(size_t)row * (N / 32) + col / 32] = ss;
         }
     } else if (EPI == EPI_STORE) {

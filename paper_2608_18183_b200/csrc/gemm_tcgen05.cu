@@ -456,24 +456,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                     float4 hcur[8];
 #pragma unroll
                     for (int v = 0; v < 8; ++v) hcur[v] = hbuf[u][v];
-                    // new residual = old + acc (one fp32 addition per element, as the reduce-add form did)
-                    float ss = 0.f;
-#pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        const float x0 = hcur[v].x + __uint_as_float(r[4 * v]);
-                        const float x1 = hcur[v].y + __uint_as_float(r[4 * v + 1]);
-                        const float x2 = hcur[v].z + __uint_as_float(r[4 * v + 2]);
-                        const float x3 = hcur[v].w + __uint_as_float(r[4 * v + 3]);
-                        ss += x0 * x0;
-                        ss += x1 * x1;
-                        ss += x2 * x2;
-                        ss += x3 * x3;
-                        r[4 * v] = __float_as_uint(x0);
-                        r[4 * v + 1] = __float_as_uint(x1);
-                        r[4 * v + 2] = __float_as_uint(x2);
-                        r[4 * v + 3] = __float_as_uint(x3);
-                    }
-                    ssq4[u] = ss;
+                    ssq4[u] = residual_chunk(hcur, r);  // new residual = old + acc
                     // one bulk tensor store per tile (the pair is one bulk group: of two buffers, the one used two chunks
                     // ago is free once at most one group is still reading); rows past the buffers' capacity are clipped
                     if (lane == 0) {
@@ -914,7 +897,7 @@ void set_norm(GemmArgs& g, const NormIn& nin, int K) {
 }  // namespace
 
 int gemm_tcgen05_head(const bf16* A, const bf16* W, float* C, int M, int N, int K, int m_cap, const NormIn& nin,
-                      int32_t* error_flag, cudaStream_t s, char* err, size_t errlen) {
+                      int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile) {
     GemmArgs g{};
     g.C = C;
     g.M = M;
@@ -923,11 +906,11 @@ int gemm_tcgen05_head(const bf16* A, const bf16* W, float* C, int M, int N, int 
     g.error_flag = error_flag;
     g.w_constant = 1;
     set_norm(g, nin, K);
-    return run(EPI_STORE, A, W, g, 0, 256, m_cap, s, err, errlen);
+    return run(EPI_STORE, A, W, g, tile, 256, m_cap, s, err, errlen);
 }
 
 int gemm_tcgen05_addnorm(const bf16* A, const bf16* W, float* h, bf16* hb, float* ssq_out, int M, int N, int K,
-                         int m_cap, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen) {
+                         int m_cap, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile) {
     if (((uintptr_t)h | (uintptr_t)hb) & 15) {
         snprintf(err, errlen, "gemm: residual buffers must be 16-byte aligned");
         return -1;
@@ -941,11 +924,11 @@ int gemm_tcgen05_addnorm(const bf16* A, const bf16* W, float* h, bf16* hb, float
     g.K = K;
     g.error_flag = error_flag;
     g.w_constant = 1;
-    return run(EPI_ADDNORM, A, W, g, 0, 256, m_cap, s, err, errlen);
+    return run(EPI_ADDNORM, A, W, g, tile, 256, m_cap, s, err, errlen);
 }
 
 int gemm_tcgen05_swiglu(const bf16* A, const bf16* W13_interleaved, bf16* act, int M, int F2, int K, int m_cap,
-                        const NormIn& nin, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen) {
+                        const NormIn& nin, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile) {
     GemmArgs g{};
     set_norm(g, nin, K);
     g.out = act;
@@ -954,12 +937,12 @@ int gemm_tcgen05_swiglu(const bf16* A, const bf16* W13_interleaved, bf16* act, i
     g.K = K;
     g.error_flag = error_flag;
     g.w_constant = 1;
-    return run(EPI_SWIGLU, A, W13_interleaved, g, 0, 256, m_cap, s, err, errlen);
+    return run(EPI_SWIGLU, A, W13_interleaved, g, tile, 256, m_cap, s, err, errlen);
 }
 
 int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, int S, int layer,
                      const float* rope_cs, const KvView& kv, int m_cap, const NormIn& nin, int32_t* error_flag,
-                     cudaStream_t s, char* err, size_t errlen) {
+                     cudaStream_t s, char* err, size_t errlen, int tile) {
     GemmArgs g{};
     set_norm(g, nin, st.D);
     g.out = q;
@@ -976,7 +959,7 @@ int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, 
     // a tile must lie inside one of the q / k / v sections and start on a rotation-pair boundary
     int max_bn = 256;
     while (st.D % max_bn != 0) max_bn >>= 1;
-    return run(EPI_QKV, A, Wqkv, g, 0, max_bn, m_cap, s, err, errlen);
+    return run(EPI_QKV, A, Wqkv, g, tile, max_bn, m_cap, s, err, errlen);
 }
 
 }  // namespace hbsjd

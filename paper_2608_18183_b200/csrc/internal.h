@@ -171,20 +171,21 @@ struct NormIn {
     const float* ssq;  // [M][K / 32] partial sums of squares of the fp32 rows
     float eps;
 };
+// (tile: as gemm_tcgen05_run's force_bn, here and below)
 // act[M, F] bf16 = silu(gate) * up, from A[M,K] . W13i^T where W13i[2F, K] holds gate row f at 2f, up row f at 2f+1.
 int gemm_tcgen05_swiglu(const bf16* A, const bf16* W13_interleaved, bf16* act, int M, int F2, int K, int m_cap,
-                        const NormIn& nin, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen);
+                        const NormIn& nin, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile = 0);
 // logits[M, N] fp32 = norm(x) . W^T with the norm folded as above.
 int gemm_tcgen05_head(const bf16* A, const bf16* W, float* C, int M, int N, int K, int m_cap, const NormIn& nin,
-                      int32_t* error_flag, cudaStream_t s, char* err, size_t errlen);
+                      int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile = 0);
 // Residual update h[M, N] fp32 += A[M,K] . W^T, which also leaves what the next folded norm needs: hb = bf16(h)
 // and ssq_out[M][N / 32] = sums of squares of the new h over each 32-column chunk (fixed order, no atomics).
 int gemm_tcgen05_addnorm(const bf16* A, const bf16* W, float* h, bf16* hb, float* ssq_out, int M, int N, int K,
-                         int m_cap, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen);
+                         int m_cap, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile = 0);
 // QKV projection of the normed activations A[M, D] with the 2D RoPE and the paged KV write fused:
 // q[M, D] bf16 rotated; rotated k and v stored at each row's (cache row, sequence index).
 int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, int S, int layer,
                      const float* rope_cs, const KvView& kv, int m_cap, const NormIn& nin, int32_t* error_flag,
-                     cudaStream_t s, char* err, size_t errlen);
+                     cudaStream_t s, char* err, size_t errlen, int tile = 0);
 
 }  // namespace hbsjd

@@ -213,3 +213,42 @@ def test_layer0_full_size_shapes(name, ks, fold):
     w = synth.WORKLOADS[name]
     errs, longest = run_case(w, ks, fold)
     check(errs, longest, w.shape.head_dim, name, fold)
+
+
+@pytest.mark.parametrize("fold", [False, True])
+@pytest.mark.parametrize("head", [64, 32])
+def test_every_epilogue_gives_the_same_bits_in_both_gemm_kernels(fold, head):
+    """The two bf16 GEMM kernels take over from one another by the number of rows, so Full and Compact execution and an
+    image's independence of its batch need equal bits in every fused epilogue: rotated q, k and v, silu(gate) up, the
+    residual update with its bf16 copy and sums of squares, the row factor and the head, two layers behind one another.
+    Weights spread over 2^+-4, so that the rotation cancels and the gates saturate."""
+    s = synth.ModelShape(2, 256, 256 // head, 512, 1024, 12, 12, 10, "bf16")
+    img = synth.make_weights(s, 5, target_entropy=None)
+    rng = np.random.default_rng(7)
+    for name, r, c, off in synth.tensor_table(s)[0]:
+        if name.split(".")[-1].startswith("w_"):
+            m = img[off:off + r * c * 2].view(np.uint16)
+            m += (rng.integers(-4, 5, size=r * c) << 7).astype(np.uint16)  # exponents; N(0, 0.02) stays normal
+    w = synth.with_shape(synth.WORKLOADS["small_bf16"], shape=s)
+    ks = np.array([0, 1, 31, 64, 65, 100, 141], dtype=np.int32)
+    toks, _, lab = synth.make_inputs(w, seed=3, batch=len(ks))
+    what = {0: (binding.DBG_ACT_Q, binding.DBG_KV_K, binding.DBG_KV_V, binding.DBG_ACT_O, binding.DBG_ACT_H, binding.DBG_ACT_A),
+            1: (binding.DBG_ACT_FFN, binding.DBG_ACT_H, binding.DBG_ACT_A)}
+    seen = {}
+    for tile in (64, 0, 16032, 16064, 32032, 32064):
+        ctx = binding.Context(s, img, len(ks), 13)
+        ctx.hbsjd_debug_fold_norm(fold)
+        ctx.hbsjd_debug_force_tile(tile)
+        ctx.hbsjd_rollout(G.dev(toks), G.dev(ks), G.dev(lab), binding.make_params(
+            13, 12, w.cfg_scale, max_rounds=0, seed=2, exec_mode=binding.EXEC_FULL))
+        got = []
+        for layer in (0, 1):
+            for stage in (0, 1):
+                ctx.hbsjd_debug_forward(layer, stage)
+                got += [ctx.hbsjd_debug_read(x, i) for x in what[stage] for i in range(2 * len(ks))]
+        ctx.hbsjd_round()
+        got += [ctx.hbsjd_debug_read(binding.DBG_LOGITS, i) for i in range(2 * len(ks))]
+        ctx.hbsjd_destroy()
+        assert all(np.isfinite(x).all() for x in got)
+        for i, x in enumerate(got):
+            np.testing.assert_array_equal(x.view(np.uint32), seen.setdefault(i, x).view(np.uint32), err_msg=f"{tile} {i}")

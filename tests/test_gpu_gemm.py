@@ -158,3 +158,60 @@ def test_bounded_wait_of_the_few_row_kernel_runs_out(ctx_bf16, tile):
     ctx_bf16.hbsjd_debug_gemm(A, W, want, tile=64)
     ctx_bf16.hbsjd_debug_gemm(A, W, got, tile=tile)
     assert torch.equal(got, want)
+
+
+def _wide_operands(kind, M, N, K, g):
+    """bf16 operands on which an accumulator that aligned or rounded its products otherwise would show."""
+    import torch
+    A, W = torch.randn(M, K, generator=g, device="cuda"), torch.randn(N, K, generator=g, device="cuda")
+    spread = lambda x, e: x * torch.exp2(((torch.rand(x.shape, generator=g, device="cuda") * 2 - 1) * e).round())
+    if kind == "wide":
+        A, W = spread(A, 20), spread(W, 20)
+    elif kind == "cancelling":  # neighbours cancel, but for the last bit of some
+        A, W = spread(A, 10), spread(W, 10)
+        A[:, 1::2] = -A[:, 0::2]
+        W[:, 1::2] = W[:, 0::2] * (1 + (torch.rand(N, K // 2, generator=g, device="cuda") < 0.3) * 2.0 ** -7)
+    elif kind == "running sum":  # a large sum first, products far below its last bits behind it
+        A[:, :64] *= 2.0 ** 12
+        A[:, 64:] *= 2.0 ** -10
+    elif kind == "one large per step":
+        big = torch.randn(M, (K + 15) // 16, generator=g, device="cuda") * 2.0 ** 10
+        A *= 2.0 ** -14
+        A[:, ::16] = big
+    elif kind == "denormal":
+        A, W = A * 2.0 ** -70, W * 2.0 ** -62
+    elif kind == "overflow":
+        A, W = A * 2.0 ** 60, W * 2.0 ** 62
+    return A.bfloat16().contiguous(), W.bfloat16().contiguous()
+
+
+@pytest.mark.parametrize("kind", ["wide", "cancelling", "running sum", "one large per step", "denormal", "overflow"])
+@pytest.mark.parametrize("M,N,K", [(48, 128, 320), (301, 512, 1024)])
+def test_both_gemm_kernels_round_alike(ctx_bf16, kind, M, N, K):
+    """mma.sync and tcgen05 sum their 16 products per step alike; no document says so, hence operands of mixed magnitude,
+    not random ones of one scale.  Infinities and NaN are compared by their bits too."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    A, W = _wide_operands(kind, M, N, K, g)
+    out = []
+    for tile in (64, 256, 512, 16032, 16064, 32032, 32064):
+        if N % 256 and tile in (256, 512):
+            continue
+        C = torch.zeros(M, N, device="cuda")
+        ctx_bf16.hbsjd_debug_gemm(A, W, C, tile=tile)
+        out.append(C.view(torch.int32))
+    assert all(torch.equal(out[0], o) for o in out[1:])
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3])
+@pytest.mark.parametrize("M", [8, 600])
+def test_output_off_its_16_byte_boundary_is_refused(ctx_bf16, M, offset):
+    """A few rows or many: refused on the host, nothing launched."""
+    import torch
+    A, W = torch.ones(M, 64, device="cuda").bfloat16(), torch.ones(128, 64, device="cuda").bfloat16()
+    flat = torch.zeros(M * 128 + 4, device="cuda")
+    for accumulate in (False, True):
+        with pytest.raises(binding.HbsjdError) as e:
+            ctx_bf16.hbsjd_gemm(A, W, flat[offset:offset + M * 128].view(M, 128), accumulate=accumulate)
+        assert e.value.code == -1
+    assert not bool(flat.any())
