@@ -196,7 +196,7 @@ int hbsjd_debug_forward(hbsjd_ctx *c, int layer, int stage);
 /* Decoder GEMM as used by the round (Sec. 4.2 verifier forward): C[M,N] (+)= A[M,K] . W[N,K]^T on the
  * context's stream.  A, W: DEVICE, element type of the context (bf16: tcgen05 tensor cores, fp32
  * accumulation; fp32: CUDA cores).  C: DEVICE fp32 [M,N]; accumulate != 0 adds into C.
- * M may be any size; bf16 needs N % 64 == 0 and K % 64 == 0; A, W 16-byte aligned.  A, W and C are ordered
+ * M may be any size; bf16 needs N % 64 == 0, K % 64 == 0 and A, W, C 16-byte aligned (HBSJD_EINVAL).  A, W and C are ordered
  * like any other kernel argument behind earlier work of the stream. */
 int hbsjd_gemm(hbsjd_ctx *c, const void *A, const void *W, float *C, int M, int N, int K, int accumulate);
 
