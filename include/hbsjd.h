@@ -318,8 +318,8 @@ int hbsjd_bikl(hbsjd_ctx *c, const float *logits_s, const float *logits_t, int r
  *   per_image     DEVICE fp32 [batch] or NULL: the per-image means (0 where k_b = T)
  *   loss          HOST float: the batch mean
  * Work is enqueued on each context's own stream with event dependencies between them; contexts that share a stream run
- * side by side all the same (the student on a stream of its own, ordered between the shared stream's earlier and later
- * work).  The call returns after all of it finished.  Errors as hbsjd_rollout (arguments are validated on the host before
+ * side by side all the same (the student on a stream of its own of the same priority, ordered between the shared
+ * stream's earlier and later work).  The call returns after all of it finished.  Errors as hbsjd_rollout (arguments are validated on the host before
  * any launch). */
 int hbsjd_score(hbsjd_ctx *student, hbsjd_ctx *teacher, int batch, const int32_t *tokens, const int32_t *prefix_len,
                 const int32_t *class_labels, float *bikl_pos, float *per_image, float *loss);

@@ -59,7 +59,7 @@ struct hbsjd_ctx {
     uint32_t post_seq;    // stamp of the last round enqueued
     int min_left;         // fewest tokens left of a live image, after the last collected round
     cudaEvent_t ev0, ev1, ev2;
-    cudaStream_t side;  // stand-in for `stream` while hbsjd_score runs two contexts that share one
+    cudaStream_t side;  // stand-in for `stream` (its priority) while hbsjd_score runs two contexts that share one
     hbsjd_params P;
     bool have_rollout;
     int live, round, last_S, last_compact;
@@ -734,7 +734,11 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
         const int32_t none = 0x7fffffff;
         CK(cudaMemcpyAsync(c->tally + 1, &none, sizeof(none), cudaMemcpyHostToDevice, c->stream));
     }
-    CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+    {
+        int priority = 0;
+        CK(cudaStreamGetPriority(c->stream, &priority));
+        CK(cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, priority));
+    }
     CK(cudaEventCreate(&c->ev0));
     CK(cudaEventCreate(&c->ev1));
     CK(cudaEventCreate(&c->ev2));
