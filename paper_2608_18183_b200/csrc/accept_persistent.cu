@@ -634,7 +634,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
 bool accept_persistent_supported(const State& st) { return st.V <= NCH * CHUNK && st.V % 4 == 0; }
 
 template <bool CFG, bool PROBS>
-static void launch(const State& st, const AcceptArgs& a, int n_sms, cudaStream_t s) {
+static void launch(const State& st, const AcceptArgs& a, int n_sms, Stream& s) {
     static int configured[64] = {0};
     const int bytes = (CFG ? 2 : 1) * st.V * (int)sizeof(float) + (int)sizeof(PShared) +
                       (PROBS ? 0 : 3 * a.S * (int)sizeof(int));
@@ -643,13 +643,15 @@ static void launch(const State& st, const AcceptArgs& a, int n_sms, cudaStream_t
     launch_k(k_accept_persistent<CFG, PROBS>, dim3(items < n_sms ? items : n_sms), dim3(PT), bytes, s, st, a);
 }
 
-void launch_accept_persistent(const State& st, const AcceptArgs& a, int n_sms, cudaStream_t s) {
-    if (st.nb == 2) launch<true, false>(st, a, n_sms, s);
-    else launch<false, false>(st, a, n_sms, s);
+void launch_accept_persistent(const State& st, const AcceptArgs& a, int n_sms, Stream& s) {
+    AcceptArgs b = a;
+    b.early = a.early && s.late;
+    if (st.nb == 2) launch<true, false>(st, b, n_sms, s);
+    else launch<false, false>(st, b, n_sms, s);
 }
 
 void launch_probs_persistent(const float* lc, const float* lu, int rows, int V, float cfg_scale, float temperature,
-                             int top_k, float* p, int32_t* counters, int n_sms, cudaStream_t s) {
+                             int top_k, float* p, int32_t* counters, int n_sms, Stream& s) {
     State st{};
     st.V = V;
     st.W = 1;

@@ -31,7 +31,7 @@ struct hbsjd_ctx {
     bool fold_norm;      // bf16 model: RMSNorm folded into the GEMM epilogues (launch-bound contexts), else its own kernel
     bool unit_gains;     // every norm gain of the model is exactly 1
     bool ref_attention;  // debugging: run the one-warp-per-row attention kernel
-    cudaStream_t stream;
+    Stream stream = nullptr;
     // weights
     unsigned char* w_img;
     const void *tok_emb, *cls_emb, *g_out, *w_head;
@@ -200,7 +200,7 @@ int forward<float>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int st
     typedef float TA;
     const State& st = c->st;
     const int M = st.nb * S * st.W, D = st.D, F = st.F;
-    cudaStream_t s = c->stream;
+    Stream& s = c->stream;
     const KvView kv = kv_view(c);
     launch_embed<TA>(st, S, (const TA*)c->tok_emb, (const TA*)c->cls_emb, c->h, nullptr, nullptr, s);
     c->launches++;
@@ -260,7 +260,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
     const State& st = c->st;
     const int M = st.nb * S * st.W, D = st.D, F = st.F;
     const int Mcap = 2 * c->Bmax * c->Wmax;  // row capacity of the activation buffers
-    cudaStream_t s = c->stream;
+    Stream& s = c->stream;
     const KvView kv = kv_view(c);
     const bool fold = c->fold_norm;
     const double es = 2.0;  // bytes of a bf16 operand / output element (algorithmic byte counts of the profile)
@@ -417,7 +417,7 @@ int enqueue_round(hbsjd_ctx* c) {
     a.post_stamp = ++c->post_seq;
     a.post = c->post_dev + (a.post_stamp & 1u);
     a.tally = c->tally;
-    a.early = c->bf16_model;
+    a.early = true;  // the head projection writes none of what is read early
     {
         const int ps = prof_begin(c, HBSJD_PROF_ACCEPT, 0.0);
         launch_prob_accept(c->st, a, c->stream);

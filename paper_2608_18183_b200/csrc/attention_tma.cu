@@ -141,7 +141,8 @@ struct AttnArgs {
     const bf16* q;
     bf16* out;
     int32_t* error_flag;
-    bool few;  // the grid leaves half of the SMs free
+    bool few;    // the grid leaves half of the SMs free
+    bool early;  // the kernel before triggers late (see pdl_wait)
 };
 
 // Position `pos` of the sorted item list, the CTA's item number `stripe` -> work item.  Returns false for an inactive slot.
@@ -339,6 +340,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
     }
+    if (!a.early) pdl_wait();
     // The kernel before this one is the QKV projection, which lets this grid start only once its own wait is over: all
     // that precedes the projection is complete here, the slot tables and the keys and values of earlier rounds among it
     // (read through L2).  Queries and the window's own keys come after the wait.  The chain of look-ups and the first
@@ -496,7 +498,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
 }
 
 template <int QB>
-cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, AttnArgs a, cudaStream_t s) {
+cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, AttnArgs a, Stream& s) {
     using cfg = AttnCfg<QB>;
     constexpr int threads = (cfg::NCW + 1) * 32;
     constexpr int fixed = 1024 + cfg::STAGES * cfg::STAGE_BYTES + 16 * cfg::STAGES + 16, most = fixed + 16 * LIST_MAX;
@@ -521,7 +523,8 @@ cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, AttnArgs a, 
     a.few = 2 * grid <= device_sm_count();
     const long stripes = (items + grid - 1) / grid;
     const int smem = fixed + 16 * (int)(stripes < LIST_MAX ? stripes : LIST_MAX);
-    return launch_k(k_attention_tma<QB>, dim3((unsigned)grid), dim3(threads), (size_t)smem, s, mk, mv, a);
+    a.early = s.late;
+    return launch_kc(!a.few, k_attention_tma<QB>, dim3((unsigned)grid), dim3(threads), (size_t)smem, s, 1, mk, mv, a);
 }
 
 }  // namespace
@@ -531,7 +534,7 @@ bool attention_tma_supported(const State& st, const KvView& kv) {
 }
 
 int launch_attention_tma(const State& st, int S, int layer, const bf16* q, int q_rows_cap, KvView kv, bf16* out,
-                         int32_t* error_flag, cudaStream_t s, char* err, size_t errlen) {
+                         int32_t* error_flag, Stream& s, char* err, size_t errlen) {
     CUtensorMap mk, mv;
     const int qb = (st.W + 15) / 16;
     const long kv_rows = (long)st.L * kv.n_pages * kv.page;

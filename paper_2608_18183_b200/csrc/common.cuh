@@ -14,21 +14,30 @@ typedef __nv_bfloat16 bf16;
 // Programmatic dependent launch: every kernel of the library has a pdl_wait() (blocks until the preceding
 // grid in the stream has completed and its writes are visible) and a pdl_trigger() (lets the next grid's
 // CTAs be scheduled as SMs free up), so launch latency and kernel prologues overlap the previous kernel's
-// tail.  All but k_commit, the small fp32 GEMM and attention's small grids trigger after their own wait:
-// triggered before it, a third kernel's CTAs took the shared memory that the second's would have had (one L
-// image 39.4 -> 37.0 ms with the gate/up projection triggering late, 24 L images token by token 274.0 ->
-// 271.1, the small kernels of four tiny images 4.50 -> 4.46).  All that precedes such a kernel is complete
-// when the next one starts and may be read there before the wait; else nothing before pdl_wait() touches
-// global memory that any kernel writes.  The pairs that make use of it: embedding, RMSNorm or the folded
-// residual projection and the QKV projection; the QKV projection and attention; a forward's LM head and
-// the accept kernel; the accept kernel (or k_sync_min) and k_commit.
+// tail.  Most trigger after their own wait ("late"): triggered before it, a third kernel's CTAs take the shared memory
+// that the second's would have had (one L image 0.94 times the time with the gate/up projection late, 24 L images token
+// by token 0.99, four tiny images 0.99 with the small kernels late).
+// All that precedes a late kernel is complete when the next one starts.  Four kernels use that: the QKV projection (rows,
+// pages and rotations), attention (work list, pages, old keys), the accept kernel behind an LM head and k_commit read what
+// kernels before their predecessor have written before their own wait, through L2.  Else nothing before pdl_wait() touches
+// global memory that any kernel writes.  Stream carries which kind the last kernel was: the launchers of these four hand it
+// to the kernel, which waits first behind a kernel that triggers early.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A stream and how the kernel launched there last triggers its successor.
+struct Stream {
+    cudaStream_t s;
+    bool late;  // after its own wait; false too where it is not known (the first launch of a call)
+    Stream(cudaStream_t stream) : s(stream), late(false) {}
+    operator cudaStream_t() const { return s; }
+};
+
 // cluster_x > 1 launches thread-block clusters of that many CTAs along x.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kc(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+inline cudaError_t launch_kc(bool late, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Stream& s,
                              int cluster_x, Args&&... args) {
+    s.late = late;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -51,10 +60,14 @@ inline cudaError_t launch_kc(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// For kernels that trigger after their own wait; launch_early for the others.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                            Args&&... args) {
-    return launch_kc(kernel, grid, block, smem, s, 1, std::forward<Args>(args)...);
+inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Stream& s, Args&&... args) {
+    return launch_kc(true, kernel, grid, block, smem, s, 1, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_early(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Stream& s, Args&&... args) {
+    return launch_kc(false, kernel, grid, block, smem, s, 1, std::forward<Args>(args)...);
 }
 
 // Raises a kernel's dynamic shared-memory limit once per device (function attributes are per device).

@@ -32,6 +32,7 @@ struct GemmArgs {
     int w_constant;   // W never changes while the stream runs (model weights): its tiles may be fetched early
     unsigned int acc_wait_ns;  // 0, or a shorter limit for the epilogue's accumulator wait (time-out test)
     // QKV epilogue
+    bool early;       // the kernel before triggers late (see pdl_wait)
     State st;
     int S, layer;
     const float* rope_cs;  // [T][dh/2][2]
@@ -218,7 +219,7 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
 int skinny_tile_code(int M, int N, int sms);
 bool skinny_tile_exists(int code);
 // m_rows: row extent of A's tensor map.  Returns 0 or a negative code with a message in err.
-int gemm_skinny_launch(int epi, int code, const bf16* A, const bf16* W, const GemmArgs& g, int m_rows, cudaStream_t s,
+int gemm_skinny_launch(int epi, int code, const bf16* A, const bf16* W, const GemmArgs& g, int m_rows, Stream& s,
                        char* err, size_t errlen);
 
 }  // namespace hbsjd

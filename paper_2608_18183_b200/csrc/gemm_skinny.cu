@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
         // in order: all of it off the consumers' path).  The look-ups need nothing of the kernel before this one, and the
         // kernels that come before a QKV projection trigger after their own wait: they go before this one's.  (24 L
         // images token by token 282.9 -> 274.0 ms, one L image 40.6 -> 39.5, six XL images 783 -> 772.)
-        if (EPI != EPI_QKV) pdl_wait();
+        if (EPI != EPI_QKV || !g.early) pdl_wait();
         const int row = m0 + lane;
         if (lane < TM && row < g.M) {
             if (EPI == EPI_QKV) {
@@ -326,17 +326,18 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
 }
 
 template <int TM, int TN, int EPI>
-cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mw, const GemmArgs& g, cudaStream_t s) {
+cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mw, GemmArgs g, Stream& s) {
     using cfg = SkinnyCfg<TM, TN, EPI>;
     static int configured[64] = {0};
     cudaError_t e = ensure_dynamic_smem(k_gemm_skinny<TM, TN, EPI>, cfg::SMEM, configured);
     if (e != cudaSuccess) return e;
     const int tiles = (g.N / TN) * ((g.M + TM - 1) / TM);
+    g.early = s.late;
     return launch_k(k_gemm_skinny<TM, TN, EPI>, dim3(tiles), dim3(cfg::THREADS), (size_t)cfg::SMEM, s, ma, mw, g);
 }
 
 template <int TM, int TN>
-cudaError_t launch_epi(int epi, const CUtensorMap& ma, const CUtensorMap& mw, const GemmArgs& g, cudaStream_t s) {
+cudaError_t launch_epi(int epi, const CUtensorMap& ma, const CUtensorMap& mw, const GemmArgs& g, Stream& s) {
     switch (epi) {
         case EPI_STORE: return launch<TM, TN, EPI_STORE>(ma, mw, g, s);
         case EPI_ADD: return launch<TM, TN, EPI_ADD>(ma, mw, g, s);
@@ -366,7 +367,7 @@ int skinny_tile_code(int M, int N, int sms) {
     return 0;
 }
 
-int gemm_skinny_launch(int epi, int code, const bf16* A, const bf16* W, const GemmArgs& g, int m_rows, cudaStream_t s,
+int gemm_skinny_launch(int epi, int code, const bf16* A, const bf16* W, const GemmArgs& g, int m_rows, Stream& s,
                        char* err, size_t errlen) {
     CUtensorMap ma, mw;
     const int tm = code / 1000, tn = code % 1000, kg = tn == 32 ? 4 : 2;

@@ -724,7 +724,7 @@ bool make_map_c(CUtensorMap* map, const float* base, int rows, int N) {
 
 template <int BN, int EPI>
 cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mw, const CUtensorMap& mc, const CUtensorMap& mh,
-                   const GemmArgs& g, cudaStream_t s) {
+                   const GemmArgs& g, Stream& s) {
     static int configured[64] = {0};
     using cfg = Cfg<BN, false, EPI == EPI_ADDNORM>;
     cudaError_t e0 = ensure_dynamic_smem(k_gemm_tcgen05<BN, EPI, false>, cfg::SMEM, configured);
@@ -738,7 +738,7 @@ cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mw, const CUtensorM
 // CTA pairs: 256 x BN tiles (BN = 256 or 128), one cluster of two CTAs per pair of SMs.
 template <int BN, int EPI>
 cudaError_t launch_pair(const CUtensorMap& ma, const CUtensorMap& mw, const CUtensorMap& mc, const CUtensorMap& mh,
-                        const GemmArgs& g, cudaStream_t s) {
+                        const GemmArgs& g, Stream& s) {
     static int configured[64] = {0};
     using cfg = Cfg<BN, true, EPI == EPI_ADDNORM>;
     cudaError_t e0 = ensure_dynamic_smem(k_gemm_tcgen05<BN, EPI, true>, cfg::SMEM, configured);
@@ -746,13 +746,13 @@ cudaError_t launch_pair(const CUtensorMap& ma, const CUtensorMap& mw, const CUte
     const int tiles = (g.N / BN) * ((g.M + 2 * BM - 1) / (2 * BM));
     const int pairs = num_sms() / 2;
     const int grid = 2 * (tiles < pairs ? tiles : pairs);
-    return launch_kc(k_gemm_tcgen05<BN, EPI, true>, dim3(grid), dim3(NUM_THREADS), (size_t)cfg::SMEM, s, 2,
+    return launch_kc(true, k_gemm_tcgen05<BN, EPI, true>, dim3(grid), dim3(NUM_THREADS), (size_t)cfg::SMEM, s, 2,
                      ma, mw, mc, mh, g);
 }
 
 template <int EPI>
 cudaError_t launch_bn(int bn, const CUtensorMap& ma, const CUtensorMap& mw, const CUtensorMap& mc,
-                      const CUtensorMap& mh, const GemmArgs& g, cudaStream_t s) {
+                      const CUtensorMap& mh, const GemmArgs& g, Stream& s) {
     switch (bn) {
         case 32: return launch<32, EPI>(ma, mw, mc, mh, g, s);
         case 64: return launch<64, EPI>(ma, mw, mc, mh, g, s);
@@ -766,7 +766,7 @@ cudaError_t launch_bn(int bn, const CUtensorMap& ma, const CUtensorMap& mw, cons
 // m_cap >= M: row extent given to the A and C tensor maps (the capacity of the caller's buffers), so that one
 // cached map serves every M; rows between M and m_cap are padding (read as they are, never stored past M's
 // last 32-row block).  0: use M.
-int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int max_bn, int m_cap, cudaStream_t s,
+int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int max_bn, int m_cap, Stream& s,
         char* err, size_t errlen) {
     const int M = g.M, N = g.N, K = g.K;
     if (M <= 0) return 0;
@@ -870,7 +870,7 @@ int gemm_tcgen05_tile_n(int M, int N, int K) {
 }
 
 int gemm_tcgen05_run(const bf16* A, const bf16* W, float* C, int M, int N, int K, int accumulate, int force_bn,
-                     int m_cap, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int w_constant,
+                     int m_cap, int32_t* error_flag, Stream& s, char* err, size_t errlen, int w_constant,
                      unsigned int acc_wait_ns) {
     if ((uintptr_t)C & 15) {
         snprintf(err, errlen, "gemm: C must be 16-byte aligned");
@@ -897,7 +897,7 @@ void set_norm(GemmArgs& g, const NormIn& nin, int K) {
 }  // namespace
 
 int gemm_tcgen05_head(const bf16* A, const bf16* W, float* C, int M, int N, int K, int m_cap, const NormIn& nin,
-                      int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile) {
+                      int32_t* error_flag, Stream& s, char* err, size_t errlen, int tile) {
     GemmArgs g{};
     g.C = C;
     g.M = M;
@@ -910,7 +910,7 @@ int gemm_tcgen05_head(const bf16* A, const bf16* W, float* C, int M, int N, int 
 }
 
 int gemm_tcgen05_addnorm(const bf16* A, const bf16* W, float* h, bf16* hb, float* ssq_out, int M, int N, int K,
-                         int m_cap, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile) {
+                         int m_cap, int32_t* error_flag, Stream& s, char* err, size_t errlen, int tile) {
     if (((uintptr_t)h | (uintptr_t)hb) & 15) {
         snprintf(err, errlen, "gemm: residual buffers must be 16-byte aligned");
         return -1;
@@ -928,7 +928,7 @@ int gemm_tcgen05_addnorm(const bf16* A, const bf16* W, float* h, bf16* hb, float
 }
 
 int gemm_tcgen05_swiglu(const bf16* A, const bf16* W13_interleaved, bf16* act, int M, int F2, int K, int m_cap,
-                        const NormIn& nin, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile) {
+                        const NormIn& nin, int32_t* error_flag, Stream& s, char* err, size_t errlen, int tile) {
     GemmArgs g{};
     set_norm(g, nin, K);
     g.out = act;
@@ -942,7 +942,7 @@ int gemm_tcgen05_swiglu(const bf16* A, const bf16* W13_interleaved, bf16* act, i
 
 int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, int S, int layer,
                      const float* rope_cs, const KvView& kv, int m_cap, const NormIn& nin, int32_t* error_flag,
-                     cudaStream_t s, char* err, size_t errlen, int tile) {
+                     Stream& s, char* err, size_t errlen, int tile) {
     GemmArgs g{};
     set_norm(g, nin, st.D);
     g.out = q;

@@ -63,29 +63,30 @@ struct AcceptArgs {
     RoundPost* post;         // mapped host memory
     int32_t* tally;          // [2] device: CTAs done, fewest tokens left of a live image; left at {0, INT_MAX}
     uint32_t post_stamp;
-    bool early;  // the kernel before is a forward's LM head, which triggers after its own wait (see pdl_wait)
+    bool early;  // the kernel before writes none of the state, tables and probabilities that are read here (an LM head);
+                 // in the kernels: and it triggers late (see pdl_wait)
 };
 
 // ---- row operations (model_kernels.cu)
-void launch_setup(const State& st, int phase /*0 round, 1 prefill*/, int compact, cudaStream_t s);
+void launch_setup(const State& st, int phase /*0 round, 1 prefill*/, int compact, Stream& s);
 // hb / ssq (bf16 model, may be null): the bf16 copy of the embedded rows and their partial sums of squares per
 // 32-column chunk, as the folded RMSNorm of the first projection wants them
 template <typename TA>
 void launch_embed(const State& st, int S, const TA* tok_emb, const TA* cls_emb, float* h, bf16* hb, float* ssq,
-                  cudaStream_t s);
+                  Stream& s);
 template <typename TA>
-void launch_rmsnorm(const float* h, const TA* gain, TA* out, int M, int D, float eps, cudaStream_t s);
+void launch_rmsnorm(const float* h, const TA* gain, TA* out, int M, int D, float eps, Stream& s);
 template <typename TA>
 void launch_rope_kv(const State& st, int S, int layer, const float* qkv, const float* rope_cs, TA* q, KvView kv,
-                    cudaStream_t s);
+                    Stream& s);
 template <typename TA>
-void launch_attention_ref(const State& st, int S, int layer, const TA* q, KvView kv, TA* out, cudaStream_t s);
+void launch_attention_ref(const State& st, int S, int layer, const TA* q, KvView kv, TA* out, Stream& s);
 template <typename TA>
-void launch_swiglu(const float* gu, TA* act, int M, int F, cudaStream_t s);
+void launch_swiglu(const float* gu, TA* act, int M, int F, Stream& s);
 // w_constant: W is a model weight (never written while the stream runs): fetched before the preceding kernel has finished
 template <typename TA>
 void launch_gemm_simt(const TA* A, const TA* W, float* C, int M, int N, int K, int accumulate, int w_constant,
-                      cudaStream_t s);
+                      Stream& s);
 
 // Scratch of the stand-alone verification step, carved from one allocation.
 struct VerifyScratch {
@@ -104,51 +105,51 @@ struct VerifyDesc {  // mirrors hbsjd_verify_desc
 // Enqueues set-up, probability/accept and commit kernels on caller state with the given scratch.
 cudaError_t verify_enqueue(const VerifyDesc& d, const VerifyScratch& sc, const float* logits, const float* q_prev,
                            float* p_out, int32_t* cursor, int32_t* seq, uint8_t* delta, int32_t* qbase,
-                           int32_t* m_out, cudaStream_t s);
+                           int32_t* m_out, Stream& s);
 
 // ---- persistent tensor-core ragged attention, bf16, head size 64 (attention_tma.cu)
 bool attention_tma_supported(const State& st, const KvView& kv);
-// To be launched directly behind a QKV projection of the same forward (whose late trigger it relies on, see pdl_wait).
+// To be launched directly behind a QKV projection of the same forward (which writes no tables and no old keys).
 // q_rows_cap: row capacity of the q buffer.  Returns 0 or a negative code with a message in err.
 int launch_attention_tma(const State& st, int S, int layer, const bf16* q, int q_rows_cap, KvView kv, bf16* out,
-                         int32_t* error_flag, cudaStream_t s, char* err, size_t errlen);
+                         int32_t* error_flag, Stream& s, char* err, size_t errlen);
 
 // ---- state kernels (state_kernels.cu)
 void launch_init_state(const State& st, const int32_t* prefix_tokens, const int32_t* prefix_len,
-                       const int32_t* labels, cudaStream_t s);
-void launch_prefill_advance(const State& st, int S, cudaStream_t s);
-void launch_init_window(const State& st, uint32_t seed_lo, uint32_t seed_hi, cudaStream_t s);
-void launch_export_tokens(const State& st, int32_t* out, cudaStream_t s);
+                       const int32_t* labels, Stream& s);
+void launch_prefill_advance(const State& st, int S, Stream& s);
+void launch_init_window(const State& st, uint32_t seed_lo, uint32_t seed_hi, Stream& s);
+void launch_export_tokens(const State& st, int32_t* out, Stream& s);
 // synthetic state for the threshold calibration: the first `live` images at cursor T/2, the rest finished
-void launch_calib_state(const State& st, int live, cudaStream_t s);
-void launch_prob_accept(const State& st, const AcceptArgs& a, cudaStream_t s);
-void launch_commit(const State& st, const AcceptArgs& a, cudaStream_t s);
+void launch_calib_state(const State& st, int live, Stream& s);
+void launch_prob_accept(const State& st, const AcceptArgs& a, Stream& s);
+void launch_commit(const State& st, const AcceptArgs& a, Stream& s);
 // smallest commit over the live slots of this round, from the accept flags (batch-synchronous progress)
-void launch_sync_min(const State& st, const AcceptArgs& a, int32_t* m_sync, cudaStream_t s);
+void launch_sync_min(const State& st, const AcceptArgs& a, int32_t* m_sync, Stream& s);
 int accept_smem_bytes(int V);
 // persistent form of launch_prob_accept for vocabularies up to 16384 (accept_persistent.cu)
 bool accept_persistent_supported(const State& st);
-void launch_accept_persistent(const State& st, const AcceptArgs& a, int n_sms, cudaStream_t s);
+void launch_accept_persistent(const State& st, const AcceptArgs& a, int n_sms, Stream& s);
 // streaming multiprocessors of the current device
 int device_sm_count();
 // counters: place of CNT_ERROR (a bounded wait that gave up), in memory that the host can read
 void launch_probs(const float* lc, const float* lu, int rows, int V, float cfg_scale, float temperature, int top_k,
-                  float* p, int32_t* counters, cudaStream_t s);
+                  float* p, int32_t* counters, Stream& s);
 void launch_probs_persistent(const float* lc, const float* lu, int rows, int V, float cfg_scale, float temperature,
-                             int top_k, float* p, int32_t* counters, int n_sms, cudaStream_t s);
+                             int top_k, float* p, int32_t* counters, int n_sms, Stream& s);
 
 // empty kernel launched like every other (timing aid, model_kernels.cu)
-void launch_noop(cudaStream_t s);
+void launch_noop(Stream& s);
 
 // ---- distillation score (score_kernels.cu)
-void launch_bikl_rows(const float* ls, const float* lt, int rows, int V, float* out, cudaStream_t s);
+void launch_bikl_rows(const float* ls, const float* lt, int rows, int V, float* out, Stream& s);
 // terms of the inputs of one scoring chunk (slot tables of st; logits rows slot * W + i of both models)
 void launch_bikl_slots(const State& st, int S, const float* ls, const float* lt, const int32_t* prefix_len,
-                       float* pos, cudaStream_t s);
+                       float* pos, Stream& s);
 void launch_score_init(const State& st, const int32_t* tokens, const int32_t* labels, const int32_t* prefix_len,
-                       float* pos, cudaStream_t s);
+                       float* pos, Stream& s);
 void launch_score_reduce(int B, int T, const int32_t* prefix_len, const float* pos, float* per_image, float* loss,
-                         cudaStream_t s);
+                         Stream& s);
 
 // ---- tcgen05 GEMM (gemm_tcgen05.cu)
 // C[M,N] fp32 (+)= A[M,K] bf16 . W[N,K]^T bf16.  force_bn: 0 = choose the tile width from the shape.
@@ -158,7 +159,7 @@ void launch_score_reduce(int B, int T, const int32_t* prefix_len, const float* p
 // w_constant: W is a model weight (never written while the stream runs), so its first tiles may be fetched before
 // the preceding kernel has finished.  acc_wait_ns: 0, or a shorter limit of the epilogue's accumulator wait.
 int gemm_tcgen05_run(const bf16* A, const bf16* W, float* C, int M, int N, int K, int accumulate, int force_bn,
-                     int m_cap, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int w_constant = 1,
+                     int m_cap, int32_t* error_flag, Stream& s, char* err, size_t errlen, int w_constant = 1,
                      unsigned int acc_wait_ns = 0);
 int gemm_tcgen05_tile_n(int M, int N, int K);
 // Cached TMA descriptor of a row-major bf16 [rows, K] matrix seen as (64 columns, rows, K / 64) with a box of
@@ -174,18 +175,18 @@ struct NormIn {
 // (tile: as gemm_tcgen05_run's force_bn, here and below)
 // act[M, F] bf16 = silu(gate) * up, from A[M,K] . W13i^T where W13i[2F, K] holds gate row f at 2f, up row f at 2f+1.
 int gemm_tcgen05_swiglu(const bf16* A, const bf16* W13_interleaved, bf16* act, int M, int F2, int K, int m_cap,
-                        const NormIn& nin, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile = 0);
+                        const NormIn& nin, int32_t* error_flag, Stream& s, char* err, size_t errlen, int tile = 0);
 // logits[M, N] fp32 = norm(x) . W^T with the norm folded as above.
 int gemm_tcgen05_head(const bf16* A, const bf16* W, float* C, int M, int N, int K, int m_cap, const NormIn& nin,
-                      int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile = 0);
+                      int32_t* error_flag, Stream& s, char* err, size_t errlen, int tile = 0);
 // Residual update h[M, N] fp32 += A[M,K] . W^T, which also leaves what the next folded norm needs: hb = bf16(h)
 // and ssq_out[M][N / 32] = sums of squares of the new h over each 32-column chunk (fixed order, no atomics).
 int gemm_tcgen05_addnorm(const bf16* A, const bf16* W, float* h, bf16* hb, float* ssq_out, int M, int N, int K,
-                         int m_cap, int32_t* error_flag, cudaStream_t s, char* err, size_t errlen, int tile = 0);
+                         int m_cap, int32_t* error_flag, Stream& s, char* err, size_t errlen, int tile = 0);
 // QKV projection of the normed activations A[M, D] with the 2D RoPE and the paged KV write fused:
 // q[M, D] bf16 rotated; rotated k and v stored at each row's (cache row, sequence index).
 int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, int S, int layer,
                      const float* rope_cs, const KvView& kv, int m_cap, const NormIn& nin, int32_t* error_flag,
-                     cudaStream_t s, char* err, size_t errlen, int tile = 0);
+                     Stream& s, char* err, size_t errlen, int tile = 0);
 
 }  // namespace hbsjd

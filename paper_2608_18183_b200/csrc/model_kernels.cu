@@ -94,7 +94,7 @@ __global__ void k_setup(State st, int phase, int compact) {
     }
 }
 
-void launch_setup(const State& st, int phase, int compact, cudaStream_t s) {
+void launch_setup(const State& st, int phase, int compact, Stream& s) {
     launch_k(k_setup, dim3(1), dim3(1024), 0, s, st, phase, compact);
 }
 
@@ -102,7 +102,7 @@ __global__ void k_noop() {
     pdl_wait();
     pdl_trigger();
 }
-void launch_noop(cudaStream_t s) { launch_k(k_noop, dim3(1), dim3(32), 0, s); }
+void launch_noop(Stream& s) { launch_k(k_noop, dim3(1), dim3(32), 0, s); }
 
 // ------------------------------------------------------------------ embedding gather
 // hb / ssq (may be null): bf16 copy of the row and its sums of squares per 32-column chunk (what the RMSNorm
@@ -147,11 +147,11 @@ __global__ void __launch_bounds__(128) k_embed(State st, int S, const TA* __rest
 
 template <typename TA>
 void launch_embed(const State& st, int S, const TA* tok_emb, const TA* cls_emb, float* h, bf16* hb, float* ssq,
-                  cudaStream_t s) {
+                  Stream& s) {
     launch_k(k_embed<TA>, dim3(st.nb * S * st.W), dim3(128), 0, s, st, S, tok_emb, cls_emb, h, hb, ssq);
 }
-template void launch_embed<float>(const State&, int, const float*, const float*, float*, bf16*, float*, cudaStream_t);
-template void launch_embed<bf16>(const State&, int, const bf16*, const bf16*, float*, bf16*, float*, cudaStream_t);
+template void launch_embed<float>(const State&, int, const float*, const float*, float*, bf16*, float*, Stream&);
+template void launch_embed<bf16>(const State&, int, const bf16*, const bf16*, float*, bf16*, float*, Stream&);
 
 // ------------------------------------------------------------------ RMSNorm: out = x * rsqrt(mean(x^2)+eps) * g
 // One warp per row; the row stays in registers between the two passes (D <= 2048 through the vector path).
@@ -222,7 +222,7 @@ __global__ void k_rmsnorm(const float* __restrict__ h, const TA* __restrict__ ga
 }
 
 template <typename TA>
-void launch_rmsnorm(const float* h, const TA* gain, TA* out, int M, int D, float eps, cudaStream_t s) {
+void launch_rmsnorm(const float* h, const TA* gain, TA* out, int M, int D, float eps, Stream& s) {
     if (D % 4 == 0 && D <= 2048) {
         const int grid = (M + 7) / 8;
         if (D <= 512) launch_k(k_rmsnorm_warp<TA, 4>, dim3(grid), dim3(256), 0, s, h, gain, out, M, D, eps);
@@ -233,8 +233,8 @@ void launch_rmsnorm(const float* h, const TA* gain, TA* out, int M, int D, float
         launch_k(k_rmsnorm<TA>, dim3(M), dim3(128), 0, s, h, gain, out, D, eps);
     }
 }
-template void launch_rmsnorm<float>(const float*, const float*, float*, int, int, float, cudaStream_t);
-template void launch_rmsnorm<bf16>(const float*, const bf16*, bf16*, int, int, float, cudaStream_t);
+template void launch_rmsnorm<float>(const float*, const float*, float*, int, int, float, Stream&);
+template void launch_rmsnorm<bf16>(const float*, const bf16*, bf16*, int, int, float, Stream&);
 
 // ------------------------------------------------------------------ 2D RoPE + KV write
 // One thread per (row, rotation pair).  rope_cs: [T][dh/2][2] cos/sin by sequence index.
@@ -280,11 +280,11 @@ __global__ void k_rope_kv(State st, int S, int layer, const float* __restrict__ 
 
 template <typename TA>
 void launch_rope_kv(const State& st, int S, int layer, const float* qkv, const float* rope_cs, TA* q, KvView kv,
-                    cudaStream_t s) {
+                    Stream& s) {
     launch_k(k_rope_kv<TA>, dim3(st.nb * S * st.W), dim3(128), 0, s, st, S, layer, qkv, rope_cs, q, kv);
 }
-template void launch_rope_kv<float>(const State&, int, int, const float*, const float*, float*, KvView, cudaStream_t);
-template void launch_rope_kv<bf16>(const State&, int, int, const float*, const float*, bf16*, KvView, cudaStream_t);
+template void launch_rope_kv<float>(const State&, int, int, const float*, const float*, float*, KvView, Stream&);
+template void launch_rope_kv<bf16>(const State&, int, int, const float*, const float*, bf16*, KvView, Stream&);
 
 // ------------------------------------------------------------------ reference attention (one warp per row, head)
 // Query at sequence index s = c+i attends keys 0..s of its cache row (cached prefix + this round's
@@ -361,14 +361,14 @@ __global__ void k_attention_ref(State st, int S, int layer, const TA* __restrict
 }
 
 template <typename TA>
-void launch_attention_ref(const State& st, int S, int layer, const TA* q, KvView kv, TA* out, cudaStream_t s) {
+void launch_attention_ref(const State& st, int S, int layer, const TA* q, KvView kv, TA* out, Stream& s) {
     const int nw = 4;
     dim3 grid(st.nb * S * st.W, (st.Hh + nw - 1) / nw);
     const size_t smem = (size_t)nw * (st.T + st.dh) * sizeof(float);
     launch_k(k_attention_ref<TA>, dim3(grid), dim3(nw * 32), smem, s, st, S, layer, q, kv, out);
 }
-template void launch_attention_ref<float>(const State&, int, int, const float*, KvView, float*, cudaStream_t);
-template void launch_attention_ref<bf16>(const State&, int, int, const bf16*, KvView, bf16*, cudaStream_t);
+template void launch_attention_ref<float>(const State&, int, int, const float*, KvView, float*, Stream&);
+template void launch_attention_ref<bf16>(const State&, int, int, const bf16*, KvView, bf16*, Stream&);
 
 // ------------------------------------------------------------------ SwiGLU: act = silu(gate) * up
 template <typename TA>
@@ -383,12 +383,12 @@ __global__ void k_swiglu(const float* __restrict__ gu, TA* __restrict__ act, int
 }
 
 template <typename TA>
-void launch_swiglu(const float* gu, TA* act, int M, int F, cudaStream_t s) {
+void launch_swiglu(const float* gu, TA* act, int M, int F, Stream& s) {
     dim3 grid((F + 255) / 256, M);
     launch_k(k_swiglu<TA>, dim3(grid), dim3(256), 0, s, gu, act, F);
 }
-template void launch_swiglu<float>(const float*, float*, int, int, cudaStream_t);
-template void launch_swiglu<bf16>(const float*, bf16*, int, int, cudaStream_t);
+template void launch_swiglu<float>(const float*, float*, int, int, Stream&);
+template void launch_swiglu<bf16>(const float*, bf16*, int, int, Stream&);
 
 // ------------------------------------------------------------------ CUDA-core GEMM (fp32 model)
 // C[M,N] (+)= A[M,K] . W[N,K]^T, fp32 accumulation in increasing k, 64x64 tile, 4x4 outputs per thread.
@@ -532,13 +532,13 @@ __global__ void __launch_bounds__(64) k_gemm_simt_small(const float* __restrict_
 
 template <typename TA>
 void launch_gemm_simt(const TA* A, const TA* W, float* C, int M, int N, int K, int accumulate, int w_constant,
-                      cudaStream_t s) {
+                      Stream& s) {
     if constexpr (sizeof(TA) == 4) {
         // up to four 16 x 16 tiles per SM (they are resident together); beyond that the 64 x 64 kernel has at least 37
         // tiles and reads every operand four times less often
         const long tiles = (long)((M + SS_T - 1) / SS_T) * ((N + SS_T - 1) / SS_T);
         if (K % 4 == 0 && (((uintptr_t)A | (uintptr_t)W) & 15) == 0 && tiles <= 4L * device_sm_count()) {
-            launch_k(k_gemm_simt_small, dim3((N + SS_T - 1) / SS_T, (M + SS_T - 1) / SS_T), dim3(64), 0, s, A, W, C, M,
+            launch_early(k_gemm_simt_small, dim3((N + SS_T - 1) / SS_T, (M + SS_T - 1) / SS_T), dim3(64), 0, s, A, W, C, M,
                      N, K, accumulate, w_constant);
             return;
         }
@@ -546,6 +546,6 @@ void launch_gemm_simt(const TA* A, const TA* W, float* C, int M, int N, int K, i
     dim3 grid((N + 63) / 64, (M + 63) / 64);
     launch_k(k_gemm_simt<TA>, dim3(grid), dim3(256), 0, s, A, W, C, M, N, K, accumulate);
 }
-template void launch_gemm_simt<float>(const float*, const float*, float*, int, int, int, int, int, cudaStream_t);
+template void launch_gemm_simt<float>(const float*, const float*, float*, int, int, int, int, int, Stream&);
 
 }  // namespace hbsjd

@@ -198,22 +198,22 @@ __global__ void k_score_reduce(int B, int T, const int32_t* __restrict__ prefix_
 
 }  // namespace
 
-void launch_bikl_rows(const float* ls, const float* lt, int rows, int V, float* out, cudaStream_t s) {
+void launch_bikl_rows(const float* ls, const float* lt, int rows, int V, float* out, Stream& s) {
     launch_k(k_bikl_rows, dim3(rows), dim3(BK_THREADS), 0, s, ls, lt, V, out);
 }
 
 void launch_bikl_slots(const State& st, int S, const float* ls, const float* lt, const int32_t* prefix_len,
-                       float* pos, cudaStream_t s) {
+                       float* pos, Stream& s) {
     launch_k(k_bikl_slots, dim3(st.W, S), dim3(BK_THREADS), 0, s, st, ls, lt, prefix_len, pos);
 }
 
 void launch_score_init(const State& st, const int32_t* tokens, const int32_t* labels, const int32_t* prefix_len,
-                       float* pos, cudaStream_t s) {
+                       float* pos, Stream& s) {
     launch_k(k_score_init, dim3(st.B), dim3(128), 0, s, st, tokens, labels, prefix_len, pos);
 }
 
 void launch_score_reduce(int B, int T, const int32_t* prefix_len, const float* pos, float* per_image, float* loss,
-                         cudaStream_t s) {
+                         Stream& s) {
     launch_k(k_score_reduce, dim3(1), dim3(1024), 0, s, B, T, prefix_len, pos, per_image, loss);
 }
 

@@ -37,7 +37,7 @@ __global__ void k_init_state(State st, const int32_t* __restrict__ prefix_tokens
 }
 
 void launch_init_state(const State& st, const int32_t* prefix_tokens, const int32_t* prefix_len,
-                       const int32_t* labels, cudaStream_t s) {
+                       const int32_t* labels, Stream& s) {
     launch_k(k_init_state, dim3(st.B), dim3(128), 0, s, st, prefix_tokens, prefix_len, labels);
 }
 
@@ -50,7 +50,7 @@ __global__ void k_prefill_advance(State st, int S) {
     if (n > 0) st.pfill[st.slot_img[slot]] = st.slot_c[slot] + n;
 }
 
-void launch_prefill_advance(const State& st, int S, cudaStream_t s) {
+void launch_prefill_advance(const State& st, int S, Stream& s) {
     launch_k(k_prefill_advance, dim3((S + 127) / 128), dim3(128), 0, s, st, S);
 }
 
@@ -79,7 +79,7 @@ __global__ void k_init_window(State st, uint32_t seed_lo, uint32_t seed_hi) {
     }
 }
 
-void launch_init_window(const State& st, uint32_t seed_lo, uint32_t seed_hi, cudaStream_t s) {
+void launch_init_window(const State& st, uint32_t seed_lo, uint32_t seed_hi, Stream& s) {
     launch_k(k_init_window, dim3((st.B + 63) / 64), dim3(64), 0, s, st, seed_lo, seed_hi);
 }
 
@@ -91,7 +91,7 @@ __global__ void k_export_tokens(State st, int32_t* __restrict__ out) {
         out[(size_t)b * st.T + t] = st.seq[(size_t)b * (st.T + 1) + t + 1];
 }
 
-void launch_export_tokens(const State& st, int32_t* out, cudaStream_t s) {
+void launch_export_tokens(const State& st, int32_t* out, Stream& s) {
     launch_k(k_export_tokens, dim3(st.B), dim3(128), 0, s, st, out);
 }
 
@@ -114,7 +114,7 @@ __global__ void k_calib_state(State st, int live) {
     }
 }
 
-void launch_calib_state(const State& st, int live, cudaStream_t s) {
+void launch_calib_state(const State& st, int live, Stream& s) {
     launch_k(k_calib_state, dim3(st.B), dim3(128), 0, s, st, live);
 }
 
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(ACC_THREADS, 2) k_prob_accept(State st, Accept
 int accept_smem_bytes(int V) { return V * (int)sizeof(float) + (int)sizeof(AccShared); }
 
 void launch_probs(const float* lc, const float* lu, int rows, int V, float cfg_scale, float temperature, int top_k,
-                  float* p, int32_t* counters, cudaStream_t s) {
+                  float* p, int32_t* counters, Stream& s) {
     // The persistent kernel has one CTA of 1024 threads per SM, this file's k_probs two of 512: up to 4096 entries a row
     // leaves the wide CTA a group of four per thread and its latency counts (4096 rows of 4096: 67 us against 75);
     // above, its prefetched rows win (2048 rows of 8192 with guidance 62 -> 56 us, 1024 rows of 16384 56 -> 42 us
@@ -645,7 +645,7 @@ int device_sm_count() {
     return n[dev];
 }
 
-void launch_prob_accept(const State& st, const AcceptArgs& a, cudaStream_t s) {
+void launch_prob_accept(const State& st, const AcceptArgs& a, Stream& s) {
     if (accept_persistent_supported(st)) {
         launch_accept_persistent(st, a, device_sm_count(), s);
         return;
@@ -694,6 +694,7 @@ __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) 
     AccShared& sh = *(AccShared*)(smem_raw + (size_t)st.V * sizeof(float));
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int slot = blockIdx.x;
+    if (!a.early) pdl_wait();
     const int n = __ldcg(st.slot_n + slot), img = __ldcg(st.slot_img + slot), c = __ldcg(st.slot_c + slot);
     if (n == 0) {
         pdl_wait();
@@ -883,15 +884,17 @@ __global__ void k_sync_min(State st, AcceptArgs a, int32_t* __restrict__ m_sync)
     }
 }
 
-void launch_sync_min(const State& st, const AcceptArgs& a, int32_t* m_sync, cudaStream_t s) {
+void launch_sync_min(const State& st, const AcceptArgs& a, int32_t* m_sync, Stream& s) {
     launch_k(k_sync_min, dim3(1), dim3(1024), 0, s, st, a, m_sync);
 }
 
-void launch_commit(const State& st, const AcceptArgs& a, cudaStream_t s) {
+void launch_commit(const State& st, const AcceptArgs& a, Stream& s) {
     static int configured[64] = {0};
     const int bytes = accept_smem_bytes(st.V);
     ensure_dynamic_smem(k_commit, bytes, configured);
-    launch_k(k_commit, dim3(a.S), dim3(ACC_THREADS), bytes, s, st, a);
+    AcceptArgs b = a;
+    b.early = s.late;  // neither the accept kernel nor k_sync_min writes what k_commit reads first
+    launch_early(k_commit, dim3(a.S), dim3(ACC_THREADS), bytes, s, st, b);
 }
 
 // ------------------------------------------------------------------ stand-alone verification step
@@ -917,7 +920,7 @@ VerifyScratch verify_scratch_carve(void* base, int batch, int window) {
 
 cudaError_t verify_enqueue(const VerifyDesc& d, const VerifyScratch& sc, const float* logits, const float* q_prev,
                            float* p_out, int32_t* cursor, int32_t* seq, uint8_t* delta, int32_t* qbase,
-                           int32_t* m_out, cudaStream_t s) {
+                           int32_t* m_out, Stream& s) {
     State st;
     memset(&st, 0, sizeof(st));
     st.B = d.batch;
@@ -958,7 +961,7 @@ cudaError_t verify_enqueue(const VerifyDesc& d, const VerifyScratch& sc, const f
     a.post = nullptr;
     a.tally = nullptr;
     a.post_stamp = 0;
-    a.early = false;
+    a.early = false;  // the set-up kernel writes the slot tables
     // the commit counters accumulate with atomics: they must start at zero on every call
     cudaError_t e = cudaMemsetAsync(sc.counters, 0, 8 * sizeof(int32_t), s);
     if (e != cudaSuccess) return e;
@@ -1010,7 +1013,7 @@ extern "C" int hbsjd_verify_static(void* cuda_stream, const hbsjd_verify_desc* d
     VerifyDesc vd;
     memcpy(&vd, d, sizeof(vd));
     const VerifyScratch sc = verify_scratch_carve(base, d->batch, d->window);
-    cudaStream_t s = (cudaStream_t)cuda_stream;
+    Stream s((cudaStream_t)cuda_stream);
     // verify_enqueue zeroes the counters; the slot tables, flags and candidates are fully rewritten for
     // every (image, position) that is read back, so stale contents of the previous call are never used
     if (verify_enqueue(vd, sc, logits, q_prev, p_out, cursor, seq, delta, qbase, m_out, s) != cudaSuccess)
