@@ -198,7 +198,7 @@ def _gemm_context(binding, synth, s, rows):
 
 
 def bench_gemm_tiles(args):
-    """Every tile shape of the GEMM kernel on the decoder's shapes, over a range of activation rows M."""
+    """Every tile shape of the GEMM kernels on the decoder's shapes, over a range of activation rows M."""
     import torch
     from paper_2608_18183_b200 import binding, synth
     s = synth.WORKLOADS[args.workload].shape
@@ -214,9 +214,12 @@ def bench_gemm_tiles(args):
             A = torch.randn(M, K, device="cuda", generator=g).bfloat16()
             Cm = torch.zeros(M, N, device="cuda")
             us = {}
-            # 0: the library's choice; 512 / 640: 256 x 256 / 256 x 128 tiles on CTA pairs
-            for tile in (0, 32, 64, 128, 256, 512, 640):
-                if tile and N % (tile if tile < 512 else 768 - tile):
+            # 0: the library's choice; 512 / 640: 256 x 256 / 256 x 128 tiles on CTA pairs; from 16032: the kernel for few
+            # rows, rows x columns of its tile
+            few = (16032, 16064, 32032, 32064) if M <= 512 else ()
+            for tile in (0, 32, 64, 128, 256, 512, 640) + few:
+                width = tile % 1000 if tile >= 1000 else 768 - tile if tile >= 512 else tile
+                if tile and N % width:
                     continue
                 def burst():
                     ctx.hbsjd_debug_gemm(A, Wt, Cm, accumulate=acc, reps=20, tile=tile)

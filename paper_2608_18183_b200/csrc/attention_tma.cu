@@ -141,7 +141,7 @@ struct AttnArgs {
     const bf16* q;
     bf16* out;
     int32_t* error_flag;
-    bool few;    // the grid leaves half of the SMs free
+    bool few;    // a small grid of one-block windows: trigger early
     bool early;  // the kernel before triggers late (see pdl_wait)
 };
 
@@ -312,9 +312,11 @@ template <int QB>
 __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS)
     k_attention_tma(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const AttnArgs a) {
-    // Before or after the wait (see pdl_wait for what the line rests on): a grid that leaves half of the SMs free lets the
-    // next kernel's CTAs fetch their weights there early (one L image: 37.0 against 37.5 ms), a larger one is better off
-    // without them (six XL images 771 -> 767 ms, 64 B images 78.5 -> 78.1, 24 L images token by token 271.1 -> 270.3).
+    // Before or after the wait: a grid that leaves three quarters of the SMs free lets the next kernel's CTAs fetch their
+    // weights there early (rollouts of one and two L images, 16 and 32 CTAs, take 0.97 and 0.99 times the time); a larger
+    // one is better off without them (three L images, 48 CTAs: 1.007 times with them; six XL images 1.005), and so are
+    // windows of two blocks and more, whose attention lasts longer (one to three XL images of window 32, 20 to 60
+    // CTAs: 1.016, 1.004, 1.009).
     if (a.few) pdl_trigger();
     using cfg = AttnCfg<QB>;
     constexpr int NCW = cfg::NCW, HPC = cfg::HPC, STAGES = cfg::STAGES;
@@ -520,7 +522,7 @@ cudaError_t launch_qb(const CUtensorMap& mk, const CUtensorMap& mv, AttnArgs a, 
     const long items = (long)a.S * a.st.nb * a.G;
     long grid = (long)device_sm_count() * per_sm;
     if (grid > items) grid = items;
-    a.few = 2 * grid <= device_sm_count();
+    a.few = QB == 1 && 4 * grid <= device_sm_count();
     const long stripes = (items + grid - 1) / grid;
     const int smem = fixed + 16 * (int)(stripes < LIST_MAX ? stripes : LIST_MAX);
     a.early = s.late;
