@@ -1127,8 +1127,8 @@ int hbsjd_score(hbsjd_ctx* student, hbsjd_ctx* teacher, int batch, const int32_t
     // The two models are independent until their logits meet.  Contexts that share a stream would run one after the
     // other, and most of a forward of few images is latency (every forward has tails in which SMs idle), so the student
     // moves to a stream of its own for the call, behind everything the shared stream holds, and back: 9 images of B
-    // against L 11.6 -> 9.8 ms, 128 of L against XL 77.5 -> 75.2 ms.  The event
-    // times of a profile would overlap: a profiled call keeps the one stream.
+    // against L 0.84 times the time, 128 of L against XL 0.97.  The event times of a profile would overlap: a profiled
+    // call keeps the one stream.
     cudaStream_t shared = c->stream;
     const bool fork = teacher->stream == shared && !c->profiling && !teacher->profiling;
     if (fork) {

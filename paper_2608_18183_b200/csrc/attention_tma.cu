@@ -40,9 +40,9 @@ constexpr int TILE_BYTES = KB * DH * 2;  // one K or V tile of one head: 4 KB
 // Split by the window's 16-query blocks QB.  A consumer warp takes 16 queries of one head; windows above 32 inputs have
 // three or four consumer warps with one head, smaller ones two heads.  What bounds an item is the latency of its chain
 // of key blocks, so windows above 16 take two blocks at a time (see attend), at the price of registers for two CTAs per
-// SM instead of three: 6 images of 36 layers, contexts up to 576: 16.6 -> 12.9 us per launch, rollout 876 -> 832 ms;
-// scoring of 128 images (windows of 64) 80.1 -> 78.9 ms.  Up to 16 inputs three CTAs with one block at a time stay
-// ahead (two at a time: 24 images one token at a time 303 -> 307 to 317 ms, 64 images of 16 inputs 84.2 -> 85.7 ms).
+// SM instead of three: 6 images of 36 layers, contexts up to 576: 16.6 -> 12.9 us per launch, the rollout 0.95 times the
+// time; scoring of 128 images (windows of 64) 0.985.  Up to 16 inputs three CTAs with one block at a time stay
+// ahead (two at a time: 24 images one token at a time 1.01 to 1.05 times the time, 64 images of 16 inputs 1.02).
 template <int QB>
 struct AttnCfg {
     static constexpr int HPC = QB >= 3 ? 1 : 2;
@@ -94,7 +94,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 }
 // Keys and values are read once per layer and round, a stream larger than L2 at full batch: marked to be evicted first,
 // so that the layer's activations and residual stream, which the next kernels read, stay in L2 (rollout of 200 L images with
-// long prefixes 426.4 -> 420.9 ms, 128 images 632.3 -> 628.5 ms).
+// long prefixes 0.987 times the time, 128 images 0.994).
 __device__ __forceinline__ uint64_t evict_first_policy() {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
@@ -172,8 +172,8 @@ __device__ __forceinline__ bool item_at(const AttnArgs& a, uint32_t list, int st
 
 // 2^x for the softmax weights and corrections, by the one instruction.  exp2f also returns results below 2^-126; here they
 // meet a normaliser of at least 1 and outputs of the values' size, whose last bits they cannot reach, and the range
-// handling was a sixth of this kernel's instructions (rollout of six XL images 823.4 -> 813.9 ms, 24 L images one token
-// at a time 307.3 -> 303.3 ms).
+// handling was a sixth of this kernel's instructions (rollouts of six XL images and of 24 L images one token at a time
+// 0.988 times the time).
 __device__ __forceinline__ float ex2(float x) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -347,8 +347,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
     // that precedes the projection is complete here, the slot tables and the keys and values of earlier rounds among it
     // (read through L2).  Queries and the window's own keys come after the wait.  The chain of look-ups and the first
     // stages' copies, two microseconds, so lie beside the projection's tail: rollouts of 24 L images token by token
-    // 294.0 -> 284.5 ms, one L image 42.8 -> 41.0, 64 B images 82.9 -> 80.7, six XL images 813 -> 796, 128 L images 624 ->
-    // 617 ms.
+    // 0.97 times the time, one L image 0.96, 64 B images 0.97, six XL images 0.98, 128 L images 0.99.
     const int n_items = a.S * st.nb * a.G;
     const int grid = (int)gridDim.x, cta = (int)blockIdx.x;
     // stripe s of the sorted list: CTA j takes position s * grid + j, in reversed order on odd stripes

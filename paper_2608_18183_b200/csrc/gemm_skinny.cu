@@ -109,9 +109,9 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
     if (!RES && warp == cfg::NW + 2) {
         // ---------------------------------------------------------------- helper: what the epilogue needs per row
         // (slot tables, page table and rotation table sit behind one another and the norm's partial sums are added
-        // in order: all of it off the consumers' path).  The look-ups need nothing of the kernel before this one, and the
-        // kernels that come before a QKV projection trigger after their own wait: they go before this one's.  (24 L
-        // images token by token 282.9 -> 274.0 ms, one L image 40.6 -> 39.5, six XL images 783 -> 772.)
+        // in order: all of it off the consumers' path).  The look-ups need nothing of the kernel before this one, so behind a kernel
+        // that triggers late they go before the wait.  (24 L images token by token and one L image 0.97 times the time, six
+        // XL images 0.986.)
         if (EPI != EPI_QKV || !g.early) pdl_wait();
         const int row = m0 + lane;
         if (lane < TM && row < g.M) {
@@ -353,10 +353,11 @@ bool skinny_tile_exists(int code) { return code == 16032 || code == 16064 || cod
 
 // The narrowest tile whose CTAs are all resident at once (two per SM): with more CTAs the second round costs more
 // than the tcgen05 kernel's longer chain (M = 64, N 5632: 9.2 against 6.7 us; M = 128, N 3072: 8.5 against 6.3 us),
-// with fewer the chain is what is left (M = 128, N 1024 K 2816, 256 CTAs of 16 x 32: 8.7 against 12.3 us).  The LM
-// head has so many columns that only the widest tile gets close, up to 32 rows (M = 32, N 16384: 8.9 against 11.6 us).
-// Three row tiles of 16 x 64 fit where two of 32 x 32 do not (M = 48, N 5632, 264 CTAs: 5.9 against the tcgen05
-// kernel's 6.7 us; rollouts of 24 images by window 1, 306.4 -> 294.2 ms).
+// with fewer the chain is what is left (N 1024: K 2816 at M = 64, 128, 208, 288: 7.0, 8.3, 9.9, 9.9 against 11.5 to 11.8 us, K
+// 1024 at M = 288, the last that fits: 5.3 against 6.5; N 768 up to M = 384: 5.0 against 5.7; N 1280 up to M = 224: 6.2 against
+// 7.3).  The LM head has so many columns that only the widest tile gets close, up to 32 rows (M = 32, N 16384: 8.9
+// against 11.6 us).  Three row tiles of 16 x 64 fit where two of 32 x 32 do not (M = 48, N 5632, 264 CTAs: 5.9 against the
+// tcgen05 kernel's 6.7 us; rollouts of 24 images by window 1 in 0.96 times the time).
 int skinny_tile_code(int M, int N, int sms) {
     const long m16 = (M + 15) / 16, m32 = (M + 31) / 32, most = 2L * sms;
     if (N % 64 != 0) return 0;

@@ -253,8 +253,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
         }
     }
     // The rest of the first tiles' weights goes to L2 meanwhile, once per weight tile: models whose layers do not stay
-    // there read them from HBM in every round (rollouts of six XL images 796.8 -> 784.8 ms, of 64 B images 80.9 -> 80.2,
-    // of 128 L images 607 -> 604 ms).
+    // there read them from HBM in every round (rollouts of six XL images 0.985 times the time, of 64 B images 0.991, of 128 L
+    // images 0.995).
     if (warp == 1 && lane == 0 && g.w_constant && unit < tiles_n) {
         const int n0 = unit * BN + (PAIR ? (int)rank * (BN / 2) : 0);
         for (int kb = cfg::GROUPS * cfg::KG; kb < num_kb; ++kb) tma_prefetch_2d(&map_w, kb * BK, n0);
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                 tmem_ld32(tbase + (uint32_t)c0, r);
                 const int col = n0 + c0;
                 if (EPI == EPI_ADDNORM) {
-                    // this warp's staging: two buffers of (fp32 tile 4 KB, swizzled | bf16 tile 2 KB, dense)
+                    // this warp's staging: one buffer, at BN = 32 two, of (fp32 tile 4 KB, swizzled | bf16 tile 2 KB, dense)
                     const uint32_t sb32 =
                         staging + (uint32_t)(warp - 2) * (uint32_t)cfg::WARP_STAGING +
                         (cfg::WARP_STAGING > 6144 ? (uint32_t)(nchunk++ & 1u) * 6144u : 0u);
@@ -836,18 +836,18 @@ int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int ma
 
 }  // namespace
 
-// Tile width by a small cost model: waves of tiles over the SMs times the time of one tile.  Measured with the
-// phase stamps of this kernel (HBSJD_GEMM_TIMELINE): a k-block costs about 0.47 us at N = 256 (MMA rate) and no
-// less than about 0.19 us however narrow the tile is -- there the ring of operand stages is what limits it (the
-// 16 KB activation tile of every k-block has to cross from L2 whatever N is, and about 160 KB can be in flight
-// per SM); the epilogue adds about 0.15 us per 32 columns.  Large problems end up with 256 (CTA pairs), small
-// ones with the widest tile that still fits one wave.
 bool make_tensor_map_kblocks(::CUtensorMap_st* map, const void* base, int rows, int K, int box_rows, int box_kb) {
     if (box_kb == 1) return cached_map(map, MapKey{base, rows, K, box_rows, 5}, encode_map_kb<1>);
     if (box_kb == 2) return cached_map(map, MapKey{base, rows, K, box_rows, 3}, encode_map_kb<2>);
     return box_kb == 4 && cached_map(map, MapKey{base, rows, K, box_rows, 4}, encode_map_kb<4>);
 }
 
+// Tile width by a small cost model: waves of tiles over the SMs times the time of one tile.  Measured with time stamps
+// in this kernel: a k-block costs about 0.47 us at N = 256 (MMA rate) and no
+// less than about 0.19 us however narrow the tile is -- there the ring of operand stages is what limits it (the
+// 16 KB activation tile of every k-block has to cross from L2 whatever N is, and about 160 KB can be in flight
+// per SM); the epilogue adds about 0.15 us per 32 columns.  Large problems end up with 256 (CTA pairs), small
+// ones with the widest tile that still fits one wave.
 int gemm_tcgen05_tile_n(int M, int N, int K) {
     const long tiles_m = (M + BM - 1) / BM;
     const int sms = num_sms(), num_kb = K / BK;

@@ -38,7 +38,7 @@ struct State {
 enum { CNT_LIVE = 0, CNT_COMMITTED = 1, CNT_REJECTS = 2, CNT_LIVE_SETUP = 3, CNT_SLOTS = 4, CNT_ERROR = 5,
        CNT_SUM_KEYS = 6 /* sum over active slots of c+n */, CNT_SUM_N = 7 /* sum of n */ };
 
-// What the host needs to know of a finished round, written by the GPU into mapped host memory; stamp last.
+// What the host needs to know of a finished round, written by the GPU into mapped host memory.
 struct RoundPost {
     // low half: the eight counters, then the fewest tokens still to commit over the images that are live after the
     // round; high half: the round's stamp.  Eight bytes are written at once: a word with the stamp is the round's.

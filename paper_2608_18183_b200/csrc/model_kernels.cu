@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(256) k_rmsnorm_warp(const float* __restrict__ 
                                                       TA* __restrict__ out, int M, int D, float eps) {
     const int lane = threadIdx.x & 31;
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    // gain read four at a time: 32 two-byte loads per thread in their place cost the rollout of 128 L images 12 of 645 ms
+    // gain read four at a time: 32 two-byte loads per thread in their place cost the rollout of 128 L images 2 %
     struct __align__(4 * sizeof(TA)) Gain4 { TA g[4]; };
     pdl_wait();
     pdl_trigger();
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(256) k_gemm_simt(const TA* __restrict__ A, con
 // ring requested before it needs the first (W's before the preceding kernel has finished when W is a model weight)
 // and runs one chain of fused multiply-adds per output in increasing k -- the sum of the 64 x 64 kernel, bit for bit.
 // A rollout of four images of the two-layer fp32 model (32 rows, N 64..384, K 64 and 192) spent 11.8 us per launch in
-// the 64 x 64 kernel and took 10.4 ms; with this one 5.9 ms.
+// the 64 x 64 kernel and takes 0.57 times the time with this one.
 constexpr int SS_T = 16, SS_K = 64, SS_PITCH = SS_K + 4, SS_STAGES = 4;
 
 __global__ void __launch_bounds__(64) k_gemm_simt_small(const float* __restrict__ A, const float* __restrict__ W,

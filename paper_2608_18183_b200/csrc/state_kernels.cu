@@ -661,9 +661,10 @@ void launch_prob_accept(const State& st, const AcceptArgs& a, Stream& s) {
 // First reject by ballot over the accept flags.  The token committed after the accepted prefix is drawn
 // here, at that one position: the replacement ~ [p_j - q]+ (point-mass proposal: p_j with the draft removed)
 // at the first reject j (Eq. 5 and the sentence after it), else the bonus token ~ p_{n-1}, both with word 1
-// of (image, position, round); the probabilities are read back from this round's p rows.  Thread 0 then
+// of (image, position, round); the probabilities are read back from this round's p rows.  Warp 0 then
 // commits, advances the cursor -- the KV commit is this cursor move: entries at and after the new cursor are
 // recomputed by the next forward (Sec. 4.2 "Independent progress") -- and rebuilds the window.
+
 // One thread of every CTA of k_commit, when the CTA's slot is done (left: tokens the slot's image still has to commit,
 // INT_MAX if it has none or no image).  The last one hands the round's counters to the host, which polls the words in
 // its own memory, in place of a copy and a stream synchronisation.
@@ -686,7 +687,8 @@ __device__ __forceinline__ void post_round(const State& st, const AcceptArgs& a,
 // What bounds it is a chain of look-ups, each a round trip to L2, with one token to draw in between.  The slot's entries
 // and the old window are therefore read before the wait (the kernel before this one triggers after its own, see
 // pdl_wait), flags and candidates together behind it, and the new window is put together in shared memory (rollouts of
-// four tiny images 4.74 -> 4.60 ms, one L image 40.9 -> 40.7, 64 B images 80.1 -> 79.9).
+// four tiny images 0.97 times the time, one L image 0.995, 64 B images 0.998).  The eight vectors of p and q in flight take
+// all 128 registers of a thread and spill 28 bytes; with four the segment of a 16384-entry row takes two trips.
 __global__ void __launch_bounds__(ACC_THREADS) k_commit(State st, AcceptArgs a) {
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
