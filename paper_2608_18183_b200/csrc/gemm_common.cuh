@@ -66,31 +66,15 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {  // as mbar_try, which may sleep a while first
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
 // Bounded wait (about one second unless a shorter limit is given).  Returns false when it gave up or another
 // role raised `abort`.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort,
                                           unsigned long long limit_ns = 1000000000ull) {
-    if (limit_ns < 1000000ull) {  // a short limit is checked after every poll
-        const unsigned long long t0 = globaltimer_ns();
-        while (!mbar_test(bar, parity))
-            if (*abort || globaltimer_ns() - t0 > limit_ns) return false;
-        return true;
-    }
     if (mbar_try(bar, parity)) return true;
     const unsigned long long t0 = globaltimer_ns();
+    const int polls = limit_ns < 1000000ull ? 1 : 128;  // a short limit is checked after every poll
     for (;;) {
-        for (int it = 0; it < 128; ++it)
+        for (int it = 0; it < polls; ++it)
             if (mbar_try(bar, parity)) return true;
         if (*abort) return false;
         if (globaltimer_ns() - t0 > limit_ns) return false;

@@ -73,6 +73,26 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], uint32
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// A wait with a limit shorter than the time that mbar_try may sleep (time-out test; in a function of its own: this poll inside
+// mbar_wait cost the tcgen05 epilogue 0.5 % of a rollout of six XL images).
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_wait_brief(uint32_t bar, uint32_t parity, volatile uint32_t* abort, uint32_t limit_ns) {
+    const unsigned long long t0 = globaltimer_ns();
+    while (!mbar_test(bar, parity))
+        if (*abort || globaltimer_ns() - t0 > limit_ns) return false;
+    return true;
+}
+
 template <int TM, int TN, int EPI>
 __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
     k_gemm_skinny(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
@@ -208,11 +228,11 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
             return ring + ((uint32_t)(kb / KG) % cfg::STAGES) * cfg::STAGE_BYTES + KG * cfg::A_BYTES +
                    (uint32_t)(kb % KG) * cfg::W_BYTES + b_row;
         };
-        const unsigned long long limit = g.acc_wait_ns ? g.acc_wait_ns : 1000000000ull;
         auto ready = [&](int kb) {  // the k-block's stage has landed: one answer for the warp, whose lanes stay together
             if (kb % KG) return true;
             const uint32_t gi = (uint32_t)(kb / KG);
-            const bool in = mbar_wait(full0 + 8 * (gi % cfg::STAGES), (gi / cfg::STAGES) & 1u, abort_flag, limit);
+            const uint32_t bar = full0 + 8 * (gi % cfg::STAGES), ph = (gi / cfg::STAGES) & 1u;
+            const bool in = g.acc_wait_ns ? mbar_wait_brief(bar, ph, abort_flag, g.acc_wait_ns) : mbar_wait(bar, ph, abort_flag);
             return __all_sync(0xffffffffu, in) != 0;
         };
         bool ok = ready(0);
