@@ -18,7 +18,8 @@ __global__ void k_setup(State st, int phase, int compact) {
     __shared__ int carry, sum_keys, sum_n;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (tid == 0) carry = sum_keys = sum_n = 0;
-    const bool failed = phase == 0 && __ldcg(st.counters + CNT_ERROR) != 0;
+    const int32_t uncollected = __ldcg(st.counters + CNT_ERROR);  // (in flight over the barrier, beside the cursors)
+    auto failed = [&] { return phase == 0 && uncollected != 0; };
     __syncthreads();
     for (int base = 0; base < st.B; base += blockDim.x) {
         const int b = base + tid;
@@ -30,7 +31,7 @@ __global__ void k_setup(State st, int phase, int compact) {
                     atomicExch(&st.counters[CNT_ERROR], 16);
                     c = st.T;
                 }
-                n = c < st.T && !failed ? min(st.W, st.T - c) : 0;
+                n = c < st.T && !failed() ? min(st.W, st.T - c) : 0;
             } else {
                 c = st.pfill[b];
                 n = c < st.klen[b] ? min(st.W, st.klen[b] - c) : 0;
@@ -54,7 +55,7 @@ __global__ void k_setup(State st, int phase, int compact) {
         for (int w = 0; w < wid; ++w) before += warp_tot[w];
         const int pos = before + incl - act;
         if (b < st.B) {
-            if (compact && !failed) {
+            if (compact && !failed()) {
                 if (act) {
                     st.slot_img[pos] = b;
                     st.slot_c[pos] = c;
@@ -74,7 +75,7 @@ __global__ void k_setup(State st, int phase, int compact) {
     // from this list so that every CTA streams about the same number of key blocks
     if (st.slot_sorted != nullptr) {
         __syncthreads();
-        const int n_slots = compact && !failed ? carry : st.B;
+        const int n_slots = compact && !failed() ? carry : st.B;
         for (int s0 = tid; s0 < n_slots; s0 += blockDim.x) {
             const int n0 = st.slot_n[s0], c0 = st.slot_c[s0], len = n0 > 0 ? c0 + n0 : -1;
             int rank = 0;
