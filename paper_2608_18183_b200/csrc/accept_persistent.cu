@@ -164,25 +164,28 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
     __syncthreads();
 
     // slot tables of the round in shared memory: the item walk below reads them at every step
-    int* s_n = (int*)(smem_raw + (size_t)(CFG ? 2 : 1) * V * sizeof(float) + sizeof(PShared));
-    int* s_img = s_n + a.S;
-    int* s_c = s_img + a.S;
+    // (image and n share a word: n is at most 64, images are far fewer than 2^25)
+    int* s_imgn = (int*)(smem_raw + (size_t)(CFG ? 2 : 1) * V * sizeof(float) + sizeof(PShared));
+    int* s_row = s_imgn + a.S;
+    int* s_c = s_row + a.S;
     for (int sidx = tid; !PROBS && sidx < a.S; sidx += PT) {
-        s_n[sidx] = __ldcg(st.slot_n + sidx);
-        s_img[sidx] = __ldcg(st.slot_img + sidx);
+        s_imgn[sidx] = __ldcg(st.slot_img + sidx) << 7 | __ldcg(st.slot_n + sidx);
+        s_row[sidx] = st.first_row(sidx);
         s_c[sidx] = __ldcg(st.slot_c + sidx);
     }
     __syncthreads();
+    auto n_of = [&](int slot) { return s_imgn[slot] & 127; };
+    auto img_of = [&](int slot) { return (int)((unsigned int)s_imgn[slot] >> 7); };
 
     const int total = a.S * W;
-    auto valid = [&](int it) { return PROBS || (it % W) < s_n[it / W]; };
+    auto valid = [&](int it) { return PROBS || (it % W) < n_of(it / W); };
     auto issue = [&](int it) {  // thread 0: both rows of item `it` into the staging area
-        const int slot = it / W, i = it % W;
+        const size_t row = PROBS ? (size_t)it : (size_t)s_row[it / W] + it % W;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
                      "r"(CFG ? 2u * row_bytes : row_bytes)
                      : "memory");
-        bulk_load(smem_addr(stage_c), a.logits + ((size_t)slot * W + i) * V, row_bytes, bar);
-        if (CFG) bulk_load(smem_addr(stage_u), a.logits_u + ((size_t)slot * W + i) * V, row_bytes, bar);
+        bulk_load(smem_addr(stage_c), a.logits + row * V, row_bytes, bar);
+        if (CFG) bulk_load(smem_addr(stage_u), a.logits_u + row * V, row_bytes, bar);
     };
     // The state an item needs besides its logits -- the draft token under test, whether its proposal is a point
     // mass, the proposal row and the proposal's entry q(z) -- sits behind three levels of dependent global loads.
@@ -192,8 +195,8 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
     auto fetch_raw = [&](int it) {
         Raw r = {0, 0, 0};
         const int slot = it / W, i = it % W;
-        if (i < s_n[slot] - 1) {  // the last input of a window has no draft to verify
-            const int img = s_img[slot];
+        if (i < n_of(slot) - 1) {  // the last input of a window has no draft to verify
+            const int img = img_of(slot);
             const size_t at = (size_t)img * (st.T + 1) + s_c[slot] + i + 1;
             r.z = __ldcg(st.seq + at);
             r.dl = __ldcg(st.delta + at);
@@ -205,13 +208,13 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
     auto fetch_qz = [&](int it, const Raw& r) {
         const int slot = it / W, i = it % W;
         float qz = 1.0f;
-        if (i < s_n[slot] - 1 && r.z >= 0 && r.z < V && ((r.z % CHUNK) >> 2) == tid && r.dl == 0 && !a.greedy) {
+        if (i < n_of(slot) - 1 && r.z >= 0 && r.z < V && ((r.z % CHUNK) >> 2) == tid && r.dl == 0 && !a.greedy) {
             const int qi = s_c[slot] + i + 1 - r.qb - 1;  // row of the previous round's probabilities
             if (qi < 0 || qi >= st.Wmax) {
                 atomicExch(&st.counters[CNT_ERROR], ERR_BAD_PROPOSAL_ROW);
                 qz = INFINITY;  // alpha = 0: rejected
             } else {
-                qz = __ldcg(a.pprev + ((size_t)s_img[slot] * st.Wmax + qi) * V + r.z);
+                qz = __ldcg(a.pprev + ((size_t)img_of(slot) * st.Wmax + qi) * V + r.z);
             }
         }
         return qz;
@@ -229,7 +232,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
     // random words of an item (Philox keyed by image, position, round): computed one item ahead by one thread
     auto make_words = [&](int it, uint32_t* dst) {
         const int slot = it / W, i = it % W;
-        philox4x32_10((uint32_t)s_img[slot], (uint32_t)(s_c[slot] + i + 1), a.round, 0u, a.seed_lo, a.seed_hi, dst);
+        philox4x32_10((uint32_t)img_of(slot), (uint32_t)(s_c[slot] + i + 1), a.round, 0u, a.seed_lo, a.seed_hi, dst);
     };
     uint32_t par = 0;  // item parity
     if (!PROBS && it < total && tid == PT - 32) make_words(it, sh.words[0]);
@@ -251,8 +254,8 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
         Raw raw_next = {0, 0, 0};
         if (!PROBS && nxt < total) raw_next = fetch_raw(nxt);  // consumed after barrier (1)
         const int slot = it / W, i = it % W;
-        const bool last = PROBS || i == s_n[slot] - 1;
-        const size_t oidx = PROBS ? (size_t)it : (size_t)s_img[slot] * st.Wmax + i;
+        const bool last = PROBS || i == n_of(slot) - 1;
+        const size_t oidx = PROBS ? (size_t)it : (size_t)img_of(slot) * st.Wmax + i;
         float* pout = a.pcur + oidx * V;
 
         int z = -1;

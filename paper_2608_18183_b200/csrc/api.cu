@@ -55,9 +55,11 @@ struct hbsjd_ctx {
     int32_t* h_counters;  // pinned [8]
     RoundPost* post;      // mapped host memory [3]: by round parity the counters of the last rounds; error code of hbsjd_probs
     RoundPost* post_dev;  // the same, as the GPU addresses it
-    int32_t* tally;       // [2] device, see AcceptArgs
+    int32_t* tally;       // [3] device, see AcceptArgs
     uint32_t post_seq;    // stamp of the last round enqueued
     int min_left;         // fewest tokens left of a live image, after the last collected round
+    int rows;             // inputs per branch of the round that follows the last collected one.  Windows only shorten, so
+                          // it is enough for every later round too
     cudaEvent_t ev0, ev1, ev2;
     cudaStream_t side;  // stand-in for `stream` (its priority) while hbsjd_score runs two contexts that share one
     hbsjd_params P;
@@ -188,7 +190,7 @@ int gemm<bf16>(hbsjd_ctx* c, const void* A, const void* W, float* C, int M, int 
     return rc == 0 ? 0 : (rc == -1 ? HBSJD_EINVAL : HBSJD_ECUDA);
 }
 
-// One batched verifier forward over S slots (Sec. 4.2 "Batched verification").
+// One batched verifier forward over S slots and c->st.R rows per branch (Sec. 4.2 "Batched verification").
 // stop_layer >= 0 (debugging): return after the attention sub-block (stop_stage 0) or the whole block
 // (stop_stage 1) of that layer, leaving the activation buffers as that point found them.
 template <typename TA>
@@ -199,10 +201,10 @@ template <>
 int forward<float>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int stop_stage) {
     typedef float TA;
     const State& st = c->st;
-    const int M = st.nb * S * st.W, D = st.D, F = st.F;
+    const int M = st.nb * st.R, D = st.D, F = st.F;
     Stream& s = c->stream;
     const KvView kv = kv_view(c);
-    launch_embed<TA>(st, S, (const TA*)c->tok_emb, (const TA*)c->cls_emb, c->h, nullptr, nullptr, s);
+    launch_embed<TA>(st, (const TA*)c->tok_emb, (const TA*)c->cls_emb, c->h, nullptr, nullptr, s);
     c->launches++;
     auto norm = [&](const float* x, const void* gain) {
         const int ps = prof_begin(c, HBSJD_PROF_OTHER, (double)M * D * (4.0 + sizeof(TA)));
@@ -215,11 +217,11 @@ int forward<float>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int st
         int rc;
         norm(c->h, w.g_attn);
         if ((rc = gemm<TA>(c, c->a, w.w_qkv, c->qkv, M, 3 * D, D, 0))) return rc;
-        launch_rope_kv<TA>(st, S, l, c->qkv, c->rope_cs, (TA*)c->q, kv, s);
+        launch_rope_kv<TA>(st, l, c->qkv, c->rope_cs, (TA*)c->q, kv, s);
         c->launches++;
         {
             const int ps = prof_begin(c, HBSJD_PROF_ATTENTION, 0.0);
-            launch_attention_ref<TA>(st, S, l, (const TA*)c->q, kv, (TA*)c->o, s);
+            launch_attention_ref<TA>(st, l, (const TA*)c->q, kv, (TA*)c->o, s);
             prof_end(c, ps);
             c->launches++;
         }
@@ -258,7 +260,7 @@ int forward<float>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int st
 template <>
 int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int stop_stage) {
     const State& st = c->st;
-    const int M = st.nb * S * st.W, D = st.D, F = st.F;
+    const int M = st.nb * st.R, D = st.D, F = st.F;
     const int Mcap = 2 * c->Bmax * c->Wmax;  // row capacity of the activation buffers
     Stream& s = c->stream;
     const KvView kv = kv_view(c);
@@ -290,7 +292,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
         c->launches++;
         return rc;
     };
-    launch_embed<bf16>(st, S, (const bf16*)c->tok_emb, (const bf16*)c->cls_emb, c->h, fold ? a : nullptr,
+    launch_embed<bf16>(st, (const bf16*)c->tok_emb, (const bf16*)c->cls_emb, c->h, fold ? a : nullptr,
                        fold ? c->ssq : nullptr, s);
     c->launches++;
     for (int l = 0; l < st.L; ++l) {
@@ -299,7 +301,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
         if (!fold) norm(w.g_attn);
         ps = prof_begin(c, HBSJD_PROF_GEMM, 2.0 * M * 3 * D * D, M,
                         es * ((double)M * D + 3.0 * D * D) + es * 3.0 * M * D);  // q, k, v written
-        rc = gemm_tcgen05_qkv(a, (const bf16*)w.w_qkv, (bf16*)c->q, st, S, l, c->rope_cs, kv, Mcap, nin, eflag, s,
+        rc = gemm_tcgen05_qkv(a, (const bf16*)w.w_qkv, (bf16*)c->q, st, l, c->rope_cs, kv, Mcap, nin, eflag, s,
                               c->err, sizeof(c->err), c->force_tile);
         prof_end(c, ps);
         if (rc) return done(rc);
@@ -309,7 +311,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
                                       sizeof(c->err));
             if (rc) return HBSJD_ECUDA;
         } else {
-            launch_attention_ref<bf16>(st, S, l, (const bf16*)c->q, kv, (bf16*)c->o, s);
+            launch_attention_ref<bf16>(st, l, (const bf16*)c->q, kv, (bf16*)c->o, s);
         }
         prof_end(c, ps);
         c->launches += 2;
@@ -389,6 +391,7 @@ int sync_counters(hbsjd_ctx* c) {
 int enqueue_round(hbsjd_ctx* c) {
     const int compact = choose_compact(c, c->live);
     const int S = compact ? c->live : c->st.B;
+    c->st.R = c->rows;
     launch_setup(c->st, 0, compact, c->stream);
     if (c->round == c->fail_round) {  // code 1: a bounded wait that gave up
         c->fail_round = -1;
@@ -399,7 +402,7 @@ int enqueue_round(hbsjd_ctx* c) {
     if (rc) return rc;
     AcceptArgs a;
     a.logits = c->logits;
-    a.logits_u = c->logits + (size_t)S * c->st.W * c->st.V;
+    a.logits_u = c->logits + (size_t)c->st.R * c->st.V;
     a.pcur = c->pbuf[c->parity];
     a.pprev = c->pbuf[c->parity ^ 1];
     a.flag = c->flag;
@@ -459,7 +462,7 @@ int collect_round(hbsjd_ctx* c, uint32_t stamp, Wait wait) {
     } else {
         // the stream is asked now and then: after a CUDA error nothing will be posted
         unsigned spins = 0;
-        for (int x = 8; x >= 0; --x) {
+        for (int x = 9; x >= 0; --x) {
             unsigned long long w;
             while ((uint32_t)((w = word[x]) >> 32) != stamp) {
                 if (wait == YIELD) sched_yield();
@@ -476,9 +479,9 @@ int collect_round(hbsjd_ctx* c, uint32_t stamp, Wait wait) {
         }
         if ((rc = check_error(c))) return rc;
     }
-    if (c->h_counters[CNT_LIVE_SETUP] != c->live) {
-        snprintf(c->err, sizeof(c->err), "live count mismatch: host %d device %d", c->live,
-                 c->h_counters[CNT_LIVE_SETUP]);
+    if (c->h_counters[CNT_LIVE_SETUP] != c->live || c->h_counters[CNT_SUM_N] > c->rows) {
+        snprintf(c->err, sizeof(c->err), "live count mismatch: host %d device %d, rows %d and %d", c->live,
+                 c->h_counters[CNT_LIVE_SETUP], c->rows, c->h_counters[CNT_SUM_N]);
         return HBSJD_ESTATE;
     }
     c->stats.rounds += 1;
@@ -489,6 +492,7 @@ int collect_round(hbsjd_ctx* c, uint32_t stamp, Wait wait) {
     c->stats.rejects = c->h_counters[CNT_REJECTS];
     c->live = c->h_counters[CNT_LIVE];
     c->min_left = (int)(uint32_t)word[8];
+    c->rows = (int)(uint32_t)word[9];
     return 0;
 }
 
@@ -530,7 +534,7 @@ int run_rounds(hbsjd_ctx* c, int max_rounds) {
 
 void free_all(hbsjd_ctx* c) {
     void* ptrs[] = {c->w_img, c->rope_cs, c->kc, c->vc, c->page_table, c->st.cursor, c->st.seq, c->st.delta,
-                    c->st.qbase, c->st.label, c->st.klen, c->st.pfill, c->st.slot_img, c->st.slot_c, c->st.slot_n, c->st.slot_sorted,
+                    c->st.qbase, c->st.label, c->st.klen, c->st.pfill, c->st.slot_img, c->st.slot_c, c->st.slot_n, c->st.slot_row, c->st.row_pos, c->st.slot_sorted,
                     c->st.counters, c->st.m_last, c->st.j_last, c->pbuf[0], c->pbuf[1], c->flag, c->cand_rep,
                     c->cand_ref, c->h, c->qkv, c->gu, c->logits, c->a, c->q, c->o, c->act, c->ssq,
                     c->stage_tok, c->stage_len, c->stage_lab, c->stage_out, c->verify_scratch,
@@ -687,6 +691,7 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
         (rc = dev_alloc(c, &st.label, Bm)) || (rc = dev_alloc(c, &st.klen, Bm)) ||
         (rc = dev_alloc(c, &st.pfill, Bm)) || (rc = dev_alloc(c, &st.slot_img, Bm)) ||
         (rc = dev_alloc(c, &st.slot_c, Bm)) || (rc = dev_alloc(c, &st.slot_n, Bm)) ||
+        (rc = dev_alloc(c, &st.slot_row, Bm)) || (rc = dev_alloc(c, &st.row_pos, 2 * Bm * Wm)) ||
         (rc = dev_alloc(c, &st.slot_sorted, Bm)) ||
         (rc = dev_alloc(c, &st.counters, (size_t)8)) || (rc = dev_alloc(c, &st.m_last, Bm)) ||
         (rc = dev_alloc(c, &st.j_last, Bm)) || (rc = dev_alloc(c, &c->pbuf[0], Bm * Wm * V)) ||
@@ -729,7 +734,7 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
     CK(cudaHostAlloc((void**)&c->post, 3 * sizeof(RoundPost), cudaHostAllocMapped));
     memset(c->post, 0, 3 * sizeof(RoundPost));
     CK(cudaHostGetDevicePointer((void**)&c->post_dev, c->post, 0));
-    if ((rc = dev_alloc(c, &c->tally, (size_t)2))) return rc;
+    if ((rc = dev_alloc(c, &c->tally, (size_t)3))) return rc;
     {
         const int32_t none = 0x7fffffff;
         CK(cudaMemcpyAsync(c->tally + 1, &none, sizeof(none), cudaMemcpyHostToDevice, c->stream));
@@ -840,7 +845,7 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
     CK(cudaMemcpyAsync(ht.data(), prefix_tokens, (size_t)batch * T * sizeof(int32_t), cudaMemcpyDeviceToHost,
                        c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    int live = 0, min_left = T;
+    int live = 0, min_left = T, rows = 0;
     for (int b = 0; b < batch; ++b) {
         if (hk[b] < 0 || hk[b] > T || hl[b] < 0 || hl[b] > c->d.n_classes) {
             snprintf(c->err, sizeof(c->err), "image %d: prefix_len %d or label %d out of range", b, hk[b], hl[b]);
@@ -854,6 +859,7 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
         if (hk[b] < T) {
             ++live;
             min_left = std::min(min_left, T - hk[b]);
+            rows += std::min(p->window, T - hk[b]);
         }
     }
     c->P = *p;
@@ -878,6 +884,7 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
     c->parity = 0;
     c->live = live;
     c->min_left = min_left;
+    c->rows = rows;
     c->have_rollout = false;
 
     CK(cudaEventRecord(c->ev0, c->stream));
@@ -886,7 +893,12 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
     // prefix pre-filling: cache sequence indices 0..k-1 in chunks of W (no LM head)
     for (int pr = 0;; ++pr) {
         int act = 0;
-        for (int b = 0; b < batch; ++b) act += hk[b] > pr * p->window;
+        st.R = 0;
+        for (int b = 0; b < batch; ++b) {
+            const int n = std::min(p->window, hk[b] - pr * p->window);
+            act += n > 0;
+            st.R += std::max(n, 0);
+        }
         if (act == 0) break;
         const int compact = choose_compact(c, act);
         const int S = compact ? act : batch;
@@ -1036,6 +1048,7 @@ int score_run(hbsjd_ctx* student, hbsjd_ctx* teacher, int batch, const int32_t* 
         st.W = W;
         st.H = 1;
         st.nb = 1;
+        st.R = batch * W;
         x->have_rollout = false;
         x->live = 0;
         launch_score_init(st, tokens, class_labels, prefix_len, x == student ? pos : nullptr, x->stream);
@@ -1216,6 +1229,7 @@ int hbsjd_calibrate_gamma(hbsjd_ctx* c, int batch, int window, int guidance, int
     int gamma = 0;
     for (int p = 0; p < 5; ++p) {
         const int live = points[p] < 1 ? 1 : points[p];
+        st.R = live * std::min(window, st.T - st.T / 2);
         float best[2] = {0.f, 0.f};
         for (int compact = 0; compact < 2; ++compact) {
             const int S = compact ? live : batch;
@@ -1283,7 +1297,7 @@ int hbsjd_set_state(hbsjd_ctx* c, const int32_t* cursor, const int32_t* seq, con
     if (!c || !cursor || !seq || !delta || !qbase) return HBSJD_EINVAL;
     if (!c->have_rollout) return HBSJD_ESTATE;
     const size_t B = c->st.B, T1 = c->T + 1;
-    int live = 0;
+    int live = 0, rows = 0;
     for (size_t b = 0; b < B; ++b) {
         if (cursor[b] < 0 || cursor[b] > c->T || qbase[b] < 0 || qbase[b] > cursor[b]) {
             snprintf(c->err, sizeof(c->err), "set_state: image %zu cursor/qbase out of range", b);
@@ -1301,6 +1315,7 @@ int hbsjd_set_state(hbsjd_ctx* c, const int32_t* cursor, const int32_t* seq, con
                 return HBSJD_EINVAL;
             }
         live += cursor[b] < c->T;
+        rows += std::min(c->st.W, c->T - cursor[b]);
     }
     CK(cudaMemcpyAsync(c->st.cursor, cursor, B * 4, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->st.seq, seq, B * T1 * 4, cudaMemcpyHostToDevice, c->stream));
@@ -1308,6 +1323,7 @@ int hbsjd_set_state(hbsjd_ctx* c, const int32_t* cursor, const int32_t* seq, con
     CK(cudaMemcpyAsync(c->st.qbase, qbase, B * 4, cudaMemcpyHostToDevice, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     c->live = live;
+    c->rows = rows;
     c->round = round;
     return HBSJD_OK;
 }
@@ -1319,8 +1335,9 @@ int hbsjd_debug_forward(hbsjd_ctx* c, int layer, int stage) {
         snprintf(c->err, sizeof(c->err), "hbsjd_debug_forward: layer or stage out of range");
         return HBSJD_EINVAL;
     }
+    c->st.R = c->rows;
     launch_setup(c->st, 0, 0, c->stream);
-    const int rc = forward_any(c, c->st.B, false, layer, stage);
+    const int rc = c->rows > 0 ? forward_any(c, c->st.B, false, layer, stage) : 0;
     if (rc) return rc;
     CK(cudaGetLastError());
     c->last_S = c->st.B;
@@ -1332,7 +1349,7 @@ int hbsjd_debug_forward(hbsjd_ctx* c, int layer, int stage) {
 int hbsjd_debug_read(hbsjd_ctx* c, int what, int index, void* host_dst, size_t max_bytes) {
     if (!c || !host_dst) return HBSJD_EINVAL;
     if (!c->have_rollout || (c->round == 0 && c->dbg_layer < 0)) return HBSJD_ESTATE;
-    const int S = c->last_S, W = c->st.W, V = c->d.vocab;
+    const int S = c->last_S, V = c->d.vocab;
     std::vector<int32_t> slots((size_t)3 * S);
     CK(cudaMemcpyAsync(slots.data(), c->st.slot_img, S * 4, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaMemcpyAsync(slots.data() + S, c->st.slot_c, S * 4, cudaMemcpyDeviceToHost, c->stream));
@@ -1352,10 +1369,12 @@ int hbsjd_debug_read(hbsjd_ctx* c, int what, int index, void* host_dst, size_t m
     if (slot < 0) return 0;
     const int n = slots[2 * S + slot];
     if (n == 0) return 0;
+    size_t row0 = 0;  // first row of the slot's inputs
+    for (int s = 0; s < slot; ++s) row0 += slots[2 * S + s];
+    row0 += (size_t)branch * c->st.R;
     if (what >= HBSJD_DBG_ACT_A && what <= HBSJD_DBG_ACT_H) {
         // rows of the slot in an activation buffer, as the last (partial) forward left them
         const size_t es = c->bf16_model ? 2 : 4, D = c->d.dim, F = c->d.ffn_hidden;
-        const size_t row0 = (size_t)(branch * S + slot) * W;
         const unsigned char* src;
         size_t width;
         switch (what) {
@@ -1395,7 +1414,7 @@ int hbsjd_debug_read(hbsjd_ctx* c, int what, int index, void* host_dst, size_t m
     if (max_bytes < bytes) return HBSJD_EINVAL;
     const float* src;
     if (what == HBSJD_DBG_PROBS) src = c->pbuf[c->parity ^ 1] + (size_t)img * c->Wmax * V;
-    else if (what == HBSJD_DBG_LOGITS) src = c->logits + ((size_t)(branch * S + slot) * W) * V;
+    else if (what == HBSJD_DBG_LOGITS) src = c->logits + row0 * V;
     else return HBSJD_EINVAL;
     CK(cudaMemcpyAsync(host_dst, src, bytes, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));

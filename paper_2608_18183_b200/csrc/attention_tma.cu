@@ -1,7 +1,7 @@
 // Ragged attention over paged per-image KV caches (Sec. 4.2 "Batched verification"), bf16, head size 64:
 // persistent, warp-specialised, K/V blocks moved by TMA.
 //
-// Work item = one physical row (branch, slot) x HPC heads.  The items of a forward are dealt to the CTAs from a
+// Work item = one (branch, slot) x HPC heads.  The items of a forward are dealt to the CTAs from a
 // list sorted by context length (longest first, alternate stripes reversed), so every CTA streams about the
 // same number of key blocks.  Inside a CTA
 //   warp 0 (one lane)   producer: for every item, its keys in stages of one or two blocks of 32, K and V of a block and
@@ -145,29 +145,37 @@ struct AttnArgs {
     bool early;  // the kernel before triggers late (see pdl_wait)
 };
 
-// Position `pos` of the sorted item list, the CTA's item number `stripe` -> work item.  Returns false for an inactive slot.
 struct Item {
-    int prow, crow, c, n, head0;
+    int row0, crow, c, n, head0;
 };
-__device__ __forceinline__ bool item_at(const AttnArgs& a, uint32_t list, int stripe, int pos, Item& it) {
+// (first row, n + 128 x first head, c, cache row) of the item at position `pos`, from the slot with that rank of context length
+__device__ __forceinline__ int4 item_entry(const AttnArgs& a, int pos) {
     const State& st = a.st;
     const int per_slot = st.nb * a.G;
     const int r = pos / per_slot, rem = pos % per_slot;
     const int br = rem / a.G, g = rem % a.G;
-    // slot, n, c, image of the slot with the r-th longest context
+    const int4 e = __ldcg(st.slot_sorted + r);  // first row, n, c, image
+    return make_int4(br * st.R + e.x, e.y | (g * a.hpc) << 7, e.z, br * st.Bmax + e.w);
+}
+// Stripe s of the sorted list: CTA j takes position s * grid + j, in reversed order on odd stripes.
+__device__ __forceinline__ int position(int stripe) {
+    const int grid = (int)gridDim.x, cta = (int)blockIdx.x;
+    return stripe * grid + ((stripe & 1) ? grid - 1 - cta : cta);
+}
+// The CTA's item of a stripe.  Returns false for an inactive slot.
+__device__ __forceinline__ bool item_at(const AttnArgs& a, uint32_t list, int stripe, Item& it) {
     int4 e;
     if (stripe < LIST_MAX)
         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(e.x), "=r"(e.y), "=r"(e.z), "=r"(e.w)
                      : "r"(list + 16u * stripe));
     else
-        e = __ldcg(st.slot_sorted + r);
-    it.n = e.y;
-    if (it.n == 0) return false;
+        e = item_entry(a, position(stripe));
+    it.n = e.y & 127;
     it.c = e.z;
-    it.prow = br * a.S + e.x;
-    it.crow = br * st.Bmax + e.w;
-    it.head0 = g * a.hpc;
-    return true;
+    it.row0 = e.x;
+    it.crow = e.w;
+    it.head0 = e.y >> 7;
+    return it.n != 0;
 }
 
 // 2^x for the softmax weights and corrections, by the one instruction.  exp2f also returns results below 2^-126; here they
@@ -329,7 +337,7 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
     const uint32_t full0 = bars, empty0 = bars + 8 * STAGES;
     unsigned char* tail = smem_raw + (bars - raw) + 16 * STAGES;
     volatile uint32_t* abort_flag = (volatile uint32_t*)tail;
-    const uint32_t list = bars + 16 * STAGES + 16;  // [min(stripes, LIST_MAX)] int4: slots of this CTA's items
+    const uint32_t list = bars + 16 * STAGES + 16;  // [min(stripes, LIST_MAX)] int4: this CTA's items
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -349,14 +357,11 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
     // stages' copies, two microseconds, so lie beside the projection's tail: rollouts of 24 L images token by token
     // 0.97 times the time, one L image 0.96, 64 B images 0.97, six XL images 0.98, 128 L images 0.99.
     const int n_items = a.S * st.nb * a.G;
-    const int grid = (int)gridDim.x, cta = (int)blockIdx.x;
-    // stripe s of the sorted list: CTA j takes position s * grid + j, in reversed order on odd stripes
-    auto position = [&](int stripe) { return stripe * grid + ((stripe & 1) ? grid - 1 - cta : cta); };
+    int stripes = n_items / (int)gridDim.x;  // stripes with an item of this CTA: the whole ones, and perhaps the last
+    if (position(stripes) < n_items) ++stripes;
     // (warp 0 has the barriers to set up)
-    for (int s = threadIdx.x - 32; warp > 0 && s < LIST_MAX && s * grid < n_items; s += NCW * 32) {
-        const int pos = position(s);
-        if (pos < n_items) ((int4*)(tail + 16))[s] = __ldcg(st.slot_sorted + pos / (st.nb * a.G));
-    }
+    for (int s = threadIdx.x - 32; warp > 0 && s < LIST_MAX && s < stripes; s += NCW * 32)
+        ((int4*)(tail + 16))[s] = item_entry(a, position(s));
     __syncthreads();
 
     if (warp == 0) {
@@ -365,10 +370,9 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
             const uint64_t policy = evict_first_policy();
             uint32_t gc = 0;  // K/V stages issued so far
             bool ok = true, waited = false;
-            for (int stripe = 0; ok && stripe * grid < n_items; ++stripe) {
-                const int pos = position(stripe);
+            for (int stripe = 0; ok && stripe < stripes; ++stripe) {
                 Item it;
-                if (pos >= n_items || !item_at(a, list, stripe, pos, it)) continue;
+                if (!item_at(a, list, stripe, it)) continue;
                 const int keys = it.c + it.n, nstages = (keys + SK - 1) / SK;
                 const int32_t* pages = a.kv.table + (size_t)it.crow * a.kv.pages_per_row;
                 const int layer_row0 = a.layer * a.kv.n_pages * a.kv.page;
@@ -418,19 +422,18 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
         const int wh = cw / QB, wq = cw % QB;  // head within the item, q-block
         uint32_t gc = 0;
         bool ok = true;
-        for (int stripe = 0; ok && stripe * grid < n_items; ++stripe) {
-            const int pos = position(stripe);
+        for (int stripe = 0; ok && stripe < stripes; ++stripe) {
             Item it;
-            if (pos >= n_items || !item_at(a, list, stripe, pos, it)) continue;
+            if (!item_at(a, list, stripe, it)) continue;
             const int c = it.c, n = it.n;
             const int keys = c + n, nstages = (keys + SK - 1) / SK;
-            // ---- this warp's queries: 16 rows x 64 dims as A fragments.  Rows at or past n hold whatever the buffer
-            // holds (finite values of older forwards): their results are never written back.
+            // ---- this warp's queries: 16 rows x 64 dims as A fragments.  Fragment rows at or past n repeat the last input:
+            // their results are never written back.
             const int i0 = wq * 16 + (lane >> 2), i1 = i0 + 8;
             uint32_t qa[4][4];
             {
-                const bf16* qrow0 = a.q + ((size_t)it.prow * st.W + min(i0, st.W - 1)) * st.D + (it.head0 + wh) * DH;
-                const bf16* qrow1 = a.q + ((size_t)it.prow * st.W + min(i1, st.W - 1)) * st.D + (it.head0 + wh) * DH;
+                const bf16* qrow0 = a.q + (size_t)(it.row0 + min(i0, n - 1)) * st.D + (it.head0 + wh) * DH;
+                const bf16* qrow1 = a.q + (size_t)(it.row0 + min(i1, n - 1)) * st.D + (it.head0 + wh) * DH;
 #pragma unroll
                 for (int kc = 0; kc < 4; ++kc) {
                     const int d = kc * 16 + (lane & 3) * 2;
@@ -441,16 +444,17 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
                 }
             }
             {   // the next item's query rows towards L1 while this item's keys stream (one 128-byte line per row)
-                const int pos2 = (stripe + 1) * grid < n_items ? position(stripe + 1) : n_items;
                 Item nx;
-                if (lane < 16 && pos2 < n_items && item_at(a, list, stripe + 1, pos2, nx)) {
-                    const bf16* nq = a.q + ((size_t)nx.prow * st.W + min(wq * 16 + lane, st.W - 1)) * st.D +
-                                     (nx.head0 + wh) * DH;
+                if (lane < 16 && stripe + 1 < stripes && item_at(a, list, stripe + 1, nx)) {
+                    const bf16* nq = a.q + (size_t)(nx.row0 + min(wq * 16 + lane, nx.n - 1)) * st.D + (nx.head0 + wh) * DH;
                     asm volatile("prefetch.global.L1 [%0];" ::"l"(nq));
                 }
             }
-            const bool warp_active = wq * 16 < n;  // q-blocks wholly past the window only keep the ring moving
             const int s0 = c + i0, s1 = c + i1;    // sequence index of this thread's two query rows
+            // Keys behind the last one visible to this warp contribute nothing: skip the math (an all-masked
+            // block is an exact no-op of the online softmax, so skipping changes no bits).  q-blocks wholly past the
+            // window only keep the ring moving.
+            const int smax_warp = wq * 16 < n ? c + min(wq * 16 + 15, n - 1) : -1;
             float o[8][4];
 #pragma unroll
             for (int t = 0; t < 8; ++t) o[t][0] = o[t][1] = o[t][2] = o[t][3] = 0.f;
@@ -463,13 +467,10 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
                 const bool in = mbar_wait(full0 + 8 * gs, ph, abort_flag);
                 __syncwarp();
                 const int key0 = sg * SK;
-                // keys behind the last one visible to this warp contribute nothing: skip the math (an all-masked
-                // block is an exact no-op of the online softmax, so skipping changes no bits)
-                const int smax_warp = c + min(wq * 16 + 15, n - 1);
                 const uint32_t kt = ring + gs * cfg::STAGE_BYTES + wh * TILE_BYTES, vt = kt + HPC * TILE_BYTES;
-                if (cfg::NBLK == 2 && warp_active && key0 + KB <= smax_warp)
+                if (cfg::NBLK == 2 && key0 + KB <= smax_warp)
                     attend<cfg::NBLK>(kt, vt, cfg::BLOCK_BYTES, key0, s0, s1, c + wq * 16, lane, qa, o, m0, m1, l0, l1);
-                else if (warp_active && key0 <= smax_warp)
+                else if (key0 <= smax_warp)
                     attend<1>(kt, vt, cfg::BLOCK_BYTES, key0, s0, s1, c + wq * 16, lane, qa, o, m0, m1, l0, l1);
                 if (!__all_sync(0xffffffffu, in)) {
                     ok = false;
@@ -478,15 +479,16 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
                 if (lane == 0) mbar_arrive(empty0 + 8 * gs);  // this warp is done with the stage
             }
             if (!ok) break;
-            if (warp_active) {
+            if (smax_warp >= 0) {
                 const float inv0 = 1.0f / l0, inv1 = 1.0f / l1;
-                bf16* orow0 = a.out + ((size_t)it.prow * st.W + i0) * st.D + (it.head0 + wh) * DH;
-                bf16* orow1 = a.out + ((size_t)it.prow * st.W + i1) * st.D + (it.head0 + wh) * DH;
+                item_at(a, list, stripe, it);  // (again: its fields kept over the loop cost spills)
+                bf16* orow0 = a.out + (size_t)(it.row0 + i0) * st.D + (it.head0 + wh) * DH;
+                bf16* orow1 = a.out + (size_t)(it.row0 + i1) * st.D + (it.head0 + wh) * DH;
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
                     const int d = t * 8 + (lane & 3) * 2;
-                    if (i0 < n) *reinterpret_cast<uint32_t*>(orow0 + d) = pack_bf16(o[t][0] * inv0, o[t][1] * inv0);
-                    if (i1 < n) *reinterpret_cast<uint32_t*>(orow1 + d) = pack_bf16(o[t][2] * inv1, o[t][3] * inv1);
+                    if (i0 < it.n) *reinterpret_cast<uint32_t*>(orow0 + d) = pack_bf16(o[t][0] * inv0, o[t][1] * inv0);
+                    if (i1 < it.n) *reinterpret_cast<uint32_t*>(orow1 + d) = pack_bf16(o[t][2] * inv1, o[t][3] * inv1);
                 }
             }
         }

@@ -34,7 +34,7 @@ struct GemmArgs {
     // QKV epilogue
     bool early;       // the kernel before triggers late (see pdl_wait)
     State st;
-    int S, layer;
+    int layer;
     const float* rope_cs;  // [T][dh/2][2]
     KvView kv;
 };
@@ -121,13 +121,12 @@ __device__ __forceinline__ RowDst qkv_row(const GemmArgs& g, int row, bool valid
     rd.kvoff = 0;
     if (valid) {
         const State& st = g.st;
-        const int i = row % st.W;
-        const int slot = (row / st.W) % g.S;
-        const int br = row / (st.W * g.S);
-        rd.valid = i < __ldcg(st.slot_n + slot);  // (through L2: may be read before the grid wait)
+        int br;
+        const int2 at = st.pos_of(row, br);  // (through L2: may be read before the grid wait)
+        rd.valid = at.x >= 0;
         if (rd.valid) {
-            rd.s = __ldcg(st.slot_c + slot) + i;
-            rd.kvoff = g.kv.offset(g.layer, br * st.Bmax + __ldcg(st.slot_img + slot), rd.s);
+            rd.s = at.y;
+            rd.kvoff = g.kv.offset(g.layer, br * st.Bmax + at.x, rd.s);
         }
     }
     return rd;

@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(SkinnyCfg<TM, TN, EPI>::THREADS, 2)
         dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
     } else {  // EPI_QKV
         const size_t kvoff = row_off[lane];
-        if (kvoff == ~(size_t)0) return;  // no input in this row of the slot's window
+        if (kvoff == ~(size_t)0) return;  // no input in this row
         const int D = g.st.D;
         const int sec = col / D, cs = col % D;  // 0 q, 1 k, 2 v; a chunk never straddles sections
         uint32_t o[16];

@@ -940,19 +940,18 @@ int gemm_tcgen05_swiglu(const bf16* A, const bf16* W13_interleaved, bf16* act, i
     return run(EPI_SWIGLU, A, W13_interleaved, g, tile, 256, m_cap, s, err, errlen);
 }
 
-int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, int S, int layer,
+int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, int layer,
                      const float* rope_cs, const KvView& kv, int m_cap, const NormIn& nin, int32_t* error_flag,
                      Stream& s, char* err, size_t errlen, int tile) {
     GemmArgs g{};
     set_norm(g, nin, st.D);
     g.out = q;
-    g.M = st.nb * S * st.W;
+    g.M = st.nb * st.R;
     g.N = 3 * st.D;
     g.K = st.D;
     g.error_flag = error_flag;
     g.w_constant = 1;
     g.st = st;
-    g.S = S;
     g.layer = layer;
     g.rope_cs = rope_cs;
     g.kv = kv;

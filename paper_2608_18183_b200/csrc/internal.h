@@ -12,13 +12,16 @@ namespace hbsjd {
 
 // Device-side rollout state and per-round slot tables.  A "slot" is the place of one image in the
 // physical batch of a forward: Full execution has one slot per image of the batch (finished images
-// get n = 0), Compact execution one slot per live image.  Token row of (branch, slot, i) =
-// (branch * S + slot) * W + i.
+// get n = 0), Compact execution one slot per live image.  The rows of a forward hold inputs only, slot behind slot: token
+// row of (branch, slot, i < n) = branch * R + slot_row[slot] + i.  Windows shorten at a sequence's end, and rows of W inputs
+// per slot were 8 % padding in a rollout of 128 L images, a third where 16 to 80 tokens follow a long prefix (the rollouts
+// take 0.95 and 0.84 times the time without them).
 struct State {
     int B, T, V, D, Hh, dh, F, L, C;  // batch, tokens per image, vocab, dim, heads, head dim, ffn, layers, classes
     int Bmax, Wmax;
     int W, H;        // window (inputs per image per round), history offset
     int nb;          // branches: 1, or 2 under classifier-free guidance
+    int R;           // rows per branch of the forward; at least the inputs that it has (rows behind them are unused)
     int32_t* cursor;   // [Bmax] committed tokens
     int32_t* seq;      // [Bmax][T+1] tokens by 1-based position (committed, then drafts)
     uint8_t* delta;    // [Bmax][T+1] draft carries a point-mass proposal
@@ -29,7 +32,15 @@ struct State {
     int32_t* slot_img; // [Bmax]
     int32_t* slot_c;   // [Bmax] first sequence index of the slot's inputs
     int32_t* slot_n;   // [Bmax] number of inputs (0: inactive slot)
-    int4* slot_sorted; // [Bmax] (slot, n, c, image) by context length c + n, longest first (null: not built)
+    int32_t* slot_row; // [Bmax] first row of the slot's inputs (null: W rows per slot)
+    int2* row_pos;     // [rows per branch] (image, sequence index) of a row; image -1: unused (null: not built)
+    int4* slot_sorted; // [Bmax] (first row, n, c, image) by context length c + n, longest first (null: not built)
+    __device__ __forceinline__ int first_row(int slot) const { return slot_row ? __ldcg(slot_row + slot) : slot * W; }
+    // (image, sequence index) of row `row` of all branches, and its branch
+    __device__ __forceinline__ int2 pos_of(int row, int& br) const {
+        br = row >= R;
+        return __ldcg(row_pos + (row - (br ? R : 0)));
+    }
     int32_t* counters; // [8], see CNT_*
     int32_t* m_last;   // [Bmax] tokens committed in the last round
     int32_t* j_last;   // [Bmax] first-reject index of the last round (-1 none)
@@ -40,15 +51,16 @@ enum { CNT_LIVE = 0, CNT_COMMITTED = 1, CNT_REJECTS = 2, CNT_LIVE_SETUP = 3, CNT
 
 // What the host needs to know of a finished round, written by the GPU into mapped host memory.
 struct RoundPost {
-    // low half: the eight counters, then the fewest tokens still to commit over the images that are live after the
-    // round; high half: the round's stamp.  Eight bytes are written at once: a word with the stamp is the round's.
-    unsigned long long word[9];
-    unsigned long long pad[7];
+    // low half: the eight counters, then over the images that are live after the round the fewest tokens still to commit
+    // and the inputs of the next round; high half: the round's stamp.  Eight bytes are written at once: a word with the
+    // stamp is the round's.
+    unsigned long long word[10];
+    unsigned long long pad[6];
 };
 
 struct AcceptArgs {
-    const float* logits;    // [S][W][V], conditional
-    const float* logits_u;  // [S][W][V], unconditional (guidance)
+    const float* logits;    // [rows][V], conditional (rows as first_row says)
+    const float* logits_u;  // [rows][V], unconditional (guidance)
     float* pcur;          // [Bmax][Wmax][V] this round's probabilities (next round's proposals)
     const float* pprev;   // [Bmax][Wmax][V]
     uint8_t* flag;        // [Bmax][Wmax] 1 = draft accepted
@@ -61,7 +73,8 @@ struct AcceptArgs {
     const int32_t* m_sync;  // batch-synchronous progress: the smallest commit of the batch (null: independent)
     // k_commit's last CTA posts the round's counters to the host (null: not wanted)
     RoundPost* post;         // mapped host memory
-    int32_t* tally;          // [2] device: CTAs done, fewest tokens left of a live image; left at {0, INT_MAX}
+    int32_t* tally;          // [3] device: CTAs done, fewest tokens left of a live image, inputs of the next round; left at
+                             // {0, INT_MAX, 0}
     uint32_t post_stamp;
     bool early;  // the kernel before writes none of the state, tables and probabilities that are read here (an LM head);
                  // in the kernels: and it triggers late (see pdl_wait)
@@ -72,15 +85,13 @@ void launch_setup(const State& st, int phase /*0 round, 1 prefill*/, int compact
 // hb / ssq (bf16 model, may be null): the bf16 copy of the embedded rows and their partial sums of squares per
 // 32-column chunk, as the folded RMSNorm of the first projection wants them
 template <typename TA>
-void launch_embed(const State& st, int S, const TA* tok_emb, const TA* cls_emb, float* h, bf16* hb, float* ssq,
-                  Stream& s);
+void launch_embed(const State& st, const TA* tok_emb, const TA* cls_emb, float* h, bf16* hb, float* ssq, Stream& s);
 template <typename TA>
 void launch_rmsnorm(const float* h, const TA* gain, TA* out, int M, int D, float eps, Stream& s);
 template <typename TA>
-void launch_rope_kv(const State& st, int S, int layer, const float* qkv, const float* rope_cs, TA* q, KvView kv,
-                    Stream& s);
+void launch_rope_kv(const State& st, int layer, const float* qkv, const float* rope_cs, TA* q, KvView kv, Stream& s);
 template <typename TA>
-void launch_attention_ref(const State& st, int S, int layer, const TA* q, KvView kv, TA* out, Stream& s);
+void launch_attention_ref(const State& st, int layer, const TA* q, KvView kv, TA* out, Stream& s);
 template <typename TA>
 void launch_swiglu(const float* gu, TA* act, int M, int F, Stream& s);
 // w_constant: W is a model weight (never written while the stream runs): fetched before the preceding kernel has finished
@@ -185,7 +196,7 @@ int gemm_tcgen05_addnorm(const bf16* A, const bf16* W, float* h, bf16* hb, float
                          int m_cap, int32_t* error_flag, Stream& s, char* err, size_t errlen, int tile = 0);
 // QKV projection of the normed activations A[M, D] with the 2D RoPE and the paged KV write fused:
 // q[M, D] bf16 rotated; rotated k and v stored at each row's (cache row, sequence index).
-int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, int S, int layer,
+int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, int layer,
                      const float* rope_cs, const KvView& kv, int m_cap, const NormIn& nin, int32_t* error_flag,
                      Stream& s, char* err, size_t errlen, int tile = 0);
 

@@ -7,17 +7,18 @@
 namespace hbsjd {
 
 // ------------------------------------------------------------------ set-up / compaction (Sec. 4.3)
-// One block.  Builds the slot tables of the next forward.  Full: slot b = image b, n = 0 for inactive
-// images.  Compact: active images gathered in increasing image order (block-wide exclusive scan).
+// One block.  Builds the slot and row tables of the next forward.  Full: slot b = image b, n = 0 for inactive
+// images.  Compact: active images gathered in increasing image order (block-wide exclusive scan).  Either way the inputs'
+// rows follow one another without gaps (the scan of n).
 // Behind an error that the host has not collected yet (it may run one round ahead) no image is active: the state
 // stays the failed round's.
 __global__ void k_setup(State st, int phase, int compact) {
     pdl_wait();
     pdl_trigger();
-    __shared__ int warp_tot[32];
-    __shared__ int carry, sum_keys, sum_n;
+    __shared__ int warp_tot[32], warp_rows[32];
+    __shared__ int carry, carry_rows, sum_keys;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if (tid == 0) carry = sum_keys = sum_n = 0;
+    if (tid == 0) carry = carry_rows = sum_keys = 0;
     const int32_t uncollected = __ldcg(st.counters + CNT_ERROR);  // (in flight over the barrier, beside the cursors)
     auto failed = [&] { return phase == 0 && uncollected != 0; };
     __syncthreads();
@@ -38,39 +39,58 @@ __global__ void k_setup(State st, int phase, int compact) {
             }
         }
         const int act = n > 0;
-        if (act) {
-            atomicAdd(&sum_keys, c + n);
-            atomicAdd(&sum_n, n);
-        }
-        // exclusive scan of act over the block
-        int incl = act;
+        if (act) atomicAdd(&sum_keys, c + n);
+        // exclusive scans of act and n over the block
+        int incl = act, incl_rows = n;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
+            const int t = __shfl_up_sync(0xffffffffu, incl, o), tr = __shfl_up_sync(0xffffffffu, incl_rows, o);
+            if (lane >= o) {
+                incl += t;
+                incl_rows += tr;
+            }
         }
-        if (lane == 31) warp_tot[wid] = incl;
+        if (lane == 31) {
+            warp_tot[wid] = incl;
+            warp_rows[wid] = incl_rows;
+        }
         __syncthreads();
-        int before = carry;
-        for (int w = 0; w < wid; ++w) before += warp_tot[w];
-        const int pos = before + incl - act;
+        int before = carry, rows_before = carry_rows;
+        for (int w = 0; w < wid; ++w) {
+            before += warp_tot[w];
+            rows_before += warp_rows[w];
+        }
+        const int pos = before + incl - act, row0 = rows_before + incl_rows - n;
         if (b < st.B) {
-            if (compact && !failed()) {
-                if (act) {
-                    st.slot_img[pos] = b;
-                    st.slot_c[pos] = c;
-                    st.slot_n[pos] = n;
-                }
-            } else {
-                st.slot_img[b] = b;
-                st.slot_c[b] = c;
-                st.slot_n[b] = n;
+            const bool gather = compact && !failed();
+            const int slot = gather ? pos : b;
+            if (act || !gather) {
+                st.slot_img[slot] = b;
+                st.slot_c[slot] = c;
+                st.slot_n[slot] = n;
+                if (st.slot_row != nullptr) st.slot_row[slot] = row0;
+            }
+        }
+        if (st.row_pos != nullptr) {
+            // the warp writes its images' rows, one image after the other
+            for (unsigned int left = __ballot_sync(0xffffffffu, act); left; left &= left - 1) {
+                const int src = __ffs(left) - 1;
+                const int ib = base + wid * 32 + src;
+                const int ic = __shfl_sync(0xffffffffu, c, src), in = __shfl_sync(0xffffffffu, n, src);
+                const int ir = __shfl_sync(0xffffffffu, row0, src);
+                for (int i = lane; i < in; i += 32)
+                    if (ir + i < st.R) st.row_pos[ir + i] = make_int2(ib, ic + i);
             }
         }
         __syncthreads();
-        if (tid == blockDim.x - 1) carry = before + incl;
+        if (tid == blockDim.x - 1) {
+            carry = before + incl;
+            carry_rows = rows_before + incl_rows;
+        }
         __syncthreads();
     }
+    if (st.row_pos != nullptr)  // rows that the host has allowed for and no input takes
+        for (int r = carry_rows + tid; r < st.R; r += blockDim.x) st.row_pos[r] = make_int2(-1, 0);
     // slots by context length, longest first (ties by slot index): the attention kernel deals its work items
     // from this list so that every CTA streams about the same number of key blocks
     if (st.slot_sorted != nullptr) {
@@ -83,7 +103,7 @@ __global__ void k_setup(State st, int phase, int compact) {
                 const int l1 = st.slot_n[s1] > 0 ? st.slot_c[s1] + st.slot_n[s1] : -1;
                 rank += (l1 > len) || (l1 == len && s1 < s0);
             }
-            st.slot_sorted[rank] = make_int4(s0, n0, c0, st.slot_img[s0]);
+            st.slot_sorted[rank] = make_int4(st.first_row(s0), n0, c0, st.slot_img[s0]);
         }
     }
     if (tid == 0) {
@@ -91,7 +111,7 @@ __global__ void k_setup(State st, int phase, int compact) {
         st.counters[CNT_SLOTS] = compact ? carry : st.B;
         st.counters[CNT_LIVE] = 0;
         st.counters[CNT_SUM_KEYS] = sum_keys;
-        st.counters[CNT_SUM_N] = sum_n;
+        st.counters[CNT_SUM_N] = carry_rows;
     }
 }
 
@@ -109,22 +129,19 @@ void launch_noop(Stream& s) { launch_k(k_noop, dim3(1), dim3(32), 0, s); }
 // hb / ssq (may be null): bf16 copy of the row and its sums of squares per 32-column chunk (what the RMSNorm
 // folded into the first projection reads).  Warp w of the block owns chunks w, w + 4, ...; lane l element l.
 template <typename TA>
-__global__ void __launch_bounds__(128) k_embed(State st, int S, const TA* __restrict__ tok_emb,
+__global__ void __launch_bounds__(128) k_embed(State st, const TA* __restrict__ tok_emb,
                                                const TA* __restrict__ cls_emb, float* __restrict__ h,
                                                bf16* __restrict__ hb, float* __restrict__ ssq) {
     pdl_wait();
     pdl_trigger();
     const int row = blockIdx.x;
-    const int i = row % st.W;
-    const int slot = (row / st.W) % S;
-    const int br = row / (st.W * S);
-    const int n = st.slot_n[slot];
+    int br;
+    const int2 at = st.pos_of(row, br);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     float* dst = h + (size_t)row * st.D;
     const TA* src = nullptr;
-    if (i < n) {
-        const int img = st.slot_img[slot];
-        const int s = st.slot_c[slot] + i;
+    if (at.x >= 0) {
+        const int img = at.x, s = at.y;
         if (s == 0) {
             const int cls = br ? st.C : st.label[img];
             src = cls_emb + (size_t)cls * st.D;
@@ -147,12 +164,11 @@ __global__ void __launch_bounds__(128) k_embed(State st, int S, const TA* __rest
 }
 
 template <typename TA>
-void launch_embed(const State& st, int S, const TA* tok_emb, const TA* cls_emb, float* h, bf16* hb, float* ssq,
-                  Stream& s) {
-    launch_k(k_embed<TA>, dim3(st.nb * S * st.W), dim3(128), 0, s, st, S, tok_emb, cls_emb, h, hb, ssq);
+void launch_embed(const State& st, const TA* tok_emb, const TA* cls_emb, float* h, bf16* hb, float* ssq, Stream& s) {
+    launch_k(k_embed<TA>, dim3(st.nb * st.R), dim3(128), 0, s, st, tok_emb, cls_emb, h, hb, ssq);
 }
-template void launch_embed<float>(const State&, int, const float*, const float*, float*, bf16*, float*, Stream&);
-template void launch_embed<bf16>(const State&, int, const bf16*, const bf16*, float*, bf16*, float*, Stream&);
+template void launch_embed<float>(const State&, const float*, const float*, float*, bf16*, float*, Stream&);
+template void launch_embed<bf16>(const State&, const bf16*, const bf16*, float*, bf16*, float*, Stream&);
 
 // ------------------------------------------------------------------ RMSNorm: out = x * rsqrt(mean(x^2)+eps) * g
 // One warp per row; the row stays in registers between the two passes (D <= 2048 through the vector path).
@@ -240,27 +256,24 @@ template void launch_rmsnorm<bf16>(const float*, const bf16*, bf16*, int, int, f
 // ------------------------------------------------------------------ 2D RoPE + KV write
 // One thread per (row, rotation pair).  rope_cs: [T][dh/2][2] cos/sin by sequence index.
 template <typename TA>
-__global__ void k_rope_kv(State st, int S, int layer, const float* __restrict__ qkv,
+__global__ void k_rope_kv(State st, int layer, const float* __restrict__ qkv,
                           const float* __restrict__ rope_cs, TA* __restrict__ q, KvView kv) {
     pdl_wait();
     pdl_trigger();
     const int row = blockIdx.x;
-    const int i = row % st.W;
-    const int slot = (row / st.W) % S;
-    const int br = row / (st.W * S);
-    const int n = st.slot_n[slot];
+    int br;
+    const int2 at = st.pos_of(row, br);
     const int D = st.D, half = st.dh / 2;
     TA* qo = q + (size_t)row * D;
-    if (i >= n) {
+    if (at.x < 0) {
         for (int pe = threadIdx.x; pe < D / 2; pe += blockDim.x) {
             qo[2 * pe] = from_f<TA>(0.f);
             qo[2 * pe + 1] = from_f<TA>(0.f);
         }
         return;
     }
-    const int img = st.slot_img[slot];
-    const int s = st.slot_c[slot] + i;
-    const int crow = br * st.Bmax + img;
+    const int s = at.y;
+    const int crow = br * st.Bmax + at.x;
     const size_t off = kv.offset(layer, crow, s);
     TA* ko = (TA*)kv.k + off;
     TA* vo = (TA*)kv.v + off;
@@ -280,19 +293,17 @@ __global__ void k_rope_kv(State st, int S, int layer, const float* __restrict__ 
 }
 
 template <typename TA>
-void launch_rope_kv(const State& st, int S, int layer, const float* qkv, const float* rope_cs, TA* q, KvView kv,
-                    Stream& s) {
-    launch_k(k_rope_kv<TA>, dim3(st.nb * S * st.W), dim3(128), 0, s, st, S, layer, qkv, rope_cs, q, kv);
+void launch_rope_kv(const State& st, int layer, const float* qkv, const float* rope_cs, TA* q, KvView kv, Stream& s) {
+    launch_k(k_rope_kv<TA>, dim3(st.nb * st.R), dim3(128), 0, s, st, layer, qkv, rope_cs, q, kv);
 }
-template void launch_rope_kv<float>(const State&, int, int, const float*, const float*, float*, KvView, Stream&);
-template void launch_rope_kv<bf16>(const State&, int, int, const float*, const float*, bf16*, KvView, Stream&);
+template void launch_rope_kv<float>(const State&, int, const float*, const float*, float*, KvView, Stream&);
+template void launch_rope_kv<bf16>(const State&, int, const float*, const float*, bf16*, KvView, Stream&);
 
 // ------------------------------------------------------------------ reference attention (one warp per row, head)
 // Query at sequence index s = c+i attends keys 0..s of its cache row (cached prefix + this round's
 // window up to itself).  Two passes with the scores in shared memory; the reduction order depends on s only.
 template <typename TA>
-__global__ void k_attention_ref(State st, int S, int layer, const TA* __restrict__ q, KvView kv,
-                                TA* __restrict__ out) {
+__global__ void k_attention_ref(State st, int layer, const TA* __restrict__ q, KvView kv, TA* __restrict__ out) {
     pdl_wait();
     pdl_trigger();
     extern __shared__ float smem[];
@@ -300,21 +311,18 @@ __global__ void k_attention_ref(State st, int S, int layer, const TA* __restrict
     const int row = blockIdx.x;
     const int head = blockIdx.y * nw + wid;
     if (head >= st.Hh) return;
-    const int i = row % st.W;
-    const int slot = (row / st.W) % S;
-    const int br = row / (st.W * S);
-    const int n = st.slot_n[slot];
+    int br;
+    const int2 at = st.pos_of(row, br);
     const int dh = st.dh;
     TA* o = out + (size_t)row * st.D + head * dh;
-    if (i >= n) {
+    if (at.x < 0) {
         for (int e = lane; e < dh; e += 32) o[e] = from_f<TA>(0.f);
         return;
     }
     float* sc = smem + (size_t)wid * (st.T + dh);
     float* qs = sc + st.T;
-    const int img = st.slot_img[slot];
-    const int s = st.slot_c[slot] + i;
-    const int crow = br * st.Bmax + img;
+    const int s = at.y;
+    const int crow = br * st.Bmax + at.x;
     const TA* qv = q + (size_t)row * st.D + head * dh;
     for (int e = lane; e < dh; e += 32) qs[e] = to_f<TA>(qv[e]);
     __syncwarp();
@@ -362,14 +370,14 @@ __global__ void k_attention_ref(State st, int S, int layer, const TA* __restrict
 }
 
 template <typename TA>
-void launch_attention_ref(const State& st, int S, int layer, const TA* q, KvView kv, TA* out, Stream& s) {
+void launch_attention_ref(const State& st, int layer, const TA* q, KvView kv, TA* out, Stream& s) {
     const int nw = 4;
-    dim3 grid(st.nb * S * st.W, (st.Hh + nw - 1) / nw);
+    dim3 grid(st.nb * st.R, (st.Hh + nw - 1) / nw);
     const size_t smem = (size_t)nw * (st.T + st.dh) * sizeof(float);
-    launch_k(k_attention_ref<TA>, dim3(grid), dim3(nw * 32), smem, s, st, S, layer, q, kv, out);
+    launch_k(k_attention_ref<TA>, dim3(grid), dim3(nw * 32), smem, s, st, layer, q, kv, out);
 }
-template void launch_attention_ref<float>(const State&, int, int, const float*, KvView, float*, Stream&);
-template void launch_attention_ref<bf16>(const State&, int, int, const bf16*, KvView, bf16*, Stream&);
+template void launch_attention_ref<float>(const State&, int, const float*, KvView, float*, Stream&);
+template void launch_attention_ref<bf16>(const State&, int, const bf16*, KvView, bf16*, Stream&);
 
 // ------------------------------------------------------------------ SwiGLU: act = silu(gate) * up
 template <typename TA>

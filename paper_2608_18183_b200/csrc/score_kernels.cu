@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(BK_THREADS) k_bikl_slots(State st, const float
     const int img = st.slot_img[slot];
     const int idx = st.slot_c[slot] + i;
     if (idx < prefix_len[img]) return;
-    const size_t row = (size_t)slot * st.W + i;
+    const size_t row = (size_t)st.first_row(slot) + i;
     const float d = bikl_row(ls + row * st.V, lt + row * st.V, st.V);
     if (threadIdx.x == 0) pos[(size_t)img * st.T + idx] = d;
 }

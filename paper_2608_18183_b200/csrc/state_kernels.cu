@@ -544,8 +544,9 @@ __global__ void __launch_bounds__(ACC_THREADS, 2) k_prob_accept(State st, Accept
     const int V = st.V;
     const int img = st.slot_img[slot], c = st.slot_c[slot];
     const int t = c + i + 1;  // token position this distribution decides
-    const float* lc = a.logits + ((size_t)slot * st.W + i) * V;
-    const float* lu = st.nb == 2 ? a.logits_u + ((size_t)slot * st.W + i) * V : nullptr;
+    const size_t row = (size_t)st.first_row(slot) + i;
+    const float* lc = a.logits + row * V;
+    const float* lu = st.nb == 2 ? a.logits_u + row * V : nullptr;
     if (tid == 0) philox4x32_10((uint32_t)img, (uint32_t)t, a.round, 0u, a.seed_lo, a.seed_hi, sh.words);
 
     float* pout = a.pcur + ((size_t)img * st.Wmax + i) * V;
@@ -670,7 +671,10 @@ void launch_prob_accept(const State& st, const AcceptArgs& a, Stream& s) {
 // its own memory, in place of a copy and a stream synchronisation.
 __device__ __forceinline__ void post_round(const State& st, const AcceptArgs& a, int left) {
     if (a.post == nullptr) return;
-    if (left != 0x7fffffff) atomicMin(&a.tally[1], left);
+    if (left != 0x7fffffff) {
+        atomicMin(&a.tally[1], left);
+        atomicAdd(&a.tally[2], min(st.W, left));
+    }
     __threadfence();
     if (atomicAdd(&a.tally[0], 1) != (int)gridDim.x - 1) return;
     __threadfence();
@@ -680,8 +684,10 @@ __device__ __forceinline__ void post_round(const State& st, const AcceptArgs& a,
 #pragma unroll
     for (int x = 0; x < 8; ++x) w[x] = stamp | *(volatile uint32_t*)&st.counters[x];
     w[8] = stamp | *(volatile uint32_t*)&a.tally[1];
+    w[9] = stamp | *(volatile uint32_t*)&a.tally[2];
     a.tally[0] = 0;
     a.tally[1] = 0x7fffffff;
+    a.tally[2] = 0;
 }
 
 // What bounds it is a chain of look-ups, each a round trip to L2, with one token to draw in between.  The slot's entries

@@ -311,3 +311,25 @@ def test_a_process_that_asked_for_blocking_waits_does_not_poll():
         out[flags] = r.stdout.split()
     assert float(out[4][0]) < 0.5, out
     assert out[0][1] == out[2][1] == out[4][1]
+
+
+@pytest.mark.parametrize("window,cfg,mode", [(1, 1.0, "COMPACT"), (5, 3.0, "HYBRID"), (13, 1.0, "FULL"), (16, 3.0, "FULL"),
+                                             (33, 3.0, "COMPACT")])
+def test_windows_of_every_length_side_by_side(window, cfg, mode):
+    """The rows of a forward hold the live images' inputs only, one image behind the other: windows cut short by the end of
+    the sequence, whole ones, complete images and empty prefixes in one batch, token for token the oracle's."""
+    w = synth.WORKLOADS["tiny"]
+    T = w.shape.T
+    k = np.array([T - 1, T - window, 0, T, T - window + 1, 3, max(0, T - window - 1), T - 2, 17], dtype=np.int32)
+    rng = np.random.default_rng(window)
+    toks = rng.integers(0, w.shape.vocab, (len(k), T)).astype(np.int32)
+    lab = rng.integers(0, w.shape.n_classes, len(k)).astype(np.int32)
+    wl = synth.with_shape(w, batch=len(k), window=window, cfg_scale=cfg)
+    ctx = _ctx(wl)
+    out, st = ctx.hbsjd_rollout(G.dev(toks), G.dev(k), G.dev(lab),
+                                G.gpu_params(wl, 11, exec_mode=getattr(binding, "EXEC_" + mode), gamma=3))
+    r = O.Rollout(O.Model(w.shape, G.weights_for(w)), toks, k, lab, G.orc_params(wl, 11))
+    r.run()
+    np.testing.assert_array_equal(out.cpu().numpy(), r.tokens())
+    assert st["committed"] == sum(T - k)
+    ctx.hbsjd_destroy()
