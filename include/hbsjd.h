@@ -87,7 +87,8 @@ typedef struct {
     int64_t rejects;           /* image-rounds that ended in a rejection */
     int64_t full_rounds;       /* rounds executed in Full form */
     int64_t compact_rounds;    /* rounds executed in Compact form */
-    int64_t prefill_forwards;  /* batched forwards spent on prefix pre-filling */
+    int64_t prefill_forwards;  /* steps of `window` tokens that pre-filling the longest prefix takes (several steps share
+                                * one batched forward) */
     int64_t kernel_launches;   /* kernels of this library launched by the call */
     float ms_total;            /* GPU time of the call (CUDA events on the context's stream) */
     float ms_prefill;          /* of which state init + prefix pre-filling */
@@ -308,7 +309,7 @@ int hbsjd_bikl(hbsjd_ctx *c, const float *logits_s, const float *logits_t, int r
  * tokens and class label (no guidance, temperature 1, no top-k), then the mean over the images of the batch that
  * generated anything (k_b < T).  This is the step that follows the rollout in the on-policy distillation loop.
  *   student, teacher  two contexts with the same grid (T) and vocabulary; batch <= max_batch of both.  Both
- *                     models run full-sequence causal forwards in chunks of min(64, 2 min(max_window)) inputs per image
+ *                     models run full-sequence causal forwards, in as few parts as their activation rows allow,
  *                     through the same kernels as the rollout; their rollout state and KV caches are
  *                     overwritten (a stepped rollout cannot be continued afterwards).
  *   tokens        DEVICE int32 [batch, T]   completed trajectories (e.g. hbsjd_rollout's out_tokens)

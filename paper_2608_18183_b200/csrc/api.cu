@@ -17,6 +17,7 @@ using namespace hbsjd;
 namespace {
 
 constexpr int PAGE_TOKENS = 64;
+constexpr int PASS_ROWS = 4096;  // see create_impl
 
 struct LayerW {
     const void *g_attn, *w_qkv, *w_o, *g_ffn, *w_13, *w_2;
@@ -27,6 +28,7 @@ struct LayerW {
 struct hbsjd_ctx {
     hbsjd_model_desc d;
     int T, dh, Bmax, Wmax;
+    int rows_cap;        // rows of the activation buffers
     bool bf16_model;
     bool fold_norm;      // bf16 model: RMSNorm folded into the GEMM epilogues (launch-bound contexts), else its own kernel
     bool unit_gains;     // every norm gain of the model is exactly 1
@@ -202,6 +204,7 @@ int forward<float>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int st
     typedef float TA;
     const State& st = c->st;
     const int M = st.nb * st.R, D = st.D, F = st.F;
+    const bool kv_only = !want_logits && stop_layer < 0;  // pre-filling: of the last layer only keys and values are wanted
     Stream& s = c->stream;
     const KvView kv = kv_view(c);
     launch_embed<TA>(st, (const TA*)c->tok_emb, (const TA*)c->cls_emb, c->h, nullptr, nullptr, s);
@@ -219,6 +222,7 @@ int forward<float>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int st
         if ((rc = gemm<TA>(c, c->a, w.w_qkv, c->qkv, M, 3 * D, D, 0))) return rc;
         launch_rope_kv<TA>(st, l, c->qkv, c->rope_cs, (TA*)c->q, kv, s);
         c->launches++;
+        if (kv_only && l == st.L - 1) break;
         {
             const int ps = prof_begin(c, HBSJD_PROF_ATTENTION, 0.0);
             launch_attention_ref<TA>(st, l, (const TA*)c->q, kv, (TA*)c->o, s);
@@ -261,7 +265,7 @@ template <>
 int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int stop_stage) {
     const State& st = c->st;
     const int M = st.nb * st.R, D = st.D, F = st.F;
-    const int Mcap = 2 * c->Bmax * c->Wmax;  // row capacity of the activation buffers
+    const int Mcap = c->rows_cap;
     Stream& s = c->stream;
     const KvView kv = kv_view(c);
     const bool fold = c->fold_norm;
@@ -295,6 +299,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
     launch_embed<bf16>(st, (const bf16*)c->tok_emb, (const bf16*)c->cls_emb, c->h, fold ? a : nullptr,
                        fold ? c->ssq : nullptr, s);
     c->launches++;
+    const bool kv_only = !want_logits && stop_layer < 0;  // pre-filling: of the last layer only keys and values are wanted
     for (int l = 0; l < st.L; ++l) {
         const LayerW& w = c->layers[l];
         int rc, ps;
@@ -305,6 +310,8 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
                               c->err, sizeof(c->err), c->force_tile);
         prof_end(c, ps);
         if (rc) return done(rc);
+        c->launches++;
+        if (kv_only && l == st.L - 1) break;
         ps = prof_begin(c, HBSJD_PROF_ATTENTION, 0.0);
         if (attention_tma_supported(st, kv)) {
             rc = launch_attention_tma(st, S, l, (const bf16*)c->q, Mcap, kv, (bf16*)c->o, eflag, s, c->err,
@@ -314,7 +321,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
             launch_attention_ref<bf16>(st, l, (const bf16*)c->q, kv, (bf16*)c->o, s);
         }
         prof_end(c, ps);
-        c->launches += 2;
+        c->launches++;
         if ((rc = residual(c->o, w.w_o, D))) return done(rc);
         if (l == stop_layer && stop_stage == 0) return 0;
         if (!fold) norm(w.g_ffn);
@@ -357,6 +364,40 @@ int choose_compact(const hbsjd_ctx* c, int live) {
     return live > c->P.gamma ? 0 : 1;  // Eq. 6
 }
 
+// The next forward of a pass over the inputs done .. len[b] - 1 of every image (pre-filling, scoring): up to `span` inputs per
+// image in slots of `width`, `rows` and `slots` of them in all.
+struct PassShape {
+    int span, width, rows, slots;
+};
+PassShape pass_shape(const std::vector<int32_t>& len, int done, int len_max, int rows_cap) {
+    auto rows = [&](int span) {
+        long r = 0;
+        for (const int32_t l : len) r += std::max(0, std::min(span, l - done));
+        return r;
+    };
+    int lo = 1, hi = len_max - done;  // the longest span whose rows fit
+    while (lo < hi) {
+        const int mid = lo + (hi - lo + 1) / 2;
+        if (rows(mid) <= rows_cap) lo = mid;
+        else hi = mid - 1;
+    }
+    PassShape p;
+    p.span = lo;
+    // whole slots, but for the last forward; slots of 64 read an image's keys and values least often
+    p.width = p.span >= 64 ? 64 : (p.span + 15) / 16 * 16;
+    const int left = len_max - done;
+    if (p.span < left && p.span > 16) {
+        p.width = p.span >= 64 ? 64 : p.span / 16 * 16;
+        p.span -= p.span % p.width;
+        const int passes = (left + p.span - 1) / p.span;  // of equal size
+        p.span = ((left + passes - 1) / passes + p.width - 1) / p.width * p.width;
+    }
+    p.rows = (int)rows(p.span);
+    p.slots = 0;
+    for (const int32_t l : len) p.slots += (std::max(0, std::min(p.span, l - done)) + p.width - 1) / p.width;
+    return p;
+}
+
 // Error counter of the device (as read into h_counters) -> return code; clears it.
 int check_error(hbsjd_ctx* c) {
     if (c->h_counters[CNT_ERROR] == 0) return 0;
@@ -391,7 +432,8 @@ int sync_counters(hbsjd_ctx* c) {
 int enqueue_round(hbsjd_ctx* c) {
     const int compact = choose_compact(c, c->live);
     const int S = compact ? c->live : c->st.B;
-    c->st.R = c->rows;
+    c->st.R = compact ? c->rows : S * c->st.W;
+    c->st.multi = false;
     launch_setup(c->st, 0, compact, c->stream);
     if (c->round == c->fail_round) {  // code 1: a bounded wait that gave up
         c->fail_round = -1;
@@ -684,22 +726,24 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
     }
     // state
     const size_t Bm = c->Bmax, Wm = c->Wmax, T1 = c->T + 1;
+    // Activation rows: the largest round, 2 branches x max_batch slots x max_window inputs; and at least PASS_ROWS (or all
+    // that the batch has), so that contexts of few images or short windows pre-fill and score in few forwards.
+    const size_t Mmax = std::max(2 * Bm * Wm, std::min((size_t)PASS_ROWS, 2 * Bm * c->T)), Sm = max_slots(Bm, Mmax);
+    c->rows_cap = (int)Mmax;
     int rc;
     State& st = c->st;
     if ((rc = dev_alloc(c, &st.cursor, Bm)) || (rc = dev_alloc(c, &st.seq, Bm * T1)) ||
         (rc = dev_alloc(c, &st.delta, Bm * T1)) || (rc = dev_alloc(c, &st.qbase, Bm)) ||
         (rc = dev_alloc(c, &st.label, Bm)) || (rc = dev_alloc(c, &st.klen, Bm)) ||
-        (rc = dev_alloc(c, &st.pfill, Bm)) || (rc = dev_alloc(c, &st.slot_img, Bm)) ||
-        (rc = dev_alloc(c, &st.slot_c, Bm)) || (rc = dev_alloc(c, &st.slot_n, Bm)) ||
-        (rc = dev_alloc(c, &st.slot_row, Bm)) || (rc = dev_alloc(c, &st.row_pos, 2 * Bm * Wm)) ||
-        (rc = dev_alloc(c, &st.slot_sorted, Bm)) ||
+        (rc = dev_alloc(c, &st.pfill, Bm)) || (rc = dev_alloc(c, &st.slot_img, Sm)) ||
+        (rc = dev_alloc(c, &st.slot_c, Sm)) || (rc = dev_alloc(c, &st.slot_n, Sm)) ||
+        (rc = dev_alloc(c, &st.slot_row, Sm)) || (rc = dev_alloc(c, &st.row_pos, Mmax)) ||
+        (rc = dev_alloc(c, &st.slot_sorted, Sm)) ||
         (rc = dev_alloc(c, &st.counters, (size_t)8)) || (rc = dev_alloc(c, &st.m_last, Bm)) ||
         (rc = dev_alloc(c, &st.j_last, Bm)) || (rc = dev_alloc(c, &c->pbuf[0], Bm * Wm * V)) ||
         (rc = dev_alloc(c, &c->pbuf[1], Bm * Wm * V)) || (rc = dev_alloc(c, &c->flag, Bm * Wm)) ||
         (rc = dev_alloc(c, &c->cand_rep, Bm * Wm)) || (rc = dev_alloc(c, &c->cand_ref, Bm * Wm)))
         return rc;
-    // activations for the largest forward: 2 branches x max_batch slots x max_window inputs
-    const size_t Mmax = 2 * Bm * Wm;
     unsigned char *a, *q, *o, *act;
     const size_t f32_only = c->bf16_model ? 0 : 1;  // fp32 GEMM outputs the fused bf16 epilogues never materialise
     if ((rc = dev_alloc(c, &c->h, Mmax * D)) || (rc = dev_alloc(c, &c->qkv, f32_only * Mmax * 3 * D)) ||
@@ -890,29 +934,26 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
     CK(cudaEventRecord(c->ev0, c->stream));
     launch_init_state(st, prefix_tokens, prefix_len, class_labels, c->stream);
     c->launches++;
-    // prefix pre-filling: cache sequence indices 0..k-1 in chunks of W (no LM head)
-    for (int pr = 0;; ++pr) {
-        int act = 0;
-        st.R = 0;
-        for (int b = 0; b < batch; ++b) {
-            const int n = std::min(p->window, hk[b] - pr * p->window);
-            act += n > 0;
-            st.R += std::max(n, 0);
-        }
-        if (act == 0) break;
-        const int compact = choose_compact(c, act);
-        const int S = compact ? act : batch;
-        launch_setup(st, 1, compact, c->stream);
-        const int rc = forward_any(c, S, false);
+    // prefix pre-filling: cache sequence indices 0..k-1 in as few forwards as the activation rows allow (no LM head)
+    const int k_max = *std::max_element(hk.begin(), hk.end());
+    c->stats.prefill_forwards = (k_max + p->window - 1) / p->window;
+    for (int done = 0, span; done < k_max; done += span) {
+        const PassShape sh = pass_shape(hk, done, k_max, c->rows_cap / st.nb);
+        span = sh.span;
+        st.W = sh.width;
+        st.R = sh.rows;
+        st.multi = span > st.W;
+        launch_setup(st, 1, 1, c->stream, span);
+        const int rc = forward_any(c, sh.slots, false);
         if (rc) return rc;
-        launch_prefill_advance(st, S, c->stream);
+        launch_prefill_advance(st, span, c->stream);
         c->launches += 2;
-        c->stats.prefill_forwards += 1;
         if (c->profiling) {  // fold this forward's event pairs while its byte counters are current
             const int rs = sync_counters(c);
             if (rs) return rs;
         }
     }
+    st.W = p->window;
     launch_init_window(st, (uint32_t)(p->seed & 0xffffffffu), (uint32_t)(p->seed >> 32), c->stream);
     c->launches++;
     CK(cudaEventRecord(c->ev1, c->stream));
@@ -1024,11 +1065,7 @@ int score_run(hbsjd_ctx* student, hbsjd_ctx* teacher, int batch, const int32_t* 
               const int32_t* class_labels, float* bikl_pos, float* per_image, float* loss) {
     hbsjd_ctx* c = student;
     const int T = c->T, V = c->d.vocab;
-    // inputs per image per chunk: one branch only, so the activation buffers (sized for two branches of
-    // max_window inputs) hold twice the rollout's window
-    int W = 2 * (c->Wmax < teacher->Wmax ? c->Wmax : teacher->Wmax);
-    if (W > 64) W = 64;
-    if (W > T) W = T;
+    const std::vector<int32_t> len(batch, T);  // every token of the sequences is an input
     float* pos = bikl_pos ? bikl_pos : c->score_pos;
     float* img = per_image ? per_image : c->score_img;
     hbsjd_ctx* both[2] = {student, teacher};
@@ -1045,20 +1082,23 @@ int score_run(hbsjd_ctx* student, hbsjd_ctx* teacher, int batch, const int32_t* 
         st.C = x->d.n_classes;
         st.Bmax = x->Bmax;
         st.Wmax = x->Wmax;
-        st.W = W;
         st.H = 1;
         st.nb = 1;
-        st.R = batch * W;
         x->have_rollout = false;
         x->live = 0;
         launch_score_init(st, tokens, class_labels, prefix_len, x == student ? pos : nullptr, x->stream);
         x->launches++;
     }
-    for (int done = 0; done < T; done += W) {
+    for (int done = 0, span; done < T; done += span) {
+        const PassShape sh = pass_shape(len, done, T, std::min(c->rows_cap, teacher->rows_cap));
+        span = sh.span;
         for (hbsjd_ctx* x : both) {
-            launch_setup(x->st, 1, 0, x->stream);
+            x->st.W = sh.width;
+            x->st.R = sh.rows;
+            x->st.multi = span > sh.width;
+            launch_setup(x->st, 1, 1, x->stream, span);
             x->launches++;
-            const int rc = forward_any(x, batch, true);
+            const int rc = forward_any(x, sh.slots, true);
             if (rc) {
                 if (x != c) snprintf(c->err, sizeof(c->err), "teacher forward: %.200s", x->err);
                 return rc;
@@ -1075,14 +1115,14 @@ int score_run(hbsjd_ctx* student, hbsjd_ctx* teacher, int batch, const int32_t* 
         {
             // timed with the vocabulary-wide class: 2 V floats read per input, as the byte count of that class
             const int ps = prof_begin(c, HBSJD_PROF_ACCEPT, 0.0);
-            launch_bikl_slots(c->st, batch, c->logits, teacher->logits, prefix_len, pos, c->stream);
+            launch_bikl_inputs(c->st, c->logits, teacher->logits, prefix_len, pos, c->stream);
             prof_end(c, ps);
         }
         c->launches++;
         CK(cudaEventRecord(c->ev2, c->stream));
         CK(cudaStreamWaitEvent(teacher->stream, c->ev2, 0));
         for (hbsjd_ctx* x : both) {
-            launch_prefill_advance(x->st, batch, x->stream);
+            launch_prefill_advance(x->st, span, x->stream);
             x->launches++;
         }
     }
@@ -1225,14 +1265,15 @@ int hbsjd_calibrate_gamma(hbsjd_ctx* c, int batch, int window, int guidance, int
     st.W = window;
     st.H = 1;
     st.nb = guidance ? 2 : 1;
+    st.multi = false;
     const int points[5] = {batch, (3 * batch) / 4, batch / 2, batch / 4, batch / 8};
     int gamma = 0;
     for (int p = 0; p < 5; ++p) {
         const int live = points[p] < 1 ? 1 : points[p];
-        st.R = live * std::min(window, st.T - st.T / 2);
         float best[2] = {0.f, 0.f};
         for (int compact = 0; compact < 2; ++compact) {
             const int S = compact ? live : batch;
+            st.R = compact ? live * std::min(window, st.T - st.T / 2) : batch * window;
             for (int rep = 0; rep < 4; ++rep) {  // the first repetition warms up
                 launch_calib_state(st, live, c->stream);
                 launch_setup(st, 0, compact, c->stream);
@@ -1335,9 +1376,10 @@ int hbsjd_debug_forward(hbsjd_ctx* c, int layer, int stage) {
         snprintf(c->err, sizeof(c->err), "hbsjd_debug_forward: layer or stage out of range");
         return HBSJD_EINVAL;
     }
-    c->st.R = c->rows;
+    c->st.R = c->st.B * c->st.W;
+    c->st.multi = false;
     launch_setup(c->st, 0, 0, c->stream);
-    const int rc = c->rows > 0 ? forward_any(c, c->st.B, false, layer, stage) : 0;
+    const int rc = forward_any(c, c->st.B, false, layer, stage);
     if (rc) return rc;
     CK(cudaGetLastError());
     c->last_S = c->st.B;
@@ -1350,10 +1392,11 @@ int hbsjd_debug_read(hbsjd_ctx* c, int what, int index, void* host_dst, size_t m
     if (!c || !host_dst) return HBSJD_EINVAL;
     if (!c->have_rollout || (c->round == 0 && c->dbg_layer < 0)) return HBSJD_ESTATE;
     const int S = c->last_S, V = c->d.vocab;
-    std::vector<int32_t> slots((size_t)3 * S);
+    std::vector<int32_t> slots((size_t)3 * S), first_row(S);
     CK(cudaMemcpyAsync(slots.data(), c->st.slot_img, S * 4, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaMemcpyAsync(slots.data() + S, c->st.slot_c, S * 4, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaMemcpyAsync(slots.data() + 2 * S, c->st.slot_n, S * 4, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(first_row.data(), c->st.slot_row, S * 4, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     if (what == HBSJD_DBG_SLOTS) {
         if (max_bytes < slots.size() * 4) return HBSJD_EINVAL;
@@ -1369,9 +1412,7 @@ int hbsjd_debug_read(hbsjd_ctx* c, int what, int index, void* host_dst, size_t m
     if (slot < 0) return 0;
     const int n = slots[2 * S + slot];
     if (n == 0) return 0;
-    size_t row0 = 0;  // first row of the slot's inputs
-    for (int s = 0; s < slot; ++s) row0 += slots[2 * S + s];
-    row0 += (size_t)branch * c->st.R;
+    const size_t row0 = (size_t)branch * c->st.R + first_row[slot];
     if (what >= HBSJD_DBG_ACT_A && what <= HBSJD_DBG_ACT_H) {
         // rows of the slot in an activation buffer, as the last (partial) forward left them
         const size_t es = c->bf16_model ? 2 : 4, D = c->d.dim, F = c->d.ffn_hidden;

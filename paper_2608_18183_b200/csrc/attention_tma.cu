@@ -386,7 +386,8 @@ __global__ void __launch_bounds__((AttnCfg<QB>::NCW + 1) * 32, AttnCfg<QB>::CTAS
                         ok = false;
                         break;
                     }
-                    if (!waited && key0 + SK > it.c) {  // the first stage with keys of this forward
+                    // the first stage with keys of this forward (an earlier slot of the image may have written any of them)
+                    if (!waited && (st.multi || key0 + SK > it.c)) {
                         pdl_wait();
                         waited = true;
                     }

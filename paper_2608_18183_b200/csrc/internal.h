@@ -12,16 +12,17 @@ namespace hbsjd {
 
 // Device-side rollout state and per-round slot tables.  A "slot" is the place of one image in the
 // physical batch of a forward: Full execution has one slot per image of the batch (finished images
-// get n = 0), Compact execution one slot per live image.  The rows of a forward hold inputs only, slot behind slot: token
-// row of (branch, slot, i < n) = branch * R + slot_row[slot] + i.  Windows shorten at a sequence's end, and rows of W inputs
-// per slot were 8 % padding in a rollout of 128 L images, a third where 16 to 80 tokens follow a long prefix (the rollouts
-// take 0.95 and 0.84 times the time without them).
+// get n = 0), Compact execution one slot per live image.  Token row of (branch, slot, i < n) = branch * R + slot_row[slot] + i:
+// Full execution has W rows per slot, otherwise the rows hold inputs only, slot behind slot.  Windows shorten at a sequence's
+// end, and rows of W inputs per live slot were 8 % padding in a rollout of 128 L images, a third where 16 to 80 tokens follow a
+// long prefix (the rollouts take 0.95 and 0.84 times the time without them).
 struct State {
     int B, T, V, D, Hh, dh, F, L, C;  // batch, tokens per image, vocab, dim, heads, head dim, ffn, layers, classes
     int Bmax, Wmax;
     int W, H;        // window (inputs per image per round), history offset
     int nb;          // branches: 1, or 2 under classifier-free guidance
     int R;           // rows per branch of the forward; at least the inputs that it has (rows behind them are unused)
+    bool multi;      // an image may have several slots in the forward (pre-filling, scoring)
     int32_t* cursor;   // [Bmax] committed tokens
     int32_t* seq;      // [Bmax][T+1] tokens by 1-based position (committed, then drafts)
     uint8_t* delta;    // [Bmax][T+1] draft carries a point-mass proposal
@@ -29,12 +30,13 @@ struct State {
     int32_t* label;    // [Bmax]
     int32_t* klen;     // [Bmax] prefix length
     int32_t* pfill;    // [Bmax] prefill cursor
-    int32_t* slot_img; // [Bmax]
-    int32_t* slot_c;   // [Bmax] first sequence index of the slot's inputs
-    int32_t* slot_n;   // [Bmax] number of inputs (0: inactive slot)
-    int32_t* slot_row; // [Bmax] first row of the slot's inputs (null: W rows per slot)
+    // slot tables, [max_slots(..)] (stand-alone verification: [B])
+    int32_t* slot_img;
+    int32_t* slot_c;   // first sequence index of the slot's inputs
+    int32_t* slot_n;   // number of inputs (0: inactive slot)
+    int32_t* slot_row; // first row of the slot's inputs (null: W rows per slot)
     int2* row_pos;     // [rows per branch] (image, sequence index) of a row; image -1: unused (null: not built)
-    int4* slot_sorted; // [Bmax] (first row, n, c, image) by context length c + n, longest first (null: not built)
+    int4* slot_sorted; // (first row, n, c, image) by context length c + n, longest first (null: not built)
     __device__ __forceinline__ int first_row(int slot) const { return slot_row ? __ldcg(slot_row + slot) : slot * W; }
     // (image, sequence index) of row `row` of all branches, and its branch
     __device__ __forceinline__ int2 pos_of(int row, int& br) const {
@@ -45,6 +47,9 @@ struct State {
     int32_t* m_last;   // [Bmax] tokens committed in the last round
     int32_t* j_last;   // [Bmax] first-reject index of the last round (-1 none)
 };
+
+// Slots that a forward of `rows` rows may need: an image's inputs fill slots of at least 16 (or one slot), but for a last one.
+inline size_t max_slots(size_t batch, size_t rows) { return batch + rows / 16; }
 
 enum { CNT_LIVE = 0, CNT_COMMITTED = 1, CNT_REJECTS = 2, CNT_LIVE_SETUP = 3, CNT_SLOTS = 4, CNT_ERROR = 5,
        CNT_SUM_KEYS = 6 /* sum over active slots of c+n */, CNT_SUM_N = 7 /* sum of n */ };
@@ -81,7 +86,8 @@ struct AcceptArgs {
 };
 
 // ---- row operations (model_kernels.cu)
-void launch_setup(const State& st, int phase /*0 round, 1 prefill*/, int compact, Stream& s);
+// Phase 0: a round.  Phase 1: up to `span` inputs of every image behind its prefill cursor, in slots of W (gathered).
+void launch_setup(const State& st, int phase, int compact, Stream& s, int span = 0);
 // hb / ssq (bf16 model, may be null): the bf16 copy of the embedded rows and their partial sums of squares per
 // 32-column chunk, as the folded RMSNorm of the first projection wants them
 template <typename TA>
@@ -128,7 +134,7 @@ int launch_attention_tma(const State& st, int S, int layer, const bf16* q, int q
 // ---- state kernels (state_kernels.cu)
 void launch_init_state(const State& st, const int32_t* prefix_tokens, const int32_t* prefix_len,
                        const int32_t* labels, Stream& s);
-void launch_prefill_advance(const State& st, int S, Stream& s);
+void launch_prefill_advance(const State& st, int span, Stream& s);
 void launch_init_window(const State& st, uint32_t seed_lo, uint32_t seed_hi, Stream& s);
 void launch_export_tokens(const State& st, int32_t* out, Stream& s);
 // synthetic state for the threshold calibration: the first `live` images at cursor T/2, the rest finished
@@ -154,9 +160,8 @@ void launch_noop(Stream& s);
 
 // ---- distillation score (score_kernels.cu)
 void launch_bikl_rows(const float* ls, const float* lt, int rows, int V, float* out, Stream& s);
-// terms of the inputs of one scoring chunk (slot tables of st; logits rows slot * W + i of both models)
-void launch_bikl_slots(const State& st, int S, const float* ls, const float* lt, const int32_t* prefix_len,
-                       float* pos, Stream& s);
+// terms of the inputs of one scoring forward (row table of st; logits rows of both models)
+void launch_bikl_inputs(const State& st, const float* ls, const float* lt, const int32_t* prefix_len, float* pos, Stream& s);
 void launch_score_init(const State& st, const int32_t* tokens, const int32_t* labels, const int32_t* prefix_len,
                        float* pos, Stream& s);
 void launch_score_reduce(int B, int T, const int32_t* prefix_len, const float* pos, float* per_image, float* loss,

@@ -7,12 +7,14 @@
 namespace hbsjd {
 
 // ------------------------------------------------------------------ set-up / compaction (Sec. 4.3)
-// One block.  Builds the slot and row tables of the next forward.  Full: slot b = image b, n = 0 for inactive
-// images.  Compact: active images gathered in increasing image order (block-wide exclusive scan).  Either way the inputs'
-// rows follow one another without gaps (the scan of n).
+// One block.  Builds the slot and row tables of the next forward.  Full: slot b = image b with W rows, n = 0 for inactive
+// images.  Compact: active images gathered in increasing image order (block-wide exclusive scan), their inputs' rows
+// behind one another without gaps (the scan of n).  Pre-filling and scoring (phase 1) take up to `span` inputs per
+// image, in as many slots of W as they fill, always gathered: a layer's keys and values are all written before its
+// attention reads them, so the slots of one image need not wait for one another.
 // Behind an error that the host has not collected yet (it may run one round ahead) no image is active: the state
 // stays the failed round's.
-__global__ void k_setup(State st, int phase, int compact) {
+__global__ void k_setup(State st, int phase, int compact, int span) {
     pdl_wait();
     pdl_trigger();
     __shared__ int warp_tot[32], warp_rows[32];
@@ -35,12 +37,16 @@ __global__ void k_setup(State st, int phase, int compact) {
                 n = c < st.T && !failed() ? min(st.W, st.T - c) : 0;
             } else {
                 c = st.pfill[b];
-                n = c < st.klen[b] ? min(st.W, st.klen[b] - c) : 0;
+                n = c < st.klen[b] ? min(span, st.klen[b] - c) : 0;
             }
         }
-        const int act = n > 0;
-        if (act) atomicAdd(&sum_keys, c + n);
-        // exclusive scans of act and n over the block
+        const int act = phase == 0 ? n > 0 : (n + st.W - 1) / st.W;  // slots
+        if (act) {
+            int keys = 0;
+            for (int j = 0; j < act; ++j) keys += c + min(n, (j + 1) * st.W);
+            atomicAdd(&sum_keys, keys);
+        }
+        // exclusive scans of slots and inputs over the block
         int incl = act, incl_rows = n;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -64,22 +70,22 @@ __global__ void k_setup(State st, int phase, int compact) {
         if (b < st.B) {
             const bool gather = compact && !failed();
             const int slot = gather ? pos : b;
-            if (act || !gather) {
-                st.slot_img[slot] = b;
-                st.slot_c[slot] = c;
-                st.slot_n[slot] = n;
-                if (st.slot_row != nullptr) st.slot_row[slot] = row0;
+            for (int j = 0; j < (gather ? act : 1); ++j) {
+                st.slot_img[slot + j] = b;
+                st.slot_c[slot + j] = c + j * st.W;
+                st.slot_n[slot + j] = min(st.W, n - j * st.W);
+                if (st.slot_row != nullptr) st.slot_row[slot + j] = (compact ? row0 : b * st.W) + j * st.W;
             }
         }
         if (st.row_pos != nullptr) {
             // the warp writes its images' rows, one image after the other
-            for (unsigned int left = __ballot_sync(0xffffffffu, act); left; left &= left - 1) {
+            for (unsigned int left = __ballot_sync(0xffffffffu, compact ? act > 0 : b < st.B); left; left &= left - 1) {
                 const int src = __ffs(left) - 1;
                 const int ib = base + wid * 32 + src;
                 const int ic = __shfl_sync(0xffffffffu, c, src), in = __shfl_sync(0xffffffffu, n, src);
-                const int ir = __shfl_sync(0xffffffffu, row0, src);
-                for (int i = lane; i < in; i += 32)
-                    if (ir + i < st.R) st.row_pos[ir + i] = make_int2(ib, ic + i);
+                const int ir = compact ? __shfl_sync(0xffffffffu, row0, src) : ib * st.W;
+                for (int i = lane; i < (compact ? in : st.W); i += 32)
+                    if (ir + i < st.R) st.row_pos[ir + i] = i < in ? make_int2(ib, ic + i) : make_int2(-1, 0);
             }
         }
         __syncthreads();
@@ -89,7 +95,7 @@ __global__ void k_setup(State st, int phase, int compact) {
         }
         __syncthreads();
     }
-    if (st.row_pos != nullptr)  // rows that the host has allowed for and no input takes
+    if (st.row_pos != nullptr && compact)  // rows that the host has allowed for and no input takes
         for (int r = carry_rows + tid; r < st.R; r += blockDim.x) st.row_pos[r] = make_int2(-1, 0);
     // slots by context length, longest first (ties by slot index): the attention kernel deals its work items
     // from this list so that every CTA streams about the same number of key blocks
@@ -115,8 +121,8 @@ __global__ void k_setup(State st, int phase, int compact) {
     }
 }
 
-void launch_setup(const State& st, int phase, int compact, Stream& s) {
-    launch_k(k_setup, dim3(1), dim3(1024), 0, s, st, phase, compact);
+void launch_setup(const State& st, int phase, int compact, Stream& s, int span) {
+    launch_k(k_setup, dim3(1), dim3(1024), 0, s, st, phase, phase == 1 ? 1 : compact, span);
 }
 
 __global__ void k_noop() {

@@ -123,20 +123,18 @@ __global__ void __launch_bounds__(BK_THREADS) k_bikl_rows(const float* __restric
     if (threadIdx.x == 0) out[row] = d;
 }
 
-// One CTA per (slot, input i) of a scoring chunk: input i of the slot is sequence index c + i, whose output
-// is the distribution of position t = c + i + 1; the term counts when t > k (Eq. 3 sums t = k+1 .. T).
-__global__ void __launch_bounds__(BK_THREADS) k_bikl_slots(State st, const float* __restrict__ ls,
+// One CTA per row of a scoring forward: an input at sequence index s, whose output is the distribution of
+// position t = s + 1; the term counts when t > k (Eq. 3 sums t = k+1 .. T).
+__global__ void __launch_bounds__(BK_THREADS) k_bikl_inputs(State st, const float* __restrict__ ls,
                                                            const float* __restrict__ lt,
                                                            const int32_t* __restrict__ prefix_len,
                                                            float* __restrict__ pos) {
     pdl_wait();
     pdl_trigger();
-    const int i = blockIdx.x, slot = blockIdx.y;
-    if (i >= st.slot_n[slot]) return;
-    const int img = st.slot_img[slot];
-    const int idx = st.slot_c[slot] + i;
-    if (idx < prefix_len[img]) return;
-    const size_t row = (size_t)st.first_row(slot) + i;
+    const size_t row = blockIdx.x;
+    const int2 at = st.row_pos[row];
+    const int img = at.x, idx = at.y;
+    if (img < 0 || idx < prefix_len[img]) return;
     const float d = bikl_row(ls + row * st.V, lt + row * st.V, st.V);
     if (threadIdx.x == 0) pos[(size_t)img * st.T + idx] = d;
 }
@@ -202,9 +200,8 @@ void launch_bikl_rows(const float* ls, const float* lt, int rows, int V, float* 
     launch_k(k_bikl_rows, dim3(rows), dim3(BK_THREADS), 0, s, ls, lt, V, out);
 }
 
-void launch_bikl_slots(const State& st, int S, const float* ls, const float* lt, const int32_t* prefix_len,
-                       float* pos, Stream& s) {
-    launch_k(k_bikl_slots, dim3(st.W, S), dim3(BK_THREADS), 0, s, st, ls, lt, prefix_len, pos);
+void launch_bikl_inputs(const State& st, const float* ls, const float* lt, const int32_t* prefix_len, float* pos, Stream& s) {
+    launch_k(k_bikl_inputs, dim3(st.R), dim3(BK_THREADS), 0, s, st, ls, lt, prefix_len, pos);
 }
 
 void launch_score_init(const State& st, const int32_t* tokens, const int32_t* labels, const int32_t* prefix_len,

@@ -41,17 +41,15 @@ void launch_init_state(const State& st, const int32_t* prefix_tokens, const int3
     launch_k(k_init_state, dim3(st.B), dim3(128), 0, s, st, prefix_tokens, prefix_len, labels);
 }
 
-__global__ void k_prefill_advance(State st, int S) {
+__global__ void k_prefill_advance(State st, int span) {
     pdl_wait();
     pdl_trigger();
-    const int slot = blockIdx.x * blockDim.x + threadIdx.x;
-    if (slot >= S) return;
-    const int n = st.slot_n[slot];
-    if (n > 0) st.pfill[st.slot_img[slot]] = st.slot_c[slot] + n;
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < st.B) st.pfill[b] = min(st.klen[b], st.pfill[b] + span);
 }
 
-void launch_prefill_advance(const State& st, int S, Stream& s) {
-    launch_k(k_prefill_advance, dim3((S + 127) / 128), dim3(128), 0, s, st, S);
+void launch_prefill_advance(const State& st, int span, Stream& s) {
+    launch_k(k_prefill_advance, dim3((st.B + 127) / 128), dim3(128), 0, s, st, span);
 }
 
 // Initial window: every draft is the token H positions back, or a keyed uniform token where that

@@ -333,3 +333,32 @@ def test_windows_of_every_length_side_by_side(window, cfg, mode):
     np.testing.assert_array_equal(out.cpu().numpy(), r.tokens())
     assert st["committed"] == sum(T - k)
     ctx.hbsjd_destroy()
+
+
+@pytest.mark.parametrize("window", [1, 7, 32])
+def test_prefixes_and_trajectories_in_several_passes(window):
+    """Pre-filling and scoring take an image's inputs in several slots per forward and, beyond the activation rows, in several
+    forwards: 40 images of 144 tokens need two to three (pre-filling 2 x 40 x 143 rows at most, scoring 40 x 144, of 4096), the
+    same images five at a time one.  A row's arithmetic depends on its own sequence only: same bits."""
+    w = synth.with_shape(synth.WORKLOADS["small_bf16"], batch=40, window=window)
+    T = w.shape.T
+    rng = np.random.default_rng(3)
+    toks = rng.integers(0, w.shape.vocab, (40, T)).astype(np.int32)
+    k = rng.integers(0, T, 40).astype(np.int32)
+    k[:6] = [T - 1, 0, 63, 64, 65, 128]
+    lab = rng.integers(0, w.shape.n_classes, 40).astype(np.int32)
+    big, teacher = _ctx(w), _ctx(w)
+    few, few_teacher = _ctx(w, max_batch=5), _ctx(w, max_batch=5)
+    for c in (big, teacher, few, few_teacher):
+        c.hbsjd_debug_fold_norm(1)  # one form for contexts of every size
+    p = G.gpu_params(w, 0, verify_mode=1)
+    out = big.hbsjd_rollout(G.dev(toks), G.dev(k), G.dev(lab), p)[0].cpu().numpy()
+    pos = big.hbsjd_score(teacher, G.dev(out), G.dev(k), G.dev(lab))[0].cpu().numpy()
+    for b in range(0, 40, 5):
+        s = slice(b, b + 5)
+        got = few.hbsjd_rollout(G.dev(toks[s]), G.dev(k[s]), G.dev(lab[s]), p)[0].cpu().numpy()
+        np.testing.assert_array_equal(got, out[s])
+        got = few.hbsjd_score(few_teacher, G.dev(out[s]), G.dev(k[s]), G.dev(lab[s]))[0].cpu().numpy()
+        np.testing.assert_array_equal(got, pos[s])
+    for c in (big, teacher, few, few_teacher):
+        c.hbsjd_destroy()
