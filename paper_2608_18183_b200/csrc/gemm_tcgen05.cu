@@ -484,16 +484,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0 && m0 + quarter * 32 < M) {
-                        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-                                         &map_c),
-                                     "r"(col), "r"(m0 + quarter * 32), "r"(sb32)
-                                     : "memory");
-                        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-                                         &map_hb),
-                                     "r"(col), "r"(m0 + quarter * 32), "r"(sb16)
-                                     : "memory");
-                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    if (lane == 0) {
+                        if (m0 + quarter * 32 < M) {
+                            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                                             &map_c),
+                                         "r"(col), "r"(m0 + quarter * 32), "r"(sb32)
+                                         : "memory");
+                            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                                             &map_hb),
+                                         "r"(col), "r"(m0 + quarter * 32), "r"(sb16)
+                                         : "memory");
+                        }
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");  // (empty without rows: see below)
                     }
                     // The chunk three ahead takes the register slot this chunk has freed.  Requested only now, behind
                     // the proxy fence above: a fence waits for the loads its thread has in flight, so a request in
@@ -524,8 +526,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0 && m0 + quarter * 32 < M) {
-                        if (EPI == EPI_ADD)
+                    if (lane == 0) {
+                        // A warp without rows stores nothing, but commits all the same: it writes its buffers too, and the
+                        // wait above counts groups.  (Without the empty group the second chunk of such a tile overwrote
+                        // what the last chunk of the tile before was still being stored from.)
+                        const bool rows = m0 + quarter * 32 < M;
+                        if (!rows) {
+                        } else if (EPI == EPI_ADD)
                             asm volatile(
                                 "cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group "
                                 "[%0, {%1, %2}], [%3];" ::"l"(&map_c),

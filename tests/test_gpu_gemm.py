@@ -215,3 +215,20 @@ def test_output_off_its_16_byte_boundary_is_refused(ctx_bf16, M, offset):
             ctx_bf16.hbsjd_gemm(A, W, flat[offset:offset + M * 128].view(M, 128), accumulate=accumulate)
         assert e.value.code == -1
     assert not bool(flat.any())
+
+
+@pytest.mark.parametrize("tile", [32, 128, 256, 512])
+def test_epilogue_warps_without_rows_leave_the_tile_before_alone(ctx_bf16, tile):
+    """4865 rows: the last row of tiles has rows for one warp only, and CTAs come to it from whole tiles while the last of
+    those are still being stored (three k-blocks per tile: the main loop is over long before).  The other warps must not
+    write into the buffers that these stores read.  Bound: one product's sum in fp32, K = 192, whatever the tile."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(4865)
+    A = torch.randn(4865, 192, generator=g, device="cuda").bfloat16()
+    W = torch.randn(1024, 192, generator=g, device="cuda").bfloat16()
+    ref = A.float() @ W.float().T
+    for acc in (True, False) * 3:
+        C0 = torch.randn(4865, 1024, generator=g, device="cuda")
+        C = C0.clone()
+        ctx_bf16.hbsjd_debug_gemm(A, W, C, accumulate=acc, tile=tile)
+        assert float((C - (ref + C0 if acc else ref)).abs().max()) < 1e-3
