@@ -40,12 +40,13 @@ __global__ void k_setup(State st, int phase, int compact, int span) {
                 n = c < st.klen[b] ? min(span, st.klen[b] - c) : 0;
             }
         }
-        const int act = phase == 0 ? n > 0 : (n + st.W - 1) / st.W;  // slots
-        if (act) {
-            int keys = 0;
+        int act = n > 0, keys = c + n;  // slots
+        if (phase != 0) {
+            act = (n + st.W - 1) / st.W;
+            keys = 0;
             for (int j = 0; j < act; ++j) keys += c + min(n, (j + 1) * st.W);
-            atomicAdd(&sum_keys, keys);
         }
+        if (act) atomicAdd(&sum_keys, keys);
         // exclusive scans of slots and inputs over the block
         int incl = act, incl_rows = n;
 #pragma unroll
@@ -104,12 +105,13 @@ __global__ void k_setup(State st, int phase, int compact, int span) {
         const int n_slots = compact && !failed() ? carry : st.B;
         for (int s0 = tid; s0 < n_slots; s0 += blockDim.x) {
             const int n0 = st.slot_n[s0], c0 = st.slot_c[s0], len = n0 > 0 ? c0 + n0 : -1;
+            const int row0 = st.first_row(s0), img0 = st.slot_img[s0];  // (in flight beside the two above)
             int rank = 0;
             for (int s1 = 0; s1 < n_slots; ++s1) {
                 const int l1 = st.slot_n[s1] > 0 ? st.slot_c[s1] + st.slot_n[s1] : -1;
                 rank += (l1 > len) || (l1 == len && s1 < s0);
             }
-            st.slot_sorted[rank] = make_int4(st.first_row(s0), n0, c0, st.slot_img[s0]);
+            st.slot_sorted[rank] = make_int4(row0, n0, c0, img0);
         }
     }
     if (tid == 0) {
