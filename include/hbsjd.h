@@ -211,8 +211,8 @@ int hbsjd_gemm(hbsjd_ctx *c, const void *A, const void *W, float *C, int M, int 
  * then means the former).  A limit shorter than the main loop makes a healthy pipeline take the
  * time-out path: every role leaves its loop, copies and MMAs in flight are drained, TMEM is freed, the call
  * returns HBSJD_ETIMEOUT with C partly written, and the context stays usable.  Tests use it to exercise that path.
- * tile (bf16 contexts, accumulate 0 or 1): 0 = the library's own choice for the shape; 32, 64, 128, 256 = one CTA
- * per 128 x tile block of C; 512 / 640 = 256 x 256 / 256 x 128 blocks on CTA pairs (N a multiple of 256 / 128);
+ * tile (bf16 contexts, accumulate 0 or 1): 0 = the library's own choice for the shape; 32, 64, 96, 128, 160, 192, 256 = one
+ * CTA per 128 x tile block of C; 512 / 640 = 256 x 256 / 256 x 128 blocks on CTA pairs (N a multiple of 256 / 128);
  * 16032, 16064, 32032, 32064 = the kernel for few rows, 16 x 32 .. 32 x 64 blocks of C.  Every choice gives the
  * same bits (each element's products are summed in the same order); HBSJD_EINVAL for any other value. */
 int hbsjd_debug_gemm(hbsjd_ctx *c, const void *A, const void *W, float *C, int M, int N, int K, int accumulate,
@@ -233,7 +233,7 @@ int hbsjd_debug_fold_norm(hbsjd_ctx *c, int on);
  * before the first rollout of the context; HBSJD_ESTATE afterwards. */
 int hbsjd_debug_shuffle_pages(hbsjd_ctx *c, uint64_t seed);
 
-/* The tile (see hbsjd_debug_gemm: 0, 64 or one of the kernel for few rows) of every decoder GEMM of a bf16 context's
+/* The tile (see hbsjd_debug_gemm: 0, 64, 96, 160, 192 or one of the kernel for few rows) of every decoder GEMM of a bf16 context's
  * forwards, so that tests can compare the two kernels in each fused epilogue (Sec. 4.2 verifier forward).  Every choice
  * gives the same bits. */
 int hbsjd_debug_force_tile(hbsjd_ctx *c, int tile);

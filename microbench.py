@@ -217,7 +217,7 @@ def bench_gemm_tiles(args):
             # 0: the library's choice; 512 / 640: 256 x 256 / 256 x 128 tiles on CTA pairs; from 16032: the kernel for few
             # rows, rows x columns of its tile
             few = (16032, 16064, 32032, 32064) if M <= 512 else ()
-            for tile in (0, 32, 64, 128, 256, 512, 640) + few:
+            for tile in (0, 32, 64, 96, 128, 160, 192, 256, 512, 640) + few:
                 width = tile % 1000 if tile >= 1000 else 768 - tile if tile >= 512 else tile
                 if tile and N % width:
                     continue

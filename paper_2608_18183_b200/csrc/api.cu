@@ -1507,9 +1507,10 @@ int hbsjd_debug_fold_norm(hbsjd_ctx* c, int on) {
 
 int hbsjd_debug_force_tile(hbsjd_ctx* c, int tile) {
     if (!c) return HBSJD_EINVAL;
-    if (!c->bf16_model || (tile != 0 && tile != 64 && tile != 16032 && tile != 16064 && tile != 32032 && tile != 32064)) {
-        snprintf(c->err, sizeof(c->err), "hbsjd_debug_force_tile: needs a bf16 context and a tile of 0, 64, 16032, 16064, "
-                                         "32032 or 32064");
+    const int tiles[] = {0, 64, 96, 160, 192, 16032, 16064, 32032, 32064};
+    if (!c->bf16_model || std::find(std::begin(tiles), std::end(tiles), tile) == std::end(tiles)) {
+        snprintf(c->err, sizeof(c->err), "hbsjd_debug_force_tile: needs a bf16 context and a tile of 0, 64, 96, 160, 192, 16032, "
+                                         "16064, 32032 or 32064");
         return HBSJD_EINVAL;
     }
     c->force_tile = tile;

@@ -29,6 +29,7 @@ struct GemmArgs {
     // ADDNORM: C (fp32 residual) += acc, plus what the next GEMM needs
     bf16* hb;              // [M][N] bf16 copy of the updated residual
     float* ssq_out;        // [M][N / 32] sums of squares of the updated residual per 32-column chunk
+    int full_tiles;   // CTA pairs: tiles of the walk that are taken whole; the ones behind them go as two halves each
     int w_constant;   // W never changes while the stream runs (model weights): its tiles may be fetched early
     unsigned int acc_wait_ns;  // 0, or a shorter limit for the epilogue's accumulator wait (time-out test)
     // QKV epilogue

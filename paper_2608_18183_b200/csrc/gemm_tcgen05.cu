@@ -142,7 +142,7 @@ template <int BN, bool PAIR = false, bool WIDE = false>
 struct Cfg {
     // as many stages as fit beside the epilogue staging: small tiles are latency-bound (one TMA round trip per ring
     // revolution), so a narrow tile gets a deep ring
-    static constexpr int STAGES = PAIR ? 6 : (BN >= 256 ? 4 : (BN == 128 ? 6 : 8));
+    static constexpr int STAGES = PAIR ? 6 : (BN >= 160 ? 4 : (BN >= 96 ? 6 : 8));
     // k-blocks that share one full / empty barrier pair (one wait and one commit per KG x 4 MMAs).  Every group costs the
     // MMA stream about 190 clocks, as much as half a k-block of a narrow tile, so narrow tiles take four at a time.
     static constexpr int KG = !PAIR && BN <= 64 ? 4 : 2;
@@ -151,7 +151,7 @@ struct Cfg {
     static constexpr int A_BYTES = BM * BK * 2;
     static constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * BK * 2;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;  // two accumulators
+    static constexpr int TMEM_COLS = 2 * BN <= 64 ? 64 : 2 * BN <= 128 ? 128 : 2 * BN <= 256 ? 256 : 512;  // two accumulators
     // 4 epilogue warps x 2 buffers x (32 rows x 128 bytes fp32 [+ 32 rows x 64 bytes bf16]); one buffer where the second
     // would cost the ring a group: deeper groups win more than the epilogue loses (see the rule above)
     static constexpr int WARP_STAGING = WIDE ? (BN == 32 ? 2 : 1) * 6144 : 2 * 4096;
@@ -164,6 +164,7 @@ struct Cfg {
 template <int BN, int EPI, bool PAIR>
 __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_constant__ CUtensorMap map_a,
                                                               const __grid_constant__ CUtensorMap map_w,
+                                                              const __grid_constant__ CUtensorMap map_w_half,
                                                               const __grid_constant__ CUtensorMap map_c,
                                                               const __grid_constant__ CUtensorMap map_hb,
                                                               const GemmArgs g) {
@@ -189,7 +190,28 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
     const int M = g.M, N = g.N;
     const int num_kb = g.K / BK;
     const int tiles_n = N / BN, tiles_m = (M + TM - 1) / TM;
-    const int num_tiles = tiles_n * tiles_m;
+    // The tiles of the last wave of CTA pairs, where they are few, are walked as halves of BN / 2 columns.
+    constexpr bool HALVES = PAIR && BN == 256;
+    const int num_tiles = HALVES ? 2 * tiles_n * tiles_m - g.full_tiles : tiles_n * tiles_m;
+    struct Tile {
+        int m0, n0;  // first row and column
+        bool half;
+    };
+    auto tile_at = [&](int t) {
+        Tile x;
+        int off = 0;
+        x.half = HALVES && t >= g.full_tiles;
+        if (x.half) {
+            off = ((t - g.full_tiles) & 1) * (BN / 2);
+            t = g.full_tiles + (t - g.full_tiles) / 2;
+        }
+        x.m0 = (t / tiles_n) * TM;
+        x.n0 = (t % tiles_n) * BN + off;
+        return x;
+    };
+    // bytes that a k-block brings to a CTA, and the first row of W that it stages
+    auto stage_bytes = [&](bool half) { return half ? cfg::A_BYTES + cfg::B_BYTES / 2 : cfg::STAGE_BYTES; };
+    auto w_row = [&](const Tile& x) { return x.n0 + (PAIR ? (int)rank * (x.half ? BN / 4 : BN / 2) : 0); };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < cfg::STAGES; ++s) {
@@ -238,8 +260,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
     const int num_groups = (num_kb + cfg::KG - 1) / cfg::KG;  // barrier groups per tile
     int prefetched = 0;  // groups of the first tile whose W tiles are already in flight
     if (is_producer && g.w_constant) {
-        const int tile = unit;  // every CTA owns at least one tile
-        const int n0 = (tile % tiles_n) * BN + (PAIR ? (int)rank * (BN / 2) : 0);
+        const int n0 = w_row(tile_at(unit));  // every CTA owns at least one tile, the first of them whole
         prefetched = num_groups < cfg::GROUPS ? num_groups : cfg::GROUPS;
         for (int gi = 0; gi < prefetched; ++gi) {
             const int kb0 = gi * cfg::KG;
@@ -267,8 +288,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
         if (lane == 0) {
             uint32_t gc = 0;  // barrier groups issued so far
             for (int tile = unit; tile < num_tiles; tile += units) {
-                const int m0 = (tile / tiles_n) * TM + (int)rank * BM;
-                const int n0 = (tile % tiles_n) * BN + (PAIR ? (int)rank * (BN / 2) : 0);
+                const Tile x = tile_at(tile);
+                const int m0 = x.m0 + (int)rank * BM, n0 = w_row(x);
+                const CUtensorMap* mw = x.half ? &map_w_half : &map_w;
                 bool ok = true;
                 for (int kb0 = 0; kb0 < num_kb; kb0 += cfg::KG, ++gc) {
                     const int nk = num_kb - kb0 < cfg::KG ? num_kb - kb0 : cfg::KG;
@@ -285,13 +307,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                             break;
                         }
                         // in a pair both CTAs' loads complete on the leader's barrier, which expects the bytes of both
-                        if (!PAIR || rank == 0) mbar_expect_tx(full0 + 8 * gs, (PAIR ? 2 : 1) * nk * cfg::STAGE_BYTES);
+                        if (!PAIR || rank == 0) mbar_expect_tx(full0 + 8 * gs, (PAIR ? 2 : 1) * nk * stage_bytes(x.half));
                     }
                     for (int k = 0; k < nk; ++k) {
                         const uint32_t a_dst = tiles + (gs * cfg::KG + k) * cfg::STAGE_BYTES;
                         if (PAIR) {
                             tma_load_2d_pair(a_dst, &map_a, (kb0 + k) * BK, m0, bar);
-                            if (!first_rev) tma_load_2d_pair(a_dst + cfg::A_BYTES, &map_w, (kb0 + k) * BK, n0, bar);
+                            if (!first_rev) tma_load_2d_pair(a_dst + cfg::A_BYTES, mw, (kb0 + k) * BK, n0, bar);
                         } else {
                             tma_load_2d(a_dst, &map_a, (kb0 + k) * BK, m0, bar);
                             if (!first_rev) tma_load_2d(a_dst + cfg::A_BYTES, &map_w, (kb0 + k) * BK, n0, bar);
@@ -318,11 +340,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
         if (lane == 0 && rank == 0) {  // in a pair only the leader issues
-            constexpr uint32_t idesc = umma_idesc(BN, TM);
             const uint64_t desc_a0 = umma_desc(tiles);  // A tile of stage 0; every other operand tile by offset
             uint32_t gc = 0, j = 0;
             for (int tile = unit; tile < num_tiles; tile += units, ++j) {
                 const uint32_t buf = j & 1u, aph = (j >> 1) & 1u;
+                const uint32_t idesc = HALVES && tile >= g.full_tiles ? umma_idesc(BN / 2, TM) : umma_idesc(BN, TM);
                 bool ok = mbar_wait(acce0 + 8 * buf, aph ^ 1u, abort_flag);  // epilogue drained this accumulator
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t tmem_d = tmem_base + buf * BN;
@@ -379,7 +401,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
         const int quarter = warp & 3;  // TMEM lanes 32*quarter .. 32*quarter+31 belong to this warp
         uint32_t j = 0, nchunk = 0;
         for (int tile = unit; tile < num_tiles; tile += units, ++j) {
-            const int m0 = (tile / tiles_n) * TM + (int)rank * BM, n0 = (tile % tiles_n) * BN;
+            const Tile x = tile_at(tile);
+            const int m0 = x.m0 + (int)rank * BM, n0 = x.n0, width = x.half ? BN / 2 : BN;
             const uint32_t buf = j & 1u, aph = (j >> 1) & 1u;
             const int row = m0 + quarter * 32 + lane;
             const uint32_t tbase = tmem_base + buf * BN + ((uint32_t)(quarter * 32) << 16);
@@ -436,7 +459,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
 #pragma unroll 1
-            for (int cg = 0; cg < BN; cg += 32 * UNR) {
+            for (int cg = 0; cg < width; cg += 32 * UNR) {
               float ssq4[UNR];  // ADDNORM: sums of squares of this group's chunks
 #pragma unroll
               for (int u = 0; u < UNR; ++u) ssq4[u] = 0.f;
@@ -500,7 +523,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                     // The chunk three ahead takes the register slot this chunk has freed.  Requested only now, behind
                     // the proxy fence above: a fence waits for the loads its thread has in flight, so a request in
                     // front of it would cost the fence a full memory latency per chunk.
-                    if (c0 + 96 < BN && row < M) {
+                    if (c0 + 96 < width && row < M) {
                         const float4* hp = reinterpret_cast<const float4*>(g.C + (size_t)row * N + col + 96);
 #pragma unroll
                         for (int v = 0; v < 8; ++v) hbuf[(u + 3) % UNR][v] = hp[v];
@@ -571,12 +594,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
               }
               if (EPI == EPI_ADDNORM && row < M) {  // the group's partial sums: 16 contiguous bytes per row
                   float* sp = g.ssq_out + (size_t)row * (N / 32) + (n0 + cg) / 32;
-                  if (BN >= 128) {
+                  if (BN % 128 == 0) {
                       *reinterpret_cast<float4*>(sp) = make_float4(ssq4[0], ssq4[1 % UNR], ssq4[2 % UNR], ssq4[3 % UNR]);
                   } else {
 #pragma unroll
                       for (int u = 0; u < UNR; ++u)
-                          if (u * 32 < BN) sp[u] = ssq4[u];
+                          if (cg + u * 32 < BN) sp[u] = ssq4[u];
                   }
               }
             }
@@ -738,14 +761,18 @@ cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mw, const CUtensorM
     if (e0 != cudaSuccess) return e0;
     const int tiles = (g.N / BN) * ((g.M + BM - 1) / BM);
     const int grid = tiles < num_sms() ? tiles : num_sms();
-    return launch_k(k_gemm_tcgen05<BN, EPI, false>, dim3(grid), dim3(NUM_THREADS), (size_t)cfg::SMEM, s, ma, mw,
+    return launch_k(k_gemm_tcgen05<BN, EPI, false>, dim3(grid), dim3(NUM_THREADS), (size_t)cfg::SMEM, s, ma, mw, mw,
                     mc, mh, g);
 }
 
+// A last wave that half of the CTA pairs would sit out is walked in halves of its tiles (8192 rows: the QKV projection's 14 of 384
+// tiles, L, 5.55 waves in place of 6; the down projection of an XL-wide teacher 2.55 in place of 3).
+bool last_wave_in_halves(long tiles, int pairs) { return tiles > pairs && 2 * (tiles % pairs) <= pairs; }
+
 // CTA pairs: 256 x BN tiles (BN = 256 or 128), one cluster of two CTAs per pair of SMs.
 template <int BN, int EPI>
-cudaError_t launch_pair(const CUtensorMap& ma, const CUtensorMap& mw, const CUtensorMap& mc, const CUtensorMap& mh,
-                        const GemmArgs& g, Stream& s) {
+cudaError_t launch_pair(const CUtensorMap& ma, const CUtensorMap& mw, const CUtensorMap& mw_half, const CUtensorMap& mc,
+                        const CUtensorMap& mh, GemmArgs g, Stream& s) {
     static int configured[64] = {0};
     using cfg = Cfg<BN, true, EPI == EPI_ADDNORM>;
     cudaError_t e0 = ensure_dynamic_smem(k_gemm_tcgen05<BN, EPI, true>, cfg::SMEM, configured);
@@ -753,27 +780,69 @@ cudaError_t launch_pair(const CUtensorMap& ma, const CUtensorMap& mw, const CUte
     const int tiles = (g.N / BN) * ((g.M + 2 * BM - 1) / (2 * BM));
     const int pairs = num_sms() / 2;
     const int grid = 2 * (tiles < pairs ? tiles : pairs);
+    g.full_tiles = last_wave_in_halves(tiles, pairs) ? tiles - tiles % pairs : tiles;
     return launch_kc(true, k_gemm_tcgen05<BN, EPI, true>, dim3(grid), dim3(NUM_THREADS), (size_t)cfg::SMEM, s, 2,
-                     ma, mw, mc, mh, g);
+                     ma, mw, mw_half, mc, mh, g);
 }
 
 template <int EPI>
-cudaError_t launch_bn(int bn, const CUtensorMap& ma, const CUtensorMap& mw, const CUtensorMap& mc,
+cudaError_t launch_bn(int bn, const CUtensorMap& ma, const CUtensorMap& mw, const CUtensorMap& mw_half, const CUtensorMap& mc,
                       const CUtensorMap& mh, const GemmArgs& g, Stream& s) {
     switch (bn) {
         case 32: return launch<32, EPI>(ma, mw, mc, mh, g, s);
         case 64: return launch<64, EPI>(ma, mw, mc, mh, g, s);
+        case 96: return launch<96, EPI>(ma, mw, mc, mh, g, s);
         case 128: return launch<128, EPI>(ma, mw, mc, mh, g, s);
-        case 512: return launch_pair<256, EPI>(ma, mw, mc, mh, g, s);  // 256 x 256 on a CTA pair
-        case 640: return launch_pair<128, EPI>(ma, mw, mc, mh, g, s);  // 256 x 128 on a CTA pair
+        case 160: return launch<160, EPI>(ma, mw, mc, mh, g, s);
+        case 192: return launch<192, EPI>(ma, mw, mc, mh, g, s);
+        case 512: return launch_pair<256, EPI>(ma, mw, mw_half, mc, mh, g, s);  // 256 x 256 on a CTA pair
+        case 640: return launch_pair<128, EPI>(ma, mw, mw_half, mc, mh, g, s);  // 256 x 128 on a CTA pair
         default: return launch<256, EPI>(ma, mw, mc, mh, g, s);
     }
+}
+
+bool tile_exists(int code) {
+    for (const int c : {32, 64, 96, 128, 160, 192, 256, 512, 640})
+        if (code == c) return true;
+    return false;
+}
+
+// Tile of a product by a small cost model, fitted to 939 measured launches (back to back, 128 to 6000 rows of the B, L and XL
+// decoders' products, every tile; 3 to 5 % rms): a launch costs its boundary, and every wave of tiles over the SMs an
+// epilogue and its k-blocks.  The time of a k-block is shared memory's and the MMA pipe's, in that order up to 128 columns.
+// Against the best tile of each of 240 products the choice costs 0.1 %, 2.5 % at most (widths that are powers of two and CTA pairs from
+// 45 tiles on: 0.7 %; the worst were 1.25, XL's down projection at 2048 rows 27.4 -> 21.9 us with 160 columns, and 1.33, the
+// heads at 128 rows 12.4 -> 9.3 us with 128).
+int choose_tile(int M, int N, int K) {
+    struct Cost {
+        int tile;
+        float base, wave, kb;  // microseconds
+    };
+    static const Cost costs[] = {{512, 5.18f, 1.95f, 0.323f}, {256, 4.32f, 2.14f, 0.368f}, {192, 4.56f, 1.26f, 0.338f},
+                                 {160, 4.68f, 1.08f, 0.284f}, {128, 4.65f, 0.72f, 0.259f}, {96, 4.73f, 0.32f, 0.247f},
+                                 {64, 4.71f, 0.20f, 0.201f},  {32, 4.56f, 0.06f, 0.193f}};
+    const int sms = num_sms(), num_kb = K / BK;
+    int best = 32;
+    float best_cost = 0.f;
+    for (const Cost& c : costs) {
+        const int bn = c.tile == 512 ? 256 : c.tile, bm = c.tile == 512 ? 256 : 128, units = c.tile == 512 ? sms / 2 : sms;
+        if (N % bn != 0) continue;
+        const long tiles = (long)((M + bm - 1) / bm) * (N / bn), rest = tiles % units;
+        float waves = (float)((tiles + units - 1) / units), kb_waves = waves;
+        if (c.tile == 512 && rest > 0 && last_wave_in_halves(tiles, units)) kb_waves -= 0.4f;
+        const float cost = c.base + waves * c.wave + kb_waves * (float)num_kb * c.kb;
+        if (best_cost == 0.f || cost < best_cost * 0.99f) {  // the wider tile on a tie
+            best = c.tile;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
 
 // m_cap >= M: row extent given to the A and C tensor maps (the capacity of the caller's buffers), so that one
 // cached map serves every M; rows between M and m_cap are padding (read as they are, never stored past M's
 // last 32-row block).  0: use M.
-int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int max_bn, int m_cap, Stream& s,
+int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int m_cap, Stream& s,
         char* err, size_t errlen) {
     const int M = g.M, N = g.N, K = g.K;
     if (M <= 0) return 0;
@@ -792,26 +861,19 @@ int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int ma
         }
         return gemm_skinny_launch(epi, force_bn, A, W, g, map_rows, s, err, errlen);
     }
-    if (force_bn != 0 && force_bn != 32 && force_bn != 64 && force_bn != 128 && force_bn != 256 && force_bn != 512 &&
-        force_bn != 640) {
-        snprintf(err, errlen, "gemm: tile %d is not one of 32, 64, 128, 256 (one CTA), 512, 640 (CTA pair) or 16032, "
-                              "16064, 32032, 32064 (few rows)", force_bn);
+    if (force_bn != 0 && !tile_exists(force_bn)) {
+        snprintf(err, errlen, "gemm: tile %d is not one of 32, 64, 96, 128, 160, 192, 256 (one CTA), 512, 640 (CTA pair) or "
+                              "16032, 16064, 32032, 32064 (few rows)", force_bn);
         return -1;
     }
-    const bool force_pair = force_bn >= 512;
-    if (force_pair) force_bn = 768 - force_bn;  // 512 -> 256 columns, 640 -> 128
-    int bn = force_bn ? force_bn : gemm_tcgen05_tile_n(M, N, K);
-    while (bn > max_bn) bn >>= 1;
-    if (bn < 32 || N % bn != 0) {
+    const int tile = force_bn ? force_bn : choose_tile(M, N, K);
+    const bool pair = tile == 512 || tile == 640;
+    const int bn = pair ? 768 - tile : tile;  // 512 -> 256 columns, 640 -> 128
+    if (N % bn != 0) {
         snprintf(err, errlen, "gemm: N=%d is not a multiple of the tile width %d", N, bn);
         return -1;
     }
-    // large problems: 256 x 256 tiles on CTA pairs (a third less operand traffic per FLOP)
-    // (measured on the decoder's shapes: the pair tile wins from about 0.6 tiles per CTA pair upwards)
-    const long pair_tiles = N % 256 == 0 ? (long)((M + 255) / 256) * (N / 256) : 0;
-    const bool pair = force_pair || (!force_bn && max_bn >= 256 && pair_tiles * 5 >= (long)(num_sms() / 2) * 3);
-    if (pair && !force_pair) bn = 256;
-    CUtensorMap ma, mw, mc, mh;
+    CUtensorMap ma, mw, mw_half, mc, mh;
     memset(&mc, 0, sizeof(mc));
     memset(&mh, 0, sizeof(mh));
     if ((epi == EPI_STORE || epi == EPI_ADD || epi == EPI_ADDNORM) && !make_map_c(&mc, g.C, map_rows, N)) {
@@ -822,17 +884,18 @@ int run(int epi, const bf16* A, const bf16* W, GemmArgs& g, int force_bn, int ma
         snprintf(err, errlen, "gemm: cuTensorMapEncodeTiled failed for the bf16 output (M=%d N=%d)", M, N);
         return -3;
     }
-    if (!make_map(&ma, A, map_rows, K, BM) || !make_map(&mw, W, N, K, pair ? bn / 2 : bn)) {
+    if (!make_map(&ma, A, map_rows, K, BM) || !make_map(&mw, W, N, K, pair ? bn / 2 : bn) ||
+        !make_map(&mw_half, W, N, K, pair ? bn / 4 : bn)) {
         snprintf(err, errlen, "gemm: cuTensorMapEncodeTiled failed (M=%d N=%d K=%d)", M, N, K);
         return -3;
     }
     cudaError_t e;
     switch (epi) {
-        case EPI_STORE: e = launch_bn<EPI_STORE>(pair ? 768 - bn : bn, ma, mw, mc, mh, g, s); break;
-        case EPI_ADD: e = launch_bn<EPI_ADD>(pair ? 768 - bn : bn, ma, mw, mc, mh, g, s); break;
-        case EPI_SWIGLU: e = launch_bn<EPI_SWIGLU>(pair ? 768 - bn : bn, ma, mw, mc, mh, g, s); break;
-        case EPI_ADDNORM: e = launch_bn<EPI_ADDNORM>(pair ? 768 - bn : bn, ma, mw, mc, mh, g, s); break;
-        default: e = launch_bn<EPI_QKV>(pair ? 768 - bn : bn, ma, mw, mc, mh, g, s); break;
+        case EPI_STORE: e = launch_bn<EPI_STORE>(tile, ma, mw, mw_half, mc, mh, g, s); break;
+        case EPI_ADD: e = launch_bn<EPI_ADD>(tile, ma, mw, mw_half, mc, mh, g, s); break;
+        case EPI_SWIGLU: e = launch_bn<EPI_SWIGLU>(tile, ma, mw, mw_half, mc, mh, g, s); break;
+        case EPI_ADDNORM: e = launch_bn<EPI_ADDNORM>(tile, ma, mw, mw_half, mc, mh, g, s); break;
+        default: e = launch_bn<EPI_QKV>(tile, ma, mw, mw_half, mc, mh, g, s); break;
     }
     if (e != cudaSuccess) {
         snprintf(err, errlen, "gemm launch: %s", cudaGetErrorString(e));
@@ -847,33 +910,6 @@ bool make_tensor_map_kblocks(::CUtensorMap_st* map, const void* base, int rows, 
     if (box_kb == 1) return cached_map(map, MapKey{base, rows, K, box_rows, 5}, encode_map_kb<1>);
     if (box_kb == 2) return cached_map(map, MapKey{base, rows, K, box_rows, 3}, encode_map_kb<2>);
     return box_kb == 4 && cached_map(map, MapKey{base, rows, K, box_rows, 4}, encode_map_kb<4>);
-}
-
-// Tile width by a small cost model: waves of tiles over the SMs times the time of one tile.  Measured with time stamps
-// in this kernel: a k-block costs about 0.47 us at N = 256 (MMA rate) and no
-// less than about 0.19 us however narrow the tile is -- there the ring of operand stages is what limits it (the
-// 16 KB activation tile of every k-block has to cross from L2 whatever N is, and about 160 KB can be in flight
-// per SM); the epilogue adds about 0.15 us per 32 columns.  Large problems end up with 256 (CTA pairs), small
-// ones with the widest tile that still fits one wave.
-int gemm_tcgen05_tile_n(int M, int N, int K) {
-    const long tiles_m = (M + BM - 1) / BM;
-    const int sms = num_sms(), num_kb = K / BK;
-    // enough 256-wide tiles for every SM: the wide tile has the lowest operand traffic per FLOP
-    if (N % 256 == 0 && tiles_m * (N / 256) >= sms) return 256;
-    int best = 0;
-    float best_cost = 0.f;
-    for (int bn = 256; bn >= 32; bn >>= 1) {
-        if (N % bn != 0) continue;
-        const long tiles = tiles_m * (N / bn);
-        const long waves = (tiles + sms - 1) / sms;
-        const float per_kb = fmaxf(0.19f, 0.47f * (float)bn / 256.0f);  // microseconds
-        const float cost = (float)waves * (1.0f + 0.15f * (float)(bn / 32) + (float)num_kb * per_kb);
-        if (best == 0 || cost < best_cost * 0.98f) {  // prefer the wider tile on a tie
-            best = bn;
-            best_cost = cost;
-        }
-    }
-    return best ? best : 32;
 }
 
 int gemm_tcgen05_run(const bf16* A, const bf16* W, float* C, int M, int N, int K, int accumulate, int force_bn,
@@ -891,7 +927,7 @@ int gemm_tcgen05_run(const bf16* A, const bf16* W, float* C, int M, int N, int K
     g.error_flag = error_flag;
     g.w_constant = w_constant;
     g.acc_wait_ns = acc_wait_ns;
-    return run(accumulate ? EPI_ADD : EPI_STORE, A, W, g, force_bn, 256, m_cap, s, err, errlen);
+    return run(accumulate ? EPI_ADD : EPI_STORE, A, W, g, force_bn, m_cap, s, err, errlen);
 }
 
 namespace {
@@ -913,7 +949,7 @@ int gemm_tcgen05_head(const bf16* A, const bf16* W, float* C, int M, int N, int 
     g.error_flag = error_flag;
     g.w_constant = 1;
     set_norm(g, nin, K);
-    return run(EPI_STORE, A, W, g, tile, 256, m_cap, s, err, errlen);
+    return run(EPI_STORE, A, W, g, tile, m_cap, s, err, errlen);
 }
 
 int gemm_tcgen05_addnorm(const bf16* A, const bf16* W, float* h, bf16* hb, float* ssq_out, int M, int N, int K,
@@ -931,7 +967,7 @@ int gemm_tcgen05_addnorm(const bf16* A, const bf16* W, float* h, bf16* hb, float
     g.K = K;
     g.error_flag = error_flag;
     g.w_constant = 1;
-    return run(EPI_ADDNORM, A, W, g, tile, 256, m_cap, s, err, errlen);
+    return run(EPI_ADDNORM, A, W, g, tile, m_cap, s, err, errlen);
 }
 
 int gemm_tcgen05_swiglu(const bf16* A, const bf16* W13_interleaved, bf16* act, int M, int F2, int K, int m_cap,
@@ -944,7 +980,7 @@ int gemm_tcgen05_swiglu(const bf16* A, const bf16* W13_interleaved, bf16* act, i
     g.K = K;
     g.error_flag = error_flag;
     g.w_constant = 1;
-    return run(EPI_SWIGLU, A, W13_interleaved, g, tile, 256, m_cap, s, err, errlen);
+    return run(EPI_SWIGLU, A, W13_interleaved, g, tile, m_cap, s, err, errlen);
 }
 
 int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, int layer,
@@ -962,10 +998,7 @@ int gemm_tcgen05_qkv(const bf16* A, const bf16* Wqkv, bf16* q, const State& st, 
     g.layer = layer;
     g.rope_cs = rope_cs;
     g.kv = kv;
-    // a tile must lie inside one of the q / k / v sections and start on a rotation-pair boundary
-    int max_bn = 256;
-    while (st.D % max_bn != 0) max_bn >>= 1;
-    return run(EPI_QKV, A, Wqkv, g, tile, max_bn, m_cap, s, err, errlen);
+    return run(EPI_QKV, A, Wqkv, g, tile, m_cap, s, err, errlen);
 }
 
 }  // namespace hbsjd

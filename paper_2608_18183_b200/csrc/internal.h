@@ -177,7 +177,6 @@ void launch_score_reduce(int B, int T, const int32_t* prefix_len, const float* p
 int gemm_tcgen05_run(const bf16* A, const bf16* W, float* C, int M, int N, int K, int accumulate, int force_bn,
                      int m_cap, int32_t* error_flag, Stream& s, char* err, size_t errlen, int w_constant = 1,
                      unsigned int acc_wait_ns = 0);
-int gemm_tcgen05_tile_n(int M, int N, int K);
 // Cached TMA descriptor of a row-major bf16 [rows, K] matrix seen as (64 columns, rows, K / 64) with a box of
 // 64 x box_rows x box_kb (box_kb 1, 2 or 4): one copy brings box_kb consecutive 64-column blocks, each a
 // 128-byte-swizzled tile of box_rows rows; zero fill past the last one.

@@ -252,3 +252,34 @@ def test_every_epilogue_gives_the_same_bits_in_both_gemm_kernels(fold, head):
         assert all(np.isfinite(x).all() for x in got)
         for i, x in enumerate(got):
             np.testing.assert_array_equal(x.view(np.uint32), seen.setdefault(i, x).view(np.uint32), err_msg=f"{tile} {i}")
+
+
+@pytest.mark.parametrize("fold", [True, False])
+def test_every_epilogue_of_the_tiles_in_between(fold):
+    """The fused epilogues of the tiles of 96, 160 and 192 columns, which cross the sections of q, k and v: every
+    intermediate of two layers and the logits have the 128 x 64 tile's bits."""
+    s = synth.ModelShape(2, 960, 15, 960, 1920, 12, 12, 10, "bf16")
+    img = synth.make_weights(s, 5, target_entropy=None)
+    w = synth.with_shape(synth.WORKLOADS["small_bf16"], shape=s)
+    ks = np.array([0, 1, 64, 100, 141], dtype=np.int32)
+    toks, _, lab = synth.make_inputs(w, seed=3, batch=len(ks))
+    what = {0: (binding.DBG_ACT_Q, binding.DBG_KV_K, binding.DBG_KV_V, binding.DBG_ACT_O, binding.DBG_ACT_H, binding.DBG_ACT_A),
+            1: (binding.DBG_ACT_FFN, binding.DBG_ACT_H, binding.DBG_ACT_A)}
+    seen = {}
+    for tile in (64, 96, 160, 192):
+        ctx = binding.Context(s, img, len(ks), 13)
+        ctx.hbsjd_debug_fold_norm(fold)
+        ctx.hbsjd_debug_force_tile(tile)
+        ctx.hbsjd_rollout(G.dev(toks), G.dev(ks), G.dev(lab), binding.make_params(
+            13, 12, w.cfg_scale, max_rounds=0, seed=2, exec_mode=binding.EXEC_FULL))
+        got = []
+        for layer in (0, 1):
+            for stage in (0, 1):
+                ctx.hbsjd_debug_forward(layer, stage)
+                got += [ctx.hbsjd_debug_read(x, i) for x in what[stage] for i in range(2 * len(ks))]
+        ctx.hbsjd_round()
+        got += [ctx.hbsjd_debug_read(binding.DBG_LOGITS, i) for i in range(2 * len(ks))]
+        ctx.hbsjd_destroy()
+        assert all(np.isfinite(x).all() for x in got)
+        for i, x in enumerate(got):
+            np.testing.assert_array_equal(x.view(np.uint32), seen.setdefault(i, x).view(np.uint32), err_msg=f"{tile} {i}")

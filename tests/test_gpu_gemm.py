@@ -232,3 +232,55 @@ def test_epilogue_warps_without_rows_leave_the_tile_before_alone(ctx_bf16, tile)
         C = C0.clone()
         ctx_bf16.hbsjd_debug_gemm(A, W, C, accumulate=acc, tile=tile)
         assert float((C - (ref + C0 if acc else ref)).abs().max()) < 1e-3
+
+
+@pytest.mark.parametrize("tile", [96, 160, 192])
+@pytest.mark.parametrize("M,K,kind", [(1, 64, "wide"), (17, 192, "cancelling"), (63, 1088, "running sum"), (65, 64, "wide"), (129, 2816, "wide"),
+                                      (300, 1280, "cancelling"), (2100, 320, "wide"), (6000, 64, "wide")])
+def test_tiles_between_the_powers_of_two(ctx_bf16, tile, M, K, kind):
+    """Tiles whose columns are no power of two: edges of rows, 1 to 44 k-blocks against rings of 4 and 6, several tiles per CTA
+    (85 to 170 of 2100 rows, 240 of 6000); the 128 x 64 tile's bits."""
+    import torch
+    N = 960
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    A, W = _wide_operands(kind, M, N, K, g)
+    for acc in (False, True):
+        C0 = torch.randn(M, N, generator=g, device="cuda")
+        want, got = C0.clone(), C0.clone()
+        ctx_bf16.hbsjd_debug_gemm(A, W, want, accumulate=acc, tile=64)
+        ctx_bf16.hbsjd_debug_gemm(A, W, got, accumulate=acc, tile=tile)
+        assert torch.equal(got.view(torch.int32), want.view(torch.int32))
+
+
+@pytest.mark.parametrize("M", [4865, 5120, 7000, 9472, 9473])
+def test_last_wave_of_cta_pairs_in_halves(ctx_bf16, M):
+    """256 x 256 tiles on 74 CTA pairs, 80, 80, 112, 148 and 152 of them for N = 1024: a rest of 6, 6 and 4 goes as halves, a
+    rest of 38 or none whole.  The same bits as one CTA's tiles."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(M)
+    A = torch.randn(M, 192, generator=g, device="cuda").bfloat16()
+    W = torch.randn(1024, 192, generator=g, device="cuda").bfloat16()
+    for acc in (False, True):
+        C0 = torch.randn(M, 1024, generator=g, device="cuda")
+        want, got = C0.clone(), C0.clone()
+        ctx_bf16.hbsjd_debug_gemm(A, W, want, accumulate=acc, tile=128)
+        ctx_bf16.hbsjd_debug_gemm(A, W, got, accumulate=acc, tile=512)
+        assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("M", [300, 2049, 4096])
+def test_residual_update_with_norm_sums_on_every_kernel(M):
+    """The folded residual update (its bf16 copy and sums of squares come with it) at 1280 columns: one CTA per tile, and CTA
+    pairs whose last wave goes as halves (4096 rows: 80 tiles).  The sum is the plain update's."""
+    import torch
+    s = synth.ModelShape(1, 1280, 20, 64, 64, 4, 4, 3, "bf16")
+    ctx = binding.Context(s, synth.make_weights(s, 3, target_entropy=None), 64, 32)
+    g = torch.Generator(device="cuda").manual_seed(M)
+    A = torch.randn(M, 320, generator=g, device="cuda").bfloat16()
+    W = torch.randn(1280, 320, generator=g, device="cuda").bfloat16()
+    C0 = torch.randn(M, 1280, generator=g, device="cuda")
+    want, got = C0.clone(), C0.clone()
+    ctx.hbsjd_debug_gemm(A, W, want, accumulate=1, tile=64)
+    ctx.hbsjd_debug_gemm(A, W, got, accumulate=2)
+    assert torch.equal(got, want)
+    ctx.hbsjd_destroy()
