@@ -3,8 +3,17 @@
 // One CTA of 1024 threads per SM walks the (slot, window position) items of the round.  The logits of the NEXT
 // item (conditional and unconditional row, 2 x 64 KB at V = 16384) are fetched by two bulk copies into a staging
 // area in shared memory, completing on an mbarrier, while the current item is processed entirely in registers:
-// thread t owns the four float4 groups {c * 4096 + 4 t .. + 3}, c = 0..3, of the vocabulary from the guided
-// combination to the normalised probabilities, which go to global memory straight from the registers.
+// thread t owns the float4 groups {c * 4096 + 4 t .. + 3}, c = 0..3 (fewer below 8193 entries), of the vocabulary from the
+// guided combination to the normalised probabilities, which go to global memory straight from the registers.
+//
+// What bounds it: instructions, and the waits at the barriers of an item that one row in flight per SM cannot cover (128
+// images x 32 positions, V = 16384, guidance, top-k 1000: 135 million warp instructions, 0.57 issued per clock and
+// scheduler, 223 us under the profiler where 805 MB take 123).  What went into the instructions: loops without bounds, no
+// branch per entry for histogram and exponential, no divisions in the walk, the look-ups of an item by one thread, short
+// code (the unrolled waits alone were a third of it): 174 million and 263 us with them, the whole step 294 -> 255 us.
+// Taking the next row in beside the selection of the current one hides the waits but costs what it gains: 1024 threads
+// 401 us, 512 threads with twice the entries each 325 (0.43 issued: half the warps, and rows that pass through
+// shared memory).
 //
 //   guided = l_u + s (l_c - l_u); / temperature                                  (Sec. 4.2 "fused guided logits")
 //   top-k threshold, ties kept: monotone 1024-bin histogram over [guess, max] of the entries above a normal-fit
@@ -25,7 +34,7 @@ namespace {
 
 constexpr int PT = 1024;          // threads per CTA
 constexpr int PWARPS = PT / 32;
-constexpr int NCH = 4;            // float4 groups per thread
+constexpr int MAX_CH = 4;         // float4 groups per thread, at most
 constexpr int CHUNK = PT * 4;     // vocabulary entries per chunk
 constexpr unsigned int NONE = 0xFFFFFFFFu;
 
@@ -36,10 +45,13 @@ struct PShared {
     float fit[2];                  // sum and sum of squares of the sample the threshold guess is fitted to
     float redsum[PWARPS];
     unsigned int wtot[PWARPS];
-    unsigned int csum[NCH][PWARPS];  // fixed-point weight sums per chunk and warp (a row's weights total 2^30)
+    unsigned int csum[MAX_CH][PWARPS];  // fixed-point weight sums per chunk and warp (a row's weights total 2^30)
     unsigned int best[2][PWARPS];    // greedy: largest probability bits, then the lowest index holding them
     unsigned int sel_bin, sel_k, ncand, theta;  // sel_bin / sel_k: state of the radix fallback
-    uint32_t words[2][4];  // by item parity: a fast thread may start the next item while others finish this one
+    struct Draft {
+        int z, is_delta, qrow;  // the draft under test (-1: none), point-mass proposal, row of its proposal (-1: invalid)
+    } draft[3];
+    uint32_t words[3][4];  // both by item modulo 3: a fast thread may start the next item while others finish this one
     unsigned long long mbar;
 };
 
@@ -63,6 +75,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
     unsigned long long t0;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
     for (;;) {
+#pragma unroll 1  // (short code: see the head of the file)
         for (int it = 0; it < 64; ++it)
             if (mbar_try_wait(bar, parity)) return true;
         unsigned long long t1;
@@ -80,13 +93,25 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 // Bin of x >= lo in the selection histogram over [lo, lo + 1024 / scale]: a monotone map (the integer nearest to
 // (x - lo) * scale, read off the mantissa after adding 2^23; values beyond the range fall into the last bin).
 // Monotone is all the selection needs; both passes use this same function.
-__device__ __forceinline__ int sel_bin_of(float x, float lo, float scale) {
-    const float f = fminf((x - lo) * scale, (float)(SEL_BINS - 1));
-    return (int)(__float_as_uint(f + 8388608.0f) & 0x7FFFFFu);
+__device__ __forceinline__ uint32_t sel_bits(float x, float lo, float scale) {
+    return __float_as_uint(fminf(__fmaf_rn(x - lo, scale, 8388608.0f), 8388608.0f + (float)(SEL_BINS - 1)));
+}
+__device__ __forceinline__ int sel_bin_of(float x, float lo, float scale) { return (int)(sel_bits(x, lo, scale) & 0x7FFFFFu); }
+// Counts x in its bin of the histogram at this shared-memory address if x >= lo: predicated, so that a row's entries cost
+// no branches (the exponent bits of 2^23 leave the address by the subtraction).
+__device__ __forceinline__ void count_if_above(uint32_t hist, float x, float lo, float scale) {
+    const uint32_t at = hist - (0x4B000000u << 2) + (sel_bits(x, lo, scale) << 2);
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ge.f32 p, %1, %2;\n\t"
+        "@p red.shared::cta.add.u32 [%0], 1;\n\t}" ::"r"(at),
+        "f"(x), "f"(lo)
+        : "memory");
 }
 
 // Key of the k-th largest of the block's register-resident values by radix select, one byte per pass from the
 // top; exact for any input.  Only reached when the histogram's selected bin is too crowded for the exact ranking.
+template <int NCH>
 __device__ __forceinline__ unsigned int radix_select_regs(const float (&x)[NCH][4], int tid, int V, unsigned int k, PShared& sh) {
     const int lane = tid & 31, wid = tid >> 5;
     unsigned int* hist = sh.hist;  // [256] used
@@ -95,6 +120,7 @@ __device__ __forceinline__ unsigned int radix_select_regs(const float (&x)[NCH][
         sh.sel_bin = 0u;  // prefix
         sh.sel_k = k;
     }
+#pragma unroll 1
     for (int pass = 0; pass < 4; ++pass) {
         const int shift = 24 - 8 * pass;
         const unsigned int mask = pass == 0 ? 0u : (0xFFFFFFFFu << (shift + 8));
@@ -146,13 +172,16 @@ __device__ __forceinline__ unsigned int radix_select_regs(const float (&x)[NCH][
 
 // PROBS: the probability pipeline alone (hbsjd_probs): item = row of a.logits (and a.logits_u), probabilities to a.pcur;
 // st has V, W = 1 and a place for the error code.
-template <bool CFG, bool PROBS>
+// NCH: float4 groups per thread.  Rows are padded to NCH * CHUNK entries with NaN, which every comparison drops, so that the
+// loops have no bounds.
+template <bool CFG, bool PROBS, int NCH>
 __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int V = st.V, W = st.W;
+    constexpr int VP = NCH * CHUNK;
     float* stage_c = (float*)smem_raw;
-    float* stage_u = stage_c + (CFG ? V : 0);
-    PShared& sh = *(PShared*)(smem_raw + (size_t)(CFG ? 2 : 1) * V * sizeof(float));
+    float* stage_u = stage_c + (CFG ? VP : 0);
+    PShared& sh = *(PShared*)(stage_u + VP);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const uint32_t bar = smem_addr(&sh.mbar);
     const uint32_t row_bytes = (uint32_t)V * 4u;
@@ -160,12 +189,13 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    for (int v = V + tid; v < VP; v += PT) stage_c[v] = stage_u[v] = __int_as_float(0x7FFFFFFF);
     if (!a.early) pdl_wait();
     __syncthreads();
 
     // slot tables of the round in shared memory: the item walk below reads them at every step
     // (image and n share a word: n is at most 64, images are far fewer than 2^25)
-    int* s_imgn = (int*)(smem_raw + (size_t)(CFG ? 2 : 1) * V * sizeof(float) + sizeof(PShared));
+    int* s_imgn = (int*)(&sh + 1);
     int* s_row = s_imgn + a.S;
     int* s_c = s_row + a.S;
     for (int sidx = tid; !PROBS && sidx < a.S; sidx += PT) {
@@ -177,10 +207,24 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
     auto n_of = [&](int slot) { return s_imgn[slot] & 127; };
     auto img_of = [&](int slot) { return (int)((unsigned int)s_imgn[slot] >> 7); };
 
-    const int total = a.S * W;
-    auto valid = [&](int it) { return PROBS || (it % W) < n_of(it / W); };
-    auto issue = [&](int it) {  // thread 0: both rows of item `it` into the staging area
-        const size_t row = PROBS ? (size_t)it : (size_t)s_row[it / W] + it % W;
+    // An item is (slot, window position); the walk takes every gridDim.x-th of them, without a division per step.
+    struct Item { int slot, i; };
+    const int step_slot = (int)gridDim.x / W, step_i = (int)gridDim.x % W;
+    auto exists = [&](const Item& it) { return it.slot < a.S; };
+    auto missing = [&](const Item& it) { return !PROBS && it.slot < a.S && it.i >= n_of(it.slot); };
+    auto next = [&](Item it) {
+        do {
+            it.slot += step_slot;
+            it.i += step_i;
+            if (it.i >= W) {
+                it.i -= W;
+                ++it.slot;
+            }
+        } while (missing(it));
+        return it;
+    };
+    auto issue = [&](const Item& it) {  // thread 0: both rows of item `it` into the staging area
+        const size_t row = PROBS ? (size_t)it.slot : (size_t)s_row[it.slot] + it.i;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
                      "r"(CFG ? 2u * row_bytes : row_bytes)
                      : "memory");
@@ -189,87 +233,66 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
     };
     // The state an item needs besides its logits -- the draft token under test, whether its proposal is a point
     // mass, the proposal row and the proposal's entry q(z) -- sits behind three levels of dependent global loads.
-    // They are issued one item ahead (token, flag and row base while the previous item starts; q(z) by the thread
-    // that owns vocabulary entry z once those have landed), so that no item waits for them.
-    struct Raw { int z, dl, qb; };
-    auto fetch_raw = [&](int it) {
-        Raw r = {0, 0, 0};
-        const int slot = it / W, i = it % W;
+    // One thread looks it up one item ahead, with the item's random words (Philox keyed by image, position, round), while the
+    // others are in pass 1; behind the next barrier the thread that owns vocabulary entry z requests q(z).  It also records
+    // state that cannot be valid.
+    auto look_ahead = [&](const Item& it, uint32_t par) {
+        const int slot = it.slot, i = it.i, img = img_of(slot), c = s_c[slot];
+        PShared::Draft d = {-1, 0, -1};
         if (i < n_of(slot) - 1) {  // the last input of a window has no draft to verify
-            const int img = img_of(slot);
-            const size_t at = (size_t)img * (st.T + 1) + s_c[slot] + i + 1;
-            r.z = __ldcg(st.seq + at);
-            r.dl = __ldcg(st.delta + at);
-            r.qb = __ldcg(st.qbase + img);
-        }
-        return r;
-    };
-    // q(z) of item `it` for the owning thread (1 elsewhere); records state that cannot be valid
-    auto fetch_qz = [&](int it, const Raw& r) {
-        const int slot = it / W, i = it % W;
-        float qz = 1.0f;
-        if (i < n_of(slot) - 1 && r.z >= 0 && r.z < V && ((r.z % CHUNK) >> 2) == tid && r.dl == 0 && !a.greedy) {
-            const int qi = s_c[slot] + i + 1 - r.qb - 1;  // row of the previous round's probabilities
-            if (qi < 0 || qi >= st.Wmax) {
-                atomicExch(&st.counters[CNT_ERROR], ERR_BAD_PROPOSAL_ROW);
-                qz = INFINITY;  // alpha = 0: rejected
+            const size_t at = (size_t)img * (st.T + 1) + c + i + 1;
+            const int z = __ldcg(st.seq + at), qi = c + i - __ldcg(st.qbase + img);  // row of the previous round's probabilities
+            d.is_delta = __ldcg(st.delta + at);
+            if (z < 0 || z >= V) {
+                atomicExch(&st.counters[CNT_ERROR], ERR_BAD_TOKEN);
             } else {
-                qz = __ldcg(a.pprev + ((size_t)img_of(slot) * st.Wmax + qi) * V + r.z);
+                d.z = z;
+                if (qi >= 0 && qi < st.Wmax) d.qrow = img * st.Wmax + qi;
+                else if (!d.is_delta && !a.greedy) atomicExch(&st.counters[CNT_ERROR], ERR_BAD_PROPOSAL_ROW);
             }
         }
+        philox4x32_10((uint32_t)img, (uint32_t)(c + i + 1), a.round, 0u, a.seed_lo, a.seed_hi, sh.words[par]);
+        sh.draft[par] = d;
+    };
+    // q(z) for the thread that owns entry z (1 elsewhere)
+    auto fetch_qz = [&](uint32_t par) {
+        const PShared::Draft d = sh.draft[par];
+        float qz = 1.0f;
+        if (d.z >= 0 && ((d.z % CHUNK) >> 2) == tid && !d.is_delta && !a.greedy)
+            qz = d.qrow < 0 ? INFINITY /* alpha = 0: rejected */ : __ldcg(a.pprev + (size_t)d.qrow * V + d.z);
         return qz;
     };
-    int it = blockIdx.x;
-    while (it < total && !valid(it)) it += gridDim.x;
+    Item it = {(int)blockIdx.x / W, (int)blockIdx.x % W};
+    if (missing(it)) it = next(it);
     uint32_t phase = 0;
     const bool select = a.top_k > 0 && a.top_k < V;
-    Raw raw = {0, 0, 0};
     float qz = 1.0f;
-    if (!PROBS && it < total) {
-        raw = fetch_raw(it);
-        qz = fetch_qz(it, raw);
+    uint32_t par = 0;  // item modulo 3: the next item's words and draft are written while some threads may still read the last one's
+    if (!PROBS) {
+        if (exists(it) && tid == PT - 32) look_ahead(it, 0);
+        __syncthreads();
+        if (exists(it)) qz = fetch_qz(0);
     }
-    // random words of an item (Philox keyed by image, position, round): computed one item ahead by one thread
-    auto make_words = [&](int it, uint32_t* dst) {
-        const int slot = it / W, i = it % W;
-        philox4x32_10((uint32_t)img_of(slot), (uint32_t)(s_c[slot] + i + 1), a.round, 0u, a.seed_lo, a.seed_hi, dst);
-    };
-    uint32_t par = 0;  // item parity
-    if (!PROBS && it < total && tid == PT - 32) make_words(it, sh.words[0]);
     // Behind the LM head (a.early) all of the above, three levels of look-ups, lies beside its tail: that kernel lets this
     // one start only after its own wait, so slot tables, drafts and the last round's probabilities are complete (rollouts
     // of 64 B images 0.994 times the time, 24 L images token by token and one L image 0.996).
     pdl_wait();
     pdl_trigger();  // k_commit reads what precedes this kernel before its own wait
-    if (it < total && tid == 0) issue(it);
+    if (exists(it) && tid == 0) issue(it);
     sh.hist[tid] = 0u;  // SEL_BINS == PT
     // threshold guess carried from the previous item of this CTA: lower end and bin scale of the selection histogram
     float g_lo = 0.f, g_scale = 0.f;
     bool have_guess = false;
     __syncthreads();
 
-    while (it < total) {
-        int nxt = it + gridDim.x;
-        while (nxt < total && !valid(nxt)) nxt += gridDim.x;
-        Raw raw_next = {0, 0, 0};
-        if (!PROBS && nxt < total) raw_next = fetch_raw(nxt);  // consumed after barrier (1)
-        const int slot = it / W, i = it % W;
+    while (exists(it)) {
+        const Item nxt = next(it);
+        const uint32_t par_next = par == 2u ? 0u : par + 1u;
+        if (!PROBS && tid == PT - 32 && exists(nxt)) look_ahead(nxt, par_next);
+        const int slot = it.slot, i = it.i;
         const bool last = PROBS || i == n_of(slot) - 1;
-        const size_t oidx = PROBS ? (size_t)it : (size_t)img_of(slot) * st.Wmax + i;
-        float* pout = a.pcur + oidx * V;
+        const int oidx = PROBS ? slot : img_of(slot) * st.Wmax + i;
 
-        int z = -1;
-        bool is_delta = false, own_z = false;
-        if (!last) {
-            z = raw.z;
-            is_delta = raw.dl != 0;
-            if (z < 0 || z >= V) {
-                if (tid == 0) atomicExch(&st.counters[CNT_ERROR], ERR_BAD_TOKEN);
-                z = -1;
-            } else {
-                own_z = ((z % CHUNK) >> 2) == tid;
-            }
-        }
         const uint32_t* words = sh.words[par];  // written one item ahead (below), published by the barriers between
         if (tid == 0) sh.ncand = 0u;
 
@@ -283,38 +306,39 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
 #pragma unroll
         for (int ch = 0; ch < NCH; ++ch) {
             const int v = ch * CHUNK + tid * 4;
-            if (v < V) {
-                float4 lc = *reinterpret_cast<const float4*>(stage_c + v);
-                if (CFG) {
-                    const float4 lu = *reinterpret_cast<const float4*>(stage_u + v);
-                    lc.x = __fadd_rn(lu.x, __fmul_rn(a.cfg_scale, __fsub_rn(lc.x, lu.x)));
-                    lc.y = __fadd_rn(lu.y, __fmul_rn(a.cfg_scale, __fsub_rn(lc.y, lu.y)));
-                    lc.z = __fadd_rn(lu.z, __fmul_rn(a.cfg_scale, __fsub_rn(lc.z, lu.z)));
-                    lc.w = __fadd_rn(lu.w, __fmul_rn(a.cfg_scale, __fsub_rn(lc.w, lu.w)));
-                }
-                if (a.temperature != 1.0f) {
-                    lc.x = __fdiv_rn(lc.x, a.temperature);
-                    lc.y = __fdiv_rn(lc.y, a.temperature);
-                    lc.z = __fdiv_rn(lc.z, a.temperature);
-                    lc.w = __fdiv_rn(lc.w, a.temperature);
-                }
-                x[ch][0] = lc.x; x[ch][1] = lc.y; x[ch][2] = lc.z; x[ch][3] = lc.w;
-                mn = fminf(fminf(mn, lc.x), fminf(fminf(lc.y, lc.z), lc.w));
-                mx = fmaxf(fmaxf(mx, lc.x), fmaxf(fmaxf(lc.y, lc.z), lc.w));
-                if (select && wid == 0) {
-                    s1 += (lc.x + lc.y) + (lc.z + lc.w);
-                    s2 += (lc.x * lc.x + lc.y * lc.y) + (lc.z * lc.z + lc.w * lc.w);
-                }
-                if (have_guess) {  // selection histogram with the carried guess, verified after the barrier
-                    int b4[4];
+            float4 lc = *reinterpret_cast<const float4*>(stage_c + v);
+            if (CFG) {
+                const float4 lu = *reinterpret_cast<const float4*>(stage_u + v);
+                lc.x = __fadd_rn(lu.x, __fmul_rn(a.cfg_scale, __fsub_rn(lc.x, lu.x)));
+                lc.y = __fadd_rn(lu.y, __fmul_rn(a.cfg_scale, __fsub_rn(lc.y, lu.y)));
+                lc.z = __fadd_rn(lu.z, __fmul_rn(a.cfg_scale, __fsub_rn(lc.z, lu.z)));
+                lc.w = __fadd_rn(lu.w, __fmul_rn(a.cfg_scale, __fsub_rn(lc.w, lu.w)));
+            }
+            x[ch][0] = lc.x; x[ch][1] = lc.y; x[ch][2] = lc.z; x[ch][3] = lc.w;
+        }
+        if (a.temperature != 1.0f) {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) b4[e] = sel_bin_of(fmaxf(x[ch][e], g_lo), g_lo, g_scale);
+            for (int ch = 0; ch < NCH; ++ch)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        if (x[ch][e] >= g_lo) atomicAdd(&sh.hist[b4[e]], 1u);
-                }
-            } else {
-                x[ch][0] = x[ch][1] = x[ch][2] = x[ch][3] = -INFINITY;
+                for (int e = 0; e < 4; ++e) x[ch][e] = __fdiv_rn(x[ch][e], a.temperature);
+        }
+        if (have_guess) {  // selection histogram with the carried guess, verified after the barrier
+            const uint32_t hist = smem_addr(sh.hist);
+#pragma unroll
+            for (int ch = 0; ch < NCH; ++ch)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) count_if_above(hist, x[ch][e], g_lo, g_scale);
+        }
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+            mn = fminf(fminf(mn, x[ch][0]), fminf(fminf(x[ch][1], x[ch][2]), x[ch][3]));
+            mx = fmaxf(fmaxf(mx, x[ch][0]), fmaxf(fmaxf(x[ch][1], x[ch][2]), x[ch][3]));
+        }
+        if (select && wid == 0) {
+#pragma unroll
+            for (int ch = 0; ch < NCH; ++ch) {
+                s1 += (x[ch][0] + x[ch][1]) + (x[ch][2] + x[ch][3]);
+                s2 += (x[ch][0] * x[ch][0] + x[ch][1] * x[ch][1]) + (x[ch][2] * x[ch][2] + x[ch][3] * x[ch][3]);
             }
         }
         // minimum / maximum of the row: one warp reduction instruction each on the order-preserving keys
@@ -346,10 +370,9 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
             if (tid == 0) atomicExch(&st.counters[CNT_ERROR], 4);
             break;  // a copy never arrived; nothing else is in flight (the next item's copies are issued below)
         }
-        if (tid == 0 && nxt < total) issue(nxt);  // the next item's rows stream in behind the rest of this one
-        if (!PROBS && tid == PT - 32 && nxt < total) make_words(nxt, sh.words[par ^ 1u]);
+        if (tid == 0 && exists(nxt)) issue(nxt);  // the next item's rows stream in behind the rest of this one
         float qz_next = 1.0f;
-        if (!PROBS && nxt < total) qz_next = fetch_qz(nxt, raw_next);
+        if (!PROBS && exists(nxt)) qz_next = fetch_qz(par_next);
         mn = key_float(__reduce_min_sync(0xffffffffu, sh.redk[0][lane]));
         mx = key_float(__reduce_max_sync(0xffffffffu, sh.redk[1][lane]));
 
@@ -371,6 +394,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                 unsigned int theta = 0u;
                 float lo = g_lo, scale = g_scale;
                 bool found = false;
+#pragma unroll 1
                 for (int source = have_guess ? 0 : 1; source < 3; ++source) {
                     if (source > 0) {
                         if (source == 1) {
@@ -390,18 +414,12 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                         for (int ch = 0; ch < NCH; ++ch)
 #pragma unroll
                             for (int e = 0; e < 4; ++e)
-                                if (x[ch][e] >= lo) atomicAdd(&sh.hist[sel_bin_of(x[ch][e], lo, scale)], 1u);
+                                count_if_above(smem_addr(sh.hist), x[ch][e], lo, scale);
                         __syncthreads();  // (2) only without a carried guess
                     }
                     // bins from the top: warp w, lane l looks at bin 1023 - (32 w + l)
-                    const unsigned int cnt = sh.hist[SEL_BINS - 1 - (wid * 32 + lane)];
-                    unsigned int incl = cnt;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const unsigned int tt = __shfl_up_sync(0xffffffffu, incl, o);
-                        if (lane >= o) incl += tt;
-                    }
-                    if (lane == 31) sh.wtot[wid] = incl;
+                    const unsigned int tot = __reduce_add_sync(0xffffffffu, sh.hist[SEL_BINS - 1 - (wid * 32 + lane)]);
+                    if (lane == 0) sh.wtot[wid] = tot;
                     __syncthreads();  // (3)
                     // every warp locates the bin of the k-th largest by itself: first the warp-sized group of bins ...
                     unsigned int winc = sh.wtot[lane];
@@ -437,13 +455,19 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                     const float c_lo = fmaxf(lo, lo + ((float)bsel - 1.0f) * inv_scale);
                     const float c_hi = bsel == SEL_BINS - 1 ? INFINITY : lo + ((float)bsel + 1.0f) * inv_scale;
 #pragma unroll
-                    for (int ch = 0; ch < NCH; ++ch)
+                    for (int ch = 0; ch < NCH; ++ch) {
+                        bool any = false;  // few groups hold one: a branch per group, not per entry
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            if (x[ch][e] >= c_lo && x[ch][e] <= c_hi && sel_bin_of(x[ch][e], lo, scale) == bsel) {
-                                const unsigned int sidx = atomicAdd(&sh.ncand, 1u);
-                                if (sidx < (unsigned int)SEL_CAP) sh.cand[sidx] = float_key(x[ch][e]);
-                            }
+                        for (int e = 0; e < 4; ++e) any |= (x[ch][e] >= c_lo) & (x[ch][e] <= c_hi);
+                        if (any) {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (x[ch][e] >= c_lo && x[ch][e] <= c_hi && sel_bin_of(x[ch][e], lo, scale) == bsel) {
+                                    const unsigned int sidx = atomicAdd(&sh.ncand, 1u);
+                                    if (sidx < (unsigned int)SEL_CAP) sh.cand[sidx] = float_key(x[ch][e]);
+                                }
+                        }
+                    }
                     __syncthreads();  // (5)
                     sh.hist[tid] = 0u;  // every read of the histogram is behind us: clean for the next item's pass 1
                     const int nc = (int)sh.ncand;
@@ -461,6 +485,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                     } else if (nc > SEL_CAP) {
                         break;
                     } else {
+#pragma unroll 1
                         for (int u = tid; u < nc; u += PT) {
                             const unsigned int ku = sh.cand[u];
                             unsigned int gt = 0, ge = 0;
@@ -499,7 +524,8 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
         for (int ch = 0; ch < NCH; ++ch)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                x[ch][e] = x[ch][e] >= thr ? __expf(x[ch][e] - mx) : 0.f;  // entries past V are -inf: 0
+                // (dropped entries, and those past V, by exp(-inf): no branch around the exponential)
+                x[ch][e] = __expf(x[ch][e] >= thr ? x[ch][e] - mx : -INFINITY);
                 part += x[ch][e];
             }
         part = warp_sum(part);
@@ -508,6 +534,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
         const float den = warp_sum(sh.redsum[lane]);
         const float inv = 1.0f / den;
         // fixed-point weights floor(p 2^30): the whole row totals 2^30 (1 + 1e-3) at most, so 32-bit sums are exact
+        float* pout = a.pcur + (size_t)oidx * V;
         unsigned int wc[NCH];
 #pragma unroll
         for (int ch = 0; ch < NCH; ++ch) {
@@ -547,12 +574,13 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                 const int am = (int)bi;
                 a.cand_rep[oidx] = am;
                 a.cand_ref[oidx] = am;
-                a.flag[oidx] = (!last && z == am) ? 1 : 0;
+                a.flag[oidx] = (!last && sh.draft[par].z == am) ? 1 : 0;
             }
         } else {
             // accept test (Eq. 5) by the owner of entry z
+            const int z = sh.draft[par].z;
             if (!last && z < 0 && tid == 0) a.flag[oidx] = 0;  // invalid draft token: rejected
-            if (own_z) {
+            if (z >= 0 && ((z % CHUNK) >> 2) == tid) {
                 // p(z) out of the registers by a masked sum (a computed index would move the row to local memory)
                 const int zc = z / CHUNK, ze = z & 3;
                 float pz = 0.f;
@@ -560,7 +588,7 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                 for (int ch = 0; ch < NCH; ++ch)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) pz = __fmaf_rn((ch == zc && e == ze) ? 1.0f : 0.0f, x[ch][e], pz);
-                const float alpha = is_delta ? pz : fminf(1.0f, __fdiv_rn(pz, qz));
+                const float alpha = sh.draft[par].is_delta ? pz : fminf(1.0f, __fdiv_rn(pz, qz));
                 const float u = (float)(words[0] >> 8) * (1.0f / 16777216.0f);
                 a.flag[oidx] = (u < alpha) ? 1 : 0;
             }
@@ -596,54 +624,72 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                         start += ctot[ch];
                     }
                 }
-                // position of this thread's group inside the chunk: warps before it, then lanes before it
-                const unsigned int wbase = __reduce_add_sync(0xffffffffu, wsel);
-                unsigned int incl = mine;
+                // The warp whose groups hold it, warps before it counted, then lanes before its thread; the others are done
+                const unsigned int wbase = run + __reduce_add_sync(0xffffffffu, wsel);
+                if (target >= wbase && target - wbase < sh.csum[cs][wid]) {
+                    unsigned int incl = mine;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned int tt = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += tt;
-                }
-                const unsigned int start = run + wbase + incl - mine;
-                if (target >= start && target - start < mine) {  // exactly one thread
-                    unsigned int r = start;
-                    int pick = 3;
-                    bool found = false;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const unsigned int tt = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += tt;
+                    }
+                    const unsigned int start = wbase + incl - mine;
+                    if (target >= start && target - start < mine) {  // exactly one thread
+                        unsigned int r = start;
+                        int pick = 3;
+                        bool found = false;
 #pragma unroll
-                    for (int ch = 0; ch < NCH; ++ch)
-                        if (ch == cs) {
+                        for (int ch = 0; ch < NCH; ++ch)
+                            if (ch == cs) {
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                r += fixed_weight(x[ch][e]);
-                                if (!found && r > target) {
-                                    pick = e;
-                                    found = true;
+                                for (int e = 0; e < 4; ++e) {
+                                    r += fixed_weight(x[ch][e]);
+                                    if (!found && r > target) {
+                                        pick = e;
+                                        found = true;
+                                    }
                                 }
                             }
-                        }
-                    a.cand_ref[oidx] = cs * CHUNK + tid * 4 + pick;
+                        a.cand_ref[oidx] = cs * CHUNK + tid * 4 + pick;
+                    }
                 }
             }
         }
         it = nxt;
-        par ^= 1u;
-        raw = raw_next;
+        par = par_next;
         qz = qz_next;
     }
 }
 
 }  // namespace
 
-bool accept_persistent_supported(const State& st) { return st.V <= NCH * CHUNK && st.V % 4 == 0; }
+// Chunks a row is padded to: 1, 2 or 4.
+static int row_chunks(int V) { return V <= CHUNK ? 1 : V <= 2 * CHUNK ? 2 : 4; }
+static int smem_bytes(bool cfg, int V, int table_slots) {
+    return (cfg ? 2 : 1) * row_chunks(V) * CHUNK * (int)sizeof(float) + (int)sizeof(PShared) + 3 * table_slots * (int)sizeof(int);
+}
+
+// The slot tables of a round have to fit beside the rows (7000 slots at V = 16384 with guidance, 15600 up to 4096).
+bool accept_persistent_supported(const State& st, int slots) {
+    return st.V <= MAX_CH * CHUNK && st.V % 4 == 0 && slots <= 65536 && smem_bytes(st.nb == 2, st.V, slots) <= 227 * 1024;
+}
+
+template <bool CFG, bool PROBS, int NCH>
+static void launch_nch(const State& st, const AcceptArgs& a, int n_sms, Stream& s) {
+    static int configured[64] = {0};
+    const int bytes = smem_bytes(CFG, st.V, PROBS ? 0 : a.S);
+    const int items = a.S * st.W;
+    ensure_dynamic_smem(k_accept_persistent<CFG, PROBS, NCH>, bytes, configured);
+    launch_k(k_accept_persistent<CFG, PROBS, NCH>, dim3(items < n_sms ? items : n_sms), dim3(PT), bytes, s, st, a);
+}
 
 template <bool CFG, bool PROBS>
 static void launch(const State& st, const AcceptArgs& a, int n_sms, Stream& s) {
-    static int configured[64] = {0};
-    const int bytes = (CFG ? 2 : 1) * st.V * (int)sizeof(float) + (int)sizeof(PShared) +
-                      (PROBS ? 0 : 3 * a.S * (int)sizeof(int));
-    const int items = a.S * st.W;
-    ensure_dynamic_smem(k_accept_persistent<CFG, PROBS>, bytes, configured);
-    launch_k(k_accept_persistent<CFG, PROBS>, dim3(items < n_sms ? items : n_sms), dim3(PT), bytes, s, st, a);
+    switch (row_chunks(st.V)) {
+        case 1: launch_nch<CFG, PROBS, 1>(st, a, n_sms, s); break;
+        case 2: launch_nch<CFG, PROBS, 2>(st, a, n_sms, s); break;
+        default: launch_nch<CFG, PROBS, 4>(st, a, n_sms, s);
+    }
 }
 
 void launch_accept_persistent(const State& st, const AcceptArgs& a, int n_sms, Stream& s) {

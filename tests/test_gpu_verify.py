@@ -150,3 +150,41 @@ def test_commit_of_every_window_and_history_offset(W, H, greedy):
         np.testing.assert_array_equal(s2, seq[b])
         np.testing.assert_array_equal(d2[nc + 1:nc + W], dl[b][nc + 1:nc + W])
     ctx.hbsjd_destroy()
+
+
+@pytest.mark.parametrize("V,B,W,branches,top_k,greedy", [
+    (4160, 60, 13, 2, 500, False), (8256, 40, 16, 1, 100, False), (8256, 40, 16, 2, 0, False), (16384, 24, 16, 2, 1000, False),
+    (16384, 24, 16, 2, 1000, True), (64, 1100, 2, 2, 9, False), (64, 1100, 2, 1, 0, True), (64, 16500, 2, 2, 9, False)])
+def test_several_positions_per_cta(V, B, W, branches, top_k, greedy):
+    """Positions behind one another on a CTA: vocabularies that end inside a chunk and that leave threads and whole chunks
+    without entries, positions with and without a selection guess, and more slots than have their tables in shared
+    memory (16500, through the other kernel).  Probabilities as the oracle's pipeline gives them, decisions replayed on
+    them: equal."""
+    import torch
+    sh = synth.ModelShape(1, 64, 1, 64, V, 4, 4, 3, "bf16")
+    ctx = binding.Context(sh, synth.make_weights(sh, 3, target_entropy=None), B, W)
+    case = G.verify_case(V + W, B=B, W=W, T=64, V=V, branches=branches, cfg_scale=2.0 if branches == 2 else 1.0, top_k=top_k)
+    # multiples of 2^-10 below 2^7: guidance is exact in fp32, so that the k-th largest is the oracle's
+    case["logits"] = (np.round(case["logits"] * 1024) / 1024).astype(np.float32)
+    d = {k: G.dev(case[k]) for k in ("logits", "q", "cursor", "seq", "delta", "qbase")}
+    p_out = torch.zeros((B, W, V), device="cuda")
+    m_out = torch.zeros(B, dtype=torch.int32, device="cuda")
+    ctx.hbsjd_verify(G.verify_desc(case, 5, 3, greedy), d["logits"], d["q"], p_out, d["cursor"], d["seq"], d["delta"],
+                     d["qbase"], m_out)
+    p, cur, seq, dl = (x.cpu().numpy() for x in (p_out, d["cursor"], d["seq"], d["delta"]))
+    for b in range(B):
+        c = int(case["cursor"][b])
+        if c >= 64:
+            assert np.array_equal(seq[b], case["seq"][b])
+            continue
+        n = min(W, 64 - c)
+        for i in range(0, n, 3):
+            ref = O.probs(case["logits"][0, b, i], case["logits"][1, b, i] if branches == 2 else None,
+                          s=case["cfg_scale"], k=top_k)
+            assert np.all(np.abs(p[b, i] - ref) <= 1e-6 + 1e-5 * ref)
+        s2, d2 = case["seq"][b].copy(), case["delta"][b].copy()
+        nc, m, _ = O.replay_round(V, 64, W, 8, greedy, 5, b, 3, c, s2, d2, p[b, :n], case["q"][b], int(case["qbase"][b]))
+        assert nc == cur[b] and m == int(m_out[b])
+        np.testing.assert_array_equal(s2, seq[b])
+        np.testing.assert_array_equal(d2[nc + 1:nc + W], dl[b][nc + 1:nc + W])
+    ctx.hbsjd_destroy()
