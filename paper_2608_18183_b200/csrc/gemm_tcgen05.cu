@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tcgen05(const __grid_co
                 } else {  // EPI_QKV
                     const State& st = g.st;
                     const int D = st.D;
-                    const int sec = col / D, cs = col % D;  // 0 q, 1 k, 2 v; a tile never straddles sections
+                    const int sec = col / D, cs = col % D;  // 0 q, 1 k, 2 v; a chunk never straddles sections (a tile of 192 columns may)
                     uint32_t o[16];
                     if (sec < 2)  // the chunk's 16 rotation pairs: first or second half of the row's cos/sin table
                         rope_chunk(r, rscale, ((cs % st.dh) / 2) >= 16 ? rope_hi : rope_lo, o);
