@@ -314,13 +314,13 @@ __global__ void __launch_bounds__(PT, 1) k_accept_persistent(State st, AcceptArg
                 lc.z = __fadd_rn(lu.z, __fmul_rn(a.cfg_scale, __fsub_rn(lc.z, lu.z)));
                 lc.w = __fadd_rn(lu.w, __fmul_rn(a.cfg_scale, __fsub_rn(lc.w, lu.w)));
             }
+            if (a.temperature != 1.0f) {  // (here, not in a loop behind: 60 images x 16 positions 107 -> 105 us)
+                lc.x = __fdiv_rn(lc.x, a.temperature);
+                lc.y = __fdiv_rn(lc.y, a.temperature);
+                lc.z = __fdiv_rn(lc.z, a.temperature);
+                lc.w = __fdiv_rn(lc.w, a.temperature);
+            }
             x[ch][0] = lc.x; x[ch][1] = lc.y; x[ch][2] = lc.z; x[ch][3] = lc.w;
-        }
-        if (a.temperature != 1.0f) {
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) x[ch][e] = __fdiv_rn(x[ch][e], a.temperature);
         }
         if (have_guess) {  // selection histogram with the carried guess, verified after the barrier
             const uint32_t hist = smem_addr(sh.hist);
