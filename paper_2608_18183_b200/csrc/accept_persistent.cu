@@ -670,9 +670,11 @@ static int smem_bytes(bool cfg, int V, int table_slots) {
     return (cfg ? 2 : 1) * row_chunks(V) * CHUNK * (int)sizeof(float) + (int)sizeof(PShared) + 3 * table_slots * (int)sizeof(int);
 }
 
-// The slot tables of a round have to fit beside the rows (7000 slots at V = 16384 with guidance, 15600 up to 4096).
-bool accept_persistent_supported(const State& st, int slots) {
-    return st.V <= MAX_CH * CHUNK && st.V % 4 == 0 && slots <= 65536 && smem_bytes(st.nb == 2, st.V, slots) <= 227 * 1024;
+// The slot tables of a round have to fit beside the rows (7000 slots at V = 16384 with guidance, 15600 up to 4096).  The batch
+// decides, not the round's slots: the kernels add a row's terms in different orders, and Compact execution, whose slots
+// fall with the live images, has to give Full execution's bits.
+bool accept_persistent_supported(const State& st) {
+    return st.V <= MAX_CH * CHUNK && st.V % 4 == 0 && st.B <= 65536 && smem_bytes(st.nb == 2, st.V, st.B) <= 227 * 1024;
 }
 
 template <bool CFG, bool PROBS, int NCH>

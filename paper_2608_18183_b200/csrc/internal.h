@@ -145,7 +145,7 @@ void launch_commit(const State& st, const AcceptArgs& a, Stream& s);
 void launch_sync_min(const State& st, const AcceptArgs& a, int32_t* m_sync, Stream& s);
 int accept_smem_bytes(int V);
 // persistent form of launch_prob_accept for vocabularies up to 16384 (accept_persistent.cu)
-bool accept_persistent_supported(const State& st, int slots);
+bool accept_persistent_supported(const State& st);
 void launch_accept_persistent(const State& st, const AcceptArgs& a, int n_sms, Stream& s);
 // streaming multiprocessors of the current device
 int device_sm_count();

@@ -645,7 +645,7 @@ int device_sm_count() {
 }
 
 void launch_prob_accept(const State& st, const AcceptArgs& a, Stream& s) {
-    if (accept_persistent_supported(st, a.S)) {
+    if (accept_persistent_supported(st)) {
         launch_accept_persistent(st, a, device_sm_count(), s);
         return;
     }

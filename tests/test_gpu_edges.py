@@ -362,3 +362,24 @@ def test_prefixes_and_trajectories_in_several_passes(window):
         np.testing.assert_array_equal(got, pos[s])
     for c in (big, teacher, few, few_teacher):
         c.hbsjd_destroy()
+
+
+def test_a_batch_beyond_the_slot_tables_has_one_accept_kernel():
+    """18000 images are too many slots for the persistent accept kernel's tables in shared memory, the 70 that are live are
+    not: Full and Compact execution have to run the same kernel all the same.  Probabilities and state bit for bit."""
+    s = synth.ModelShape(1, 64, 1, 64, 1024, 4, 4, 3, "bf16")
+    B, W = 18000, 2
+    live = np.arange(0, B, 260)
+    rng = np.random.default_rng(18000)
+    toks = rng.integers(0, s.vocab, (B, s.T)).astype(np.int32)
+    k = np.full(B, s.T, dtype=np.int32)
+    k[live] = rng.integers(0, s.T - 4, len(live))
+    ctx = binding.Context(s, synth.make_weights(s, 3), B, W)
+    got = {}
+    for mode in (binding.EXEC_FULL, binding.EXEC_COMPACT):
+        ctx.hbsjd_rollout(G.dev(toks), G.dev(k), G.dev(np.zeros(B, dtype=np.int32)),
+                          binding.make_params(W, 4, 1.0, 0.9, 100, seed=5, exec_mode=mode, max_rounds=2))
+        got[mode] = [np.concatenate([ctx.hbsjd_debug_read(binding.DBG_PROBS, int(b)) for b in live])] + list(ctx.hbsjd_get_state())
+    for full, compact in zip(got[binding.EXEC_FULL], got[binding.EXEC_COMPACT]):
+        np.testing.assert_array_equal(full, compact)
+    ctx.hbsjd_destroy()
