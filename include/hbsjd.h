@@ -106,6 +106,11 @@ typedef struct {
  * Constraints: dim % n_heads == 0; head size 16/32/64/128 for fp32 models, 32 or 64 for bf16 models (64 runs
  * the tensor-core attention kernel, 32 a plain one); dim, ffn_hidden, vocab multiples of 64 for bf16;
  * vocab <= 32768 (a position's probabilities stay in one CTA's shared memory).
+ * Device memory, but for some KB per image: the weights; keys and values of 2 max_batch sequences of T tokens, T rounded up to
+ * 64; 16 max_batch max_window vocab bytes of logits and probabilities; and activations of R = max(2 max_batch max_window,
+ * min(4096, 2 max_batch T)) rows, so that pre-filling and scoring take few forwards: 10.125 dim + 2 ffn_hidden bytes
+ * a row for bf16 models, 28 dim + 12 ffn_hidden for fp32.  Where that does not fit, R is 2 max_batch max_window, what a
+ * round needs: the results are the same.
  * Errors: HBSJD_EINVAL, HBSJD_ENOMEM, HBSJD_ECUDA. */
 int hbsjd_create(hbsjd_ctx **out, const hbsjd_model_desc *m, const void *weights, size_t weight_bytes,
                  int max_batch, int max_window, void *cuda_stream);

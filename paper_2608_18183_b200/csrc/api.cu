@@ -17,7 +17,7 @@ using namespace hbsjd;
 namespace {
 
 constexpr int PAGE_TOKENS = 64;
-constexpr int PASS_ROWS = 4096;  // see create_impl
+constexpr int PASS_ROWS = 4096;  // see alloc_activations
 
 struct LayerW {
     const void *g_attn, *w_qkv, *w_o, *g_ffn, *w_13, *w_2;
@@ -29,6 +29,8 @@ struct hbsjd_ctx {
     hbsjd_model_desc d;
     int T, dh, Bmax, Wmax;
     int rows_cap;        // rows of the activation buffers
+    int logit_rows;      // rows of `logits`: the largest round's, 2 x max_batch x max_window
+    int score_rows;      // rows of logits that have room where a forward of hbsjd_score puts them, see alloc_activations
     bool bf16_model;
     bool fold_norm;      // bf16 model: RMSNorm folded into the GEMM epilogues (launch-bound contexts), else its own kernel
     bool unit_gains;     // every norm gain of the model is exactly 1
@@ -49,7 +51,8 @@ struct hbsjd_ctx {
     int parity;
     uint8_t* flag;
     int32_t *cand_rep, *cand_ref;
-    // activations
+    // activations, one allocation (see alloc_activations)
+    unsigned char* activations;
     float *h, *qkv, *gu, *logits;
     void *a, *q, *o, *act;  // a: normed operand (fp32 model) / bf16 copy of the residual stream (bf16 model)
     float* ssq;             // [rows][dim / 32] partial sums of squares of the residual rows (bf16 model)
@@ -127,7 +130,7 @@ void prof_resolve(hbsjd_ctx* c, double attn_bytes, double accept_bytes) {
         if (cudaEventElapsedTime(&ms, s.a, s.b) != cudaSuccess) continue;
         double work = s.work;
         if (s.cls == HBSJD_PROF_ATTENTION) work = attn_bytes;
-        if (s.cls == HBSJD_PROF_ACCEPT) work = accept_bytes;
+        if (s.cls == HBSJD_PROF_ACCEPT && work == 0.0) work = accept_bytes;
         c->prof.ms[s.cls] += ms;
         c->prof.work[s.cls] += work;
         c->prof.launches[s.cls] += 1;
@@ -192,19 +195,45 @@ int gemm<bf16>(hbsjd_ctx* c, const void* A, const void* W, float* C, int M, int 
     return rc == 0 ? 0 : (rc == -1 ? HBSJD_EINVAL : HBSJD_ECUDA);
 }
 
+// How far a forward goes: pre-filling wants the last layer's keys and values, scoring the operand of the head, whose logits it
+// takes in parts (see head), a round the logits.
+enum Until { KEYS_VALUES, HEAD_OPERAND, LOGITS };
+
 // One batched verifier forward over S slots and c->st.R rows per branch (Sec. 4.2 "Batched verification").
 // stop_layer >= 0 (debugging): return after the attention sub-block (stop_stage 0) or the whole block
 // (stop_stage 1) of that layer, leaving the activation buffers as that point found them.
 template <typename TA>
-int forward(hbsjd_ctx* c, int S, bool want_logits, int stop_layer = -1, int stop_stage = 0);
+int forward(hbsjd_ctx* c, int S, Until until, int stop_layer = -1, int stop_stage = 0);
+
+// Logits of the rows row0 .. row0 + rows - 1 of a forward that has left the head's operand, into `out` with room for `cap` rows.
+template <typename TA>
+int head(hbsjd_ctx* c, int row0, int rows, float* out, int cap);
+template <>
+int head<float>(hbsjd_ctx* c, int row0, int rows, float* out, int) {
+    const size_t D = c->d.dim;
+    return gemm<float>(c, (const float*)c->a + row0 * D, c->w_head, out, rows, c->d.vocab, c->d.dim, 0);
+}
+template <>
+int head<bf16>(hbsjd_ctx* c, int row0, int rows, float* out, int cap) {
+    const size_t D = c->d.dim, V = c->d.vocab;
+    const NormIn nin = {c->fold_norm ? c->ssq + row0 * (D / 32) : nullptr, c->d.rms_eps};
+    const int ps = prof_begin(c, HBSJD_PROF_GEMM, 2.0 * rows * V * D, rows,
+                              2.0 * ((double)rows * D + (double)V * D) + 4.0 * rows * V);
+    const int rc = gemm_tcgen05_head((const bf16*)c->a + row0 * D, (const bf16*)c->w_head, out, rows, c->d.vocab, c->d.dim,
+                                     std::min(cap, c->rows_cap - row0), nin, c->st.counters + CNT_ERROR, c->stream, c->err,
+                                     sizeof(c->err), c->force_tile);
+    prof_end(c, ps);
+    c->launches++;
+    return rc == 0 ? 0 : (rc == -1 ? HBSJD_EINVAL : HBSJD_ECUDA);
+}
 
 // fp32 model: every step its own kernel (the configuration exists for parity, not speed).
 template <>
-int forward<float>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int stop_stage) {
+int forward<float>(hbsjd_ctx* c, int S, Until until, int stop_layer, int stop_stage) {
     typedef float TA;
     const State& st = c->st;
     const int M = st.nb * st.R, D = st.D, F = st.F;
-    const bool kv_only = !want_logits && stop_layer < 0;  // pre-filling: of the last layer only keys and values are wanted
+    const bool kv_only = until == KEYS_VALUES && stop_layer < 0;  // of the last layer only keys and values are wanted
     Stream& s = c->stream;
     const KvView kv = kv_view(c);
     launch_embed<TA>(st, (const TA*)c->tok_emb, (const TA*)c->cls_emb, c->h, nullptr, nullptr, s);
@@ -238,10 +267,10 @@ int forward<float>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int st
         if ((rc = gemm<TA>(c, c->act, w.w_2, c->h, M, D, F, 1))) return rc;
         if (l == stop_layer) return 0;
     }
-    if (want_logits) {
-        norm(c->h, c->g_out);
-        int rc;
-        if ((rc = gemm<TA>(c, c->a, c->w_head, c->logits, M, st.V, D, 0))) return rc;
+    if (until != KEYS_VALUES) norm(c->h, c->g_out);
+    if (until == LOGITS) {
+        const int rc = head<TA>(c, 0, M, c->logits, c->logit_rows);
+        if (rc) return rc;
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -262,7 +291,7 @@ int forward<float>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int st
 //     what the separate kernel costs (its reads of the old residual compete with the operand stream for L2
 //     bandwidth), so the form with the exact operand rounding of the definition is kept there.
 template <>
-int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int stop_stage) {
+int forward<bf16>(hbsjd_ctx* c, int S, Until until, int stop_layer, int stop_stage) {
     const State& st = c->st;
     const int M = st.nb * st.R, D = st.D, F = st.F;
     const int Mcap = c->rows_cap;
@@ -299,7 +328,7 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
     launch_embed<bf16>(st, (const bf16*)c->tok_emb, (const bf16*)c->cls_emb, c->h, fold ? a : nullptr,
                        fold ? c->ssq : nullptr, s);
     c->launches++;
-    const bool kv_only = !want_logits && stop_layer < 0;  // pre-filling: of the last layer only keys and values are wanted
+    const bool kv_only = until == KEYS_VALUES && stop_layer < 0;  // of the last layer only keys and values are wanted
     for (int l = 0; l < st.L; ++l) {
         const LayerW& w = c->layers[l];
         int rc, ps;
@@ -335,15 +364,10 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
         if ((rc = residual(c->act, w.w_2, F))) return done(rc);
         if (l == stop_layer) return 0;
     }
-    if (want_logits) {
-        if (!fold) norm(c->g_out);
-        const int ps = prof_begin(c, HBSJD_PROF_GEMM, 2.0 * M * st.V * D, M,
-                                  es * ((double)M * D + (double)st.V * D) + 4.0 * M * st.V);
-        const int rc = gemm_tcgen05_head(a, (const bf16*)c->w_head, c->logits, M, st.V, D, Mcap, nin, eflag, s,
-                                         c->err, sizeof(c->err), c->force_tile);
-        prof_end(c, ps);
-        if (rc) return done(rc);
-        c->launches++;
+    if (until != KEYS_VALUES && !fold) norm(c->g_out);
+    if (until == LOGITS) {
+        const int rc = head<bf16>(c, 0, M, c->logits, c->logit_rows);
+        if (rc) return rc;
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -353,9 +377,9 @@ int forward<bf16>(hbsjd_ctx* c, int S, bool want_logits, int stop_layer, int sto
     return 0;
 }
 
-int forward_any(hbsjd_ctx* c, int S, bool want_logits, int stop_layer = -1, int stop_stage = 0) {
-    return c->bf16_model ? forward<bf16>(c, S, want_logits, stop_layer, stop_stage)
-                         : forward<float>(c, S, want_logits, stop_layer, stop_stage);
+int forward_any(hbsjd_ctx* c, int S, Until until, int stop_layer = -1, int stop_stage = 0) {
+    return c->bf16_model ? forward<bf16>(c, S, until, stop_layer, stop_stage)
+                         : forward<float>(c, S, until, stop_layer, stop_stage);
 }
 
 int choose_compact(const hbsjd_ctx* c, int live) {
@@ -440,7 +464,7 @@ int enqueue_round(hbsjd_ctx* c) {
         CK(cudaMemsetAsync(c->st.counters + CNT_ERROR, 1, 1, c->stream));
     }
     c->launches++;
-    int rc = forward_any(c, S, true);
+    int rc = forward_any(c, S, LOGITS);
     if (rc) return rc;
     AcceptArgs a;
     a.logits = c->logits;
@@ -577,8 +601,7 @@ int run_rounds(hbsjd_ctx* c, int max_rounds) {
 void free_all(hbsjd_ctx* c) {
     void* ptrs[] = {c->w_img, c->rope_cs, c->kc, c->vc, c->page_table, c->st.cursor, c->st.seq, c->st.delta,
                     c->st.qbase, c->st.label, c->st.klen, c->st.pfill, c->st.slot_img, c->st.slot_c, c->st.slot_n, c->st.slot_row, c->st.row_pos, c->st.slot_sorted,
-                    c->st.counters, c->st.m_last, c->st.j_last, c->pbuf[0], c->pbuf[1], c->flag, c->cand_rep,
-                    c->cand_ref, c->h, c->qkv, c->gu, c->logits, c->a, c->q, c->o, c->act, c->ssq,
+                    c->st.counters, c->st.m_last, c->st.j_last, c->flag, c->cand_rep, c->cand_ref, c->activations,
                     c->stage_tok, c->stage_len, c->stage_lab, c->stage_out, c->verify_scratch,
                     c->score_pos, c->score_img, c->score_loss, c->m_sync, c->tally};
     for (void* p : ptrs)
@@ -593,6 +616,44 @@ void free_all(hbsjd_ctx* c) {
     if (c->ev0) cudaEventDestroy(c->ev0);
     if (c->ev1) cudaEventDestroy(c->ev1);
     if (c->ev2) cudaEventDestroy(c->ev2);
+}
+
+// The activations of forwards of up to `rows` rows, the logits of the largest round and the probabilities of two, in one
+// allocation.  A row of logits is as large as three to six rows of all other activations, and only scoring wants logits of more
+// rows than a round has.  So the head's operand lies behind all that is free once the operand is there, and hbsjd_score has the
+// logits written over that, from the front, in as many parts as it takes (9 images of B against L, window 16: 2 parts and
+// 3.07 ms, where logits for 4096 rows, 260 MB more per context, took 3.03; 128 images of L against XL, window 32: 1 part).
+int alloc_activations(hbsjd_ctx* c, size_t rows) {
+    const size_t D = c->d.dim, F = c->d.ffn_hidden, V = c->d.vocab, es = c->bf16_model ? 2 : 4;
+    const size_t f32_only = c->bf16_model ? 0 : 1;  // fp32 GEMM outputs the fused bf16 epilogues never materialise
+    const size_t probs = (size_t)c->Bmax * c->Wmax * V * sizeof(float);
+    size_t bytes = 0;
+    auto take = [&](size_t n) {
+        const size_t at = bytes;
+        bytes = align256(bytes + n);
+        return at;
+    };
+    const size_t h = take(rows * D * sizeof(float)), q = take(rows * D * es), o = take(rows * D * es), act = take(rows * F * es);
+    const size_t qkv = take(f32_only * rows * 3 * D * sizeof(float)), gu = take(f32_only * rows * 2 * F * sizeof(float));
+    const size_t logits = take(2 * probs), p0 = take(probs), p1 = take(probs);
+    const size_t a = take(rows * D * es), ssq = take(c->bf16_model ? rows * (D / 32) * sizeof(float) : 0);
+    const int rc = dev_alloc(c, &c->activations, bytes);
+    if (rc) return rc;
+    unsigned char* base = c->activations;
+    c->h = (float*)(base + h);
+    c->q = base + q;
+    c->o = base + o;
+    c->act = base + act;
+    c->qkv = (float*)(base + qkv);
+    c->gu = (float*)(base + gu);
+    c->logits = (float*)(base + logits);
+    c->pbuf[0] = (float*)(base + p0);
+    c->pbuf[1] = (float*)(base + p1);
+    c->a = base + a;
+    c->ssq = (float*)(base + ssq);
+    c->rows_cap = (int)rows;
+    c->score_rows = (int)std::min(rows, a / (V * sizeof(float)));
+    return 0;
 }
 
 int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
@@ -726,10 +787,10 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
     }
     // state
     const size_t Bm = c->Bmax, Wm = c->Wmax, T1 = c->T + 1;
+    c->logit_rows = (int)(2 * Bm * Wm);
     // Activation rows: the largest round, 2 branches x max_batch slots x max_window inputs; and at least PASS_ROWS (or all
     // that the batch has), so that contexts of few images or short windows pre-fill and score in few forwards.
-    const size_t Mmax = std::max(2 * Bm * Wm, std::min((size_t)PASS_ROWS, 2 * Bm * c->T)), Sm = max_slots(Bm, Mmax);
-    c->rows_cap = (int)Mmax;
+    const size_t most_rows = std::max(2 * Bm * Wm, std::min((size_t)PASS_ROWS, 2 * Bm * c->T)), Sm = max_slots(Bm, most_rows);
     int rc;
     State& st = c->st;
     if ((rc = dev_alloc(c, &st.cursor, Bm)) || (rc = dev_alloc(c, &st.seq, Bm * T1)) ||
@@ -737,25 +798,11 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
         (rc = dev_alloc(c, &st.label, Bm)) || (rc = dev_alloc(c, &st.klen, Bm)) ||
         (rc = dev_alloc(c, &st.pfill, Bm)) || (rc = dev_alloc(c, &st.slot_img, Sm)) ||
         (rc = dev_alloc(c, &st.slot_c, Sm)) || (rc = dev_alloc(c, &st.slot_n, Sm)) ||
-        (rc = dev_alloc(c, &st.slot_row, Sm)) || (rc = dev_alloc(c, &st.row_pos, Mmax)) ||
+        (rc = dev_alloc(c, &st.slot_row, Sm)) || (rc = dev_alloc(c, &st.row_pos, most_rows)) ||
         (rc = dev_alloc(c, &st.slot_sorted, Sm)) ||
         (rc = dev_alloc(c, &st.counters, (size_t)8)) || (rc = dev_alloc(c, &st.m_last, Bm)) ||
-        (rc = dev_alloc(c, &st.j_last, Bm)) || (rc = dev_alloc(c, &c->pbuf[0], Bm * Wm * V)) ||
-        (rc = dev_alloc(c, &c->pbuf[1], Bm * Wm * V)) || (rc = dev_alloc(c, &c->flag, Bm * Wm)) ||
-        (rc = dev_alloc(c, &c->cand_rep, Bm * Wm)) || (rc = dev_alloc(c, &c->cand_ref, Bm * Wm)))
+        (rc = dev_alloc(c, &st.j_last, Bm)) || (rc = dev_alloc(c, &c->flag, Bm * Wm)) || (rc = dev_alloc(c, &c->cand_rep, Bm * Wm)) || (rc = dev_alloc(c, &c->cand_ref, Bm * Wm)))
         return rc;
-    unsigned char *a, *q, *o, *act;
-    const size_t f32_only = c->bf16_model ? 0 : 1;  // fp32 GEMM outputs the fused bf16 epilogues never materialise
-    if ((rc = dev_alloc(c, &c->h, Mmax * D)) || (rc = dev_alloc(c, &c->qkv, f32_only * Mmax * 3 * D)) ||
-        (rc = dev_alloc(c, &c->gu, f32_only * Mmax * 2 * F)) || (rc = dev_alloc(c, &c->logits, Mmax * V)) ||
-        (rc = dev_alloc(c, &a, Mmax * D * es)) || (rc = dev_alloc(c, &q, Mmax * D * es)) ||
-        (rc = dev_alloc(c, &o, Mmax * D * es)) || (rc = dev_alloc(c, &act, Mmax * F * es)))
-        return rc;
-    if ((rc = dev_alloc(c, &c->ssq, c->bf16_model ? Mmax * (D / 32) : (size_t)0))) return rc;
-    c->a = a;
-    c->q = q;
-    c->o = o;
-    c->act = act;
     if ((rc = dev_alloc(c, &c->stage_tok, Bm * (size_t)c->T)) || (rc = dev_alloc(c, &c->stage_len, Bm)) ||
         (rc = dev_alloc(c, &c->stage_lab, Bm)) || (rc = dev_alloc(c, &c->stage_out, Bm * (size_t)c->T)))
         return rc;
@@ -791,6 +838,14 @@ int create_impl(hbsjd_ctx* c, const void* weights, size_t weight_bytes) {
     CK(cudaEventCreate(&c->ev0));
     CK(cudaEventCreate(&c->ev1));
     CK(cudaEventCreate(&c->ev2));
+    // last, so that everything else has found its place where the larger size does not fit
+    rc = alloc_activations(c, most_rows);
+    if (rc == HBSJD_ENOMEM && most_rows > (size_t)c->logit_rows) {
+        (void)cudaGetLastError();
+        c->err[0] = 0;
+        rc = alloc_activations(c, (size_t)c->logit_rows);
+    }
+    if (rc) return rc;
     CK(cudaStreamSynchronize(c->stream));
     return 0;
 }
@@ -944,7 +999,7 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
         st.R = sh.rows;
         st.multi = span > st.W;
         launch_setup(st, 1, 1, c->stream, span);
-        const int rc = forward_any(c, sh.slots, false);
+        const int rc = forward_any(c, sh.slots, KEYS_VALUES);
         if (rc) return rc;
         launch_prefill_advance(st, span, c->stream);
         c->launches += 2;
@@ -1098,7 +1153,7 @@ int score_run(hbsjd_ctx* student, hbsjd_ctx* teacher, int batch, const int32_t* 
             x->st.multi = span > sh.width;
             launch_setup(x->st, 1, 1, x->stream, span);
             x->launches++;
-            const int rc = forward_any(x, sh.slots, true);
+            const int rc = forward_any(x, sh.slots, HEAD_OPERAND);
             if (rc) {
                 if (x != c) snprintf(c->err, sizeof(c->err), "teacher forward: %.200s", x->err);
                 return rc;
@@ -1108,19 +1163,33 @@ int score_run(hbsjd_ctx* student, hbsjd_ctx* teacher, int batch, const int32_t* 
                 if (rs) return rs;
             }
         }
-        // the divergence kernel reads both models' logits on the student's stream; the teacher's next
-        // forward overwrites its logits and waits for that kernel in turn
-        CK(cudaEventRecord(teacher->ev2, teacher->stream));
-        CK(cudaStreamWaitEvent(c->stream, teacher->ev2, 0));
-        {
-            // timed with the vocabulary-wide class: 2 V floats read per input, as the byte count of that class
-            const int ps = prof_begin(c, HBSJD_PROF_ACCEPT, 0.0);
-            launch_bikl_inputs(c->st, c->logits, teacher->logits, prefix_len, pos, c->stream);
+        // logits and divergence in as few parts of equal size as both contexts have room for
+        const int most = std::min(c->score_rows, teacher->score_rows), parts = (sh.rows + most - 1) / most;
+        const int step = std::min(most, ((sh.rows + parts - 1) / parts + 127) / 128 * 128);
+        for (int row0 = 0; row0 < sh.rows; row0 += step) {
+            const int rows = std::min(step, sh.rows - row0);
+            for (hbsjd_ctx* x : both) {
+                float* out = (float*)x->activations;
+                const int rc = x->bf16_model ? head<bf16>(x, row0, rows, out, x->score_rows)
+                                             : head<float>(x, row0, rows, out, x->score_rows);
+                if (rc) {
+                    if (x != c) snprintf(c->err, sizeof(c->err), "teacher head: %.200s", x->err);
+                    return rc;
+                }
+            }
+            // the divergence kernel reads both models' logits on the student's stream; the teacher's next logits or
+            // forward overwrite its own and wait for that kernel in turn
+            CK(cudaEventRecord(teacher->ev2, teacher->stream));
+            CK(cudaStreamWaitEvent(c->stream, teacher->ev2, 0));
+            // timed with the vocabulary-wide class: 2 V floats read per input
+            const int ps = prof_begin(c, HBSJD_PROF_ACCEPT, 8.0 * rows * V);
+            launch_bikl_inputs(c->st, row0, rows, (const float*)c->activations, (const float*)teacher->activations, prefix_len, pos,
+                               c->stream);
             prof_end(c, ps);
+            c->launches++;
+            CK(cudaEventRecord(c->ev2, c->stream));
+            CK(cudaStreamWaitEvent(teacher->stream, c->ev2, 0));
         }
-        c->launches++;
-        CK(cudaEventRecord(c->ev2, c->stream));
-        CK(cudaStreamWaitEvent(teacher->stream, c->ev2, 0));
         for (hbsjd_ctx* x : both) {
             launch_prefill_advance(x->st, span, x->stream);
             x->launches++;
@@ -1278,7 +1347,7 @@ int hbsjd_calibrate_gamma(hbsjd_ctx* c, int batch, int window, int guidance, int
                 launch_calib_state(st, live, c->stream);
                 launch_setup(st, 0, compact, c->stream);
                 CK(cudaEventRecord(c->ev0, c->stream));
-                const int rc = forward_any(c, S, true);
+                const int rc = forward_any(c, S, LOGITS);
                 if (rc) return rc;
                 CK(cudaEventRecord(c->ev1, c->stream));
                 const int rs = sync_counters(c);
@@ -1379,7 +1448,7 @@ int hbsjd_debug_forward(hbsjd_ctx* c, int layer, int stage) {
     c->st.R = c->st.B * c->st.W;
     c->st.multi = false;
     launch_setup(c->st, 0, 0, c->stream);
-    const int rc = forward_any(c, c->st.B, false, layer, stage);
+    const int rc = forward_any(c, c->st.B, KEYS_VALUES, layer, stage);
     if (rc) return rc;
     CK(cudaGetLastError());
     c->last_S = c->st.B;

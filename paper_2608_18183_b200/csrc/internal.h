@@ -160,8 +160,9 @@ void launch_noop(Stream& s);
 
 // ---- distillation score (score_kernels.cu)
 void launch_bikl_rows(const float* ls, const float* lt, int rows, int V, float* out, Stream& s);
-// terms of the inputs of one scoring forward (row table of st; logits rows of both models)
-void launch_bikl_inputs(const State& st, const float* ls, const float* lt, const int32_t* prefix_len, float* pos, Stream& s);
+// terms of the inputs in rows row0 .. row0 + rows - 1 of a scoring forward (row table of st; these rows' logits of both models)
+void launch_bikl_inputs(const State& st, int row0, int rows, const float* ls, const float* lt, const int32_t* prefix_len,
+                        float* pos, Stream& s);
 void launch_score_init(const State& st, const int32_t* tokens, const int32_t* labels, const int32_t* prefix_len,
                        float* pos, Stream& s);
 void launch_score_reduce(int B, int T, const int32_t* prefix_len, const float* pos, float* per_image, float* loss,

@@ -123,16 +123,16 @@ __global__ void __launch_bounds__(BK_THREADS) k_bikl_rows(const float* __restric
     if (threadIdx.x == 0) out[row] = d;
 }
 
-// One CTA per row of a scoring forward: an input at sequence index s, whose output is the distribution of
+// One CTA per row from row0 of a scoring forward on: an input at sequence index s, whose output is the distribution of
 // position t = s + 1; the term counts when t > k (Eq. 3 sums t = k+1 .. T).
-__global__ void __launch_bounds__(BK_THREADS) k_bikl_inputs(State st, const float* __restrict__ ls,
+__global__ void __launch_bounds__(BK_THREADS) k_bikl_inputs(State st, int row0, const float* __restrict__ ls,
                                                            const float* __restrict__ lt,
                                                            const int32_t* __restrict__ prefix_len,
                                                            float* __restrict__ pos) {
     pdl_wait();
     pdl_trigger();
     const size_t row = blockIdx.x;
-    const int2 at = st.row_pos[row];
+    const int2 at = st.row_pos[row0 + row];
     const int img = at.x, idx = at.y;
     if (img < 0 || idx < prefix_len[img]) return;
     const float d = bikl_row(ls + row * st.V, lt + row * st.V, st.V);
@@ -200,8 +200,9 @@ void launch_bikl_rows(const float* ls, const float* lt, int rows, int V, float* 
     launch_k(k_bikl_rows, dim3(rows), dim3(BK_THREADS), 0, s, ls, lt, V, out);
 }
 
-void launch_bikl_inputs(const State& st, const float* ls, const float* lt, const int32_t* prefix_len, float* pos, Stream& s) {
-    launch_k(k_bikl_inputs, dim3(st.R), dim3(BK_THREADS), 0, s, st, ls, lt, prefix_len, pos);
+void launch_bikl_inputs(const State& st, int row0, int rows, const float* ls, const float* lt, const int32_t* prefix_len,
+                        float* pos, Stream& s) {
+    launch_k(k_bikl_inputs, dim3(rows), dim3(BK_THREADS), 0, s, st, row0, ls, lt, prefix_len, pos);
 }
 
 void launch_score_init(const State& st, const int32_t* tokens, const int32_t* labels, const int32_t* prefix_len,

@@ -383,3 +383,61 @@ def test_a_batch_beyond_the_slot_tables_has_one_accept_kernel():
     for full, compact in zip(got[binding.EXEC_FULL], got[binding.EXEC_COMPACT]):
         np.testing.assert_array_equal(full, compact)
     ctx.hbsjd_destroy()
+
+
+def test_a_small_context_holds_no_logits_that_its_rounds_do_not_need():
+    """24 images token by token with a vocabulary of 16384: the rounds have 48 rows.  Pre-filling and scoring take up to 4096
+    rows per forward, whose logits alone would be 268 MB; scoring takes them in parts, with the bits of a context that has
+    room for more at a time."""
+    import torch
+    s = synth.ModelShape(2, 64, 1, 64, 16384, 16, 16, 3, "bf16")
+    t = synth.ModelShape(2, 128, 2, 128, 16384, 16, 16, 3, "bf16")
+    simg, timg = (synth.make_weights(x, 3 + i, target_entropy=None) for i, x in enumerate((s, t)))
+    rng = np.random.default_rng(24)
+    toks, k, lab = (G.dev(x.astype(np.int32)) for x in (rng.integers(0, s.vocab, (24, s.T)), rng.integers(0, s.T, 24),
+                                                        rng.integers(0, 3, 24)))
+    wide = binding.Context(s, simg, 24, 32), binding.Context(t, timg, 24, 32)
+    assert wide[0].fold_norm  # one form of RMSNorm throughout
+    want = wide[0].hbsjd_score(wide[1], toks, k, lab)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    narrow = [binding.Context(s, simg, 24, 1)]
+    used = free - torch.cuda.mem_get_info()[0]
+    # weights 4.5 MB, keys and values 6 MB, logits and probabilities 6 MB, activations 3 MB, allocation granules
+    assert used < 64e6, used
+    narrow.append(binding.Context(t, timg, 24, 1))
+    for _ in range(2):
+        got = narrow[0].hbsjd_score(narrow[1], toks, k, lab)
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1]) and got[2] == want[2]
+        out = [c.hbsjd_rollout(toks, k, lab, binding.make_params(1, 16, 2.0, 1.0, 50, seed=1))[0] for c in (wide[0], narrow[0])]
+        assert torch.equal(out[0], out[1])
+    for c in (*wide, *narrow):
+        c.hbsjd_destroy()
+
+
+def test_a_context_whose_larger_activations_do_not_fit_takes_the_smaller():
+    """Activations for forwards of 4096 rows are for speed only (75 MB here): with 40 MB less free than the context would take
+    it is created all the same, and its tokens are the same."""
+    import torch
+    s = synth.ModelShape(1, 1024, 16, 4096, 64, 48, 48, 3, "bf16")
+    img = synth.make_weights(s, 3, target_entropy=None)
+    toks = torch.randint(0, 64, (1, s.T), device="cuda", dtype=torch.int32)
+    k, lab = (torch.tensor([x], device="cuda", dtype=torch.int32) for x in (2250, 1))
+    p = binding.make_params(1, 48, 1.0, 1.0, 0, seed=1)
+    out = [torch.empty_like(toks) for _ in range(2)]
+    binding.Context(s, img, 1, 1).hbsjd_destroy()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    ctx = binding.Context(s, img, 1, 1)
+    ctx.hbsjd_rollout(toks, k, lab, p, out[0])
+    taken = before - torch.cuda.mem_get_info()[0]
+    ctx.hbsjd_destroy()
+    torch.cuda.synchronize()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - taken + 40 * 2 ** 20, dtype=torch.uint8, device="cuda")
+    ctx = binding.Context(s, img, 1, 1)
+    ctx.hbsjd_rollout(toks, k, lab, p, out[1])
+    assert torch.equal(out[0], out[1])
+    ctx.hbsjd_destroy()
+    del filler
+    torch.cuda.empty_cache()
