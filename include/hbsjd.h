@@ -87,8 +87,8 @@ typedef struct {
     int64_t rejects;           /* image-rounds that ended in a rejection */
     int64_t full_rounds;       /* rounds executed in Full form */
     int64_t compact_rounds;    /* rounds executed in Compact form */
-    int64_t prefill_forwards;  /* steps of `window` tokens that pre-filling the longest prefix takes (several steps share
-                                * one batched forward) */
+    int64_t prefill_forwards;  /* longest prefix / window, rounded up: the forwards of a pre-filling window by window.  NOT the
+                                * forwards that ran, which take many windows at a time: hbsjd_prefill_passes */
     int64_t kernel_launches;   /* kernels of this library launched by the call */
     float ms_total;            /* GPU time of the call (CUDA events on the context's stream) */
     float ms_prefill;          /* of which state init + prefix pre-filling */
@@ -129,6 +129,10 @@ int hbsjd_create(hbsjd_ctx **out, const hbsjd_model_desc *m, const void *weights
  * prefix token out of range, non-positive temperature; HBSJD_ECUDA; HBSJD_ETIMEOUT. */
 int hbsjd_rollout(hbsjd_ctx *c, int batch, const int32_t *prefix_tokens, const int32_t *prefix_len,
                   const int32_t *class_labels, const hbsjd_params *p, int32_t *out_tokens, hbsjd_stats *stats);
+
+/* *passes (HOST) = the batched forwards that pre-filled the prefixes of the last hbsjd_rollout of the context (0 before the
+ * first; of one that failed, those that were enqueued). */
+int hbsjd_prefill_passes(hbsjd_ctx *c, int64_t *passes);
 
 /* hbsjd_rollout for callers whose buffers live in HOST memory (pinned memory makes the copies
  * asynchronous): copies the three inputs to staging buffers of the context, runs the rollout, and copies

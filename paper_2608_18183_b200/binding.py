@@ -17,7 +17,7 @@ EXEC_FULL, EXEC_COMPACT, EXEC_HYBRID, EXEC_SYNC = 0, 1, 2, 3
 DBG_PROBS, DBG_LOGITS, DBG_SLOTS = 0, 1, 2
 DBG_ACT_A, DBG_ACT_Q, DBG_ACT_O, DBG_ACT_FFN, DBG_ACT_H, DBG_KV_K, DBG_KV_V = 3, 4, 5, 6, 7, 8, 9
 
-EXPORTS = ["hbsjd_create", "hbsjd_rollout", "hbsjd_rollout_host", "hbsjd_profile", "hbsjd_profile_read", "hbsjd_profile_launch_floor", "hbsjd_probs", "hbsjd_verify", "hbsjd_verify_static", "hbsjd_calibrate_gamma", "hbsjd_round", "hbsjd_tokens", "hbsjd_destroy", "hbsjd_get_state",
+EXPORTS = ["hbsjd_create", "hbsjd_rollout", "hbsjd_prefill_passes", "hbsjd_rollout_host", "hbsjd_profile", "hbsjd_profile_read", "hbsjd_profile_launch_floor", "hbsjd_probs", "hbsjd_verify", "hbsjd_verify_static", "hbsjd_calibrate_gamma", "hbsjd_round", "hbsjd_tokens", "hbsjd_destroy", "hbsjd_get_state",
            "hbsjd_set_state", "hbsjd_debug_read", "hbsjd_debug_forward", "hbsjd_debug_gemm",
            "hbsjd_debug_shuffle_pages", "hbsjd_debug_fold_norm", "hbsjd_debug_fail_round",
            "hbsjd_debug_force_tile", "hbsjd_gemm", "hbsjd_bikl", "hbsjd_score", "hbsjd_strerror",
@@ -88,6 +88,7 @@ def load():
         L.hbsjd_rollout.argtypes = [vp, C.c_int, vp, vp, vp, C.POINTER(hbsjd_params), vp, C.POINTER(hbsjd_stats)]
         L.hbsjd_rollout_host.argtypes = [vp, C.c_int, vp, vp, vp, C.POINTER(hbsjd_params), vp,
                                          C.POINTER(hbsjd_stats)]
+        L.hbsjd_prefill_passes.argtypes = [vp, C.POINTER(C.c_int64)]
         L.hbsjd_profile.argtypes = [vp, C.c_int]
         L.hbsjd_profile_read.argtypes = [vp, C.POINTER(hbsjd_kernel_profile)]
         L.hbsjd_profile_launch_floor.argtypes = [vp, C.c_int, C.POINTER(C.c_float)]
@@ -198,6 +199,12 @@ class Context:
         self._check(rc, "hbsjd_rollout_host")
         self.batch, self.window = B, params.window
         return out_tokens, st.as_dict()
+
+    def hbsjd_prefill_passes(self) -> int:
+        """Batched forwards that pre-filled the prefixes of the last rollout."""
+        n = C.c_int64(0)
+        self._check(self.lib.hbsjd_prefill_passes(self.h, C.byref(n)), "hbsjd_prefill_passes")
+        return n.value
 
     def hbsjd_profile(self, enable: bool):
         self._check(self.lib.hbsjd_profile(self.h, 1 if enable else 0), "hbsjd_profile")

@@ -75,6 +75,7 @@ struct hbsjd_ctx {
     int dbg_layer;  // layer of the last hbsjd_debug_forward (-1: none); selects the KV rows of hbsjd_debug_read
     hbsjd_stats stats;
     long long launches;
+    int64_t prefill_passes;  // forwards that pre-filled for the last rollout
     // host-buffer staging
     int32_t *stage_tok, *stage_len, *stage_lab, *stage_out;
     void* verify_scratch;
@@ -902,6 +903,7 @@ int hbsjd_create(hbsjd_ctx** out, const hbsjd_model_desc* m, const void* weights
     c->dbg_layer = -1;
     c->force_tile = 0;
     c->fail_round = -1;
+    c->prefill_passes = 0;
     c->err[0] = 0;
     const int rc = create_impl(c, weights, weight_bytes);
     if (rc != 0) {
@@ -992,6 +994,7 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
     // prefix pre-filling: cache sequence indices 0..k-1 in as few forwards as the activation rows allow (no LM head)
     const int k_max = *std::max_element(hk.begin(), hk.end());
     c->stats.prefill_forwards = (k_max + p->window - 1) / p->window;
+    c->prefill_passes = 0;
     for (int done = 0, span; done < k_max; done += span) {
         const PassShape sh = pass_shape(hk, done, k_max, c->rows_cap / st.nb);
         span = sh.span;
@@ -1001,6 +1004,7 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
         launch_setup(st, 1, 1, c->stream, span);
         const int rc = forward_any(c, sh.slots, KEYS_VALUES);
         if (rc) return rc;
+        c->prefill_passes++;
         launch_prefill_advance(st, span, c->stream);
         c->launches += 2;
         if (c->profiling) {  // fold this forward's event pairs while its byte counters are current
@@ -1032,6 +1036,12 @@ int hbsjd_rollout(hbsjd_ctx* c, int batch, const int32_t* prefix_tokens, const i
     CK(cudaEventElapsedTime(&c->stats.ms_total, c->ev0, c->ev2));
     c->stats.kernel_launches = c->launches;
     if (stats) *stats = c->stats;
+    return HBSJD_OK;
+}
+
+int hbsjd_prefill_passes(hbsjd_ctx* c, int64_t* passes) {
+    if (!c || !passes) return HBSJD_EINVAL;
+    *passes = c->prefill_passes;
     return HBSJD_OK;
 }
 

@@ -441,3 +441,20 @@ def test_a_context_whose_larger_activations_do_not_fit_takes_the_smaller():
     ctx.hbsjd_destroy()
     del filler
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("batch,k_max,passes", [(4, 0, 0), (4, 1, 1), (4, 128, 1), (40, 128, 3)])
+def test_prefill_passes_are_the_forwards_that_ran(batch, k_max, passes):
+    """Window 1, prefixes of up to 128 tokens: 128 steps of a window, but one forward while the inputs of both branches fit
+    4096 rows (of 40 images 51 each do, in slots of 48: 48, 48 and 32 tokens).  A pass runs attention in every layer but the last: counted by the profile."""
+    w = synth.with_shape(synth.WORKLOADS["small_bf16"], batch=batch, window=1, cfg_scale=3.0)
+    toks, _, lab = synth.make_inputs(w, seed=3, batch=batch)
+    k = np.full(batch, k_max, dtype=np.int32)
+    k[0] //= 2
+    ctx = _ctx(w)
+    assert ctx.hbsjd_prefill_passes() == 0
+    ctx.hbsjd_profile(True)
+    _, st = ctx.hbsjd_rollout(G.dev(toks), G.dev(k), G.dev(lab), G.gpu_params(w, 1, max_rounds=0))
+    assert ctx.hbsjd_profile_read()["attention"]["launches"] == passes * (w.shape.n_layers - 1)
+    assert ctx.hbsjd_prefill_passes() == passes and st["prefill_forwards"] == k_max
+    ctx.hbsjd_destroy()
