@@ -210,7 +210,7 @@ int hbsjd_debug_forward(hbsjd_ctx *c, int layer, int stage);
  * like any other kernel argument behind earlier work of the stream. */
 int hbsjd_gemm(hbsjd_ctx *c, const void *A, const void *W, float *C, int M, int N, int K, int accumulate);
 
-/* accumulate = 2 (bf16 contexts, N = dim, M within the context's activation rows): the residual-update form the
+/* accumulate = 2 (bf16 contexts, N = dim, M <= 2 max_batch max_window): the residual-update form the
  * forward itself uses, C += A W^T together with the bf16 copy and the per-row partial sums of squares of the new C
  * (written to buffers of the context), so that it can be timed and checked alone.
  * hbsjd_gemm `reps` times back to back before the one synchronisation (micro-benchmarks time the decoder's GEMM
@@ -220,7 +220,7 @@ int hbsjd_gemm(hbsjd_ctx *c, const void *A, const void *W, float *C, int M, int 
  * then means the former).  A limit shorter than the main loop makes a healthy pipeline take the
  * time-out path: every role leaves its loop, copies and MMAs in flight are drained, TMEM is freed, the call
  * returns HBSJD_ETIMEOUT with C partly written, and the context stays usable.  Tests use it to exercise that path.
- * tile (bf16 contexts, accumulate 0 or 1): 0 = the library's own choice for the shape; 32, 64, 96, 128, 160, 192, 256 = one
+ * tile (bf16 contexts): 0 = the library's own choice for the shape; 32, 64, 96, 128, 160, 192, 256 = one
  * CTA per 128 x tile block of C; 512 / 640 = 256 x 256 / 256 x 128 blocks on CTA pairs (N a multiple of 256 / 128);
  * 16032, 16064, 32032, 32064 = the kernel for few rows, 16 x 32 .. 32 x 64 blocks of C.  Every choice gives the
  * same bits (each element's products are summed in the same order); HBSJD_EINVAL for any other value. */
@@ -242,7 +242,7 @@ int hbsjd_debug_fold_norm(hbsjd_ctx *c, int on);
  * before the first rollout of the context; HBSJD_ESTATE afterwards. */
 int hbsjd_debug_shuffle_pages(hbsjd_ctx *c, uint64_t seed);
 
-/* The tile (see hbsjd_debug_gemm: 0, 64, 96, 160, 192 or one of the kernel for few rows) of every decoder GEMM of a bf16 context's
+/* The tile (see hbsjd_debug_gemm: 0, 64, 96, 160, 192, 512 or one of the kernel for few rows) of every decoder GEMM of a bf16 context's
  * forwards, so that tests can compare the two kernels in each fused epilogue (Sec. 4.2 verifier forward).  Every choice
  * gives the same bits. */
 int hbsjd_debug_force_tile(hbsjd_ctx *c, int tile);

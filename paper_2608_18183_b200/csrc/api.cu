@@ -1550,7 +1550,7 @@ int hbsjd_debug_gemm(hbsjd_ctx* c, const void* A, const void* W, float* C, int M
     if (!c || !A || !W || !C || M < 1 || N < 1 || K < 1 || reps < 1) return HBSJD_EINVAL;
     if (accumulate == 2 && (!c->bf16_model || N != c->d.dim || M > 2 * c->Bmax * c->Wmax)) {
         snprintf(c->err, sizeof(c->err), "hbsjd_debug_gemm: the residual-update form needs a bf16 context, N = dim and "
-                                         "M within the context's activation rows");
+                                         "at most 2 x max_batch x max_window rows");
         return HBSJD_EINVAL;
     }
     for (int r = 0; r < reps; ++r) {
@@ -1560,7 +1560,7 @@ int hbsjd_debug_gemm(hbsjd_ctx* c, const void* A, const void* W, float* C, int M
             // sums of squares of the new rows (into the context's own buffers)
             c->launches++;
             rc = gemm_tcgen05_addnorm((const bf16*)A, (const bf16*)W, C, (bf16*)c->a, c->ssq, M, N, K, 0,
-                                      c->st.counters + CNT_ERROR, c->stream, c->err, sizeof(c->err));
+                                      c->st.counters + CNT_ERROR, c->stream, c->err, sizeof(c->err), tile);
             if (rc) rc = rc == -1 ? HBSJD_EINVAL : HBSJD_ECUDA;
         } else {
             // W is the caller's buffer, possibly written by earlier work of the stream: no early fetch of its tiles
@@ -1586,10 +1586,10 @@ int hbsjd_debug_fold_norm(hbsjd_ctx* c, int on) {
 
 int hbsjd_debug_force_tile(hbsjd_ctx* c, int tile) {
     if (!c) return HBSJD_EINVAL;
-    const int tiles[] = {0, 64, 96, 160, 192, 16032, 16064, 32032, 32064};
+    const int tiles[] = {0, 64, 96, 160, 192, 512, 16032, 16064, 32032, 32064};
     if (!c->bf16_model || std::find(std::begin(tiles), std::end(tiles), tile) == std::end(tiles)) {
-        snprintf(c->err, sizeof(c->err), "hbsjd_debug_force_tile: needs a bf16 context and a tile of 0, 64, 96, 160, 192, 16032, "
-                                         "16064, 32032 or 32064");
+        snprintf(c->err, sizeof(c->err), "hbsjd_debug_force_tile: needs a bf16 context and a tile of 0, 64, 96, 160, 192, 512, "
+                                         "16032, 16064, 32032 or 32064");
         return HBSJD_EINVAL;
     }
     c->force_tile = tile;

@@ -283,3 +283,38 @@ def test_every_epilogue_of_the_tiles_in_between(fold):
         assert all(np.isfinite(x).all() for x in got)
         for i, x in enumerate(got):
             np.testing.assert_array_equal(x.view(np.uint32), seen.setdefault(i, x).view(np.uint32), err_msg=f"{tile} {i}")
+
+
+@pytest.mark.parametrize("fold", [True, False])
+def test_every_epilogue_of_cta_pairs_with_a_last_wave_in_halves(fold):
+    """64 images x 32 inputs x 2 branches, 4096 rows: the tiles of every product are 80, 160 or 240 on 74 CTA pairs, so that a
+    rest of 6, 12 or 18 goes as halves of 128 columns.  Queries, keys, values, the updated residual with its bf16 copy, the
+    FFN's product and the logits (through the copy and the sums of squares of the folded norm) have the 128 x 64 tile's bits."""
+    s = synth.ModelShape(2, 1280, 20, 1280, 2560, 12, 12, 10, "bf16")
+    img = synth.make_weights(s, 5, target_entropy=None)
+    rng = np.random.default_rng(64)
+    toks = rng.integers(0, s.vocab, (64, s.T)).astype(np.int32)
+    ks = rng.integers(0, s.T, 64).astype(np.int32)
+    ks[:4] = [0, 64, s.T - 32, s.T - 1]
+    lab = rng.integers(0, s.n_classes, 64).astype(np.int32)
+    what = {0: (binding.DBG_ACT_Q, binding.DBG_KV_K, binding.DBG_KV_V, binding.DBG_ACT_O, binding.DBG_ACT_H, binding.DBG_ACT_A),
+            1: (binding.DBG_ACT_FFN, binding.DBG_ACT_H, binding.DBG_ACT_A)}
+    rows = [2 * b + br for b in (0, 1, 2, 3, 31, 33, 63) for br in (0, 1)]
+    seen = {}
+    for tile in (64, 512):
+        ctx = binding.Context(s, img, 64, 32)
+        ctx.hbsjd_debug_fold_norm(fold)
+        ctx.hbsjd_debug_force_tile(tile)
+        ctx.hbsjd_rollout(G.dev(toks), G.dev(ks), G.dev(lab), binding.make_params(
+            32, 12, 3.0, max_rounds=0, seed=2, exec_mode=binding.EXEC_FULL))
+        got = []
+        for layer in (0, 1):
+            for stage in (0, 1):
+                ctx.hbsjd_debug_forward(layer, stage)
+                got += [ctx.hbsjd_debug_read(x, i) for x in what[stage] for i in rows]
+        ctx.hbsjd_round()
+        got += [ctx.hbsjd_debug_read(binding.DBG_LOGITS, i) for i in rows]
+        ctx.hbsjd_destroy()
+        assert all(np.isfinite(x).all() for x in got)
+        for i, x in enumerate(got):
+            np.testing.assert_array_equal(x.view(np.uint32), seen.setdefault(i, x).view(np.uint32), err_msg=f"{tile} {i}")

@@ -270,8 +270,10 @@ def test_last_wave_of_cta_pairs_in_halves(ctx_bf16, M):
 
 @pytest.mark.parametrize("M", [300, 2049, 4096])
 def test_residual_update_with_norm_sums_on_every_kernel(M):
-    """The folded residual update (its bf16 copy and sums of squares come with it) at 1280 columns: one CTA per tile, and CTA
-    pairs whose last wave goes as halves (4096 rows: 80 tiles).  The sum is the plain update's."""
+    """The folded residual update (its bf16 copy and sums of squares come with it) at 1280 columns: tiles of every width that
+    one CTA takes, the few-row kernel, and CTA pairs, whose last wave goes as halves at 4096 rows (80 tiles on 74 pairs)
+    and whole at 2049 (45 tiles).  The sum is the plain update's; copy and sums of squares are compared through whole
+    forwards, in test_every_epilogue_of_cta_pairs_with_a_last_wave_in_halves."""
     import torch
     s = synth.ModelShape(1, 1280, 20, 64, 64, 4, 4, 3, "bf16")
     ctx = binding.Context(s, synth.make_weights(s, 3, target_entropy=None), 64, 32)
@@ -279,8 +281,10 @@ def test_residual_update_with_norm_sums_on_every_kernel(M):
     A = torch.randn(M, 320, generator=g, device="cuda").bfloat16()
     W = torch.randn(1280, 320, generator=g, device="cuda").bfloat16()
     C0 = torch.randn(M, 1280, generator=g, device="cuda")
-    want, got = C0.clone(), C0.clone()
+    want = C0.clone()
     ctx.hbsjd_debug_gemm(A, W, want, accumulate=1, tile=64)
-    ctx.hbsjd_debug_gemm(A, W, got, accumulate=2)
-    assert torch.equal(got, want)
+    for tile in (0, 32, 64, 128, 160, 256, 512, 640, 16032, 32064):
+        got = C0.clone()
+        ctx.hbsjd_debug_gemm(A, W, got, accumulate=2, tile=tile)
+        assert torch.equal(got, want), tile
     ctx.hbsjd_destroy()
