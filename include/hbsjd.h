@@ -230,7 +230,7 @@ int hbsjd_debug_gemm(hbsjd_ctx *c, const void *A, const void *W, float *C, int M
 /* Chooses the form of RMSNorm of a bf16 context (Sec. 4.2 verifier forward; the paper does not go below the model):
  * on = 1 folds it into the GEMM epilogues (bf16 copy of the unnormalised residual stream as the operand, gain in the
  * weights, row factor in the next epilogue), on = 0 runs it as a kernel of its own in front of the projections.
- * hbsjd_create picks the folded form for contexts of at most 2048 activation rows (2 x max_batch x max_window) and the
+ * hbsjd_create picks the folded form for contexts whose largest round has at most 2048 rows (2 x max_batch x max_window) and the
  * separate one above; this call lets tests run either form at any size.  The two forms round the GEMM operand at
  * different points (x r g against x), so their results differ at bf16-noise level; one context always uses one form,
  * so Full and Compact execution stay bit-identical.  Only before the first rollout, and only for models whose norm
@@ -318,7 +318,7 @@ int hbsjd_bikl(hbsjd_ctx *c, const float *logits_s, const float *logits_t, int r
  * tokens and class label (no guidance, temperature 1, no top-k), then the mean over the images of the batch that
  * generated anything (k_b < T).  This is the step that follows the rollout in the on-policy distillation loop.
  *   student, teacher  two contexts with the same grid (T) and vocabulary; batch <= max_batch of both.  Both
- *                     models run full-sequence causal forwards, in as few parts as their activation rows allow,
+ *                     models run full-sequence causal forwards, of as many tokens as their activation rows allow,
  *                     through the same kernels as the rollout; their rollout state and KV caches are
  *                     overwritten (a stepped rollout cannot be continued afterwards).
  *   tokens        DEVICE int32 [batch, T]   completed trajectories (e.g. hbsjd_rollout's out_tokens)

@@ -283,7 +283,7 @@ int forward<float>(hbsjd_ctx* c, int S, Until until, int stop_layer, int stop_st
 
 // bf16 model: four tensor-core GEMMs and one attention kernel per layer; RoPE + the paged KV write, SwiGLU and the
 // residual add ride in the GEMM epilogues.  RMSNorm comes in two forms, fixed per context at creation:
-//   folded (contexts of at most 2048 activation rows, which are bound by the number of launches): no kernel of its
+//   folded (contexts with rounds of at most 2048 rows, which are bound by the number of launches): no kernel of its
 //     own -- the kernels that write the residual stream (embedding gather, attention-out and FFN-down projections)
 //     also leave its bf16 copy and per-row partial sums of squares, the norm's gain is folded into the following
 //     weight matrix at load, and the following GEMM's epilogue applies the row factor rsqrt(mean(x^2) + eps);

@@ -372,12 +372,13 @@ cudaError_t launch_epi(int epi, const CUtensorMap& ma, const CUtensorMap& mw, co
 bool skinny_tile_exists(int code) { return code == 16032 || code == 16064 || code == 32032 || code == 32064; }
 
 // The narrowest tile whose CTAs are all resident at once (two per SM): with more CTAs the second round costs more
-// than the tcgen05 kernel's longer chain (M = 64, N 5632: 9.2 against 6.7 us; M = 128, N 3072: 8.5 against 6.3 us),
-// with fewer the chain is what is left (N 1024: K 2816 at M = 64, 128, 208, 288: 7.0, 8.3, 9.9, 9.9 against 11.5 to 11.8 us, K
-// 1024 at M = 288, the last that fits: 5.3 against 6.5; N 768 up to M = 384: 5.0 against 5.7; N 1280 up to M = 224: 6.2 against
-// 7.3).  The LM head has so many columns that only the widest tile gets close, up to 32 rows (M = 32, N 16384: 8.9
-// against 11.6 us).  Three row tiles of 16 x 64 fit where two of 32 x 32 do not (M = 48, N 5632, 264 CTAs: 5.9 against the
-// tcgen05 kernel's 6.7 us; rollouts of 24 images by window 1 in 0.96 times the time).
+// than the tcgen05 kernel's longer chain (back to back, best tile of each kernel: M = 64, N 5632: 8.6 against 7.8 us; M = 128,
+// N 3072: 9.1 against 7.5), with fewer the chain is what is left (N 1024: K 2816 at M = 64, 128, 208, 288: 7.3, 8.9, 10.5, 10.5
+// against 12.7 to 13.1 us, K 1024 at M = 288, the last that fits: 6.3 against 7.5; N 768 up to M = 384: 6.0 against 6.8; N 1280 up
+// to M = 224: 7.1 against 8.1).  The LM head has so many columns that only the widest tile gets close, up to 32 rows
+// (M = 32, N 16384: 8.7 against 12.2 us).  Three row tiles of 16 x 64 fit where two of 32 x 32 do not (M = 48, N 5632, 264
+// CTAs: 6.6 against 8.7 us).  Of the B, L and XL decoders' products of 16 to 512 rows the rule takes 96, at 0.73 times the
+// best tcgen05 tile's time on average and 0.90 at most, and leaves 114, where this kernel takes at least 1.07 times.
 int skinny_tile_code(int M, int N, int sms) {
     const long m16 = (M + 15) / 16, m32 = (M + 31) / 32, most = 2L * sms;
     if (N % 64 != 0) return 0;

@@ -796,7 +796,9 @@ cudaError_t launch_bn(int bn, const CUtensorMap& ma, const CUtensorMap& mw, cons
         case 160: return launch<160, EPI>(ma, mw, mc, mh, g, s);
         case 192: return launch<192, EPI>(ma, mw, mc, mh, g, s);
         case 512: return launch_pair<256, EPI>(ma, mw, mw_half, mc, mh, g, s);  // 256 x 256 on a CTA pair
-        case 640: return launch_pair<128, EPI>(ma, mw, mw_half, mc, mh, g, s);  // 256 x 128 on a CTA pair
+        // 256 x 128 on a CTA pair: never chosen (1.04 to 2.1 times the best tile's time over 300 products); hbsjd_debug_gemm
+        // takes it, so that what finer pair tiles cost can be measured
+        case 640: return launch_pair<128, EPI>(ma, mw, mw_half, mc, mh, g, s);
         default: return launch<256, EPI>(ma, mw, mc, mh, g, s);
     }
 }
@@ -810,9 +812,12 @@ bool tile_exists(int code) {
 // Tile of a product by a small cost model, fitted to 939 measured launches (back to back, 128 to 6000 rows of the B, L and XL
 // decoders' products, every tile; 3 to 5 % rms): a launch costs its boundary, and every wave of tiles over the SMs an
 // epilogue and its k-blocks.  The time of a k-block is shared memory's and the MMA pipe's, in that order up to 128 columns.
-// Against the best tile of each of 240 products the choice costs 0.1 %, 2.5 % at most (widths that are powers of two and CTA pairs from
-// 45 tiles on: 0.7 %; the worst were 1.25, XL's down projection at 2048 rows 27.4 -> 21.9 us with 160 columns, and 1.33, the
-// heads at 128 rows 12.4 -> 9.3 us with 128).
+// Measured again against the best tile of each of 263 products (the decoders' from 128 to 8192 rows that the kernel for few
+// rows leaves) the choice costs 0.04 %, 3.5 % at most (widths that are powers of two and CTA pairs from 45 tiles on: 0.7 %; the
+// worst were 1.25, XL's down projection at 2048 rows 27.4 -> 21.9 us with 160 columns, and 1.33, the heads at 128 rows
+// 12.4 -> 9.3 us with 128).  Below 128 rows it is not fitted: XL's gate/up at 48 rows, 11.6 us with 64 columns, 9.4 with 96.
+// The table has the plain epilogues (store, add).  The folded residual update takes 6 to 9 us longer at 8192 rows; contexts
+// that fold have rounds of at most 2048 rows, and forwards of 4096 when they pre-fill or score.
 int choose_tile(int M, int N, int K) {
     struct Cost {
         int tile;

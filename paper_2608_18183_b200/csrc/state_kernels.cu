@@ -618,10 +618,13 @@ int accept_smem_bytes(int V) { return V * (int)sizeof(float) + (int)sizeof(AccSh
 
 void launch_probs(const float* lc, const float* lu, int rows, int V, float cfg_scale, float temperature, int top_k,
                   float* p, int32_t* counters, Stream& s) {
-    // The persistent kernel has one CTA of 1024 threads per SM, this file's k_probs two of 512: up to 4096 entries a row
-    // leaves the wide CTA a group of four per thread and its latency counts (4096 rows of 4096: 67 us against 75);
-    // above, its prefetched rows win (2048 rows of 8192 with guidance 62 -> 56 us, 1024 rows of 16384 56 -> 42 us
-    // plain and 85 -> 72 us with every option, 3 rows of 16384 26 -> 20 us).
+    // The persistent kernel has one CTA of 1024 threads per SM, this file's k_probs two of 512.  Above 4096 entries its
+    // prefetched rows win (k_probs -> persistent; 2048 rows of 8192 53 -> 46 us plain, 100 -> 81 with every option, 1024 rows of
+    // 16384 46 -> 41 and 85 -> 69, 3 rows of 16384 19.8 -> 19.6 and 27.0 -> 24.4).  At 4096 they win too since an item
+    // takes fewer instructions (4096 rows 67 -> 56 us plain, 133 -> 109 with every option; 3 rows 18.0 -> 17.6 and 21.4 -> 20.4),
+    // at 2048 by less (4096 rows 56 -> 50, 111 -> 111), at 1024 they win plain (53 -> 47) and lose with every option
+    // (103 -> 111): the line has not been moved below 4096, which would change those rows' last bits (the kernels add in
+    // different orders).
     if (V > 4096 && V <= 16384) {
         launch_probs_persistent(lc, lu, rows, V, cfg_scale, temperature, top_k, p, counters, device_sm_count(), s);
         return;
